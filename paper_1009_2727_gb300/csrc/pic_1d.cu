@@ -10,9 +10,8 @@
 //    current-sheet antenna, the lab-frame moving window.
 // Layout: node k of every component at index k (arrays padded to 32 values);
 // Ex, Ey, Bz, Jx, Jy at k, Ez, Bx, By, Jz at k + 1/2. Weights per unit area.
-// One thread per node for the fields; one thread per particle for the push,
-// whose deposit adds to the current with global atomics (1D grids are small:
-// the step is launch-bound, not bandwidth-bound).
+// A step is two launches: k1_fields (everything between two pushes, tile by tile in shared memory) and k1_push
+// (electrons, ions, antenna). 1D grids are small: the step is bound by launches and latency, not by bandwidth.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -73,123 +72,174 @@ struct Taps1 {
 };
 
 // ---------------------------------------------------------------------------
-// fields
-// moving window: every field array moves down by sh cells, keeping each component on its valid range
-template <class T>
-__global__ void k1_shift(G1 g, T* const* arr, const int* comp, int sh) {
-  const int a = blockIdx.y;
-  T* F = arr[a];
-  const int c = comp[a];
-  int lo, hi;
-  vr1(c, g.nz, lo, hi);
-  // in-place downward copy by one block per array, chunk by chunk from the bottom: a node reads a higher
-  // index than it writes, and every read of a chunk precedes its writes (1D grids are small)
-  for (int k0 = 0; k0 <= g.nz; k0 += blockDim.x) {
-    const int k = k0 + threadIdx.x;
-    T v = T(0);
-    if (k <= g.nz) {
-      const int kk = k + sh;
-      v = kk <= g.nz ? F[kk] : T(0);
-    }
-    __syncthreads();
-    if (k <= g.nz) F[k] = (k >= lo && k <= hi) ? v : T(0);
-    __syncthreads();
-  }
-}
+// fields: one launch per step
+//
+// The step's order is Faraday, push, Ampère; between two pushes the fields need Ampère of one step, the moving
+// window's shift, and Faraday, the Friedman history and the gather copies of the next. k1_fields does all of that for
+// a tile of NT1 nodes in shared memory, recomputing what the tile's halo needs (the filters' reach), so that no
+// grid-wide wait stands between the parts: it reads one set of the fields and writes the other. A step is then this
+// kernel and k1_push. On these grids (a few hundred to a few thousand nodes) a launch costs more than its arithmetic:
+// with one launch per part the fields of a step at 952 nodes (FP32, one pass on J) took 20 us of 52 us; this kernel
+// takes 6.0 us, the step 12.7 us. It is bound by latency (load, four to six barriers), not by bytes.
+constexpr int NT1 = 64;                              // nodes of a tile
+constexpr int W1MAX = NT1 + 2 * FILTER_HMAX + 5;     // staged nodes: the gather filter's reach and one more each side
+constexpr int JW1MAX = W1MAX + 2 * FILTER_HMAX;      // staged current: the current filter's reach on top
+constexpr int FB1 = 384;                             // one thread per gather copy of the tile
 
-// Faraday with E_eff = c1 E - c2 E^{n-1} + c3 E-bar and the PML: Bx(k+1/2) += dt dEy/dz,
-// By(k+1/2) -= dt dEx/dz; Bavg = (B^{n-1/2} + B^{n+1/2}) / 2 for the gather
+// E, E^{n-1}, E-bar and B (three components of n1p nodes each)
 template <class T>
-__global__ void k1_faraday(G1 g, Pml1<T> pm, const T* E, const T* Ep, const T* Eb, T* B, T* Bavg, T c1, T c2, T c3,
-                           T dtT, T idz) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > g.nz) return;
-  const int n = g.n1p;
-  for (int q = 0; q < 3; q++) {
-    const T old = B[q * n + k];
-    T nw = old;
-    if (q < 2 && k <= g.nz - 1) {
-      const int ce = q == 0 ? 1 : 0;
-      const T sgn = q == 0 ? T(1) : T(-1);
-      const T e1 = c1 * E[ce * n + k + 1] - c2 * Ep[ce * n + k + 1] + c3 * Eb[ce * n + k + 1];
-      const T e0 = c1 * E[ce * n + k] - c2 * Ep[ce * n + k] + c3 * Eb[ce * n + k];
-      const T d = sgn * (e1 - e0) * idz;
-      const T sg = pm.sgH[k];
-      nw = sg > T(0) ? pm.xiH[k] * old + pm.cfH[k] * d : old + dtT * d;
-      B[q * n + k] = nw;
-    }
-    Bavg[q * n + k] = T(0.5) * (old + nw);
-  }
-}
-
-// Friedman history (PR-1): E-bar <- (1 - theta/2) E + (theta/2) E-bar, E^{n-1} <- E
-template <class T>
-__global__ void k1_friedman(int n, const T* E, T* Ep, T* Eb, T a, T b) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const T e = E[p];
-  Eb[p] = a * e + b * Eb[p];
-  Ep[p] = e;
-}
-
-// composed filter along z on up to six components (blockIdx.y): dst = sum_m c_m src(k + (m - P) s), zero
-// off the component's valid range and off the grid
-template <class T>
-struct FiltJob1 {
-  const T* src[6];
-  T* dst[6];
-  int comp[6];
+struct Set1 {
+  T *E, *Ep, *Eb, *B;
 };
 
 template <class T>
-__global__ void k1_filter(G1 g, FiltJob1<T> jb, Taps1<T> t) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > g.nz) return;
-  const int a = blockIdx.y;
-  const T* F = jb.src[a];
-  int lo, hi;
-  vr1(jb.comp[a], g.nz, lo, hi);
-  T acc = T(0);
-  if (k >= lo && k <= hi) {
-    for (int m = 0; m <= 2 * t.P; m++) {
-      const int o = k + (m - t.P) * t.s;
-      if (o >= 0 && o <= g.nz) acc += t.c[m] * F[o];
+struct Fields1 {
+  Set1<T> in, out;
+  const T* J;      // the current deposited in the step that Ampère completes
+  T* Jz;           // the next step's current, set to zero
+  T *fE, *fB;      // gather copies
+  T c1, c2, c3;    // E_eff = c1 E - c2 E^{n-1} + c3 E-bar
+  T ha, hb;        // E-bar <- ha E + hb E-bar
+  T dt, idz, c2idz, ie0;
+  int ampere, faraday;             // the parts to run
+  int filt_j, filt_g, nodal;       // current filter, gather filter, node-interpolated gather copies
+  int shift, H;                    // window shift (cells) between the parts; reach of a filter that is on
+};
+
+template <class T>
+__global__ void __launch_bounds__(FB1) k1_fields(G1 g, Pml1<T> pm, Taps1<T> t, Fields1<T> a) {
+  __shared__ T sJ[3][JW1MAX];
+  __shared__ T sE[3][W1MAX], sEp[3][W1MAX], sEb[3][W1MAX], sB[3][W1MAX], sV[3][W1MAX];
+  __shared__ T sP[9][W1MAX];   // PML tables: sigma, xi, coefficient at integer and half nodes (Ampère), half nodes (Faraday)
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int n = g.n1p, nz = g.nz, H = a.H, sh = a.shift;
+  const int t0 = blockIdx.x * NT1;
+  const int W = NT1 + 2 * H + 5, JW = W + 2 * H;
+  // staged node i is node p0 + i before the shift and p0 + i - sh after it; staged current j is node p0 - H + j
+  const int p0 = t0 - H - 3 + sh;
+  if (a.ampere) {
+    for (int e = threadIdx.x; e < 3 * JW; e += FB1) {
+      const int q = e / JW, i = e - q * JW, k = p0 - H + i;
+      sJ[q][i] = (k >= 0 && k <= nz) ? a.J[q * n + k] : T(0);
     }
   }
-  jb.dst[a][k] = acc;
-}
-
-// 'momentum conserving' gather (Sec. 5): node values of the six gather copies, the mean of the two
-// nearest values of a half-staggered component (Ez, Bx, By); values off the grid count as zero
-template <class T>
-__global__ void k1_nodal(G1 g, const T* fE, const T* fB, T* dst) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > g.nz) return;
-  const int n = g.n1p;
-  for (int c = 0; c < 6; c++) {
-    const T* F = c < 3 ? fE + c * n : fB + (c - 3) * n;
-    dst[c * n + k] = half1(c) ? T(0.5) * ((k >= 1 ? F[k - 1] : T(0)) + F[k]) : F[k];
+  for (int e = threadIdx.x; e < 3 * W; e += FB1) {
+    const int q = e / W, i = e - q * W, k = p0 + i;
+    const bool in = k >= 0 && k <= nz;
+    sE[q][i] = in ? a.in.E[q * n + k] : T(0);
+    sB[q][i] = in ? a.in.B[q * n + k] : T(0);
+    sEp[q][i] = in ? a.in.Ep[q * n + k] : T(0);
+    sEb[q][i] = in ? a.in.Eb[q * n + k] : T(0);
   }
-}
-
-// Ampère with the PML: Ex(k) += dt (-c^2 dBy/dz - Jx/eps0), Ey(k) += dt (c^2 dBx/dz - Jy/eps0),
-// Ez(k+1/2) += -dt Jz/eps0; no current in the PML, where the curl term is damped
-template <class T>
-__global__ void k1_ampere(G1 g, Pml1<T> pm, T* E, const T* B, const T* J, T dtT, T c2idz, T ie0) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > g.nz) return;
-  const int n = g.n1p;
-  for (int q = 0; q < 3; q++) {
+  for (int e = threadIdx.x; e < 9 * W; e += FB1) {
+    const int q = e / W, i = e - q * W, k = p0 + i - (q >= 6 ? sh : 0);
+    const T* tab = q == 0 ? pm.sgI : q == 1 ? pm.xiI : q == 2 ? pm.cfI : q % 3 == 0 ? pm.sgH : q % 3 == 1 ? pm.xiH : pm.cfH;
+    if (k >= 0 && k <= nz) sP[q][i] = tab[k];
+  }
+  __syncthreads();
+  if (a.ampere) {
+    // Ampère with the PML: Ex(k) += dt (-c^2 dBy/dz - Jx/eps0), Ey(k) += dt (c^2 dBx/dz - Jy/eps0),
+    // Ez(k+1/2) += -dt Jz/eps0; no current in the PML, where the curl term is damped. Every node reads its own E and
+    // the unchanged B only, so E is updated in place.
+    for (int e = threadIdx.x; e < 3 * W; e += FB1) {
+      const int q = e / W, i = e - q * W, k = p0 + i;
+      int lo, hi;
+      vr1(q, nz, lo, hi);
+      if (k < lo || k > hi || i < 1) continue;
+      T d = T(0);
+      if (q == 0) d = -a.c2idz * (sB[1][i] - sB[1][i - 1]);
+      if (q == 1) d = a.c2idz * (sB[0][i] - sB[0][i - 1]);
+      const int pt = q == 2 ? 3 : 0;
+      const T old = sE[q][i];
+      if (sP[pt][i] > T(0)) {
+        sE[q][i] = sP[pt + 1][i] * old + sP[pt + 2][i] * d;
+      } else {
+        T j;
+        if (a.filt_j) {
+          j = T(0);
+          const T* c = sJ[q] + i + H - t.P * t.s;   // staged values off the grid are zero
+          for (int m = 0; m <= 2 * t.P; m++) j += t.c[m] * c[m * t.s];
+        } else {
+          j = sJ[q][i + H];
+        }
+        sE[q][i] = old + a.dt * (d - j * a.ie0);
+      }
+    }
+    __syncthreads();
+  }
+  if (sh > 0) {
+    // the window's shift: node k of every array takes the value of node k + sh, on the component's valid range
+    for (int e = threadIdx.x; e < 3 * W; e += FB1) {
+      const int q = e / W, i = e - q * W, k = p0 + i - sh;
+      int lo, hi;
+      vr1(q, nz, lo, hi);
+      if (k < lo || k > hi) { sE[q][i] = T(0); sEp[q][i] = T(0); sEb[q][i] = T(0); }
+      vr1(3 + q, nz, lo, hi);
+      if (k < lo || k > hi) sB[q][i] = T(0);
+    }
+    __syncthreads();
+  }
+  const int k0 = p0 - sh;   // node of staged index 0 from here on
+  if (!a.faraday) {
+    for (int e = threadIdx.x; e < 3 * NT1; e += FB1) {
+      const int q = e / NT1, i = e - q * NT1 + t0 - k0, k = k0 + i;
+      if (k > nz) continue;
+      a.out.E[q * n + k] = sE[q][i];
+      a.out.Ep[q * n + k] = sEp[q][i];
+      a.out.Eb[q * n + k] = sEb[q][i];
+      a.out.B[q * n + k] = sB[q][i];
+      a.Jz[q * n + k] = T(0);
+    }
+    return;
+  }
+  // Faraday with E_eff and the PML: Bx(k+1/2) += dt dEy/dz, By(k+1/2) -= dt dEx/dz, and the average of the old and
+  // the new B for the gather, on the tile and the filter's reach (staged indices 1 .. W - 2); the tile's own nodes
+  // are written with the Friedman history E-bar <- ha E + hb E-bar, E^{n-1} <- E
+  for (int e = threadIdx.x; e < 3 * W; e += FB1) {
+    const int q = e / W, i = e - q * W, k = k0 + i;
+    const bool in = k >= 0 && k <= nz;
+    const T old = sB[q][i];
+    T nw = old;
+    if (in && q < 2 && k <= nz - 1 && i + 1 < W) {
+      const int ce = q == 0 ? 1 : 0;
+      const T e1 = a.c1 * sE[ce][i + 1] - a.c2 * sEp[ce][i + 1] + a.c3 * sEb[ce][i + 1];
+      const T e0 = a.c1 * sE[ce][i] - a.c2 * sEp[ce][i] + a.c3 * sEb[ce][i];
+      const T d = (q == 0 ? T(1) : T(-1)) * (e1 - e0) * a.idz;
+      nw = sP[6][i] > T(0) ? sP[7][i] * old + sP[8][i] * d : old + a.dt * d;
+    }
+    sV[q][i] = in ? T(0.5) * (old + nw) : T(0);
+    if (in && k >= t0 && k < t0 + NT1) {
+      const T ev = sE[q][i];
+      a.out.B[q * n + k] = nw;
+      a.out.E[q * n + k] = ev;
+      a.out.Ep[q * n + k] = ev;
+      a.out.Eb[q * n + k] = a.ha * ev + a.hb * sEb[q][i];
+      a.Jz[q * n + k] = T(0);
+    }
+  }
+  __syncthreads();
+  // gather copies: the composed filter along z of E and of the averaged B (zero off the component's valid range), or
+  // the values themselves; for the 'momentum conserving' gather (Sec. 5) a half-staggered component (Ez, Bx, By)
+  // becomes the mean of its two nearest values (off the grid: zero)
+  for (int e = threadIdx.x; e < 6 * NT1; e += FB1) {
+    const int c = e / NT1, k = t0 + e - c * NT1, i = k - k0;
+    if (k > nz) continue;
+    const T* F = c < 3 ? sE[c] : sV[c - 3];
     int lo, hi;
-    vr1(q, g.nz, lo, hi);
-    if (k < lo || k > hi) continue;
-    T d = T(0);
-    if (q == 0) d = -c2idz * (B[1 * n + k] - (k >= 1 ? B[1 * n + k - 1] : T(0)));
-    if (q == 1) d = c2idz * (B[0 * n + k] - (k >= 1 ? B[0 * n + k - 1] : T(0)));
-    const T sg = q == 2 ? pm.sgH[k] : pm.sgI[k];
-    T& e = E[q * n + k];
-    if (sg > T(0)) e = (q == 2 ? pm.xiH[k] : pm.xiI[k]) * e + (q == 2 ? pm.cfH[k] : pm.cfI[k]) * d;
-    else e = e + dtT * (d - J[q * n + k] * ie0);
+    vr1(c, nz, lo, hi);
+    auto copy_at = [&](int kk, int ii) {
+      if (!a.filt_g) return F[ii];
+      T acc = T(0);
+      if (kk >= lo && kk <= hi) {
+        const T* w = F + ii - t.P * t.s;   // staged values off the grid are zero
+        for (int m = 0; m <= 2 * t.P; m++) acc += t.c[m] * w[m * t.s];
+      }
+      return acc;
+    };
+    T v = copy_at(k, i);
+    if (a.nodal && half1(c)) v = T(0.5) * ((k >= 1 ? copy_at(k - 1, i - 1) : T(0)) + v);
+    (c < 3 ? a.fE + c * n : a.fB + (c - 3) * n)[k] = v;
   }
 }
 
@@ -207,102 +257,6 @@ struct Ctrl1 {
   int status;
 };
 
-// one electron per thread: gather -> Boris -> move -> 1D Esirkepov; removal after the deposit when it
-// leaves [z_lo, z_hi + dz). The particles of a block are consecutive in memory and, injected row by row,
-// close in z: their current is summed in a shared window over the block's cells (one global atomic per
-// window node afterwards), else, for a block spread wider than the window, added to J directly.
-constexpr int PB1 = 128, JW1 = 320;
-template <class T, bool MC>
-__global__ void __launch_bounds__(PB1) k1_push(G1 g, const T* fE, const T* fB, T* J, Parts1<T> p, const Ctrl1* ctrl,
-                                               int order, T kq, T qe, double zlo, double zhi1) {
-  __shared__ T sJ[3][JW1];
-  __shared__ int s_lo, s_hi;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = g.n1p;
-  if (threadIdx.x == 0) { s_lo = INT_MAX; s_hi = INT_MIN; }
-  for (int e = threadIdx.x; e < 3 * JW1; e += blockDim.x) (&sJ[0][0])[e] = T(0);
-  __syncthreads();
-  const bool live = j < ctrl->count && p.w[j] > T(0);
-  double z = 0.0, Z = 0.0;
-  int f = 0;
-  if (live) {
-    z = p.z[j];
-    Z = (z - g.z0) * g.idz;
-    f = (int)floor(Z);
-    atomicMin(&s_lo, f);
-    atomicMax(&s_hi, f);
-  }
-  __syncthreads();
-  // the deposit of a particle in cell f (moving less than a cell) touches nodes f - 4 .. f + 5
-  const int base = s_lo - 5, span = s_hi - s_lo + 12;
-  const bool win = s_hi >= s_lo && span <= JW1;
-  if (live) {
-    const T w = p.w[j];
-    T EB[6];
-#pragma unroll
-    for (int c = 0; c < 6; c++) {
-      const T* F = c < 3 ? fE + c * n : fB + (c - 3) * n;
-      const double st = (!MC && half1(c)) ? 0.5 : 0.0;
-      T acc = T(0);
-      for (int k = f - 3; k <= f + 3; k++) {
-        if (k < 0 || k > g.nz) continue;
-        const T wz = shp<T>(order, T(Z - (k + st)));
-        if (wz != T(0)) acc += F[k] * wz;
-      }
-      EB[c] = acc;
-    }
-    // relativistic Boris push (textbook)
-    T u0 = p.ux[j], u1 = p.uy[j], u2 = p.uz[j];
-    const T ic2 = T(1.0 / (kC * kC));
-    const T um0 = u0 + kq * EB[0], um1 = u1 + kq * EB[1], um2 = u2 + kq * EB[2];
-    const T gm = sqrt(T(1) + (um0 * um0 + um1 * um1 + um2 * um2) * ic2);
-    const T t0 = kq * EB[3] / gm, t1 = kq * EB[4] / gm, t2 = kq * EB[5] / gm;
-    const T tt = t0 * t0 + t1 * t1 + t2 * t2;
-    const T s0 = T(2) * t0 / (T(1) + tt), s1 = T(2) * t1 / (T(1) + tt), s2 = T(2) * t2 / (T(1) + tt);
-    const T up0 = um0 + (um1 * t2 - um2 * t1), up1 = um1 + (um2 * t0 - um0 * t2), up2 = um2 + (um0 * t1 - um1 * t0);
-    const T pl0 = um0 + (up1 * s2 - up2 * s1), pl1 = um1 + (up2 * s0 - up0 * s2), pl2 = um2 + (up0 * s1 - up1 * s0);
-    u0 = pl0 + kq * EB[0]; u1 = pl1 + kq * EB[1]; u2 = pl2 + kq * EB[2];
-    const T g1 = sqrt(T(1) + (u0 * u0 + u1 * u1 + u2 * u2) * ic2);
-    const double zn = z + g.dt * (double)(u2 / g1);
-    const double Zn = (zn - g.z0) * g.idz;
-    // 1D Esirkepov: Jz(k+1/2) = -(q w/dt) sum_{k' <= k} (S1 - S0)(k'); Jx, Jy = q w v (S0 + S1)/(2 dz)
-    const T qw = qe * w;
-    const T vx = u0 / g1, vy = u1 / g1;
-    const T cz = -qw / T(g.dt), ct = qw * T(0.5) * T(g.idz);
-    const int b = (int)floor(Z < Zn ? Z : Zn) - 3;
-    T run = T(0);
-    for (int a = 0; a < 9; a++) {
-      const int k = b + a;
-      const T S0 = shp<T>(order, T(Z - k)), S1 = shp<T>(order, T(Zn - k));
-      run += S1 - S0;
-      if (k < 0 || k > g.nz) continue;
-      const T ss = S0 + S1;
-      const T jz = cz * run, jx = ct * vx * ss, jy = ct * vy * ss;
-      const int l = k - base;
-      if (win && l >= 0 && l < span) {
-        if (jz != T(0)) atomicAdd(&sJ[2][l], jz);
-        if (jx != T(0)) atomicAdd(&sJ[0][l], jx);
-        if (jy != T(0)) atomicAdd(&sJ[1][l], jy);
-      } else {
-        if (jz != T(0)) atomicAdd(J + 2 * n + k, jz);
-        if (jx != T(0)) atomicAdd(J + k, jx);
-        if (jy != T(0)) atomicAdd(J + n + k, jy);
-      }
-    }
-    p.z[j] = zn;
-    p.ux[j] = u0; p.uy[j] = u1; p.uz[j] = u2;
-    if (zn < zlo || zn >= zhi1) p.w[j] = T(0);
-  }
-  __syncthreads();
-  if (win) {
-    for (int e = threadIdx.x; e < 3 * span; e += blockDim.x) {
-      const int q = e / span, l = e - q * span, k = base + l;
-      const T v = sJ[q][l];
-      if (v != T(0) && k >= 0 && k <= g.nz) atomicAdd(J + q * n + k, v);
-    }
-  }
-}
-
 // plasma rows [m0, m0 + nrow): row m at z' = (m + 1/2) h - beta c t, density gamma n0(gamma (m + 1/2) h),
 // weight n' dz / ppc_z per unit area; rows without plasma, or below z_lo, are stored dead (w = 0)
 struct Lat1 {
@@ -319,54 +273,244 @@ __host__ __device__ inline double lab_density1(const Lat1& L, double zl) {
   return L.n0;
 }
 
+// rows waiting to be stored in the slots at .. at + nrow - 1
+struct Rows1 {
+  long long m0;
+  int nrow, at;
+  double t, zlo;
+};
+
+// state of lattice row m entering at time t
 template <class T>
-__global__ void k1_inject(Parts1<T> p, Ctrl1* ctrl, Lat1 L, long long m0, int nrow, double t, double zlo, int at) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrow) return;
-  const long long m = m0 + r;
+__device__ __forceinline__ void row_state(const Lat1& L, long long m, double t, double zlo, double& z, T& uz, T& w) {
   const double zlat = (m + 0.5) * L.h;
   const double n = L.gamma * lab_density1(L, L.gamma * zlat);
-  const double zp = zlat - L.beta * kC * t;
-  const int q = at + r;
-  p.z[q] = zp;
+  z = zlat - L.beta * kC * t;
+  uz = T(-L.gamma * L.beta * kC);
+  w = (n > 0.0 && z >= zlo) ? T(n * L.dz / (double)L.ppc) : T(0);
+}
+
+template <class T>
+__global__ void k1_inject(Parts1<T> p, Ctrl1* ctrl, Lat1 L, Rows1 r) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= r.nrow) return;
+  const int q = r.at + i;
+  double z;
+  T uz, w;
+  row_state<T>(L, r.m0 + i, r.t, r.zlo, z, uz, w);
+  p.z[q] = z;
   p.ux[q] = T(0);
   p.uy[q] = T(0);
-  p.uz[q] = T(-L.gamma * L.beta * kC);
-  p.w[q] = (n > 0.0 && zp >= zlo) ? T(n * L.dz / (double)L.ppc) : T(0);
-  p.id[q] = (uint32_t)m;
-  if (r == 0) ctrl->count = at + nrow;
+  p.uz[q] = uz;
+  p.w[q] = w;
+  p.id[q] = (uint32_t)(r.m0 + i);
+  if (i == 0) ctrl->count = r.at + r.nrow;
 }
 
-// sum over n >= 0 of S(u + n): the prefix of the shape samples (the 1D Esirkepov flux of a row)
-__device__ __forceinline__ double cum_shape1(int order, double u) {
-  const double r = order == 3 ? 2.0 : 1.0;
-  if (u >= r) return 0.0;
-  if (u <= -r) return 1.0;
-  double acc = 0.0;
-  for (int n = 0; n < 5; n++) acc += shp<double>(order, u + n);
-  return acc;
-}
+// current-sheet antenna: J_y(k) += K w_k / dz over eight nodes from k0
+struct Ant1 {
+  int k0, on;
+  double v[8];
+};
 
-// ions fixed in the lab (PR-9): J_z(k+1/2) += -(e/dt) sum over the live rows of w_m (C(Z1 - k) - C(Z0 - k))
-template <class T>
-__global__ void k1_ion_jz(G1 g, Lat1 L, int order, long long mlo, long long mhi, double t0, double t1, T* Jz) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > g.nz) return;
-  const double vsh = L.beta * kC;
-  long long m0 = (long long)floor(((k - 4) * g.dz + g.z0 + vsh * t0) / L.h - 0.5);
-  long long m1 = (long long)ceil(((k + 4) * g.dz + g.z0 + vsh * t0) / L.h - 0.5);
-  if (m0 < mlo) m0 = mlo;
-  if (m1 > mhi - 1) m1 = mhi - 1;
-  double acc = 0.0;
-  for (long long m = m0; m <= m1; m++) {
-    const double zl = (m + 0.5) * L.h;
-    const double n = L.gamma * lab_density1(L, L.gamma * zl);
-    if (n <= 0.0) continue;
-    const double w = n * L.dz / (double)L.ppc;
-    const double Z0 = (zl - vsh * t0 - g.z0) * g.idz, Z1 = (zl - vsh * t1 - g.z0) * g.idz;
-    acc += w * (cum_shape1(order, Z1 - k) - cum_shape1(order, Z0 - k));
+// the rigid ions' rows of one step (off: on = 0)
+struct Ions1 {
+  long long mlo, mhi;
+  double t0, t1;
+  int on;
+};
+
+// share of a row's shape samples on the nodes <= k (the 1D Esirkepov flux of a row at Z, in cells, through the face
+// above node k), in closed form from the four (two) weights
+template <int ORD>
+__device__ __forceinline__ double cum_shape1(double Z, int k) {
+  const double f = floor(Z), t = Z - f;
+  const int j = k - ((int)f - (ORD == 3 ? 1 : 0));   // node k in the row's stencil
+  if (j < 0) return 0.0;
+  if (ORD == 3) {
+    if (j >= 3) return 1.0;
+    const double t2 = t * t, t3 = t2 * t, s = 1.0 - t;
+    const double w0 = s * s * s * (1.0 / 6.0);
+    if (j == 0) return w0;
+    if (j == 1) return w0 + (2.0 / 3.0 - t2 + 0.5 * t3);
+    return 1.0 - t3 * (1.0 / 6.0);
   }
-  if (acc != 0.0) Jz[k] += T(-kQe / g.dt * acc);
+  return j >= 1 ? 1.0 : 1.0 - t;
+}
+
+// One electron per thread: gather -> Boris -> move -> 1D Esirkepov; removal after the deposit when it leaves
+// [z_lo, z_hi + dz). The rows that entered at the end of the last step are created in their slots here. The blocks past
+// the electrons' add the rigid ions' column current, a warp per node with its lanes over the rows: one thread per
+// node with generic shape sums took 150 us a step in FP64 at 400 nodes and 4 rows a cell. Block 0 adds the antenna.
+// Bound by the latency of one particle's chain (FP32: 10.6 us at 9100 electrons in 24,000 slots, 26.5 us with generic
+// shape functions and lanes of one cell on the same words) and, in FP64, by the FP64 pipe (17 us with the ions at 2500
+// electrons and 400 nodes; 203 us before).
+// A block takes PB1 consecutive slots (injected row by row, so close in z) and sums their current in a shared window
+// over its cells, then adds the window to J; a block spread wider than the window adds to J directly. Thread t takes
+// slot (9 t) mod PB1 of the block: neighbouring lanes then sit about a cell apart, where consecutive slots of one
+// cell would meet on every shared atomic (FP32 and FP64 shared adds retry on a collision).
+// Threads of a block: the FP64 pipe of an SM serves two lanes a cycle, so FP64 blocks are small and spread over the SMs
+// (2500 electrons, 400 nodes: 17 us in blocks of 64, 24 us in blocks of 256; FP32 11.2 us in blocks of 256, 10.6 in
+// blocks of 128).
+template <class T>
+constexpr int push_threads1() { return sizeof(T) == 8 ? 64 : 128; }
+constexpr int JW1 = 192;
+
+template <class T, int ORD, bool MC>
+__global__ void __launch_bounds__(push_threads1<T>()) k1_push(G1 g, const T* __restrict__ fE, const T* __restrict__ fB, T* J,
+                                               Parts1<T> p, int count, Ctrl1* ctrl, T kq, T qe, double zlo,
+                                               double zhi1, Lat1 L, Rows1 rows, Ions1 ions, Ant1 ant, int nbp) {
+  constexpr int NG = ORD + 1, ND = NG + 1, OFF = ORD == 3 ? 1 : 0, PB1 = push_threads1<T>();
+  static_assert((PB1 & (PB1 - 1)) == 0, "(9 t) mod PB1 visits every slot once");
+  const int n = g.n1p;
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  if ((int)blockIdx.x >= nbp) {
+    // ions fixed in the lab (PR-9): J_z(k+1/2) += -(e/dt) sum over the live rows of w_m (C(Z1, k) - C(Z0, k))
+    const int k = ((int)blockIdx.x - nbp) * (PB1 / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k > g.nz) return;   // warp-uniform
+    const double vsh = L.beta * kC;
+    long long m0 = (long long)floor(((k - 4) * g.dz + g.z0 + vsh * ions.t0) / L.h - 0.5);
+    long long m1 = (long long)ceil(((k + 4) * g.dz + g.z0 + vsh * ions.t0) / L.h - 0.5);
+    if (m0 < ions.mlo) m0 = ions.mlo;
+    if (m1 > ions.mhi - 1) m1 = ions.mhi - 1;
+    double acc = 0.0;
+    for (long long m = m0 + lane; m <= m1; m += 32) {
+      const double zl = (m + 0.5) * L.h;
+      const double nd = L.gamma * lab_density1(L, L.gamma * zl);
+      if (nd <= 0.0) continue;
+      const double w = nd * L.dz / (double)L.ppc;
+      const double Z0 = (zl - vsh * ions.t0 - g.z0) * g.idz, Z1 = (zl - vsh * ions.t1 - g.z0) * g.idz;
+      acc += w * (cum_shape1<ORD>(Z1, k) - cum_shape1<ORD>(Z0, k));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0 && acc != 0.0) atomicAdd(J + 2 * n + k, T(-kQe / g.dt * acc));
+    return;
+  }
+  __shared__ T sJ[3][JW1];
+  __shared__ int s_lo, s_hi;
+  if (threadIdx.x == 0) { s_lo = INT_MAX; s_hi = INT_MIN; }
+  for (int e = threadIdx.x; e < 3 * JW1; e += PB1) (&sJ[0][0])[e] = T(0);
+  const int j = blockIdx.x * PB1 + ((9 * threadIdx.x) & (PB1 - 1));
+  T w = T(0), u0 = T(0), u1 = T(0), u2 = T(0);
+  double z = 0.0;
+  if (j < count) {
+    const int r = j - rows.at;
+    if (rows.nrow > 0 && r >= 0 && r < rows.nrow) {
+      row_state<T>(L, rows.m0 + r, rows.t, rows.zlo, z, u2, w);
+      p.id[j] = (uint32_t)(rows.m0 + r);
+      p.w[j] = w;
+      if (w == T(0)) {   // a dead slot is stored whole; a live one is stored below
+        p.z[j] = z; p.ux[j] = T(0); p.uy[j] = T(0); p.uz[j] = u2;
+      }
+    } else {
+      w = p.w[j];
+      if (w > T(0)) { z = p.z[j]; u0 = p.ux[j]; u1 = p.uy[j]; u2 = p.uz[j]; }
+    }
+  }
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0 && rows.nrow > 0) ctrl->count = count;
+    if (ant.on && threadIdx.x < 8) {
+      const int k = ant.k0 + (int)threadIdx.x;
+      if (k >= 0 && k <= g.nz && ant.v[threadIdx.x] != 0.0) atomicAdd(J + n + k, T(ant.v[threadIdx.x]));
+    }
+  }
+  const bool live = w > T(0);
+  double Z = 0.0;
+  int f = 0;
+  if (live) {
+    Z = (z - g.z0) * g.idz;
+    f = (int)floor(Z);
+  }
+  const int flo = __reduce_min_sync(0xffffffffu, live ? f : INT_MAX);
+  const int fhi = __reduce_max_sync(0xffffffffu, live ? f : INT_MIN);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0 && flo <= fhi) { atomicMin(&s_lo, flo); atomicMax(&s_hi, fhi); }
+  __syncthreads();
+  if (s_hi < s_lo) return;   // block-uniform: no live electron here
+  // the deposit of a particle in cell f (moving less than a cell) touches nodes f - 2 .. f + 3
+  const int base = s_lo - 2, span = s_hi - s_lo + 6;
+  const bool win = span <= JW1;
+  if (live) {
+    // shape weights from the fractional offset: integer nodes from f - OFF, half-staggered ones from fh - OFF
+    const T ti = T(Z - f);
+    const int fh = ti >= T(0.5) ? f : f - 1;
+    const T th = ti >= T(0.5) ? ti - T(0.5) : ti + T(0.5);
+    T wi[NG], wh[NG];
+    if constexpr (ORD == 3) { weights3<T>(ti, wi); weights3<T>(th, wh); }
+    else { weights1<T>(ti, wi); weights1<T>(th, wh); }
+    T EB[6];
+    const bool inside = f - OFF - 1 >= 0 && f + NG <= g.nz;
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+      const T* F = c < 3 ? fE + c * n : fB + (c - 3) * n;
+      const bool hf = !MC && half1(c);
+      const int k0 = (hf ? fh : f) - OFF;
+      T acc = T(0);
+#pragma unroll
+      for (int b = 0; b < NG; b++)
+        if (inside || (k0 + b >= 0 && k0 + b <= g.nz)) acc += F[k0 + b] * (hf ? wh[b] : wi[b]);
+      EB[c] = acc;
+    }
+    // relativistic Boris push (textbook), one division each for k / gamma and 2 / (1 + t^2)
+    const T ic2 = T(1.0 / (kC * kC));
+    const T um0 = u0 + kq * EB[0], um1 = u1 + kq * EB[1], um2 = u2 + kq * EB[2];
+    const T kg = kq / sqrt(T(1) + (um0 * um0 + um1 * um1 + um2 * um2) * ic2);
+    const T t0 = kg * EB[3], t1 = kg * EB[4], t2 = kg * EB[5];
+    const T sf = T(2) / (T(1) + (t0 * t0 + t1 * t1 + t2 * t2));
+    const T s0 = sf * t0, s1 = sf * t1, s2 = sf * t2;
+    const T up0 = um0 + (um1 * t2 - um2 * t1), up1 = um1 + (um2 * t0 - um0 * t2), up2 = um2 + (um0 * t1 - um1 * t0);
+    const T pl0 = um0 + (up1 * s2 - up2 * s1), pl1 = um1 + (up2 * s0 - up0 * s2), pl2 = um2 + (up0 * s1 - up1 * s0);
+    u0 = pl0 + kq * EB[0]; u1 = pl1 + kq * EB[1]; u2 = pl2 + kq * EB[2];
+    const T ig = T(1) / sqrt(T(1) + (u0 * u0 + u1 * u1 + u2 * u2) * ic2);
+    const double zn = z + g.dt * (double)(u2 * ig);
+    const double Zn = (zn - g.z0) * g.idz;
+    p.z[j] = zn;
+    p.ux[j] = u0; p.uy[j] = u1; p.uz[j] = u2;
+    if (zn < zlo || zn >= zhi1) p.w[j] = T(0);
+    // 1D Esirkepov: Jz(k+1/2) = -(q w/dt) sum_{k' <= k} (S1 - S0)(k'); Jx, Jy = q w v (S0 + S1)/(2 dz)
+    const int fn = (int)floor(Zn);
+    const int b0 = (f < fn ? f : fn) - OFF;
+    T wn[NG];
+    const T tn = T(Zn - fn);
+    if constexpr (ORD == 3) weights3<T>(tn, wn);
+    else weights1<T>(tn, wn);
+    const T qw = qe * w;
+    const T cz = -qw / T(g.dt), ct = qw * T(0.5) * T(g.idz);
+    const T cx = ct * (u0 * ig), cy = ct * (u1 * ig);
+    const bool o0 = f - OFF > b0, o1 = fn - OFF > b0;
+    T run = T(0);
+#pragma unroll
+    for (int a = 0; a < ND; a++) {
+      // a stencil starts at b0 or one node above
+      const T S0 = o0 ? (a >= 1 ? wi[a - 1] : T(0)) : (a < NG ? wi[a] : T(0));
+      const T S1 = o1 ? (a >= 1 ? wn[a - 1] : T(0)) : (a < NG ? wn[a] : T(0));
+      run += S1 - S0;
+      const int k = b0 + a;
+      if (k < 0 || k > g.nz) continue;
+      const T ss = S0 + S1;
+      const T jz = a < ND - 1 ? cz * run : T(0), jx = cx * ss, jy = cy * ss;
+      const int l = k - base;
+      if (win && l >= 0 && l < span) {
+        if (jz != T(0)) atomicAdd(&sJ[2][l], jz);
+        if (jx != T(0)) atomicAdd(&sJ[0][l], jx);
+        if (jy != T(0)) atomicAdd(&sJ[1][l], jy);
+      } else {
+        if (jz != T(0)) atomicAdd(J + 2 * n + k, jz);
+        if (jx != T(0)) atomicAdd(J + k, jx);
+        if (jy != T(0)) atomicAdd(J + n + k, jy);
+      }
+    }
+  }
+  __syncthreads();
+  if (win) {
+    for (int e = threadIdx.x; e < 3 * span; e += PB1) {
+      const int q = e / span, l = e - q * span, k = base + l;
+      const T v = sJ[q][l];
+      if (v != T(0) && k >= 0 && k <= g.nz) atomicAdd(J + q * n + k, v);
+    }
+  }
 }
 
 // charge density: electrons and the ion rows at time t
@@ -401,18 +545,6 @@ __global__ void k1_rho_i(G1 g, Lat1 L, int order, long long mlo, long long mhi, 
     acc += n * L.dz / (double)L.ppc * shp<double>(order, (zl - vsh * t - g.z0) * g.idz - k);
   }
   rho[k] += kQe * acc * g.idz;
-}
-
-// current-sheet antenna: J_y(k) += K w_k / dz over eight nodes from k0
-struct Ant1 {
-  int k0;
-  double v[8];
-};
-template <class T>
-__global__ void k1_antenna(G1 g, Ant1 a, T* Jy) {
-  const int i = threadIdx.x;
-  const int k = a.k0 + i;
-  if (i < 8 && k >= 0 && k <= g.nz && a.v[i] != 0.0) Jy[k] += T(a.v[i]);
 }
 
 // diagnostics: [0] live electrons, [1] field energy per unit area, [2] weight above the lab gamma threshold
@@ -602,11 +734,15 @@ class Sim1 : public Sim3Api {
     taps.s = wide ? 1 : c->filter_stride;
     nodal = c->gather_scheme == 1;
     const int n = g.n1p;
-    E = dal<T>(3 * n); B = dal<T>(3 * n); J = dal<T>(3 * n); Jf = dal<T>(3 * n); Ep = dal<T>(3 * n);
-    Eb = dal<T>(3 * n); Bavg = dal<T>(3 * n); fE = dal<T>(3 * n); fB = dal<T>(3 * n); nF = dal<T>(6 * n);
+    // two sets of the fields and of the current: k1_fields reads one and writes the other
+    for (int q = 0; q < 2; q++) {
+      fs2[q].E = dal<T>(3 * n); fs2[q].Ep = dal<T>(3 * n); fs2[q].Eb = dal<T>(3 * n); fs2[q].B = dal<T>(3 * n);
+      J2[q] = dal<T>(3 * n);
+      if (!fs2[q].E || !fs2[q].Ep || !fs2[q].Eb || !fs2[q].B || !J2[q]) return fail(PIC_ENOMEM, "allocation failed");
+    }
+    fE = dal<T>(3 * n); fB = dal<T>(3 * n);
     rho = dal<double>(n); outd = dal<double>(n); sred = dal<double>(4); ctrl = dal<Ctrl1>(1);
-    if (!E || !B || !J || !Jf || !Ep || !Eb || !Bavg || !fE || !fB || !nF || !rho || !outd || !sred || !ctrl)
-      return fail(PIC_ENOMEM, "allocation failed");
+    if (!fE || !fB || !rho || !outd || !sred || !ctrl) return fail(PIC_ENOMEM, "allocation failed");
     // PML tables at integer and half positions
     std::vector<T> sg(2 * n, T(0)), xi(2 * n, T(1)), cf(2 * n, T(g.dt));
     for (int h = 0; h < 2; h++)
@@ -635,19 +771,6 @@ class Sim1 : public Sim3Api {
     cudaStreamSynchronize(s);
     pm.sgI = dsg; pm.xiI = dxi; pm.cfI = dcf;
     pm.sgH = dsg + n; pm.xiH = dxi + n; pm.cfH = dcf + n;
-    shift_arr = dal<T*>(12);
-    shift_comp = dal<int>(12);
-    if (!shift_arr || !shift_comp) return fail(PIC_ENOMEM, "allocation failed");
-    T* arrs[12];
-    int comps[12];
-    for (int q = 0; q < 3; q++) {
-      arrs[q] = E + q * n; comps[q] = q;
-      arrs[3 + q] = B + q * n; comps[3 + q] = 3 + q;
-      arrs[6 + q] = Ep + q * n; comps[6 + q] = q;
-      arrs[9 + q] = Eb + q * n; comps[9 + q] = q;
-    }
-    cudaMemcpyAsync(shift_arr, arrs, sizeof(arrs), cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(shift_comp, comps, sizeof(comps), cudaMemcpyHostToDevice, s);
     return cudaStreamSynchronize(s) == cudaSuccess ? PIC_OK : fail(PIC_ECUDA, "CUDA error in 1D init");
   }
 
@@ -705,20 +828,28 @@ class Sim1 : public Sim3Api {
     const int c = read_count();
     if (c < 0) return fail(PIC_ECUDA, "CUDA error in compaction");
     count_ub = c;
-    live_est = c;
     compactions++;
     return PIC_OK;
   }
 
+  // rows [m0, m1) enter at time t: their slots are taken now, their state is written by the next step's k1_push, or by
+  // k1_inject (store_rows) before anything else reads or moves the particles
   int inject(long long m0, long long m1, double t) {
     if (m1 <= m0) return PIC_OK;
     const long nrow = (long)(m1 - m0);
+    if (store_rows() != PIC_OK) return st;
     if (count_ub + nrow > cap && grow(count_ub + nrow) != PIC_OK) return st;
-    k1_inject<T><<<nb1(nrow, 128), 128, 0, s>>>(P2[cur], ctrl, lat, m0, (int)nrow, t, z_lo(), (int)count_ub);
-    nl++;
+    pend.m0 = m0; pend.nrow = (int)nrow; pend.at = (int)count_ub; pend.t = t; pend.zlo = z_lo();
     count_ub += nrow;
-    live_est += nrow;
     return PIC_OK;
+  }
+
+  int store_rows() {
+    if (pend.nrow == 0) return PIC_OK;
+    k1_inject<T><<<nb1(pend.nrow, 128), 128, 0, s>>>(P2[cur], ctrl, lat, pend);
+    nl++;
+    pend.nrow = 0;
+    return cudaGetLastError() == cudaSuccess ? PIC_OK : fail(PIC_ECUDA, "CUDA error in 1D inflow");
   }
 
   int load_plasma(const pic_plasma* p) override {
@@ -737,7 +868,7 @@ class Sim1 : public Sim3Api {
     const long want = (long)(m_end - m_beg) * 2 + 4096;
     if (alloc_parts(want) != PIC_OK) return fail(PIC_ENOMEM, "particle allocation failed");
     count_ub = 0;
-    if (inject(m_beg, m_end, t) != PIC_OK) return st;
+    if (inject(m_beg, m_end, t) != PIC_OK || store_rows() != PIC_OK) return st;
     row_next = m_end;
     mlo = m_beg;
     loaded = true;
@@ -800,92 +931,92 @@ class Sim1 : public Sim3Api {
     tev.clear();
   }
 
-  int one_step() {
-    const int n = g.n1p, n1 = g.nz + 1;
+  // a kernel that may begin launching while the one before it on the stream ends (it waits for it on the device)
+  template <class... KA, class... A>
+  void chain(void (*k)(KA...), unsigned blocks, unsigned threads, const A&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(blocks);
+    c.blockDim = dim3(threads);
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, k, KA(args)...);
+    nl++;
+  }
+
+  // moving window (lab frame): the grid moves down by whole cells at the start of a step
+  int window_shift() {
+    if (!cfg.moving_window) return 0;
+    const long long want = (long long)std::floor(cfg.window_beta * kC * time_of(step) / g.dz);
+    const long long sh = want - shifts;
+    if (sh <= 0) return 0;
+    shifts = want;
+    g.z0 = want * g.dz;
+    return (int)std::min<long long>(sh, g.nz + 1);
+  }
+
+  // the fields between two pushes: Ampère of the step before (ampere), the window's shift, Faraday, the Friedman
+  // history and the gather copies of the step to come (faraday)
+  void fields(bool ampere, bool faraday, int shift) {
     const double th = cfg.theta;
-    const double tn = time_of(step), tn1 = time_of(step + 1);
-    // moving window (lab frame): the grid moves down by whole cells
-    if (cfg.moving_window) {
-      const long long want = (long long)std::floor(cfg.window_beta * kC * tn / g.dz);
-      const long long sh = want - shifts;
-      if (sh > 0) {
-        k1_shift<T><<<dim3(1, 12), 1024, 0, s>>>(g, shift_arr, shift_comp, (int)std::min<long long>(sh, g.nz + 1));
-        nl++;
-        shifts = want;
-        g.z0 = want * g.dz;
-      }
-    }
+    Fields1<T> a;
+    a.in = fs2[fc]; a.out = fs2[1 - fc];
+    a.J = J2[jc]; a.Jz = J2[1 - jc];
+    a.fE = fE; a.fB = fB;
+    a.c1 = T(1.0 + th / 4.0); a.c2 = T(0.5); a.c3 = T(0.5 - th / 4.0);
+    a.ha = T(1.0 - th / 2.0); a.hb = T(th / 2.0);
+    a.dt = T(g.dt); a.idz = T(g.idz); a.c2idz = T(kC * kC * g.idz); a.ie0 = T(1.0 / kEps0);
+    a.ampere = ampere; a.faraday = faraday;
+    a.filt_j = cfg.filter_J && P > 0; a.filt_g = cfg.filter_gather && P > 0; a.nodal = nodal;
+    a.shift = shift;
+    a.H = a.filt_j || a.filt_g ? taps.P * taps.s : 0;
     tbeg(1);
-    // 1. Faraday + Friedman + PML-B, B average
-    k1_faraday<T><<<nb1(n1, 256), 256, 0, s>>>(g, pm, E, Ep, Eb, B, Bavg, T(1.0 + th / 4.0), T(0.5),
-                                               T(0.5 - th / 4.0), T(g.dt), T(g.idz));
-    k1_friedman<T><<<nb1(3 * n, 256), 256, 0, s>>>(3 * n, E, Ep, Eb, T(1.0 - th / 2.0), T(th / 2.0));
-    nl += 2;
-    // 2. gather copies (filtered; node-interpolated for the 'momentum conserving' gather)
-    const T* gE = E;
-    const T* gB = Bavg;
-    if (cfg.filter_gather && P > 0) {
-      FiltJob1<T> jb;
-      for (int q = 0; q < 3; q++) {
-        jb.src[q] = E + q * n; jb.dst[q] = fE + q * n; jb.comp[q] = q;
-        jb.src[3 + q] = Bavg + q * n; jb.dst[3 + q] = fB + q * n; jb.comp[3 + q] = 3 + q;
-      }
-      k1_filter<T><<<dim3(nb1(n1, 256), 6), 256, 0, s>>>(g, jb, taps);
-      nl++;
-      gE = fE; gB = fB;
-    }
-    if (nodal) {
-      k1_nodal<T><<<nb1(n1, 256), 256, 0, s>>>(g, gE, gB, nF);
-      nl++;
-      gE = nF; gB = nF + 3 * n;
-    }
+    chain(k1_fields<T>, nb1(g.nz + 1, NT1), FB1, g, pm, taps, a);
     tend(1);
-    // 3. particles
-    cudaMemsetAsync(J, 0, sizeof(T) * 3 * n, s);
-    tbeg(0);
-    if (loaded && count_ub > 0) {
-      const T kq = T(-kQe * g.dt / (2.0 * kMe));
-      if (nodal)
-        k1_push<T, true><<<nb1(count_ub, PB1), PB1, 0, s>>>(g, gE, gB, J, P2[cur], ctrl, cfg.shape_order, kq,
-                                                           T(-kQe), z_lo(), z_hi() + g.dz);
-      else
-        k1_push<T, false><<<nb1(count_ub, PB1), PB1, 0, s>>>(g, gE, gB, J, P2[cur], ctrl, cfg.shape_order, kq,
-                                                            T(-kQe), z_lo(), z_hi() + g.dz);
-      nl++;
-    }
-    tend(0);
-    // ions fixed in the lab: no current in the lab frame (beta = 0); 32-thread blocks spread the rows' FP64
-    // sums over more SMs
-    if (loaded && ions && row_next > mlo && beta > 0.0) {
-      k1_ion_jz<T><<<nb1(n1, 32), 32, 0, s>>>(g, lat, cfg.shape_order, mlo, row_next, tn, tn1, J + 2 * n);
-      nl++;
-    }
-    // 4. antenna
+    fc = 1 - fc;
+    if (faraday) jc = 1 - jc;   // the next deposit goes to the current just set to zero
+  }
+
+  template <int ORD, bool MC>
+  void launch_push(const Ions1& io, const Ant1& an) {
+    constexpr int PB1 = push_threads1<T>();
+    const unsigned nbp = std::max(1u, nb1(count_ub, PB1));
+    const unsigned nbi = io.on ? nb1(g.nz + 1, PB1 / 32) : 0;
+    chain(k1_push<T, ORD, MC>, nbp + nbi, PB1, g, fE, fB, J2[jc], P2[cur], (int)count_ub, ctrl,
+          T(-kQe * g.dt / (2.0 * kMe)), T(-kQe), z_lo(), z_hi() + g.dz, lat, pend, io, an, (int)nbp);
+    pend.nrow = 0;
+  }
+
+  // push of the electrons (with the rows that entered at the end of the last step), ions, antenna, inflow
+  int particles() {
+    const double tn = time_of(step), tn1 = time_of(step + 1);
+    // ions fixed in the lab: no current in the lab frame (beta = 0)
+    Ions1 io{};
+    io.on = loaded && ions && row_next > mlo && beta > 0.0;
+    io.mlo = mlo; io.mhi = row_next; io.t0 = tn; io.t1 = tn1;
+    Ant1 a{};
     if (has_laser && las.z_antenna >= z_lo() && las.z_antenna < z_hi()) {
       const double Z = (las.z_antenna - g.z0) / g.dz;
       const int f = (int)std::floor(Z);
       const double K = -2.0 * kEps0 * kC * emit(0.5 * (tn + tn1));
-      Ant1 a;
+      a.on = 1;
       a.k0 = f - 3;
       for (int i = 0; i < 8; i++) a.v[i] = K * shape_h(cfg.shape_order, Z - (a.k0 + i)) / g.dz;
-      k1_antenna<T><<<1, 32, 0, s>>>(g, a, J + n);
-      nl++;
     }
-    // 5. current filter, Ampère + PML-E
-    tbeg(1);
-    const T* Ja = J;
-    if (cfg.filter_J && P > 0) {
-      FiltJob1<T> jb;
-      for (int q = 0; q < 3; q++) { jb.src[q] = J + q * n; jb.dst[q] = Jf + q * n; jb.comp[q] = 6 + q; }
-      k1_filter<T><<<dim3(nb1(n1, 256), 3), 256, 0, s>>>(g, jb, taps);
-      nl++;
-      Ja = Jf;
+    tbeg(0);
+    if (cfg.shape_order == 3) {
+      if (nodal) launch_push<3, true>(io, a);
+      else launch_push<3, false>(io, a);
+    } else {
+      if (nodal) launch_push<1, true>(io, a);
+      else launch_push<1, false>(io, a);
     }
-    k1_ampere<T><<<nb1(n1, 256), 256, 0, s>>>(g, pm, E, B, Ja, T(g.dt), T(kC * kC * g.idz), T(1.0 / kEps0));
-    nl++;
-    tend(1);
+    tend(0);
     step++;
-    // 6. ion rows that left, plasma rows entering through z_hi
+    // ion rows that left, plasma rows entering through z_hi
     if (loaded) {
       while (mlo < row_next && (mlo + 0.5) * lat.h - beta * kC * tn1 < z_lo()) mlo++;
       const long long m_end = rows_inside(tn1);
@@ -895,7 +1026,7 @@ class Sim1 : public Sim3Api {
       }
       // the dead slots (left the domain, or rows without plasma) are squeezed out now and then
       if (count_ub > 65536 && (step & 63) == 0) {
-        if (compact() != PIC_OK) return st;
+        if (store_rows() != PIC_OK || compact() != PIC_OK) return st;
       }
     }
     return PIC_OK;
@@ -903,8 +1034,14 @@ class Sim1 : public Sim3Api {
 
   int run(int nsteps) override {
     if (st != PIC_OK) return st;
-    for (int q = 0; q < nsteps; q++)
-      if (one_step() != PIC_OK) return st;
+    int r = PIC_OK;
+    for (int q = 0; q < nsteps && r == PIC_OK; q++) {
+      fields(q > 0, true, window_shift());
+      r = particles();
+    }
+    // the last step's Ampère and inflow, so that the state is whole between calls
+    if (nsteps > 0) fields(true, false, 0);
+    if (store_rows() != PIC_OK || r != PIC_OK) return st;
     return cudaGetLastError() == cudaSuccess ? PIC_OK : fail(PIC_ECUDA, "CUDA error in 1D step");
   }
 
@@ -918,9 +1055,9 @@ class Sim1 : public Sim3Api {
 
   T* comp_ptr(int comp) {
     const int n = g.n1p;
-    if (comp < 3) return E + comp * n;
-    if (comp < 6) return B + (comp - 3) * n;
-    return J + (comp - 6) * n;
+    if (comp < 3) return fs2[fc].E + comp * n;
+    if (comp < 6) return fs2[fc].B + (comp - 3) * n;
+    return J2[jc] + (comp - 6) * n;
   }
 
   int get_field(int comp, double* dst, int on_device) override {
@@ -1004,7 +1141,7 @@ class Sim1 : public Sim3Api {
     cudaMemsetAsync(sred, 0, 4 * sizeof(double), s);
     Parts1<T> p = P2[cur];
     if (!loaded) cudaMemsetAsync(ctrl, 0, sizeof(Ctrl1), s);
-    k1_stats<T><<<64, 256, 0, s>>>(g, E, B, p, ctrl, gamma, beta, trap, sred);
+    k1_stats<T><<<64, 256, 0, s>>>(g, fs2[fc].E, fs2[fc].B, p, ctrl, gamma, beta, trap, sred);
     nl++;
     double h[4];
     cudaMemcpyAsync(h, sred, sizeof(h), cudaMemcpyDeviceToHost, s);
@@ -1056,17 +1193,18 @@ class Sim1 : public Sim3Api {
   bool nodal = false;
   Taps1<T> taps{};
   Pml1<T> pm{};
-  T *E = nullptr, *B = nullptr, *J = nullptr, *Jf = nullptr, *Ep = nullptr, *Eb = nullptr, *Bavg = nullptr;
-  T *fE = nullptr, *fB = nullptr, *nF = nullptr;
+  Set1<T> fs2[2]{};      // the current fields are fs2[fc], the step's current J2[jc]
+  T* J2[2] = {nullptr, nullptr};
+  int fc = 0, jc = 0;
+  T *fE = nullptr, *fB = nullptr;
   double *rho = nullptr, *outd = nullptr, *sred = nullptr;
   Ctrl1* ctrl = nullptr;
-  T** shift_arr = nullptr;
-  int* shift_comp = nullptr;
   Parts1<T> P2[2]{};
   int cur = 0;
   int* blk = nullptr;
   long cap = 0;
-  long count_ub = 0, live_est = 0;
+  long count_ub = 0;
+  Rows1 pend{};          // rows whose slots are taken and whose state is not yet stored
   bool loaded = false, ions = false, has_laser = false;
   Lat1 lat{};
   pic_laser las{};
