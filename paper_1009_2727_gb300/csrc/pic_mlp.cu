@@ -149,6 +149,365 @@ __global__ void k_gather_rows(int nb, const int* idx, const float* X, int dx, co
   for (int j = threadIdx.x; j < dt; j += blockDim.x) Tb[(long)r * dt + j] = T[s * dt + j];
 }
 
+// ---------------------------------------------------------------------------
+// Small batches (training minibatches, up to SB_ROWS rows). At 64 rows and widths of 256 a minibatch is 0.05 us of FP32
+// work on the whole GPU, so what counts is how many SMs share a product and how many dependent launches there are:
+// 64 x 64 tiles gave each product 4 CTAs and 14-34 us, and 21 launches made 240 us of a minibatch. Here a product is
+// cut into 8 x 16 output tiles (128 CTAs for 64 x 256), one output per thread, its sum taken in the order of the large
+// tiles (the results are bitwise theirs); the row gather, BF16 rounding, bias, GELU, loss and GELU' ride with the
+// products, and one launch takes the gradients and AdamW of every layer: 8 launches for four layers. Consecutive
+// launches overlap their start (programmatic dependent launch): each kernel fetches what its predecessor does not write
+// (weights, pre-activations, moments) before it waits for it.
+// Measured (6-256-256-256-4, batch 64): 235 -> 33 us a minibatch; each product 5.4-6.8 us alone, the gradients 9.3 us
+// (19.5 us with element-wise staging and the bias sums from global memory): bound by the eight launches' latencies.
+constexpr int SB_ROWS = 512;    // above: the 64 x 64 tiles, which re-read less
+constexpr int SB_M = 8;         // output tile: rows
+constexpr int SB_N = 16;        //              columns
+constexpr int SB_KC = 256;      // reduction slice held in shared memory (FP32)
+constexpr int SB_LD = SB_KC + 4;   // rows 16 bytes apart modulo 128: the 16-byte reads of eight rows hit all banks
+constexpr int SB_THREADS = SB_M * SB_N;
+
+// eight BF16 values of a row from p[k ..] (zero past K), read through L2 (what a kernel fetches before its wait must not
+// come from an older L1 line); vec: 16-byte loads are aligned and K is a multiple of 8
+__device__ __forceinline__ uint4 ld8(const __nv_bfloat16* p, int k, int K, bool vec) {
+  if (vec && k + 8 <= K) return __ldcg(reinterpret_cast<const uint4*>(p + k));
+  __align__(16) __nv_bfloat16 v[8];
+#pragma unroll
+  for (int q = 0; q < 8; q++) v[q] = k + q < K ? __ldcg(p + k + q) : __float2bfloat16(0.0f);
+  return *reinterpret_cast<const uint4*>(v);
+}
+__device__ __forceinline__ void unpack8(const uint4& u, float* f) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    f[2 * q] = __uint_as_float(w[q] << 16);
+    f[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
+  }
+}
+__device__ __forceinline__ void put8(float* d, const float* f) {
+  reinterpret_cast<float4*>(d)[0] = make_float4(f[0], f[1], f[2], f[3]);
+  reinterpret_cast<float4*>(d)[1] = make_float4(f[4], f[5], f[6], f[7]);
+}
+
+// acc += sum over the staged slice of a row times a row, in order
+__device__ __forceinline__ void slice_dot(const float* a, const float* b, int kn, float& acc) {
+#pragma unroll 8
+  for (int k = 0; k < kn; k += 4) {
+    const float4 x = *reinterpret_cast<const float4*>(a + k), y = *reinterpret_cast<const float4*>(b + k);
+    acc += x.x * y.x;
+    acc += x.y * y.y;
+    acc += x.z * y.z;
+    acc += x.w * y.w;
+  }
+}
+
+// one layer's forward product of M rows: Z = H W^T + b. FIRST: H is the BF16 rounding of the rows idx[r] (or r) of the
+// FP32 inputs x. Hidden layers store Z (FP32) and GELU(Z) (BF16); the last layer (LAST) stores Z and, with targets t,
+// the gradient dY = 2 (Z - t[idx[r]]) / (M N) of the mean squared error and every output's share of it (sq).
+template <bool FIRST, bool LAST>
+__global__ void __launch_bounds__(SB_THREADS) k_sb_fwd(int M, int N, int K, const __nv_bfloat16* H, const float* x,
+                                                       const int* idx, const __nv_bfloat16* W, const float* bias,
+                                                       float* Z, __nv_bfloat16* Hn, const float* t, float* dY,
+                                                       float* sq, int vec) {
+  __shared__ __align__(16) float sa[SB_M][SB_LD], sw[SB_N][SB_LD];
+  const int tid = threadIdx.x, ty = tid / SB_N, tx = tid % SB_N;
+  const int m0 = blockIdx.y * SB_M, n0 = blockIdx.x * SB_N;
+  auto stage_w = [&](int k0) {
+    for (int e = tid; e < SB_N * (SB_KC / 8); e += SB_THREADS) {
+      const int r = e / (SB_KC / 8), k = k0 + (e % (SB_KC / 8)) * 8;
+      uint4 u = make_uint4(0, 0, 0, 0);
+      if (n0 + r < N && k < K) u = ld8(W + (long)(n0 + r) * K, k, K, vec);
+      float f[8];
+      unpack8(u, f);
+      put8(&sw[r][k - k0], f);
+    }
+  };
+  // the weights were last written before the predecessor began (the first layer's predecessor is their update)
+  if (!FIRST) stage_w(0);
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  float acc = 0.0f;
+  for (int k0 = 0; k0 < K; k0 += SB_KC) {
+    if (FIRST || k0 > 0) stage_w(k0);
+    for (int e = tid; e < SB_M * (SB_KC / 8); e += SB_THREADS) {
+      const int r = e / (SB_KC / 8), k = k0 + (e % (SB_KC / 8)) * 8, m = m0 + r;
+      float f[8] = {};
+      if (m < M && k < K) {
+        if (FIRST) {
+          const float* xr = x + (long)(idx ? idx[m] : m) * K;
+#pragma unroll
+          for (int q = 0; q < 8; q++) f[q] = k + q < K ? __bfloat162float(__float2bfloat16(xr[k + q])) : 0.0f;
+        } else {
+          unpack8(ld8(H + (long)m * K, k, K, vec), f);
+        }
+      }
+      put8(&sa[r][k - k0], f);
+    }
+    __syncthreads();
+    slice_dot(sa[ty], sw[tx], min(SB_KC, (K - k0 + 3) & ~3), acc);
+    __syncthreads();
+  }
+  const int m = m0 + ty, n = n0 + tx;
+  if (m >= M || n >= N) return;
+  const long o = (long)m * N + n;
+  const float z = acc + bias[n];
+  Z[o] = z;
+  if (!LAST) Hn[o] = __float2bfloat16(0.5f * z * (1.0f + erff(z * 0.70710678118654752f)));
+  if (LAST && t) {
+    const float nd = (float)((long)M * N), d = z - t[(long)(idx ? idx[m] : m) * N + n];
+    dY[o] = 2.0f * d / nd;
+    sq[o] = d * d / nd;
+  }
+}
+
+// input gradient through the GELU of the layer below: dZ'(m, i) = (sum_o dZ(m, o) W(o, i)) GELU'(Z'(m, i)),
+// GELU'(z) = Phi(z) + z phi(z); M rows, K outputs o, N inputs i
+__global__ void __launch_bounds__(SB_THREADS) k_sb_dx(int M, int N, int K, const float* dZ, const __nv_bfloat16* W,
+                                                      const float* Zl, float* dZl, int vec, int vecz) {
+  __shared__ __align__(16) float sa[SB_M][SB_LD], sw[SB_N][SB_LD];   // sw: the weights' columns as rows
+  const int tid = threadIdx.x, ty = tid / SB_N, tx = tid % SB_N;
+  const int m0 = blockIdx.y * SB_M, n0 = blockIdx.x * SB_N;
+  auto stage_w = [&](int k0) {
+    for (int e = tid; e < SB_KC * (SB_N / 8); e += SB_THREADS) {
+      const int k = e % SB_KC, c = (e / SB_KC) * 8;
+      uint4 u = make_uint4(0, 0, 0, 0);
+      if (k0 + k < K && n0 + c < N) u = ld8(W + (long)(k0 + k) * N, n0 + c, N, vec);
+      float f[8];
+      unpack8(u, f);
+#pragma unroll
+      for (int q = 0; q < 8; q++) sw[c + q][k] = f[q];
+    }
+  };
+  // weights and pre-activations were written before the predecessor began
+  stage_w(0);
+  const int m = m0 + ty, n = n0 + tx;
+  const float z = m < M && n < N ? __ldcg(Zl + (long)m * N + n) : 0.0f;
+  const float d = 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  float acc = 0.0f;
+  for (int k0 = 0; k0 < K; k0 += SB_KC) {
+    if (k0 > 0) stage_w(k0);
+    for (int e = tid; e < SB_M * (SB_KC / 4); e += SB_THREADS) {
+      const int r = e / (SB_KC / 4), k = k0 + (e % (SB_KC / 4)) * 4, mr = m0 + r;
+      float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (mr < M && k < K) {
+        const float* p = dZ + (long)mr * K + k;
+        if (vecz && k + 4 <= K) {
+          f = *reinterpret_cast<const float4*>(p);
+        } else {
+          f.x = p[0];
+          if (k + 1 < K) f.y = p[1];
+          if (k + 2 < K) f.z = p[2];
+          if (k + 3 < K) f.w = p[3];
+        }
+      }
+      *reinterpret_cast<float4*>(&sa[r][k - k0]) = f;
+    }
+    __syncthreads();
+    slice_dot(sa[ty], sw[tx], min(SB_KC, (K - k0 + 3) & ~3), acc);
+    __syncthreads();
+  }
+  if (m < M && n < N) dZl[(long)m * N + n] = acc * d;
+}
+
+// AdamW's constants; the bias corrections c1 = 1 - b1^t, c2 = 1 - b2^t come from a host-computed table at step
+// (*eidx) * nbat + kk (the form a captured epoch replays)
+struct AdamC {
+  float lr, b1, b2, eps, wd;
+  const float2* ctab;
+  const int* eidx;
+  int nbat, kk;
+};
+
+__device__ __forceinline__ float adamw_one(float pi, float gi, float& m, float& v, const AdamC& a, float2 c) {
+  // roundings written out, so that this is k_adamw bit for bit
+  m = fmaf(1.0f - a.b1, gi, __fmul_rn(a.b1, m));
+  v = fmaf(__fmul_rn(1.0f - a.b2, gi), gi, __fmul_rn(a.b2, v));
+  return fmaf(-a.lr, fmaf(a.wd, pi, (m / c.x) / (sqrtf(v / c.y) + a.eps)), pi);
+}
+
+struct SbLayer {
+  const float* dZ;            // M x N
+  const __nv_bfloat16* H;     // M x K (layers above the first)
+  long off_w, off_b;
+  int N, K, blocks, tk;       // tiles (tk along the inputs) end at block `blocks` of the launch
+  int vz, vh;                 // four values of a row of dZ, of H load together (widths and bases aligned)
+};
+struct SbNet {
+  SbLayer l[16];
+  int L;
+};
+
+// gradients of every layer, dW(o, i) = sum_r dZ(r, o) H(r, i) and db(o) = sum_r dZ(r, o), on 32 x 32 tiles of the
+// weights (rows summed in order); then AdamW and the BF16 copies (p given), or the gradient stored (g given). The first
+// layer's H are the BF16-rounded rows idx[r] (or r) of x. The last
+// block (a tile of the small last layer) sums the minibatch's loss, 256 outputs at a time.
+constexpr int SB_GT = 32, SB_GR = 64;
+__global__ void __launch_bounds__(256) k_sb_grad(SbNet net, int M, const float* x, const int* idx, float* p,
+                                                 __nv_bfloat16* pb, float* mo, float* vo, float* g, AdamC a,
+                                                 const float* sq, long nsq, float* loss) {
+  __shared__ float sz[SB_GR][SB_GT + 1], sh[SB_GR][SB_GT + 1];   // padded: the bias sums read sz by columns
+  __shared__ float red[256], sdb[SB_GT];
+  int li = 0;
+  while (li + 1 < net.L && (int)blockIdx.x >= net.l[li].blocks) li++;
+  const SbLayer& L = net.l[li];
+  const int b = (int)blockIdx.x - (li > 0 ? net.l[li - 1].blocks : 0);
+  const int o0 = (b / L.tk) * SB_GT, i0 = (b % L.tk) * SB_GT;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  // the tile's parameters and moments were last written before the predecessors began
+  float pv[2][2], mv[2][2], vv[2][2], bp = 0.f, bm = 0.f, bv = 0.f;
+  const bool bias = i0 == 0 && tid < SB_GT && o0 + tid < L.N;
+  float2 c = make_float2(1.0f, 1.0f);
+  if (p) {
+    c = __ldcg(a.ctab + (long)__ldcg(a.eidx) * a.nbat + a.kk);
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+#pragma unroll
+      for (int w = 0; w < 2; w++) {
+        const int o = o0 + ty + 16 * u, i = i0 + tx + 16 * w;
+        pv[u][w] = mv[u][w] = vv[u][w] = 0.0f;
+        if (o < L.N && i < L.K) {
+          const long q = L.off_w + (long)o * L.K + i;
+          pv[u][w] = __ldcg(p + q); mv[u][w] = __ldcg(mo + q); vv[u][w] = __ldcg(vo + q);
+        }
+      }
+    if (bias) {
+      const long q = L.off_b + o0 + tid;
+      bp = __ldcg(p + q); bm = __ldcg(mo + q); bv = __ldcg(vo + q);
+    }
+  }
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  float acc[2][2] = {};
+  for (int r0 = 0; r0 < M; r0 += SB_GR) {
+    const int nr = min(SB_GR, M - r0);
+    // four values of a row of either operand per thread and pass, every load of the slice issued together
+    constexpr int NP = SB_GR * SB_GT / 4 / 256;
+    const int q = (tid & 7) * 4;
+    float fz[NP][4], fh[NP][4];
+#pragma unroll
+    for (int u = 0; u < NP; u++) {
+      const int r = (tid >> 3) + 32 * u, m = r0 + r;
+#pragma unroll
+      for (int j = 0; j < 4; j++) fz[u][j] = fh[u][j] = 0.0f;
+      if (r >= nr) continue;
+      const float* pz = L.dZ + (long)m * L.N + o0 + q;
+      if (L.vz && o0 + q + 4 <= L.N) {
+        const float4 f = *reinterpret_cast<const float4*>(pz);
+        fz[u][0] = f.x; fz[u][1] = f.y; fz[u][2] = f.z; fz[u][3] = f.w;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; j++) if (o0 + q + j < L.N) fz[u][j] = pz[j];
+      }
+      if (li == 0) {
+        const float* px = x + (long)(idx ? idx[m] : m) * L.K + i0 + q;
+#pragma unroll
+        for (int j = 0; j < 4; j++) if (i0 + q + j < L.K) fh[u][j] = __bfloat162float(__float2bfloat16(px[j]));
+      } else {
+        const __nv_bfloat16* ph = L.H + (long)m * L.K + i0 + q;
+        if (L.vh && i0 + q + 4 <= L.K) {
+          const uint2 w = *reinterpret_cast<const uint2*>(ph);
+          fh[u][0] = __uint_as_float(w.x << 16); fh[u][1] = __uint_as_float(w.x & 0xffff0000u);
+          fh[u][2] = __uint_as_float(w.y << 16); fh[u][3] = __uint_as_float(w.y & 0xffff0000u);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; j++) if (i0 + q + j < L.K) fh[u][j] = __bfloat162float(ph[j]);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < NP; u++) {
+      const int r = (tid >> 3) + 32 * u;
+#pragma unroll
+      for (int j = 0; j < 4; j++) { sz[r][q + j] = fz[u][j]; sh[r][q + j] = fh[u][j]; }
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int r = 0; r < SB_GR; r++) {   // rows past nr are zero
+#pragma unroll
+      for (int u = 0; u < 2; u++)
+#pragma unroll
+        for (int w = 0; w < 2; w++) acc[u][w] += sz[r][ty + 16 * u] * sh[r][tx + 16 * w];
+    }
+    __syncthreads();
+  }
+  if (i0 == 0) {
+    // db: rows 256 apart, then halves of 256 slots added pairwise; a warp per output, slot lane + 32 j
+    const int lane = tid & 31;
+    for (int q = tid >> 5; q < SB_GT; q += 8) {
+      if (o0 + q >= L.N) break;
+      float v[8];
+      if (M <= SB_GR) {   // the staged rows (zero past M)
+        v[0] = sz[lane][q] + sz[lane + 32][q];
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          v[j] = 0.0f;
+          for (int r = lane + 32 * j; r < M; r += 256) v[j] += L.dZ[(long)r * L.N + o0 + q];
+        }
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+          for (int j = 0; j < h; j++) v[j] += v[j + h];
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_down_sync(0xffffffffu, v[0], o);
+      if (lane == 0) sdb[q] = v[0];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int u = 0; u < 2; u++)
+#pragma unroll
+    for (int w = 0; w < 2; w++) {
+      const int o = o0 + ty + 16 * u, i = i0 + tx + 16 * w;
+      if (o >= L.N || i >= L.K) continue;
+      const long q = L.off_w + (long)o * L.K + i;
+      if (p) {
+        const float n = adamw_one(pv[u][w], acc[u][w], mv[u][w], vv[u][w], a, c);
+        p[q] = n; mo[q] = mv[u][w]; vo[q] = vv[u][w];
+        pb[q] = __float2bfloat16(n);
+      } else {
+        g[q] = acc[u][w];
+      }
+    }
+  if (bias) {
+    const long q = L.off_b + o0 + tid;
+    const float db = sdb[tid];
+    if (p) {
+      const float n = adamw_one(bp, db, bm, bv, a, c);
+      p[q] = n; mo[q] = bm; vo[q] = bv;
+      pb[q] = __float2bfloat16(n);
+    } else {
+      g[q] = db;
+    }
+  }
+  if (blockIdx.x == gridDim.x - 1) {
+    float* d = p ? loss + *a.eidx : loss;
+    float sum = *d;
+    for (long c0 = 0; c0 < nsq; c0 += 256) {
+      red[tid] = c0 + tid < nsq ? sq[c0 + tid] : 0.0f;
+      __syncthreads();
+      if (tid < 32) {
+        // halves of 256 added pairwise: slots 128, 64, 32 apart, then across the lanes
+        float w[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) w[j] = red[tid + 32 * j];
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+          for (int j = 0; j < h; j++) w[j] += w[j + h];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) w[0] += __shfl_down_sync(0xffffffffu, w[0], o);
+        sum += w[0];
+      }
+      __syncthreads();
+    }
+    if (tid == 0) *d = sum;
+  }
+}
+
 uint64_t splitmix64(uint64_t& s) {
   uint64_t z = (s += 0x9e3779b97f4a7c15ULL);
   z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
@@ -384,8 +743,10 @@ struct pic_mlp {
   std::vector<__nv_bfloat16*> Hb;       // activations per layer (BF16); Hb[0] is the input
   float* dA = nullptr;                  // gradient work buffers
   float* dB = nullptr;
+  std::vector<float*> dZ;               // small batches: the gradient of every layer's pre-activations
   float* out = nullptr;
   float* loss = nullptr;
+  float* sq = nullptr;                  // small batches: every output's share of the loss
   int* idx = nullptr;
   int* perm = nullptr;                  // shuffled sample order of one epoch (training)
   int perm_cap = 0;
@@ -454,6 +815,14 @@ bool ensure_batch(pic_mlp* m, int n) {
   m->tb = mlp_al<float>(m, (size_t)n * m->w[m->L]);
   m->idx = mlp_al<int>(m, (size_t)n);
   if (!m->dA || !m->dB || !m->out || !m->xb || !m->tb || !m->idx) return false;
+  m->dZ.assign(m->L + 1, nullptr);
+  const int ns = n < SB_ROWS ? n : SB_ROWS;
+  for (int l = 1; l <= m->L; l++) {
+    m->dZ[l] = mlp_al<float>(m, (size_t)ns * m->w[l]);
+    if (!m->dZ[l]) return false;
+  }
+  m->sq = mlp_al<float>(m, (size_t)ns * m->w[m->L]);
+  if (!m->sq) return false;
   m->cap = n;
   return true;
 }
@@ -501,6 +870,71 @@ void backward(pic_mlp* m, const float* T, int n, float* loss, const int* eidx = 
       dH = t;
     }
   }
+}
+
+// a kernel whose launch may overlap the end of its predecessor on the stream (it waits for it on the device)
+template <class... KA, class... A>
+void sb_launch(pic_mlp* m, void (*k)(KA...), dim3 grid, int threads, const A&... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.stream = m->s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, k, KA(args)...);
+}
+
+// loss and gradients of n <= SB_ROWS rows (idx[r], or r) of X against T, then AdamW (adam given) or the gradient in
+// m->g; the loss is added to *loss (adam: to loss[epoch])
+void small_pass(pic_mlp* m, const float* X, const float* T, const int* idx, int n, float* loss, const AdamC* adam) {
+  const int L = m->L, ty = (n + SB_M - 1) / SB_M;
+  auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
+  for (int l = 1; l <= L; l++) {
+    const int in = m->w[l - 1], ou = m->w[l];
+    const dim3 grid((ou + SB_N - 1) / SB_N, ty);
+    const __nv_bfloat16* W = m->pb + m->off_w[l - 1];
+    const float* b = m->p + m->off_b[l - 1];
+    const __nv_bfloat16* H = m->Hb[l - 1];
+    const int vec = in % 8 == 0 && al16(W) && al16(H);
+    const bool last = l == L;
+    float* Z = last ? m->out : m->Z[l];
+    __nv_bfloat16* Hn = last ? nullptr : m->Hb[l];
+    const float* t = last ? T : nullptr;
+    float* dY = last ? m->dZ[L] : nullptr;
+    if (l == 1 && last) sb_launch(m, k_sb_fwd<true, true>, grid, SB_THREADS, n, ou, in, H, X, idx, W, b, Z, Hn, t, dY, m->sq, vec);
+    else if (l == 1) sb_launch(m, k_sb_fwd<true, false>, grid, SB_THREADS, n, ou, in, H, X, idx, W, b, Z, Hn, t, dY, m->sq, vec);
+    else if (last) sb_launch(m, k_sb_fwd<false, true>, grid, SB_THREADS, n, ou, in, H, X, idx, W, b, Z, Hn, t, dY, m->sq, vec);
+    else sb_launch(m, k_sb_fwd<false, false>, grid, SB_THREADS, n, ou, in, H, X, idx, W, b, Z, Hn, t, dY, m->sq, vec);
+  }
+  for (int l = L; l >= 2; l--) {
+    const int in = m->w[l - 1], ou = m->w[l];
+    const __nv_bfloat16* W = m->pb + m->off_w[l - 1];
+    const int vec = in % 8 == 0 && al16(W), vecz = ou % 4 == 0 && al16(m->dZ[l]);
+    sb_launch(m, k_sb_dx, dim3((in + SB_N - 1) / SB_N, ty), SB_THREADS, n, in, ou, m->dZ[l], W, m->Z[l - 1],
+              m->dZ[l - 1], vec, vecz);
+  }
+  SbNet net{};
+  net.L = L;
+  int blocks = 0;
+  for (int l = 1; l <= L; l++) {
+    SbLayer& q = net.l[l - 1];
+    q.dZ = m->dZ[l];
+    q.H = m->Hb[l - 1];
+    q.off_w = m->off_w[l - 1];
+    q.off_b = m->off_b[l - 1];
+    q.N = m->w[l];
+    q.K = m->w[l - 1];
+    q.tk = (q.K + SB_GT - 1) / SB_GT;
+    q.vz = q.N % 4 == 0 && al16(q.dZ);
+    q.vh = q.K % 4 == 0 && al16(q.H);
+    blocks += q.tk * ((q.N + SB_GT - 1) / SB_GT);
+    q.blocks = blocks;
+  }
+  sb_launch(m, k_sb_grad, dim3(blocks), 256, net, n, X, idx, adam ? m->p : nullptr, m->pb, m->m, m->v, m->g,
+            adam ? *adam : AdamC{}, m->sq, (long)n * m->w[L], loss);
 }
 
 }  // namespace
@@ -658,9 +1092,13 @@ int pic_mlp_status(pic_mlp* m) {
 int pic_mlp_grad(pic_mlp* m, const float* x, const float* t, int n, float* loss_host, float* grad_host) {
   if (!m || !x || !t || n < 1) return PIC_EINVAL;
   if (!ensure_batch(m, n)) return PIC_ENOMEM;
-  forward(m, x, n);
   cudaMemsetAsync(m->loss, 0, sizeof(float), m->s);
-  backward(m, t, n, m->loss);
+  if (n <= SB_ROWS) {
+    small_pass(m, x, t, nullptr, n, m->loss, nullptr);
+  } else {
+    forward(m, x, n);
+    backward(m, t, n, m->loss);
+  }
   if (loss_host) cudaMemcpyAsync(loss_host, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->s);
   if (grad_host) cudaMemcpyAsync(grad_host, m->g, m->np * sizeof(float), cudaMemcpyDeviceToHost, m->s);
   return cudaStreamSynchronize(m->s) == cudaSuccess ? PIC_OK : PIC_ECUDA;
@@ -707,12 +1145,18 @@ int pic_mlp_train(pic_mlp* m, const float* x, const float* t, int n, int epochs,
   if (nsteps > 0)
     cudaMemcpyAsync(m->ctab, ctab.data(), (size_t)nsteps * sizeof(float2), cudaMemcpyHostToDevice, m->s);
   cudaMemsetAsync(m->eidx, 0, sizeof(int), m->s);
-  // one epoch's launches (nbat batches of gather, forward, backward, AdamW, then the epoch counter), with
+  // one epoch's launches (per batch of up to SB_ROWS rows the small-batch products with AdamW, else gather, forward,
+  // backward and AdamW; then the epoch counter), with
   // the epoch index and the step's bias corrections read on the device
   auto epoch_launches = [&](cudaStream_t s) {
     cudaStream_t keep = m->s;
     m->s = s;
     for (int k = 0; k < nbat; k++) {
+      if (batch <= SB_ROWS) {
+        const AdamC a{lr, b1, b2, eps, weight_decay, m->ctab, m->eidx, nbat, k};
+        small_pass(m, x, t, m->perm + (long)k * batch, batch, m->curve, &a);
+        continue;
+      }
       k_gather_rows<<<batch, 64, 0, s>>>(batch, m->perm + (long)k * batch, x, m->w[0], t, m->w[m->L], m->xb, m->tb);
       forward(m, m->xb, batch);
       backward(m, m->tb, batch, m->curve, m->eidx);
@@ -722,8 +1166,8 @@ int pic_mlp_train(pic_mlp* m, const float* x, const float* t, int n, int epochs,
     k_next_epoch<<<1, 1, 0, s>>>(m->eidx);
     m->s = keep;
   };
-  // The epoch is captured once in a CUDA graph on a private stream and replayed (about 20 launches per
-  // batch otherwise: at batch 64 the step is launch-bound). Where capture is not possible, the same
+  // The epoch is captured once in a CUDA graph on a private stream and replayed (8 launches per batch for four layers:
+  // at batch 64 the step is launch-bound). Where capture is not possible, the same
   // launches run directly on the caller's stream.
   cudaStream_t ts = nullptr;
   cudaGraphExec_t ge = nullptr;
