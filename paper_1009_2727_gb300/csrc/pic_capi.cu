@@ -364,6 +364,14 @@ struct Sim : SimBase {
       q->id = al<uint32_t>(cap);
       if (!okp || !q->ux || !q->uy || !q->uz || !q->w || !q->id) return c->fail(PIC_ENOMEM, "particle allocation failed");
     }
+    if (!CellPos<T>::value) {
+      // FP64: a block's time is its particles times the SM's narrow FP64 pipe (1024 particles of cubic order took 320 us),
+      // so chunks are small enough for every SM to take several: 64 chunks of up to 1024 left 88 SMs idle
+      int dev = 0, nsm = 1;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+      chunk_max = std::min(1024, std::max(128, (cap / (16 * nsm) + 127) / 128 * 128));
+    }
     const int ntiles = sb.ntx * sb.ntz;
     const int xblocks = (g.gx_hi - g.gx_lo + ip.xblock - 1) / ip.xblock;
     const int inj_chunks = xblocks * 4;

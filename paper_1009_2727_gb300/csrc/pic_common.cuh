@@ -215,6 +215,7 @@ struct Ctrl {
 // Constants of the particle push (one run, one step).
 struct PushConst {
   double dx, dz, dt, z0;            // FP64 path
+  double idx, idz;                  // 1/dx, 1/dz
   double xlo, xhi, zlo, zhi;        // FP64 path removal bounds [m]
   int cx_lo, cx_hi, cz_lo, cz_hi;   // mixed path removal bounds [cells, hi exclusive]
   float dtdx, dtdz;                 // mixed path

@@ -20,6 +20,10 @@ namespace picgb {
 namespace {
 
 constexpr int PB_THREADS = 256;
+// Blocks per SM the push is compiled for. FP32: five hide the shared-memory latency best (48 registers). FP64: the FP64
+// pipe serves two lanes a cycle and SM, so that two blocks keep it busy; at 128 registers nothing of a particle spills.
+template <class T>
+constexpr int push_blocks() { return sizeof(T) == 8 ? 2 : 5; }
 
 template <int ORDER>
 struct St;
@@ -97,6 +101,14 @@ __device__ __forceinline__ void interp2(const typename Vec2<T>::type* F, int ld,
 }
 
 
+// Tests on the bits: a comparison of doubles runs on the FP64 pipe, which serves two lanes a cycle and SM and bounds the
+// FP64 push. v != 0; t in [0, 1) at or above 1/2; a finite position of fewer than 2^30 cells
+__device__ __forceinline__ bool nonzero(float v) { return v != 0.0f; }
+__device__ __forceinline__ bool nonzero(double v) { return ((uint64_t)__double_as_longlong(v) << 1) != 0; }
+__device__ __forceinline__ bool upper_half(float t) { return t >= 0.5f; }
+__device__ __forceinline__ bool upper_half(double t) { return __double2hiint(t) >= 0x3fe00000; }
+__device__ __forceinline__ bool small_pos(double v) { return (__double2hiint(v) & 0x7fffffff) < 0x41d00000; }
+
 // products and differences rounded on their own (no contraction into FMA)
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
@@ -155,7 +167,7 @@ __device__ __forceinline__ void deposit(T* Jx, long cs, int ld, const T* S0x, co
 #pragma unroll
       for (int a = 0; a < NDX - 1; a++) {
         const T v = Px[a] * fzb;
-        if (v != T(0)) atomicAdd(Jx + (Idx)a * ld + b, v);
+        if (nonzero(v)) atomicAdd(Jx + (Idx)a * ld + b, v);
       }
     }
   }
@@ -167,7 +179,7 @@ __device__ __forceinline__ void deposit(T* Jx, long cs, int ld, const T* S0x, co
 #pragma unroll
       for (int b = 0; b < ND; b++) {
         const T v = ay * S0z[b] + by * DSz[b];
-        if (v != T(0)) atomicAdd(Jy + (Idx)a * ld + b, v);
+        if (nonzero(v)) atomicAdd(Jy + (Idx)a * ld + b, v);
       }
     }
   }
@@ -187,7 +199,7 @@ __device__ __forceinline__ void deposit(T* Jx, long cs, int ld, const T* S0x, co
         T v;
         if (JZ == 2) v = sub_rn(mul_rn(fxa, Pz[b]), mul_rn(Sxi[a], Pzi[b]));
         else v = fxa * Pz[b];
-        if (v != T(0)) atomicAdd(Jz + (Idx)a * ld + b, v);
+        if (nonzero(v)) atomicAdd(Jz + (Idx)a * ld + b, v);
       }
     }
   }
@@ -399,14 +411,15 @@ __device__ __forceinline__ bool push_one(const T* __restrict__ Eb, const T* __re
     fzh = tz >= T(0.5) ? fz : fz - 1; tzh = tz >= T(0.5) ? tz - T(0.5) : tz + T(0.5);
   } else {
     x = p.x[pi]; z = p.z[pi];
-    X = x / pc.dx; Z = (z - pc.z0) / pc.dz;
-    if (SMEM && (!(X == X) || !(Z == Z) || fabs(X) > 1e9 || fabs(Z) > 1e9)) return false;
-    fx = (int)floor(X); fz = (int)floor(Z);
+    X = x * pc.idx; Z = (z - pc.z0) * pc.idz;
+    if (SMEM && (!small_pos(X) || !small_pos(Z))) return false;
+    const double Xf = floor(X), Zf = floor(Z);
+    fx = (int)Xf; fz = (int)Zf;
     if (SMEM && !box.in(fx, fz)) return false;
-    tx = T(X - fx); tz = T(Z - fz);
-    const double Xh = X - 0.5, Zh = Z - 0.5;
-    fxh = (int)floor(Xh); fzh = (int)floor(Zh);
-    txh = T(Xh - fxh); tzh = T(Zh - fzh);
+    tx = T(X - Xf); tz = T(Z - Zf);
+    const bool ux2 = upper_half(tx), uz2 = upper_half(tz);
+    fxh = ux2 ? fx : fx - 1; txh = tx + (ux2 ? T(-0.5) : T(0.5));
+    fzh = uz2 ? fz : fz - 1; tzh = tz + (uz2 ? T(-0.5) : T(0.5));
   }
   T ux = pword<ST>(p.ux, pi, rec, RW_UX), uy = pword<ST>(p.uy, pi, rec, RW_UY), uz = pword<ST>(p.uz, pi, rec, RW_UZ);
   T wxi[NG], wzi[NG], wxh[NG], wzh[NG];
@@ -490,8 +503,8 @@ __device__ __forceinline__ bool push_one(const T* __restrict__ Eb, const T* __re
     vz = (uz - u0 * __fdividef(dg, pc.g0_f)) * ig1;
   } else {
     T umx = ux + k * Ex, umy = uy + k * Ey, umz = uz + k * Ez;
-    const T gm = sqrt(T(1) + (umx * umx + umy * umy + umz * umz) * ic2);
-    const T tbx = k * Bx / gm, tby = k * By / gm, tbz = k * Bz / gm;
+    const T kig = k * rsqrt(T(1) + (umx * umx + umy * umy + umz * umz) * ic2);
+    const T tbx = kig * Bx, tby = kig * By, tbz = kig * Bz;
     const T t2 = tbx * tbx + tby * tby + tbz * tbz;
     const T sf = T(2) / (T(1) + t2);
     const T sbx = sf * tbx, sby = sf * tby, sbz = sf * tbz;
@@ -502,8 +515,8 @@ __device__ __forceinline__ bool push_one(const T* __restrict__ Eb, const T* __re
     const T ply = umy + (upz * sbx - upx * sbz);
     const T plz = umz + (upx * sby - upy * sbx);
     ux = plx + k * Ex; uy = ply + k * Ey; uz = plz + k * Ez;
-    const T g1 = sqrt(T(1) + (ux * ux + uy * uy + uz * uz) * ic2);
-    vx = ux / g1; vy = uy / g1; vz = uz / g1;
+    const T ig1 = rsqrt(T(1) + (ux * ux + uy * uy + uz * uz) * ic2);
+    vx = ux * ig1; vy = uy * ig1; vz = uz * ig1;
   }
   // move
   int fxn, fzn;
@@ -524,9 +537,10 @@ __device__ __forceinline__ bool push_one(const T* __restrict__ Eb, const T* __re
   } else {
     xn = x + pc.dt * (double)vx;
     zn = z + pc.dt * (double)vz;
-    const double Xn = xn / pc.dx, Zn = (zn - pc.z0) / pc.dz;
-    fxn = (int)floor(Xn); fzn = (int)floor(Zn);
-    txn = T(Xn - fxn); tzn = T(Zn - fzn);
+    const double Xn = xn * pc.idx, Zn = (zn - pc.z0) * pc.idz;
+    const double Xf = floor(Xn), Zf = floor(Zn);
+    fxn = (int)Xf; fzn = (int)Zf;
+    txn = T(Xn - Xf); tzn = T(Zn - Zf);
   }
   // the lab-fixed ion of the particle's lattice site (mixed path): J_z of the
   // pair is exactly zero when electron and ion made the same move (the cold
@@ -642,7 +656,7 @@ __device__ __forceinline__ bool particle_cell(const Particles<T>& p, int pi, con
     frame_z(c, oz, pc.fr0_sz, pc.fr0_fz, fz, tz);
     return true;
   } else {
-    const double X = p.x[pi] / pc.dx, Z = (p.z[pi] - pc.z0) / pc.dz;
+    const double X = p.x[pi] * pc.idx, Z = (p.z[pi] - pc.z0) * pc.idz;
     if (!(X == X) || !(Z == Z) || fabs(X) > 1e9 || fabs(Z) > 1e9) return false;
     fx = (int)floor(X); fz = (int)floor(Z);
     return true;
@@ -808,7 +822,7 @@ __device__ __forceinline__ void push_chunk(const GridP& g, const T* gE, const T*
 }
 
 template <class T, int ORDER, bool MC>
-__global__ void __launch_bounds__(PB_THREADS, 5) k_push(GridP g, const T* gE, const T* gB, T* gJ, Particles<T> p,
+__global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push(GridP g, const T* gE, const T* gB, T* gJ, Particles<T> p,
                                                      Chunk* chunks, Ctrl* ctrl, int cap_nodes, int tile_z,
                                                      PushDefer pd, PushConst pc) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -920,8 +934,8 @@ __global__ void k_sort_key(GridP g, Particles<T> p, SortBufs sb, const Ctrl* ctr
     cx = cell_x(c);
     frame_z(c, oz, g.fr_sz, g.fr_fz, cz, tz);
   } else {
-    cx = (int)floor(p.x[i] / g.dx);
-    cz = (int)floor((p.z[i] - g.z0) / g.dz);
+    cx = (int)floor(p.x[i] * g.idx);
+    cz = (int)floor((p.z[i] - g.z0) * g.idz);
   }
   cx = min(max(cx, 0), g.nx - 1);
   cz = min(max(cz, 0), g.nz - 1);
@@ -1101,8 +1115,8 @@ __device__ __forceinline__ void inject_block(const GridP& g, const Particles<T>&
     Chunk c;
     c.p0 = (int)start; c.p1 = (int)(start + cnt);
     c.ix0 = g.gx_lo + cx0; c.ix1 = g.gx_lo + cx0 + ncx - 1;
-    const double za = ((ip.m_beg + r0 + 0.5) * ip.h - ip.beta * kC * ip.t - g.z0) / gdz;
-    const double zb = ((ip.m_beg + r0 + nr - 1 + 0.5) * ip.h - ip.beta * kC * ip.t - g.z0) / gdz;
+    const double za = ((ip.m_beg + r0 + 0.5) * ip.h - ip.beta * kC * ip.t - g.z0) * g.idz;
+    const double zb = ((ip.m_beg + r0 + nr - 1 + 0.5) * ip.h - ip.beta * kC * ip.t - g.z0) * g.idz;
     c.iz0 = (int)floor(za); c.iz1 = (int)floor(zb);
     chunks[ci] = c;
   }
@@ -1132,7 +1146,7 @@ __global__ void k_push_batch_reset(const StepArgs<T>* a, int nruns, int* counter
 // the window kernel over all runs' chunks: blocks take (run, chunk) pairs from one queue; the run's push
 // constants, geometry and particle arrays are copied to shared memory when a block changes run
 template <class T, int ORDER>
-__global__ void __launch_bounds__(PB_THREADS, 5) k_push_batch(const StepArgs<T>* a, int nruns, int* counter,
+__global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push_batch(const StepArgs<T>* a, int nruns, int* counter,
                                                            int cap_nodes, int tile_z) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
@@ -1269,6 +1283,7 @@ PushConst push_const(const GridP& g, double q, double m, double gamma_b, int fr1
                      int mlo) {
   PushConst pc;
   pc.dx = g.dx; pc.dz = g.dz; pc.dt = g.dt; pc.z0 = g.z0;
+  pc.idx = g.idx; pc.idz = g.idz;
   pc.xlo = g.gx_lo * g.dx; pc.xhi = g.gx_hi * g.dx;
   pc.zlo = g.z0 + g.gz_lo * g.dz; pc.zhi = g.z0 + g.gz_hi * g.dz + g.dz;
   pc.cx_lo = g.gx_lo; pc.cx_hi = g.gx_hi; pc.cz_lo = g.gz_lo; pc.cz_hi = g.gz_hi + 1;
