@@ -201,6 +201,11 @@ struct Sim : SimBase {
     if (filt_gather) ok = ok && block(f.fE) && block(f.fB);
     nodal = cf.gather_scheme == 1;
     if (nodal) ok = ok && block(f.nE) && block(f.nB);
+    if ((filt_gather || filt_J) && filter_is_wide<T>(fs)) {
+      f.wide = al<T>(6 * N);
+      ok = ok && f.wide;
+      if (filt_J) ok = ok && block(f.Jf);
+    }
     if (!ok) return c->fail(PIC_ENOMEM, "field allocation failed");
     if (cf.pml_cells > 0) {
       f.Byx = grid(); f.Byz = grid(); f.Eyx = grid(); f.Eyz = grid();
@@ -625,7 +630,7 @@ struct Sim : SimBase {
     tstart(1);
     const bool fused = launch_faraday_fused<T>(g, f, pt, h.a2, h.b2, cf.theta, friedman, fs, filt_gather, tmaps,
                                                ctrl, c->stream);
-    if (!fused) launch_faraday<T>(g, f, pt, h.a2, h.b2, cf.theta, friedman, c->stream);
+    if (!fused) launch_faraday<T>(g, f, pt, h.a2, h.b2, cf.theta, friedman, tmaps, ctrl, c->stream);
     // 2. gather copies (interpolated to the nodes for the 'momentum conserving' gather): B_avg, and E^n
     //    unless the fused kernel filtered it
     launch_filter_fields<T>(g, f, fs, filt_gather, tmaps, ctrl, c->stream, fused ? 3 : 0);

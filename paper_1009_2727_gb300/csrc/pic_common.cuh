@@ -95,6 +95,8 @@ struct FieldPtrs {
   T* nE[3];     // 'momentum conserving' gather: the copies interpolated to the nodes (3 x cs each, contiguous)
   T* nB[3];
   T* Byx; T* Byz; T* Eyx; T* Eyz;  // split PML parts (full-size, used in the PML only)
+  T* wide;      // scratch of the wide filters' x pass (6 x cs), null when the tile kernels filter
+  T* Jf[3];     // the filtered current (wide filters of the current)
 };
 
 struct FilterSpec {
@@ -261,9 +263,6 @@ __device__ __forceinline__ void weights1(R t, R* w) {
 
 // ---------------------------------------------------------------------------
 // Launchers (defined in the .cu files, instantiated for float and double).
-template <class T>
-void launch_faraday(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, double a2, double b2,
-                    double theta, bool friedman, cudaStream_t s);
 // TMA descriptors of the 3-component blocks read by the tile kernels (a 3D tensor
 // (nz+1) x (nx+1) x 3 per block; out-of-range elements read as zero)
 struct TileMaps {
@@ -279,6 +278,9 @@ struct TileMaps {
   bool ok, r_ok;
 };
 template <class T>
+void launch_faraday(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, double a2, double b2,
+                    double theta, bool friedman, const TileMaps& tm, Ctrl* ctrl, cudaStream_t s);
+template <class T>
 bool make_tile_maps(const GridP& g, const FieldPtrs<T>& f, int H, TileMaps& tm);
 // the gather filter of components c_first..5 (E^n: 0..2, B_avg: 3..5)
 template <class T>
@@ -289,6 +291,10 @@ template <class T>
 bool launch_faraday_fused(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, double a2, double b2,
                           double theta, bool friedman, const FilterSpec& fs, bool filt_gather, const TileMaps& tm,
                           Ctrl* ctrl, cudaStream_t s);
+// a filter the tile kernels have no unrolled form for, with a halo of at least eight cells: it takes the two-pass
+// kernels, with f.wide (and f.Jf for the current) allocated
+template <class T>
+bool filter_is_wide(const FilterSpec& fs);
 template <class T>
 void launch_ampere(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, const FilterSpec& fs, bool filter_on,
                    const double* ion_x, const double* ion_c, double ion_coef, const TileMaps& tm, Ctrl* ctrl,

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(FT_Z* FT_TY) k_filter_fields(GridP g, FieldPtr
 // and, under Friedman damping, E^{n-1} and E-bar on the tile and a one-node halo (boxes of FT_X + 2 rows
 // by FT_Z + 8 columns, starting 16-byte aligned at k0 - 4). E_eff (Eq. 7) is formed in place of the
 // staged E^{n-1}; B, B_avg and E-bar are updated as in k_faraday, then F(E^n) is written for the gather
-// (k_filter_fields then filters B_avg only).
+// (k_filter_fields then filters B_avg only). PT = 0: no filter, E^n on the small boxes too.
 template <class T, bool FRIED, bool CK, int PT>
 __device__ __forceinline__ void faraday_fused_tile(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt,
                                                    const FarK<T>& q, const FilterTaps<T>& ft,
@@ -526,7 +526,7 @@ __device__ __forceinline__ void faraday_fused_tile(const GridP& g, const FieldPt
   constexpr int SX = FT_X + 2, SZ = FT_Z + 2, RZ = FT_Z + 8;
   // the staged boxes' geometry as constants: a stride-1 filter of PT passes has halo H = PT (the host
   // checks that the tile maps were built for it), the boxes are FT_X + 2 H rows of FT_Z + 2 HZ
-  constexpr int H = PT, HZ = (PT + 3) & ~3, BX = FT_X + 2 * H, BZ = FT_Z + 2 * HZ;
+  constexpr int H = PT > 0 ? PT : 1, HZ = (H + 3) & ~3, BX = FT_X + 2 * H, BZ = FT_Z + 2 * HZ;
   constexpr int LINE = 128 / (int)sizeof(T), stride = (BX * BZ + LINE - 1) / LINE * LINE;
   extern __shared__ __align__(128) unsigned char smraw[];
   const int rstride = ring_stride<T>();
@@ -612,6 +612,7 @@ __device__ __forceinline__ void faraday_fused_tile(const GridP& g, const FieldPt
     esz = BZ;
   }
   faraday_update<T, CK>(g, f, pt, q, Eep, esz, i0, k0, bold);
+  if constexpr (PT == 0) return;
   // the gather copies of E^n: the filter of the staged boxes (its scratch overwrites E_eff: every thread's
   // B update has read it first)
   __syncthreads();
@@ -630,11 +631,12 @@ __global__ void __launch_bounds__(FT_Z* FT_TY, 4) k_faraday_fused(GridP g, Field
 }
 
 // Ampere + PML-E, with the current (plus the ion column current) filtered in the tile first
-template <class T, bool FILT, int PT>
+// DIRECT: the current comes filtered from f.Jf (no staging), one component per block
+template <class T, bool FILT, int PT, bool DIRECT = false>
 __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt,
                                             const FilterTaps<T>& ft, const double* ion_x, const double* ion_c,
                                             double ion_coef, const CUtensorMap* pmapJ, const TileMaps& tm,
-                                            Ctrl* ctrl, int tile_k, int tile_i) {
+                                            Ctrl* ctrl, int tile_k, int tile_i, int c_first = 0, int c_last = 2) {
   extern __shared__ __align__(128) unsigned char smraw[];
   T* tile0 = reinterpret_cast<T*>(align128(smraw));
   T* tile1 = tile0 + tile_stride<T>(tm);
@@ -651,30 +653,31 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (leader) stage<T>(tile0, pmapJ, 0, gk0, gi0, &bar[0], tm);
+  if (!DIRECT && leader) stage<T>(tile0, pmapJ, 0, gk0, gi0, &bar[0], tm);
   const T dt = grid_dt<T>(g);
   const T c2 = T(kC * kC);
   const T ie0 = T(1.0 / kEps0);
   const T idx = grid_idx<T>(g), idz = grid_idz<T>(g);
   const double c2d = kC * kC;
   const int k = k0 + threadIdx.x;
-  for (int c = 0; c < 3; c++) {
+  for (int c = c_first; c <= c_last; c++) {
     T* A = (c & 1) ? tile1 : tile0;
-    if (leader && c + 1 < 3) stage<T>((c & 1) ? tile0 : tile1, pmapJ, c + 1, gk0, gi0, &bar[(c + 1) & 1], tm);
+    if (!DIRECT && leader && c + 1 < 3) stage<T>((c & 1) ? tile0 : tile1, pmapJ, c + 1, gk0, gi0, &bar[(c + 1) & 1], tm);
     int vi0, vi1, vk0, vk1;
     valid_range(c, g.nx, g.nz, vi0, vi1, vk0, vk1);
     // E^n and the B^{n+1/2} values of the curl for the thread's rows, loaded before the wait for the
     // staged current and the filter, so that their latency overlaps both
     constexpr int NR = FT_X / FT_TY;
-    T e0[NR], ba[NR], bb[NR], bc[NR], bd[NR];
+    T e0[NR], ba[NR], bb[NR], bc[NR], bd[NR], jd[NR];
 #pragma unroll
     for (int r = 0; r < NR; r++) {
       const int i = i0 + threadIdx.y + r * FT_TY;
       const long p = (long)i * g.ld + k;
       const bool v = i <= g.nx && k <= g.nz && i >= vi0 && i <= vi1 && k >= vk0 && k <= vk1;
-      e0[r] = ba[r] = bb[r] = bc[r] = bd[r] = T(0);
+      e0[r] = ba[r] = bb[r] = bc[r] = bd[r] = jd[r] = T(0);
       if (v) {
         e0[r] = f.E[c][p];
+        if (DIRECT) jd[r] = f.Jf[c][p];
         if (c == 0) {
           ba[r] = f.B[1][p]; bb[r] = f.B[1][p - 1];
         } else if (c == 2) {
@@ -684,11 +687,11 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
         }
       }
     }
-    if (!block_wait(&bar[c & 1], (c >> 1) & 1)) {
+    if (!DIRECT && !block_wait(&bar[c & 1], (c >> 1) & 1)) {
       tile_timeout(ctrl, &bar[0], &bar[1]);
       return;
     }
-    if (c == 2 && ion_x != nullptr) {
+    if (!DIRECT && c == 2 && ion_x != nullptr) {
       // rigid ion-column current added to Jz before the filter (each thread
       // converts its columns' factors once)
       T cz[(256 + FT_Z - 1) / FT_Z];
@@ -726,7 +729,7 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
         f.Eo[c][p] = T(0);
         continue;
       }
-      const T jv = FILT ? Zb[ti * FT_Z + threadIdx.x] : A[(ti + tm.H) * tm.BZ + threadIdx.x + tm.HZ];
+      const T jv = DIRECT ? jd[r] : FILT ? Zb[ti * FT_Z + threadIdx.x] : A[(ti + tm.H) * tm.BZ + threadIdx.x + tm.HZ];
       const T eo = e0[r];
       T en;
       if (c == 0) {
@@ -755,8 +758,15 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
     };
     if (clear) rows(std::false_type{});
     else rows(std::true_type{});
-    __syncthreads();
+    if (!DIRECT) __syncthreads();
   }
+}
+
+template <class T>
+__global__ void __launch_bounds__(FT_Z* FT_TY) k_ampere_direct(GridP g, FieldPtrs<T> f, PmlTabs pt, FilterTaps<T> ft,
+                                                              TileMaps tm, Ctrl* ctrl) {
+  ampere_tile<T, false, 0, true>(g, f, pt, ft, nullptr, nullptr, 0.0, nullptr, tm, ctrl, blockIdx.x, blockIdx.y,
+                                 blockIdx.z, blockIdx.z);
 }
 
 template <class T, bool FILT, int PT>
@@ -765,6 +775,238 @@ __global__ void __launch_bounds__(FT_Z* FT_TY, sizeof(T) == 4 ? 4 : 2) k_ampere(
                                                         const __grid_constant__ CUtensorMap mapJ, TileMaps tm,
                                                         Ctrl* ctrl) {
   ampere_tile<T, FILT, PT>(g, f, pt, ft, ion_x, ion_c, ion_coef, &mapJ, tm, ctrl, blockIdx.x, blockIdx.y);
+}
+
+// ---------------------------------------------------------------------------
+// Wide filters (halo above six cells, or strided): along x into a scratch block, then along z, one launch each for all
+// components. The tile kernels above stage a 16 x 64 tile with its halo on both axes; with the 35-cell halo of S(1:2:4)
+// that is 86 x 136 nodes read and 220 products per output, a third of which refill the halo. Here the halo is paid along
+// one axis at a time, each thread sums 16 outputs from a register window (128 products per eight inputs and 15 or 23
+// taps), in the order of the taps, and the intermediate stays in L2. 1536 x 224 nodes, S(1:2:4), FP32, E and
+// B: 152 -> 32 us; the current with Ampère: 98 -> 38 us. Bound by the FMA pipe and the staging round.
+constexpr int WTAPS = 2 * FILTER_HMAX + 1;
+constexpr int WPAD = 16;                  // zeros before the taps in shared memory (at least the outputs of a thread)
+constexpr int WXR = 8, WXC = 32, WXG = 8;     // x pass: consecutive rows of a thread, threads along z, groups of rows
+constexpr int WZR = 16, WZT = 32, WZB = 4;    // z pass: consecutive columns of a thread, threads and rows of a block
+
+// dense taps at offsets -H .. H
+template <class T>
+struct WideTaps {
+  T c[WTAPS];
+  int H;
+};
+
+template <class T>
+struct WideJob {
+  const T* src[6];
+  T* dst[6];
+  // the rigid ion-column current added to component ion (-1: none) as it is read: T(coef ion_x[i]) T(ion_c[k])
+  const double *ion_x, *ion_c;
+  double coef;
+  int ion;
+};
+
+// a thread's value: two z columns in FP32 (8-byte loads), one in FP64
+template <class T>
+struct WideV;
+template <>
+struct WideV<float> { typedef float2 type; static constexpr int n = 2; };
+template <>
+struct WideV<double> { typedef double type; static constexpr int n = 1; };
+__device__ __forceinline__ void wide_fma(float2& a, float t, const float2& v) {
+  a = __ffma2_rn(make_float2(t, t), v, a);
+}
+__device__ __forceinline__ void wide_fma(float& a, float t, float v) { a += t * v; }
+__device__ __forceinline__ void wide_fma(double& a, double t, double v) { a += t * v; }
+
+// acc[r] += sum over m = m0 .. m0 + 7 of c[m - r] v[m - m0], r < NR, for the terms with LO <= (m - m0) - r <= HI (the
+// block's part of the tap range: terms off it are left out, not multiplied by zero); sc[WPAD + q] = c[q]
+template <class T, class V, int NR, int LO, int HI>
+__device__ __forceinline__ void wide_block(const T* sc, int m0, const V* v, V* acc) {
+  constexpr int NT = NR + 8;   // t[j] = c[m0 - NR + j], one more in front so that the loads are whole vectors
+  static_assert(NT % 4 == 0 && WPAD % 4 == 0 && NR % 4 == 0 && NR <= WPAD, "aligned tap vectors");
+  T t[NT];
+  const T* p = sc + WPAD + m0 - NR;
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int j = 0; j < NT; j += 4) {
+      const float4 f = *reinterpret_cast<const float4*>(p + j);
+      t[j] = f.x; t[j + 1] = f.y; t[j + 2] = f.z; t[j + 3] = f.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < NT; j += 2) {
+      const double2 f = *reinterpret_cast<const double2*>(p + j);
+      t[j] = f.x; t[j + 1] = f.y;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 8; q++)
+#pragma unroll
+    for (int r = 0; r < NR; r++)
+      if (q - r >= LO && q - r <= HI) wide_fma(acc[r], t[q - r + NR], v[q]);
+}
+
+// The sums over staged inputs in(0), in(1), ...: acc[r] = sum_m c[m] in(m + r), m = 0 .. 2H. HM = H mod 4 makes the
+// first and last blocks' ranges constants; the last block of the tap range is block A = 2H / 8, and A >= NR / 8 keeps
+// the first and last blocks apart.
+template <class T, class V, int NR, int HM, class In>
+__device__ __forceinline__ void wide_sums(const T* sc, int H, const In& in, V* acc) {
+  constexpr int NB = NR / 8, ALL = 64;
+  const int A = H >> 2;
+#pragma unroll
+  for (int r = 0; r < NR; r++) acc[r] = V{};
+  V v[8];
+  auto at = [&](auto lo, auto hi, int b) {
+    in(8 * b, v);
+    wide_block<T, V, NR, decltype(lo)::value, decltype(hi)::value>(sc, 8 * b, v, acc);
+  };
+  typedef std::integral_constant<int, -ALL> None;
+  typedef std::integral_constant<int, ALL> Any;
+  at(std::integral_constant<int, 0>{}, Any{}, 0);
+  if constexpr (NB > 1) at(std::integral_constant<int, -8>{}, Any{}, 1);
+  for (int b = NB; b < A; b++) at(None{}, Any{}, b);
+  at(None{}, std::integral_constant<int, 2 * HM>{}, A);
+  if constexpr (2 * HM - 8 >= -(NR - 1)) at(None{}, std::integral_constant<int, 2 * HM - 8>{}, A + 1);
+  if constexpr (2 * HM - 16 >= -(NR - 1)) at(None{}, std::integral_constant<int, 2 * HM - 16>{}, A + 2);
+}
+// halo from which the wide kernels' blocks do not overlap
+constexpr int WMINH = 8;
+
+template <class T>
+__device__ __forceinline__ void wide_taps_to(T* sc, const WideTaps<T>& w, int tid, int nthr, int n) {
+  for (int e = tid; e < n; e += nthr) sc[e] = (e >= WPAD && e < WPAD + WTAPS) ? w.c[e - WPAD] : T(0);
+}
+constexpr int WSC = (WPAD + WTAPS + 2 * WPAD + 3) / 4 * 4;
+
+template <class T, int HM>
+__global__ void __launch_bounds__(WXC* WXG) k_wide_x(GridP g, const __grid_constant__ WideTaps<T> w,
+                                                         const __grid_constant__ WideJob<T> job) {
+  typedef typename WideV<T>::type V;
+  constexpr int CV = WideV<T>::n, NX = WXG * WXR, NIN = NX + 2 * FILTER_HMAX + 8;   // output rows; staged rows
+  __shared__ V s[NIN][WXC];
+  __shared__ __align__(16) T sc[WSC];
+  const int c = blockIdx.z, i0 = blockIdx.y * NX, k0 = blockIdx.x * WXC * CV;
+  const int lane = threadIdx.x, gy = threadIdx.y;
+  const int H = w.H, k = k0 + lane * CV;
+  wide_taps_to(sc, w, gy * WXC + lane, WXC * WXG, WSC);
+  const T* F = job.src[c];
+  const bool ion = c == job.ion;
+  T cz[CV];
+#pragma unroll
+  for (int q = 0; q < CV; q++) cz[q] = (ion && k + q <= g.nz) ? T(job.ion_c[k + q]) : T(0);
+  const int n = NX + 2 * H + 8;
+  // six rows' loads of a thread in flight
+  constexpr int U = 6;
+  for (int l0 = gy; l0 < n; l0 += WXG * U) {
+    T v[U][CV];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int li = l0 + u * WXG, i = i0 - H + li;
+      const bool in = li < n && i >= 0 && i <= g.nx;
+#pragma unroll
+      for (int q = 0; q < CV; q++) v[u][q] = T(0);
+      if (!in || k > g.nz) continue;
+      // rows are padded past nz: the pair's second value is loaded and dropped there
+      const V x = *reinterpret_cast<const V*>(F + (long)i * g.ld + k);
+      const T* xp = reinterpret_cast<const T*>(&x);
+#pragma unroll
+      for (int q = 0; q < CV; q++) v[u][q] = k + q <= g.nz ? xp[q] : T(0);
+      if (ion) {
+        const T ix = T(job.coef * job.ion_x[i]);
+#pragma unroll
+        for (int q = 0; q < CV; q++) v[u][q] += ix * cz[q];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int li = l0 + u * WXG;
+      if (li >= n) break;
+      V x;
+      T* xp = reinterpret_cast<T*>(&x);
+#pragma unroll
+      for (int q = 0; q < CV; q++) xp[q] = v[u][q];
+      s[li][lane] = x;
+    }
+  }
+  __syncthreads();
+  if (i0 + gy * WXR > g.nx || k > g.nz) return;
+  V acc[WXR];
+  wide_sums<T, V, WXR, HM>(sc, H, [&](int m, V* v) {
+#pragma unroll
+    for (int q = 0; q < 8; q++) v[q] = s[gy * WXR + m + q][lane];
+  }, acc);
+  T* D = job.dst[c];
+#pragma unroll
+  for (int r = 0; r < WXR; r++) {
+    const int i = i0 + gy * WXR + r;
+    if (i > g.nx) break;
+    T* d = D + (long)i * g.ld + k;
+    if (k + CV - 1 <= g.nz) *reinterpret_cast<V*>(d) = acc[r];
+    else *d = *reinterpret_cast<const T*>(&acc[r]);
+  }
+}
+
+template <class T, int HM>
+__global__ void __launch_bounds__(WZT* WZB) k_wide_z(GridP g, const __grid_constant__ WideTaps<T> w,
+                                                         const __grid_constant__ WideJob<T> job) {
+  // a row's staged values in groups of sixteen, four values apart, so that the 16-byte reads of eight threads (sixteen
+  // columns apart) fall in different banks
+  constexpr int NZ = WZT * WZR, NG = (NZ + 2 * FILTER_HMAX + 8 + 15) / 16, GS = 20;
+  __shared__ __align__(16) T s[WZB][NG * GS];
+  __shared__ __align__(16) T sc[WSC];
+  const int c = blockIdx.z, k0 = blockIdx.x * NZ;
+  const int t = threadIdx.x, ry = threadIdx.y;
+  const int H = w.H, i = blockIdx.y * WZB + ry;
+  wide_taps_to(sc, w, ry * WZT + t, WZT * WZB, WSC);
+  const T* F = job.src[c];
+  const int n = NZ + 2 * H + 8;
+  constexpr int U = 8;
+  for (int l0 = t; l0 < n; l0 += WZT * U) {
+    T v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int l = l0 + u * WZT, k = k0 - H + l;
+      v[u] = (l < n && i <= g.nx && k >= 0 && k <= g.nz) ? F[(long)i * g.ld + k] : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int l = l0 + u * WZT;
+      if (l < n) s[ry][(l >> 4) * GS + (l & 15)] = v[u];
+    }
+  }
+  __syncthreads();
+  const int kt = k0 + t * WZR;
+  if (i > g.nx || kt > g.nz) return;
+  T acc[WZR];
+  wide_sums<T, T, WZR, HM>(sc, H, [&](int m, T* v) {
+    const T* p = s[ry] + (t + (m >> 4)) * GS + (m & 15);   // m is a multiple of 8
+    if constexpr (sizeof(T) == 4) {
+      const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; q += 2) {
+        const double2 a = *reinterpret_cast<const double2*>(p + q);
+        v[q] = a.x; v[q + 1] = a.y;
+      }
+    }
+  }, acc);
+  T* D = job.dst[c] + (long)i * g.ld + kt;   // 16-byte aligned: ld is padded to 128 bytes
+  if (kt + WZR - 1 <= g.nz) {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int r = 0; r < WZR; r += 4)
+        *reinterpret_cast<float4*>(D + r) = make_float4(acc[r], acc[r + 1], acc[r + 2], acc[r + 3]);
+    } else {
+#pragma unroll
+      for (int r = 0; r < WZR; r += 2) *reinterpret_cast<double2*>(D + r) = make_double2(acc[r], acc[r + 1]);
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < WZR; r++)
+      if (kt + r <= g.nz) D[r] = acc[r];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -923,12 +1165,28 @@ FarK<T> faraday_coefs(double a2, double b2, double theta) {
   return q;
 }
 
+template <class T, bool CK>
+static void run_faraday_staged(dim3 grd, dim3 blk, cudaStream_t s, const GridP& g, const FieldPtrs<T>& f,
+                               const PmlTabs& pt, const FarK<T>& q, const TileMaps& tm, Ctrl* ctrl) {
+  const size_t sm = (size_t)9 * ring_stride<T>() * sizeof(T) + 128;
+  const int e = tm.Ebase[0] == (const void*)f.E[0] ? 0 : 1, b = tm.Ebbase[0] == (const void*)f.Eb[0] ? 0 : 1;
+  cudaFuncSetAttribute(k_faraday_fused<T, true, CK, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_faraday_fused<T, true, CK, 0><<<grd, blk, sm, s>>>(g, f, pt, q, FilterTaps<T>{}, tm.Er[e], tm.Er[1 - e], tm.Eb[b],
+                                                        ctrl);
+}
+
 template <class T>
 void launch_faraday(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, double a2, double b2, double theta,
-                    bool friedman, cudaStream_t s) {
+                    bool friedman, const TileMaps& tm, Ctrl* ctrl, cudaStream_t s) {
   const FarK<T> q = faraday_coefs<T>(a2, b2, theta);
   dim3 blk(FT_Z, FT_TY), grd((g.nz + 1 + FT_Z - 1) / FT_Z, (g.nx + 1 + FT_X - 1) / FT_X);
   const bool ck = b2 != 0.0;
+  if (friedman && tm.ok && tm.r_ok) {
+    // Friedman's nine components staged by TMA (30 -> 26 us at 1536 x 224 nodes, FP32, against loads by the threads)
+    if (ck) run_faraday_staged<T, true>(grd, blk, s, g, f, pt, q, tm, ctrl);
+    else run_faraday_staged<T, false>(grd, blk, s, g, f, pt, q, tm, ctrl);
+    return;
+  }
   if (friedman) {
     if (ck) k_faraday<T, true, true><<<grd, blk, 0, s>>>(g, f, pt, q);
     else k_faraday<T, true, false><<<grd, blk, 0, s>>>(g, f, pt, q);
@@ -1070,11 +1328,58 @@ static void run_filter_fields(dim3 grd, dim3 blk, size_t sm, cudaStream_t s, con
   k_filter_fields<T, PT><<<grd, blk, sm, s>>>(g, f, ft, mE, tm.Bavg, tm, ctrl, c_first);
 }
 
+// the taps at offsets -H .. H, strides written out
+template <class T>
+static WideTaps<T> wide_taps(const FilterTaps<T>& ft) {
+  WideTaps<T> w{};
+  w.H = ft.H;
+  for (int j = 0; j <= 2 * ft.P; j++) w.c[j * ft.s] = ft.c[j];
+  return w;
+}
+
+template <class T, int HM>
+static void run_wide_h(const GridP& g, const WideTaps<T>& w, WideJob<T> job, T* scratch, int ncomp, cudaStream_t s) {
+  T* dst[6];
+  for (int c = 0; c < ncomp; c++) { dst[c] = job.dst[c]; job.dst[c] = scratch + c * g.cs; }
+  constexpr int XC = WXC * WideV<T>::n, XR = WXG * WXR, ZC = WZT * WZR;
+  k_wide_x<T, HM><<<dim3((g.nz + XC) / XC, (g.nx + XR) / XR, ncomp), dim3(WXC, WXG), 0, s>>>(g, w, job);
+  for (int c = 0; c < ncomp; c++) { job.src[c] = job.dst[c]; job.dst[c] = dst[c]; }
+  job.ion = -1;
+  k_wide_z<T, HM><<<dim3((g.nz + ZC) / ZC, (g.nx + WZB) / WZB, ncomp), dim3(WZT, WZB), 0, s>>>(g, w, job);
+}
+
+template <class T>
+static void run_wide(const GridP& g, const WideTaps<T>& w, const WideJob<T>& job, T* scratch, int ncomp,
+                     cudaStream_t s) {
+  switch (w.H & 3) {
+    case 0: run_wide_h<T, 0>(g, w, job, scratch, ncomp, s); break;
+    case 1: run_wide_h<T, 1>(g, w, job, scratch, ncomp, s); break;
+    case 2: run_wide_h<T, 2>(g, w, job, scratch, ncomp, s); break;
+    default: run_wide_h<T, 3>(g, w, job, scratch, ncomp, s); break;
+  }
+}
+
+template <class T>
+bool filter_is_wide(const FilterSpec& fs) {
+  const FilterTaps<T> ft = make_taps<T>(fs);
+  return ft.H >= WMINH && filter_pt(ft) == 0;
+}
+
 template <class T>
 void launch_filter_fields(const GridP& g, const FieldPtrs<T>& f, const FilterSpec& fs, bool enabled,
                           const TileMaps& tm, Ctrl* ctrl, cudaStream_t s, int c_first) {
   if (!enabled) return;
   const FilterTaps<T> ft = make_taps<T>(fs);
+  if (f.wide) {
+    WideJob<T> job{};
+    for (int c = 0; c < 3; c++) {
+      job.src[c] = f.E[c]; job.dst[c] = f.fE[c];
+      job.src[3 + c] = f.Bavg[c]; job.dst[3 + c] = f.fB[c];
+    }
+    job.ion = -1;
+    run_wide<T>(g, wide_taps(ft), job, f.wide, 6, s);
+    return;
+  }
   dim3 grd((g.nz + 1 + FT_Z - 1) / FT_Z, (g.nx + 1 + FT_X - 1) / FT_X), blk(FT_Z, FT_TY);
   const size_t sm = tile_smem<T>(tm, ft.H);
   const CUtensorMap& mE = tm.Ebase[0] == (const void*)f.E[0] ? tm.E[0] : tm.E[1];
@@ -1170,6 +1475,15 @@ void launch_ampere(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, con
   dim3 grd((g.nz + 1 + FT_Z - 1) / FT_Z, (g.nx + 1 + FT_X - 1) / FT_X), blk(FT_Z, FT_TY);
   const CUtensorMap& mJ = tm.Jbase[0] == (const void*)f.J[0] ? tm.J[0] : tm.J[1];
   const size_t sm = tile_smem<T>(tm, filter_on ? ft.H : 0);
+  if (filter_on && f.wide) {
+    WideJob<T> job{};
+    for (int c = 0; c < 3; c++) { job.src[c] = f.J[c]; job.dst[c] = f.Jf[c]; }
+    job.ion = ion_x ? 2 : -1;
+    job.ion_x = ion_x; job.ion_c = ion_c; job.coef = ion_coef;
+    run_wide<T>(g, wide_taps(ft), job, f.wide, 3, s);
+    k_ampere_direct<T><<<dim3(grd.x, grd.y, 3), blk, 0, s>>>(g, f, pt, ft, tm, ctrl);
+    return;
+  }
   if (!filter_on) {
     run_ampere<T, false, 0>(grd, blk, sm, s, g, f, pt, ft, ion_x, ion_c, ion_coef, mJ, tm, ctrl);
     return;
@@ -1186,9 +1500,9 @@ void launch_ampere(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, con
 }
 
 template void launch_faraday<float>(const GridP&, const FieldPtrs<float>&, const PmlTabs&, double, double, double,
-                                    bool, cudaStream_t);
+                                    bool, const TileMaps&, Ctrl*, cudaStream_t);
 template void launch_faraday<double>(const GridP&, const FieldPtrs<double>&, const PmlTabs&, double, double, double,
-                                     bool, cudaStream_t);
+                                     bool, const TileMaps&, Ctrl*, cudaStream_t);
 template <class T>
 FilterTaps<T> filter_taps(const FilterSpec& fs) { return make_taps<T>(fs); }
 template <class T>
@@ -1198,6 +1512,7 @@ size_t tile_smem_bytes(const TileMaps& tm, int H) { return tile_smem<T>(tm, H); 
 
 #define INSTF(T)                                                                                                 \
   template FarK<T> faraday_coefs<T>(double, double, double);                                                     \
+  template bool filter_is_wide<T>(const FilterSpec&);                                                            \
   template FilterTaps<T> filter_taps<T>(const FilterSpec&);                                                      \
   template int filter_taps_class<T>(const FilterTaps<T>&);                                                       \
   template size_t tile_smem_bytes<T>(const TileMaps&, int);                                                      \
