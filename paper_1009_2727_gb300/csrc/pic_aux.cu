@@ -509,6 +509,8 @@ __global__ void k_shift_chunks(Chunk* c, const Ctrl* ctrl, int sh) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= ctrl->nchunks) return;
   if (c[j].ix0 <= c[j].ix1) { c[j].iz0 -= sh; c[j].iz1 -= sh; }
+  c[j].zlo -= (uint32_t)sh << 16;   // the stored cells shift with the grid (k_shift_particles)
+  c[j].zhi -= (uint32_t)sh << 16;
 }
 
 template <class T>

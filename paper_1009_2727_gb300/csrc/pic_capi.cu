@@ -369,13 +369,16 @@ struct Sim : SimBase {
       q->id = al<uint32_t>(cap);
       if (!okp || !q->ux || !q->uy || !q->uz || !q->w || !q->id) return c->fail(PIC_ENOMEM, "particle allocation failed");
     }
-    if (!CellPos<T>::value) {
-      // FP64: a block's time is its particles times the SM's narrow FP64 pipe (1024 particles of cubic order took 320 us),
-      // so chunks are small enough for every SM to take several: 64 chunks of up to 1024 left 88 SMs idle
+    {
+      // Chunks small enough for every SM to take several. FP64: a block's time is its particles times the SM's narrow
+      // FP64 pipe (1024 particles of cubic order took 320 us; 64 chunks of up to 1024 left 88 SMs idle). Mixed: below 512
+      // particles the window's staging outweighs the balance (638 thousand electrons on 8 x 32 tiles: 215 us per step
+      // in chunks of up to 1024, 202 in 512, 203 in 256; ensembles of 3 million per run are fastest in whole tiles).
       int dev = 0, nsm = 1;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-      chunk_max = std::min(1024, std::max(128, (cap / (16 * nsm) + 127) / 128 * 128));
+      if (CellPos<T>::value) chunk_max = std::min(4096, std::max(512, (cap / (8 * nsm) + 255) / 256 * 256));
+      else chunk_max = std::min(1024, std::max(128, (cap / (16 * nsm) + 127) / 128 * 128));
     }
     const int ntiles = sb.ntx * sb.ntz;
     const int xblocks = (g.gx_hi - g.gx_lo + ip.xblock - 1) / ip.xblock;

@@ -126,10 +126,19 @@ struct FilterTaps {
 
 // Particle chunk: a contiguous particle range and the bounding box of the
 // cells its particles occupy (inclusive, grid-relative cells).
+// rest (mixed path): every live particle is an electron at rest at its lattice
+// site with its ion (zero momentum deviation, the site's stored position);
+// zlo, zhi are then the least and greatest stored z, 16.16 fixed point modulo
+// 2^16 cells (exact: a site's offset is an odd multiple of 1/(2 ppc_z)).
 struct Chunk {
   int p0, p1;
   int ix0, ix1, iz0, iz1;
+  int rest;
+  uint32_t zlo, zhi;
 };
+__host__ __device__ inline uint32_t z_key(int cell, float oz) {
+  return ((uint32_t)cell << 16) | (uint32_t)(oz * 65536.0f);
+}
 
 // Particle storage (structure of arrays). The FP64 path keeps absolute
 // positions; the mixed path keeps a cell (iz | ix << 16) and the FP32 offset
