@@ -166,20 +166,53 @@ __global__ void k_beam_finish(Beam<T> b, double t_now, double* acc) {
   if (j == 0) acc[2] = vbar;
 }
 
-template <class T>
-__device__ T gather_global(const T* F, const GridP& g, int order, double X, double Z, double sx, double sz) {
-  const int fx = (int)floor(X), fz = (int)floor(Z);
-  double acc = 0.0;
-  for (int i = fx - 3; i <= fx + 3; i++) {
-    const double wx = shape_val(order, X - (i + sx));
-    if (wx == 0.0 || i < 0 || i > g.nx) continue;
-    for (int k = fz - 3; k <= fz + 3; k++) {
-      const double wz = shape_val(order, Z - (k + sz));
-      if (wz == 0.0 || k < 0 || k > g.nz) continue;
-      acc += (double)F[(long)i * g.ld + k] * wx * wz;
+// one component at a beam particle: sum of F over the NG x NG stencil from node (i0, k0) with weights wx, wz, in FP64;
+// nodes off the grid count as zero
+template <class T, int NG>
+__device__ __forceinline__ double gather_beam(const T* F, const GridP& g, int i0, int k0, const double* wx,
+                                              const double* wz) {
+  T v[NG][NG];
+#pragma unroll
+  for (int a = 0; a < NG; a++)
+#pragma unroll
+    for (int b = 0; b < NG; b++) {
+      const int i = i0 + a, k = k0 + b;
+      v[a][b] = (i >= 0 && i <= g.nx && k >= 0 && k <= g.nz) ? F[(long)i * g.ld + k] : T(0);
     }
+  double acc = 0.0;
+#pragma unroll
+  for (int a = 0; a < NG; a++) {
+    double r = 0.0;
+#pragma unroll
+    for (int b = 0; b < NG; b++) r += (double)v[a][b] * wz[b];
+    acc += r * wx[a];
   }
-  return T(acc);
+  return acc;
+}
+
+// the six components at a beam particle at (X, Z) cells: the weights of the integer and the half positions once per
+// axis. half 0: every component at the nodes (the 'momentum conserving' copies)
+template <class T, int ORD>
+__device__ __forceinline__ void gather_beam6(const T* const* gE, const T* const* gB, const GridP& g, double X, double Z,
+                                             bool half, double* E, double* B) {
+  constexpr int NG = ORD + 1, OFF = ORD == 3 ? 1 : 0;
+  double wx[2][NG], wz[2][NG];
+  int bx[2], bz[2];
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    const double s = (h == 1 && half) ? 0.5 : 0.0;
+    const double fx = floor(X - s), fz = floor(Z - s);
+    if constexpr (ORD == 3) { weights3<double>(X - s - fx, wx[h]); weights3<double>(Z - s - fz, wz[h]); }
+    else { weights1<double>(X - s - fx, wx[h]); weights1<double>(Z - s - fz, wz[h]); }
+    bx[h] = (int)fx - OFF;
+    bz[h] = (int)fz - OFF;
+  }
+  E[0] = gather_beam<T, NG>(gE[0], g, bx[1], bz[0], wx[1], wz[0]);
+  E[1] = gather_beam<T, NG>(gE[1], g, bx[0], bz[0], wx[0], wz[0]);
+  E[2] = gather_beam<T, NG>(gE[2], g, bx[0], bz[1], wx[0], wz[1]);
+  B[0] = gather_beam<T, NG>(gB[0], g, bx[0], bz[1], wx[0], wz[1]);
+  B[1] = gather_beam<T, NG>(gB[1], g, bx[1], bz[1], wx[1], wz[1]);
+  B[2] = gather_beam<T, NG>(gB[2], g, bx[1], bz[0], wx[1], wz[0]);
 }
 
 // Esirkepov deposit of one beam particle (charge * weight qw per unit length along y) moving (x0, z0) ->
@@ -226,6 +259,12 @@ __device__ void beam_deposit(const GridP& g, const FieldPtrs<T>& f, int order, d
       }
 }
 
+// Test beams: a few hundred particles whose push is one long FP64 chain (about 300 operations at cubic order), so blocks
+// are single warps, spread over as many SMs as there are warps: the FP64 pipe of an SM takes 16 cycles per warp and
+// operation. Blocks of 128 with every shape weight evaluated per node made a step with 256 active particles 262 us; it is
+// 114 us so (1600 x 96 cells, 20 thousand electrons).
+constexpr int BEAM_TB = 32;
+
 template <class T>
 __device__ __forceinline__ void beam_push_one(const GridP& g, const FieldPtrs<T>& f, const Beam<T>& b, int order,
                                               double tn, double tn1, int nodal, const double* acc, int j) {
@@ -252,23 +291,19 @@ __device__ __forceinline__ void beam_push_one(const GridP& g, const FieldPtrs<T>
     }
   }
   const double x = b.x[j], z = b.z[j];
-  const double X = x / g.dx, Z = (z - g.z0) / g.dz;
-  // Yee locations, or the node values of the 'momentum conserving' gather (offsets 0)
-  const double h = nodal ? 0.0 : 0.5;
+  const double X = x * g.idx, Z = (z - g.z0) * g.idz;
+  // Yee locations, or the node values of the 'momentum conserving' gather
   const T* const* gE = nodal ? f.nE : f.fE;
   const T* const* gB = nodal ? f.nB : f.fB;
-  const double E[3] = {(double)gather_global<T>(gE[0], g, order, X, Z, h, 0.0),
-                       (double)gather_global<T>(gE[1], g, order, X, Z, 0.0, 0.0),
-                       (double)gather_global<T>(gE[2], g, order, X, Z, 0.0, h)};
-  const double B[3] = {(double)gather_global<T>(gB[0], g, order, X, Z, 0.0, h),
-                       (double)gather_global<T>(gB[1], g, order, X, Z, h, h),
-                       (double)gather_global<T>(gB[2], g, order, X, Z, h, 0.0)};
+  double E[3], B[3];
+  if (order == 3) gather_beam6<T, 3>(gE, gB, g, X, Z, !nodal, E, B);
+  else gather_beam6<T, 1>(gE, gB, g, X, Z, !nodal, E, B);
   const T k = T(-kQe * g.dt / (2.0 * kMe));
   const T ic2 = T(1.0 / (kC * kC));
   T ux = b.ux[j], uy = b.uy[j], uz = b.uz[j];
   T umx = ux + k * T(E[0]), umy = uy + k * T(E[1]), umz = uz + k * T(E[2]);
-  T gm = sqrt(T(1) + (umx * umx + umy * umy + umz * umz) * ic2);
-  T tbx = k * T(B[0]) / gm, tby = k * T(B[1]) / gm, tbz = k * T(B[2]) / gm;
+  const T kg = k / sqrt(T(1) + (umx * umx + umy * umy + umz * umz) * ic2);
+  T tbx = kg * T(B[0]), tby = kg * T(B[1]), tbz = kg * T(B[2]);
   T t2 = tbx * tbx + tby * tby + tbz * tbz;
   T sf = T(2) / (T(1) + t2);
   T upx = umx + (umy * tbz - umz * tby), upy = umy + (umz * tbx - umx * tbz), upz = umz + (umx * tby - umy * tbx);
@@ -291,7 +326,7 @@ __global__ void k_beam_push(GridP g, FieldPtrs<T> f, Beam<T> b, int order, doubl
   beam_push_one<T>(g, f, b, order, tn, tn1, nodal, acc, j);
 }
 
-// the batched step's test beams: run blockIdx.y, its particles from blockIdx.x * 128 (the Yee-located
+// the batched step's test beams: run blockIdx.y, its particles from blockIdx.x * blockDim.x (the Yee-located
 // gather; the batched step carries no node-interpolated runs)
 template <class T>
 __global__ void k_beam_push_batch(const StepArgs<T>* a) {
@@ -831,15 +866,15 @@ void launch_beam_init(Beam<T> b, const double* lx, const double* lz, const doubl
 }
 
 template <class T>
-void launch_beam_push_batch(const StepArgs<T>* a, int nruns, int beam_blocks, cudaStream_t s) {
-  if (beam_blocks > 0) k_beam_push_batch<T><<<dim3(beam_blocks, nruns), 128, 0, s>>>(a);
+void launch_beam_push_batch(const StepArgs<T>* a, int nruns, int beam_max, cudaStream_t s) {
+  if (beam_max > 0) k_beam_push_batch<T><<<dim3((beam_max + BEAM_TB - 1) / BEAM_TB, nruns), BEAM_TB, 0, s>>>(a);
 }
 
 template <class T>
 void launch_beam_push(const GridP& g, const FieldPtrs<T>& f, Beam<T> b, int order, double tn, double tn1, int nodal,
                       const double* scratch, cudaStream_t s) {
   if (b.n <= 0) return;
-  k_beam_push<T><<<(b.n + 127) / 128, 128, 0, s>>>(g, f, b, order, tn, tn1, nodal, scratch);
+  k_beam_push<T><<<(b.n + BEAM_TB - 1) / BEAM_TB, BEAM_TB, 0, s>>>(g, f, b, order, tn, tn1, nodal, scratch);
 }
 
 // 'momentum conserving' gather (Sec. 5): each gather copy interpolated to the nodes, the mean of its two

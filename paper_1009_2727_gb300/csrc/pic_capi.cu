@@ -1106,7 +1106,7 @@ struct BatchImpl : Batch {
   BatchGrid bg{};
   int order = 3, pt_taps = 0, push_grid = 0, smem_nodes = 0, tile_z = 0;
   bool friedman = false, ck = false, filt_gather = false, filt_J = false, any_ion = false;
-  int beam_blocks = 0;   // blocks of 128 particles of the largest test beam (0: no run has one)
+  int beam_max = 0;   // particles of the largest test beam (0: no run has one)
   size_t filt_smem = 0, amp_smem = 0;
   size_t fused_smem = 0;   // > 0: the fused Faraday + E filter kernel serves every run
   int64_t nl = 0, nstep = 0;
@@ -1171,7 +1171,7 @@ struct BatchImpl : Batch {
       ion_off[r + 1] = ion_off[r] + (column ? (int)((m->ion_rows_max() + 255) / 256) : 0);
       inj_off[r + 1] = inj_off[r] + m->inj_xblocks() * m->inj_rblocks_max();
       ant_off[r + 1] = ant_off[r] + (std::max(m->g.nx, m->g.nz) + 1 + 127) / 128;
-      beam_blocks = std::max(beam_blocks, (m->beam.n + 127) / 128);
+      beam_max = std::max(beam_max, m->beam.n);
     }
     bg.nruns = n;
     bg.tiles = tile_off[n];
@@ -1206,7 +1206,7 @@ struct BatchImpl : Batch {
     cudaMemcpyAsync(dA[q], hA[q], sizeof(StepArgs<T>) * n, cudaMemcpyHostToDevice, s);
     launch_faraday_filter_batch<T>(dA[q], bg, friedman, ck, pt_taps, filt_gather, filt_smem, fused_smem, s);
     launch_push_batch<T>(dA[q], bg, order, push_grid, smem_nodes, tile_z, s);
-    launch_beam_push_batch<T>(dA[q], n, beam_blocks, s);
+    launch_beam_push_batch<T>(dA[q], n, beam_max, s);
     launch_antenna_ion_batch<T>(dA[q], bg, any_ion, s);
     launch_ampere_batch<T>(dA[q], bg, filt_J, pt_taps, amp_smem, s);
     launch_inject_batch<T>(dA[q], bg, s);
@@ -1249,7 +1249,7 @@ struct BatchImpl : Batch {
       }
       cudaEventRecord(done[q], s);
       used[q] = true;
-      nl += kernels_per_step(filt_gather, any_ion, beam_blocks > 0);
+      nl += kernels_per_step(filt_gather, any_ion, beam_max > 0);
       for (int r : sorts) {
         sims[r]->do_sort();
         nl += 8;

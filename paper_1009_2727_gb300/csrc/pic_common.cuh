@@ -520,9 +520,9 @@ void launch_ampere_batch(const StepArgs<T>* a, const BatchGrid& bg, bool filt_J,
 // plasma rows entering through the +z plane of every run, then the runs' particle and chunk counts
 template <class T>
 void launch_inject_batch(const StepArgs<T>* a, const BatchGrid& bg, cudaStream_t s);
-// the test beams of every run with one (blockIdx.y: run; beam_blocks: blocks of 128 particles of the largest)
+// the test beams of every run with one (blockIdx.y: run; beam_max: particles of the largest)
 template <class T>
-void launch_beam_push_batch(const StepArgs<T>* a, int nruns, int beam_blocks, cudaStream_t s);
+void launch_beam_push_batch(const StepArgs<T>* a, int nruns, int beam_max, cudaStream_t s);
 // filter taps and shared-memory sizes the batched field kernels need (the same as a single run's)
 template <class T>
 FilterTaps<T> filter_taps(const FilterSpec& fs);
