@@ -2568,7 +2568,12 @@ struct Sim3 : Sim3Api {
   int get_field(int comp, double* dst, int on_device) override {
     if (comp < 0 || comp > PIC_RHO) return fail(PIC_EINVAL, "bad component");
     const long nn = nodes();
-    if (!out_d) { out_d = dal<double>(nn); if (!out_d) return fail(PIC_ENOMEM, "allocation failed"); }
+    // a device destination is written in place, a host one through out_d
+    double* o = dst;
+    if (!on_device) {
+      if (!out_d) { out_d = dal<double>(nn); if (!out_d) return fail(PIC_ENOMEM, "allocation failed"); }
+      o = out_d;
+    }
     if (comp == PIC_RHO) {
       if (!rho) { rho = dal<double>(g.cs); if (!rho) return fail(PIC_ENOMEM, "allocation failed"); }
       cudaMemsetAsync(rho, 0, sizeof(double) * g.cs, s);
@@ -2585,12 +2590,12 @@ struct Sim3 : Sim3Api {
         k3_antenna_rho<<<nblk(npair, 128), 128, 0, s>>>(g, ant_params(Dn, Dn), rho);
         nl++;
       }
-      k3_out_rho<<<nblk(nn, 256), 256, 0, s>>>(g, rho, out_d);
+      k3_out_rho<<<nblk(nn, 256), 256, 0, s>>>(g, rho, o);
     } else {
-      k3_out_field<T><<<nblk(nn, 256), 256, 0, s>>>(g, comp_ptr(comp), out_d);
+      k3_out_field<T><<<nblk(nn, 256), 256, 0, s>>>(g, comp_ptr(comp), o);
     }
     nl++;
-    cudaMemcpyAsync(dst, out_d, sizeof(double) * nn, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
+    if (!on_device) cudaMemcpyAsync(dst, out_d, sizeof(double) * nn, cudaMemcpyDeviceToHost, s);
     return cudaStreamSynchronize(s) == cudaSuccess ? PIC_OK : fail(PIC_ECUDA, "CUDA error in get_field");
   }
 

@@ -110,15 +110,7 @@ __global__ void k_ion_current(GridP g, long long mlo, long long mhi, double t0, 
 // the antenna's positions at t^n and t^{n+1}, averaged and divided by dz.
 template <class T>
 __global__ void k_antenna(GridP g, T* Jy, const double* xs, AntennaStep a) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i > g.nx) return;
-  const double kx = a.amp * xs[i];
-  if (kx == 0.0) return;
-#pragma unroll
-  for (int j = 0; j < 8; j++) {
-    const int k = a.k0 + j;
-    if (a.wz[j] != 0.0 && k >= 0 && k <= g.nz) Jy[(long)i * g.ld + k] += T(kx * a.wz[j]);
-  }
+  antenna_column<T>(g, Jy, xs, a, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -629,17 +621,7 @@ __global__ void k_antenna_batch(const StepArgs<T>* a, const int* off, int nruns)
   const int lb = blockIdx.x - off[s_r], nb = off[s_r + 1] - off[s_r];
   if (A.ion_on)
     for (int k = lb * blockDim.x + threadIdx.x; k <= A.g.nz; k += nb * blockDim.x) A.ion_C[k] = 0.0;
-  if (!A.ant_on) return;
-  const int i = lb * blockDim.x + threadIdx.x;
-  if (i > A.g.nx) return;
-  const double kx = A.ast.amp * A.ant_xs[i];
-  if (kx == 0.0) return;
-  T* Jy = A.f.J[1];
-#pragma unroll
-  for (int j = 0; j < 8; j++) {
-    const int k = A.ast.k0 + j;
-    if (A.ast.wz[j] != 0.0 && k >= 0 && k <= A.g.nz) Jy[(long)i * A.g.ld + k] += T(kx * A.ast.wz[j]);
-  }
+  if (A.ant_on) antenna_column<T>(A.g, A.f.J[1], A.ant_xs, A.ast, lb * blockDim.x + threadIdx.x);
 }
 
 // batched rigid-ion column current: rows [ion_mlo, ion_mhi) of each run, one thread per row

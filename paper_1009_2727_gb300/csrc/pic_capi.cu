@@ -159,10 +159,12 @@ struct Sim : SimBase {
   int timing_which = 0;
   std::vector<cudaEvent_t> ev;
   int64_t timed_launches = 0;
+  cudaEvent_t dst_ready = nullptr;   // get_field: the default stream's work before a device destination is written
 
   explicit Sim(pic_ctx* ctx) : c(ctx) {}
   ~Sim() override {
     for (auto e : ev) cudaEventDestroy(e);
+    if (dst_ready) cudaEventDestroy(dst_ready);
     if (hmirror) cudaFreeHost(hmirror);
     if (hstats) cudaFreeHost(hstats);
   }
@@ -439,7 +441,7 @@ struct Sim : SimBase {
         ip.m_beg = a; ip.m_end = b; ip.t = t; ip.rblock = 8;
         if ((b - a) * (long long)ip.nxl > cap) return c->fail(PIC_EOVERFLOW, "initial plasma exceeds capacity");
         launch_inject<T>(g, P, chunks, ctrl, ip, cap, chunk_cap, c->stream);
-        c->launches += 2;
+        c->launches += 1;
         count_ub = (b - a) * (long long)ip.nxl;
         do_sort();
       }
@@ -643,7 +645,9 @@ struct Sim : SimBase {
     // ion rows live during this step: those inside the particle domain at t^n
     long long mlo = std::max(row_first, (long long)std::ceil((zlo_prev + h.beta * kC * tn) / ip.h - 0.5));
     if (step == 0) mlo = row_first;
-    // 3. particles
+    // 3.-4. particles, and the antenna (with the push's second launch where there are particles)
+    AntennaStep ast{};
+    const bool ant_on = has_laser && antenna_step(tn, tn1, ast);
     if (loaded && cap > 0) {
       tstart(0);
       int fr1_sz;
@@ -651,7 +655,8 @@ struct Sim : SimBase {
       frame_of(frame_shift(step + 1), fr1_sz, fr1_fz);
       launch_push<T>(g, f, P, chunks, ctrl, cf.shape_order, push_grid, smem_nodes, sb.tz, -kQe, kMe, c->hg.gamma,
                      c->hg.beta,
-                     fr1_sz, fr1_fz, (pairs && ions) ? 1 : 0, (int)mlo, nodal ? 1 : 0, pdef, c->stream);
+                     fr1_sz, fr1_fz, (pairs && ions) ? 1 : 0, (int)mlo, nodal ? 1 : 0, pdef, ast,
+                     ant_on ? ant_xs : nullptr, c->stream);
       tstop(0);
       c->launches += 2;
     }
@@ -660,9 +665,7 @@ struct Sim : SimBase {
       launch_beam_push<T>(g, f, beam, cf.shape_order, tn, tn1, nodal ? 1 : 0, beam_scratch, c->stream);
       c->launches++;
     }
-    // 4. antenna
-    AntennaStep ast;
-    if (has_laser && antenna_step(tn, tn1, ast)) {
+    if (ant_on && !(loaded && cap > 0)) {
       launch_antenna<T>(g, f.J[1], ant_xs, ast, c->stream);
       c->launches++;
     }
@@ -701,7 +704,7 @@ struct Sim : SimBase {
         if (!ids_fit(a, b)) return c->fail(PIC_EOVERFLOW, "plasma rows exceed the 32-bit particle id space");
         ip.m_beg = a; ip.m_end = b; ip.t = tn1; ip.rblock = 4;
         launch_inject<T>(g, P, chunks, ctrl, ip, cap, chunk_cap, c->stream);
-        c->launches += 2;
+        c->launches += 1;
         count_ub += add;
       }
     }
@@ -869,25 +872,35 @@ struct Sim : SimBase {
 
   int get_field(int comp, double* dst, int on_device) {
     set_ptrs_for_step();
+    if (on_device && c->stream) {
+      // dst is written on the context's stream: after the work already queued on the default stream, where the caller's
+      // earlier use of that memory may still run
+      if (!dst_ready && cudaEventCreateWithFlags(&dst_ready, cudaEventDisableTiming) != cudaSuccess)
+        return c->fail(PIC_ECUDA, "event creation failed");
+      cudaEventRecord(dst_ready, nullptr);
+      cudaStreamWaitEvent(c->stream, dst_ready, 0);
+    }
     const size_t n = stage_n;
     if (comp >= PIC_EX && comp <= PIC_JZ) {
       const T* src = comp < 3 ? f.E[comp] : comp < 6 ? f.B[comp - 3] : f.Jn[comp - 6];
-      launch_convert<T>(src, stage, g, c->stream);
+      launch_convert<T>(src, on_device ? dst : stage, g, c->stream);
     } else if (comp == PIC_RHO) {
-      cudaMemsetAsync(stage, 0, n * 8, c->stream);
-      if (loaded) launch_rho<T>(g, P, ctrl, cap, c->cfg.shape_order, -kQe, stage, c->stream);
+      double* rho = on_device ? dst : stage;
+      cudaMemsetAsync(rho, 0, n * 8, c->stream);
+      if (loaded) launch_rho<T>(g, P, ctrl, cap, c->cfg.shape_order, -kQe, rho, c->stream);
       if (ions && loaded) {
         const double t = time_of(step);
         long long mlo = std::max(row_first, (long long)std::ceil((zlo_prev + c->hg.beta * kC * t) / ip.h - 0.5));
         if (step == 0) mlo = row_first;
         launch_ion_rows(g, mlo, row_next, t, ip, c->cfg.shape_order, ion_R0, c->stream);
-        launch_ion_rho(g, ion_x, ion_R0, kQe / (g.dx * g.dz), stage, c->stream);
+        launch_ion_rho(g, ion_x, ion_R0, kQe / (g.dx * g.dz), rho, c->stream);
       }
     } else {
       return c->fail(PIC_EINVAL, "unknown component");
     }
+    // a device destination was written in place (on this stream); the call returns when it is there
+    if (!on_device) cudaMemcpyAsync(dst, stage, n * 8, cudaMemcpyDeviceToHost, c->stream);
     cudaStreamSynchronize(c->stream);
-    cudaMemcpy(dst, stage, n * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost);
     return cudaGetLastError() == cudaSuccess ? PIC_OK : c->fail(PIC_ECUDA, "CUDA error in get_field");
   }
 
@@ -1212,7 +1225,7 @@ struct BatchImpl : Batch {
     launch_inject_batch<T>(dA[q], bg, s);
   }
   static int kernels_per_step(bool filt, bool ion, bool beam) {
-    return 1 + (filt ? 1 : 0) + 3 + (beam ? 1 : 0) + 1 + (ion ? 1 : 0) + 1 + 2;
+    return 1 + (filt ? 1 : 0) + 2 + (beam ? 1 : 0) + 1 + (ion ? 1 : 0) + 1 + 1;
   }
 
   int step(int nsteps) override {

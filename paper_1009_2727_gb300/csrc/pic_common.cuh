@@ -219,7 +219,7 @@ struct Ctrl {
   int overflow_chunks;
   int n_defer;        // particles of this step's push left for the global-memory pass
   int n_ovf;          // chunks of this step's push left for the global-memory pass (window too large)
-  int pad;
+  int inj_done;       // blocks of the running injection that have finished
   double red[8];      // reduction scratch
 };
 
@@ -309,6 +309,25 @@ void launch_ampere(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, con
                    const double* ion_x, const double* ion_c, double ion_coef, const TileMaps& tm, Ctrl* ctrl,
                    cudaStream_t s);
 
+// antenna current of one step: K_y(i) = amp * xs[i] on the rows k0 .. k0+7 with weights wz (1/dz included)
+struct AntennaStep {
+  double amp;
+  int k0;
+  double wz[8];
+};
+// J_y of column i: added atomically, the antenna runs beside other writers of the current
+template <class T>
+__device__ __forceinline__ void antenna_column(const GridP& g, T* Jy, const double* xs, const AntennaStep& a, int i) {
+  if (i > g.nx) return;
+  const double kx = a.amp * xs[i];
+  if (kx == 0.0) return;
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    const int k = a.k0 + j;
+    if (a.wz[j] != 0.0 && k >= 0 && k <= g.nz) atomicAdd(Jy + (long)i * g.ld + k, T(kx * a.wz[j]));
+  }
+}
+
 // The push runs in two launches: the shared-memory window kernel over every chunk, then a global-memory
 // pass over what it left (particles outside their chunk's box, chunks whose window exceeds the shared
 // memory), recorded in defer (particle, chunk) and ovf (chunk) lists of the given capacities.
@@ -317,10 +336,13 @@ struct PushDefer {
   int* ovf;
   int defer_cap, ovf_cap;
 };
+// The second launch also adds the antenna (ant_xs given). Both start from counters that Ampère's kernel of the step
+// before has cleared.
 template <class T>
 void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* chunks, Ctrl* ctrl, int order,
                  int grid_blocks, int smem_nodes, int tile_z, double q, double m, double gamma_b, double beta_b,
-                 int fr1_sz, float fr1_fz, int pairs, int mlo, int nodal, const PushDefer& pd, cudaStream_t s);
+                 int fr1_sz, float fr1_fz, int pairs, int mlo, int nodal, const PushDefer& pd, const AntennaStep& ant,
+                 const double* ant_xs, cudaStream_t s);
 
 struct SortBufs {
   int* cell_cnt;       // ntiles*tx*tz, cells in tile-major order: particles per cell
@@ -350,7 +372,6 @@ struct InjectP {
 template <class T>
 void launch_inject(const GridP& g, Particles<T> p, Chunk* chunks, Ctrl* ctrl, const InjectP& ip, int cap,
                    int chunk_cap, cudaStream_t s);
-void launch_add_counts(Ctrl* ctrl, int dcount, int dchunks, cudaStream_t s);
 
 void launch_ion_column(const GridP& g, long long mlo, long long mhi, double t0, double t1, const InjectP& ip,
                        int order, double* C, cudaStream_t s);
@@ -361,12 +382,6 @@ void launch_ion_rows(const GridP& g, long long mlo, long long mhi, double t, con
 struct LaserP {
   double lambda0, a0, w0, tau, t_peak, x_center, phase, z_antenna, beta_s;
   double gamma, beta;
-};
-// antenna current of one step: K_y(i) = amp * xs[i] on the rows k0 .. k0+7 with weights wz (1/dz included)
-struct AntennaStep {
-  double amp;
-  int k0;
-  double wz[8];
 };
 template <class T>
 void launch_antenna(const GridP& g, T* Jy, const double* xs, const AntennaStep& a, cudaStream_t s);
@@ -487,7 +502,7 @@ struct BatchGrid {
   const int* inj_off;      // injection blocks
   const int* ant_off;      // antenna blocks
   int nruns, tiles, ion_blocks, inj_blocks, ant_blocks;
-  int* push_counter;       // the push's (run, chunk) queue head
+  int* push_counter;       // the push's (run, chunk) queue head, cleared by Ampère's kernel of the step before
 };
 // the push's constants for one step (q, m: charge and mass; fr1: frame shift at t^{n+1}; pairs, mlo: the
 // electron-ion pairs and the first live ion row)

@@ -647,6 +647,8 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
   const int i0 = tile_i * FT_X, k0 = tile_k * FT_Z;
   const int gi0 = i0 - tm.H, gk0 = k0 - tm.HZ;
   const bool leader = threadIdx.x == 0 && threadIdx.y == 0;
+  // the push is over: its queue and lists start empty in the next step
+  if (leader && c_first == 0 && tile_k == 0 && tile_i == 0) ctrl->next_chunk = ctrl->n_defer = ctrl->n_ovf = 0;
   if (leader) {
     mbar_init(&bar[0]);
     mbar_init(&bar[1]);
@@ -1063,9 +1065,11 @@ __global__ void __launch_bounds__(FT_Z* FT_TY) k_filter_fields_batch(const StepA
 }
 
 template <class T, bool FILT, int PT>
-__global__ void __launch_bounds__(FT_Z* FT_TY, sizeof(T) == 4 ? 4 : 2) k_ampere_batch(const StepArgs<T>* a, const int* off, int nruns) {
+__global__ void __launch_bounds__(FT_Z* FT_TY, sizeof(T) == 4 ? 4 : 2) k_ampere_batch(const StepArgs<T>* a, const int* off, int nruns,
+                                                                                  int* push_counter) {
   __shared__ int s_r;
   if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (blockIdx.x == 0) *push_counter = 0;
     s_r = batch_run(off, nruns, blockIdx.x);
     tensormap_acquire(&a[s_r].tm.J[a[s_r].mapJ]);
   }
@@ -1134,7 +1138,7 @@ void launch_ampere_batch(const StepArgs<T>* a, const BatchGrid& bg, bool filt_J,
   dim3 blk(FT_Z, FT_TY);
 #define ABATCH(F, PTV)                                                                                   \
   cudaFuncSetAttribute(k_ampere_batch<T, F, PTV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)amp_smem); \
-  k_ampere_batch<T, F, PTV><<<bg.tiles, blk, amp_smem, s>>>(a, bg.tile_off, bg.nruns);
+  k_ampere_batch<T, F, PTV><<<bg.tiles, blk, amp_smem, s>>>(a, bg.tile_off, bg.nruns, bg.push_counter);
   if (!filt_J) {
     ABATCH(false, 0)
     return;

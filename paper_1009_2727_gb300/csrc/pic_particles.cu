@@ -924,20 +924,28 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push(GridP g, 
   }
 }
 
-// The global-memory pass after k_push: whole chunks whose window did not fit in shared memory (one block
-// each), then single particles that were outside their chunk's box (one thread each). Both add their
+// The global-memory pass after k_push: whole chunks whose window did not fit in shared memory (OVF_SLICES
+// blocks each), then single particles that were outside their chunk's box (one thread each); the blocks past nblk add
+// the antenna. Both add their
 // current with global atomics and widen their chunk's box atomically (k_push has written the box of the
 // particles it pushed; an overflow chunk's box starts empty).
+constexpr int OVF_SLICES = 8;
 template <class T, int ORDER, bool MC>
 __global__ void __launch_bounds__(PB_THREADS) k_push_deferred(GridP g, const T* gE, const T* gB, T* gJ,
                                                                Particles<T> p, Chunk* chunks, Ctrl* ctrl,
-                                                               PushDefer pd, PushConst pc) {
+                                                               PushDefer pd, PushConst pc, int nblk,
+                                                               AntennaStep ant, const double* ant_xs) {
+  if ((int)blockIdx.x >= nblk) {
+    antenna_column<T>(g, gJ + g.cs, ant_xs, ant, ((int)blockIdx.x - nblk) * PB_THREADS + threadIdx.x);
+    return;
+  }
   const int novf = min(ctrl->n_ovf, pd.ovf_cap), ndef = min(ctrl->n_defer, pd.defer_cap);
-  for (int j = blockIdx.x; j < novf; j += gridDim.x) {
-    const int c = pd.ovf[j];
+  // a chunk's particles are shared by OVF_SLICES blocks
+  for (int j = blockIdx.x; j < novf * OVF_SLICES; j += nblk) {
+    const int c = pd.ovf[j / OVF_SLICES];
     const Chunk ch = chunks[c];
     BoxI acc;
-    for (int pi = ch.p0 + threadIdx.x; pi < ch.p1; pi += blockDim.x)
+    for (int pi = ch.p0 + (j % OVF_SLICES) * PB_THREADS + threadIdx.x; pi < ch.p1; pi += OVF_SLICES * PB_THREADS)
       push_global_guarded<T, ORDER, MC>(gE, gB, gJ, g, p, pi, pc, ctrl, acc);
     int bx0 = acc.x0, bx1 = acc.x1, bz0 = acc.z0, bz1 = acc.z1;
     bx0 = __reduce_min_sync(0xffffffffu, bx0); bx1 = __reduce_max_sync(0xffffffffu, bx1);
@@ -947,7 +955,7 @@ __global__ void __launch_bounds__(PB_THREADS) k_push_deferred(GridP g, const T* 
       atomicMin(&chunks[c].iz0, bz0); atomicMax(&chunks[c].iz1, bz1);
     }
   }
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < ndef; j += gridDim.x * blockDim.x) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < ndef; j += nblk * blockDim.x) {
     const int2 e = pd.defer[j];
     BoxI acc;
     push_global_guarded<T, ORDER, MC>(gE, gB, gJ, g, p, e.x, pc, ctrl, acc);
@@ -1154,7 +1162,8 @@ __device__ double lab_density(const InjectP& ip, double zl) {
 
 template <class T>
 __device__ __forceinline__ void inject_block(const GridP& g, const Particles<T>& p, Chunk* chunks, Ctrl* ctrl,
-                                             const InjectP& ip, int cap, int chunk_cap, int xb, int rb, int nxb) {
+                                             const InjectP& ip, int cap, int chunk_cap, int xb, int rb, int nxb,
+                                             int nblocks) {
   const long long nrows = ip.m_end - ip.m_beg;
   const long long r0 = (long long)rb * ip.rblock;
   const int nr = (int)min((long long)ip.rblock, nrows - r0);
@@ -1196,7 +1205,9 @@ __device__ __forceinline__ void inject_block(const GridP& g, const Particles<T>&
   }
   if (threadIdx.x == 0 && cnt > 0) {
     const int ci = ctrl->nchunks + rb * nxb + xb;
-    if (ci >= chunk_cap || start + cnt > cap) { atomicOr(&ctrl->status, ST_OVERFLOW); return; }
+    if (ci >= chunk_cap || start + cnt > cap) {
+      atomicOr(&ctrl->status, ST_OVERFLOW);
+    } else {
     Chunk c;
     c.p0 = (int)start; c.p1 = (int)(start + cnt);
     c.ix0 = g.gx_lo + cx0; c.ix1 = g.gx_lo + cx0 + ncx - 1;
@@ -1215,29 +1226,29 @@ __device__ __forceinline__ void inject_block(const GridP& g, const Particles<T>&
       c.rest = 1;
     }
     chunks[ci] = c;
+    }
+  }
+  // the last of the injection's nblocks blocks to finish adds the counts (every block has read them by then)
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&ctrl->inj_done, 1) == nblocks - 1) {
+      ctrl->inj_done = 0;
+      ctrl->count += (int)(nrows * ip.nxl);
+      ctrl->nchunks += nblocks;
+    }
   }
 }
 
 template <class T>
 __global__ void k_inject(GridP g, Particles<T> p, Chunk* chunks, Ctrl* ctrl, InjectP ip, int cap, int chunk_cap) {
-  inject_block<T>(g, p, chunks, ctrl, ip, cap, chunk_cap, blockIdx.x, blockIdx.y, gridDim.x);
-}
-
-__global__ void k_add_counts(Ctrl* ctrl, int dcount, int dchunks) {
-  ctrl->count += dcount;
-  ctrl->nchunks += dchunks;
+  inject_block<T>(g, p, chunks, ctrl, ip, cap, chunk_cap, blockIdx.x, blockIdx.y, gridDim.x,
+                  gridDim.x * gridDim.y);
 }
 
 // ---------------------------------------------------------------------------
 // batched particle kernels of an ensemble step
 constexpr int MAX_BATCH_RUNS = 512;
-
-template <class T>
-__global__ void k_push_batch_reset(const StepArgs<T>* a, int nruns, int* counter) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r == 0) *counter = 0;
-  if (r < nruns && a[r].push_on) { a[r].ctrl->n_defer = 0; a[r].ctrl->n_ovf = 0; }
-}
 
 // the window kernel over all runs' chunks: blocks take (run, chunk) pairs from one queue; the run's push
 // constants, geometry and particle arrays are copied to shared memory when a block changes run
@@ -1299,11 +1310,11 @@ __global__ void __launch_bounds__(PB_THREADS) k_push_deferred_batch(const StepAr
     const StepArgs<T>& A = a[r];
     if (!A.push_on) continue;
     const int novf = min(A.ctrl->n_ovf, A.pd.ovf_cap), ndef = min(A.ctrl->n_defer, A.pd.defer_cap);
-    for (int j = blockIdx.x; j < novf; j += gridDim.x) {
-      const int c = A.pd.ovf[j];
+    for (int j = blockIdx.x; j < novf * OVF_SLICES; j += gridDim.x) {
+      const int c = A.pd.ovf[j / OVF_SLICES];
       const Chunk ch = A.chunks[c];
       BoxI acc;
-      for (int pi = ch.p0 + threadIdx.x; pi < ch.p1; pi += blockDim.x)
+      for (int pi = ch.p0 + (j % OVF_SLICES) * PB_THREADS + threadIdx.x; pi < ch.p1; pi += OVF_SLICES * PB_THREADS)
         push_global_guarded<T, ORDER, false>(A.f.fE[0], A.f.fB[0], A.f.J[0], A.g, A.p, pi, A.pc, A.ctrl, acc);
       int bx0 = acc.x0, bx1 = acc.x1, bz0 = acc.z0, bz1 = acc.z1;
       bx0 = __reduce_min_sync(0xffffffffu, bx0); bx1 = __reduce_max_sync(0xffffffffu, bx1);
@@ -1338,16 +1349,7 @@ __global__ void k_inject_batch(const StepArgs<T>* a, const int* off, int nruns) 
   const int lb = blockIdx.x - off[s_r];
   const int xb = lb % A.inj_xblocks, rb = lb / A.inj_xblocks;
   if ((long long)rb * A.ip.rblock >= A.ip.m_end - A.ip.m_beg) return;
-  inject_block<T>(A.g, A.p, A.chunks, A.ctrl, A.ip, A.cap, A.chunk_cap, xb, rb, A.inj_xblocks);
-}
-
-template <class T>
-__global__ void k_add_counts_batch(const StepArgs<T>* a, int nruns) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < nruns && a[r].inj_on) {
-    a[r].ctrl->count += a[r].add_count;
-    a[r].ctrl->nchunks += a[r].add_chunks;
-  }
+  inject_block<T>(A.g, A.p, A.chunks, A.ctrl, A.ip, A.cap, A.chunk_cap, xb, rb, A.inj_xblocks, A.add_chunks);
 }
 
 }  // namespace
@@ -1356,7 +1358,6 @@ template <class T>
 void launch_push_batch(const StepArgs<T>* a, const BatchGrid& bg, int order, int grid_blocks, int smem_nodes,
                        int tile_z, cudaStream_t s) {
   const size_t sm = (size_t)9 * smem_nodes * sizeof(T) + push_stage_bytes<T>();
-  k_push_batch_reset<T><<<(bg.nruns + 255) / 256, 256, 0, s>>>(a, bg.nruns, bg.push_counter);
   const int gb = grid_blocks < 304 ? grid_blocks : 304;
   if (order == 3) {
     cudaFuncSetAttribute(k_push_batch<T, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -1372,7 +1373,6 @@ void launch_push_batch(const StepArgs<T>* a, const BatchGrid& bg, int order, int
 template <class T>
 void launch_inject_batch(const StepArgs<T>* a, const BatchGrid& bg, cudaStream_t s) {
   k_inject_batch<T><<<bg.inj_blocks, 256, 0, s>>>(a, bg.inj_off, bg.nruns);
-  k_add_counts_batch<T><<<(bg.nruns + 127) / 128, 128, 0, s>>>(a, bg.nruns);
 }
 
 PushConst push_const(const GridP& g, double q, double m, double gamma_b, int fr1_sz, float fr1_fz, int pairs,
@@ -1403,12 +1403,11 @@ PushConst push_const(const GridP& g, double q, double m, double gamma_b, int fr1
 template <class T>
 void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* chunks, Ctrl* ctrl, int order,
                  int grid_blocks, int smem_nodes, int tile_z, double q, double m, double gamma_b, double beta_b,
-                 int fr1_sz, float fr1_fz, int pairs, int mlo, int nodal, const PushDefer& pd, cudaStream_t s) {
+                 int fr1_sz, float fr1_fz, int pairs, int mlo, int nodal, const PushDefer& pd,
+                 const AntennaStep& ant, const double* ant_xs, cudaStream_t s) {
   (void)beta_b;
   const PushConst pc = push_const(g, q, m, gamma_b, fr1_sz, fr1_fz, pairs, mlo);
   const size_t sm = (size_t)9 * smem_nodes * sizeof(T) + push_stage_bytes<T>();
-  cudaMemsetAsync(&ctrl->next_chunk, 0, sizeof(int), s);
-  cudaMemsetAsync(&ctrl->n_defer, 0, 2 * sizeof(int), s);
   // 'momentum conserving' gather: the node-interpolated copies; else the Yee-located gather copies
   const T* gE = nodal ? f.nE[0] : f.fE[0];
   const T* gB = nodal ? f.nB[0] : f.fB[0];
@@ -1425,12 +1424,16 @@ void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* c
     cudaFuncSetAttribute(k_push<T, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     k_push<T, 1, true><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
   }
-  // the global-memory pass over what the window kernel left (usually nothing: the blocks exit at once)
+  // the global-memory pass over what the window kernel left (usually nothing: its blocks exit at once), and the antenna
   const int gb = grid_blocks < 304 ? grid_blocks : 304;
-  if (order == 3 && !nodal) k_push_deferred<T, 3, false><<<gb, PB_THREADS, 0, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, pd, pc);
-  else if (order == 3) k_push_deferred<T, 3, true><<<gb, PB_THREADS, 0, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, pd, pc);
-  else if (!nodal) k_push_deferred<T, 1, false><<<gb, PB_THREADS, 0, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, pd, pc);
-  else k_push_deferred<T, 1, true><<<gb, PB_THREADS, 0, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, pd, pc);
+  const int ga = gb + (ant_xs ? (g.nx + PB_THREADS) / PB_THREADS : 0);
+  auto second = [&](auto kernel) {
+    kernel<<<ga, PB_THREADS, 0, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, pd, pc, gb, ant, ant_xs);
+  };
+  if (order == 3 && !nodal) second(k_push_deferred<T, 3, false>);
+  else if (order == 3) second(k_push_deferred<T, 3, true>);
+  else if (!nodal) second(k_push_deferred<T, 1, false>);
+  else second(k_push_deferred<T, 1, true>);
 }
 
 int push_occupancy(int order, bool dbl, int smem_nodes) {
@@ -1490,17 +1493,12 @@ void launch_inject(const GridP& g, Particles<T> p, Chunk* chunks, Ctrl* ctrl, co
   const int ncx = g.gx_hi - g.gx_lo;
   dim3 grd((ncx + ip.xblock - 1) / ip.xblock, (unsigned)((nrows + ip.rblock - 1) / ip.rblock));
   k_inject<T><<<grd, 256, 0, s>>>(g, p, chunks, ctrl, ip, cap, chunk_cap);
-  launch_add_counts(ctrl, (int)(nrows * ip.nxl), (int)(grd.x * grd.y), s);
-}
-
-void launch_add_counts(Ctrl* ctrl, int dcount, int dchunks, cudaStream_t s) {
-  k_add_counts<<<1, 1, 0, s>>>(ctrl, dcount, dchunks);
 }
 
 #define INST(T)                                                                                                 \
   template void launch_push<T>(const GridP&, const FieldPtrs<T>&, Particles<T>, Chunk*, Ctrl*, int, int, int,   \
                                int, double, double, double, double, int, float, int, int, int, const PushDefer&, \
-                               cudaStream_t);                                                                   \
+                               const AntennaStep&, const double*, cudaStream_t);                                                                   \
   template void launch_sort<T>(const GridP&, Particles<T>, Particles<T>, SortBufs, Chunk*, Ctrl*, int, int, int,\
                                cudaStream_t);                                                                   \
   template void launch_inject<T>(const GridP&, Particles<T>, Chunk*, Ctrl*, const InjectP&, int, int, cudaStream_t); \
