@@ -271,6 +271,31 @@ __device__ __forceinline__ void weights1(R t, R* w) {
 }
 
 // ---------------------------------------------------------------------------
+// The kernels of a 2D step are launched so that each may begin while its predecessor on the stream ends (programmatic
+// dependent launch) and wait for it here, before the first access to anything that a step changes: launch latency and
+// block set-up overlap the predecessor's tail. A kernel launched without the attribute returns from the wait at once.
+__device__ __forceinline__ void chain_wait() {
+#if __CUDA_ARCH__ >= 900
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+#endif
+}
+template <class... KA, class... A>
+inline void launch_chained(void (*k)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, k, KA(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Launchers (defined in the .cu files, instantiated for float and double).
 // TMA descriptors of the 3-component blocks read by the tile kernels (a 3D tensor
 // (nz+1) x (nx+1) x 3 per block; out-of-range elements read as zero)

@@ -174,6 +174,7 @@ __device__ __forceinline__ void faraday_tile(const GridP& g, const FieldPtrs<T>&
 
 template <class T, bool FRIED, bool CK>
 __global__ void __launch_bounds__(FT_Z* FT_TY) k_faraday(GridP g, FieldPtrs<T> f, PmlTabs pt, FarK<T> q) {
+  chain_wait();
   faraday_tile<T, FRIED, CK>(g, f, pt, q, blockIdx.x, blockIdx.y);
 }
 
@@ -509,6 +510,7 @@ __global__ void __launch_bounds__(FT_Z* FT_TY) k_filter_fields(GridP g, FieldPtr
                                                                const __grid_constant__ CUtensorMap mapE,
                                                                const __grid_constant__ CUtensorMap mapB, TileMaps tm,
                                                                Ctrl* ctrl, int c_first) {
+  chain_wait();
   filter_fields_tile<T, PT>(g, f, ft, &mapE, &mapB, tm, ctrl, blockIdx.x, blockIdx.y, c_first);
 }
 
@@ -627,6 +629,7 @@ __global__ void __launch_bounds__(FT_Z* FT_TY, 4) k_faraday_fused(GridP g, Field
                                                                const __grid_constant__ CUtensorMap mapEo,
                                                                const __grid_constant__ CUtensorMap mapEb,
                                                                Ctrl* ctrl) {
+  chain_wait();
   faraday_fused_tile<T, FRIED, CK, PT>(g, f, pt, q, ft, &mapE, &mapEo, &mapEb, ctrl, blockIdx.x, blockIdx.y);
 }
 
@@ -767,6 +770,7 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
 template <class T>
 __global__ void __launch_bounds__(FT_Z* FT_TY) k_ampere_direct(GridP g, FieldPtrs<T> f, PmlTabs pt, FilterTaps<T> ft,
                                                               TileMaps tm, Ctrl* ctrl) {
+  chain_wait();
   ampere_tile<T, false, 0, true>(g, f, pt, ft, nullptr, nullptr, 0.0, nullptr, tm, ctrl, blockIdx.x, blockIdx.y,
                                  blockIdx.z, blockIdx.z);
 }
@@ -776,6 +780,7 @@ __global__ void __launch_bounds__(FT_Z* FT_TY, sizeof(T) == 4 ? 4 : 2) k_ampere(
                                                         const double* ion_x, const double* ion_c, double ion_coef,
                                                         const __grid_constant__ CUtensorMap mapJ, TileMaps tm,
                                                         Ctrl* ctrl) {
+  chain_wait();
   ampere_tile<T, FILT, PT>(g, f, pt, ft, ion_x, ion_c, ion_coef, &mapJ, tm, ctrl, blockIdx.x, blockIdx.y);
 }
 
@@ -892,6 +897,7 @@ __global__ void __launch_bounds__(WXC* WXG) k_wide_x(GridP g, const __grid_const
   const int lane = threadIdx.x, gy = threadIdx.y;
   const int H = w.H, k = k0 + lane * CV;
   wide_taps_to(sc, w, gy * WXC + lane, WXC * WXG, WSC);
+  chain_wait();
   const T* F = job.src[c];
   const bool ion = c == job.ion;
   T cz[CV];
@@ -961,6 +967,7 @@ __global__ void __launch_bounds__(WZT* WZB) k_wide_z(GridP g, const __grid_const
   const int t = threadIdx.x, ry = threadIdx.y;
   const int H = w.H, i = blockIdx.y * WZB + ry;
   wide_taps_to(sc, w, ry * WZT + t, WZT * WZB, WSC);
+  chain_wait();
   const T* F = job.src[c];
   const int n = NZ + 2 * H + 8;
   constexpr int U = 8;
@@ -1175,7 +1182,7 @@ static void run_faraday_staged(dim3 grd, dim3 blk, cudaStream_t s, const GridP& 
   const size_t sm = (size_t)9 * ring_stride<T>() * sizeof(T) + 128;
   const int e = tm.Ebase[0] == (const void*)f.E[0] ? 0 : 1, b = tm.Ebbase[0] == (const void*)f.Eb[0] ? 0 : 1;
   cudaFuncSetAttribute(k_faraday_fused<T, true, CK, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_faraday_fused<T, true, CK, 0><<<grd, blk, sm, s>>>(g, f, pt, q, FilterTaps<T>{}, tm.Er[e], tm.Er[1 - e], tm.Eb[b],
+  launch_chained(k_faraday_fused<T, true, CK, 0>, grd, blk, sm, s, g, f, pt, q, FilterTaps<T>{}, tm.Er[e], tm.Er[1 - e], tm.Eb[b],
                                                         ctrl);
 }
 
@@ -1192,11 +1199,11 @@ void launch_faraday(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, do
     return;
   }
   if (friedman) {
-    if (ck) k_faraday<T, true, true><<<grd, blk, 0, s>>>(g, f, pt, q);
-    else k_faraday<T, true, false><<<grd, blk, 0, s>>>(g, f, pt, q);
+    if (ck) launch_chained(k_faraday<T, true, true>, grd, blk, 0, s, g, f, pt, q);
+    else launch_chained(k_faraday<T, true, false>, grd, blk, 0, s, g, f, pt, q);
   } else {
-    if (ck) k_faraday<T, false, true><<<grd, blk, 0, s>>>(g, f, pt, q);
-    else k_faraday<T, false, false><<<grd, blk, 0, s>>>(g, f, pt, q);
+    if (ck) launch_chained(k_faraday<T, false, true>, grd, blk, 0, s, g, f, pt, q);
+    else launch_chained(k_faraday<T, false, false>, grd, blk, 0, s, g, f, pt, q);
   }
 }
 
@@ -1329,7 +1336,7 @@ static void run_filter_fields(dim3 grd, dim3 blk, size_t sm, cudaStream_t s, con
                               const FilterTaps<T>& ft, const CUtensorMap& mE, const TileMaps& tm, Ctrl* ctrl,
                               int c_first) {
   cudaFuncSetAttribute(k_filter_fields<T, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_filter_fields<T, PT><<<grd, blk, sm, s>>>(g, f, ft, mE, tm.Bavg, tm, ctrl, c_first);
+  launch_chained(k_filter_fields<T, PT>, grd, blk, sm, s, g, f, ft, mE, tm.Bavg, tm, ctrl, c_first);
 }
 
 // the taps at offsets -H .. H, strides written out
@@ -1346,10 +1353,10 @@ static void run_wide_h(const GridP& g, const WideTaps<T>& w, WideJob<T> job, T* 
   T* dst[6];
   for (int c = 0; c < ncomp; c++) { dst[c] = job.dst[c]; job.dst[c] = scratch + c * g.cs; }
   constexpr int XC = WXC * WideV<T>::n, XR = WXG * WXR, ZC = WZT * WZR;
-  k_wide_x<T, HM><<<dim3((g.nz + XC) / XC, (g.nx + XR) / XR, ncomp), dim3(WXC, WXG), 0, s>>>(g, w, job);
+  launch_chained(k_wide_x<T, HM>, dim3((g.nz + XC) / XC, (g.nx + XR) / XR, ncomp), dim3(WXC, WXG), 0, s, g, w, job);
   for (int c = 0; c < ncomp; c++) { job.src[c] = job.dst[c]; job.dst[c] = dst[c]; }
   job.ion = -1;
-  k_wide_z<T, HM><<<dim3((g.nz + ZC) / ZC, (g.nx + WZB) / WZB, ncomp), dim3(WZT, WZB), 0, s>>>(g, w, job);
+  launch_chained(k_wide_z<T, HM>, dim3((g.nz + ZC) / ZC, (g.nx + WZB) / WZB, ncomp), dim3(WZT, WZB), 0, s, g, w, job);
 }
 
 template <class T>
@@ -1425,7 +1432,7 @@ static bool run_faraday_fused(dim3 grd, dim3 blk, cudaStream_t s, const GridP& g
   const CUtensorMap& mEo = cur0 ? tm.Er[1] : tm.Er[0];
   const CUtensorMap& mEb = tm.Ebbase[0] == (const void*)f.Eb[0] ? tm.Eb[0] : tm.Eb[1];
   cudaFuncSetAttribute(k_faraday_fused<T, FRIED, CK, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_faraday_fused<T, FRIED, CK, PT><<<grd, blk, sm, s>>>(g, f, pt, q, ft, mE, mEo, mEb, ctrl);
+  launch_chained(k_faraday_fused<T, FRIED, CK, PT>, grd, blk, sm, s, g, f, pt, q, ft, mE, mEo, mEb, ctrl);
   return true;
 }
 
@@ -1468,7 +1475,7 @@ static void run_ampere(dim3 grd, dim3 blk, size_t sm, cudaStream_t s, const Grid
                        const PmlTabs& pt, const FilterTaps<T>& ft, const double* ion_x, const double* ion_c,
                        double ion_coef, const CUtensorMap& mJ, const TileMaps& tm, Ctrl* ctrl) {
   cudaFuncSetAttribute(k_ampere<T, FILT, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_ampere<T, FILT, PT><<<grd, blk, sm, s>>>(g, f, pt, ft, ion_x, ion_c, ion_coef, mJ, tm, ctrl);
+  launch_chained(k_ampere<T, FILT, PT>, grd, blk, sm, s, g, f, pt, ft, ion_x, ion_c, ion_coef, mJ, tm, ctrl);
 }
 
 template <class T>
@@ -1485,7 +1492,7 @@ void launch_ampere(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, con
     job.ion = ion_x ? 2 : -1;
     job.ion_x = ion_x; job.ion_c = ion_c; job.coef = ion_coef;
     run_wide<T>(g, wide_taps(ft), job, f.wide, 3, s);
-    k_ampere_direct<T><<<dim3(grd.x, grd.y, 3), blk, 0, s>>>(g, f, pt, ft, tm, ctrl);
+    launch_chained(k_ampere_direct<T>, dim3(grd.x, grd.y, 3), blk, 0, s, g, f, pt, ft, tm, ctrl);
     return;
   }
   if (!filter_on) {

@@ -911,6 +911,7 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push(GridP g, 
   T* sm = reinterpret_cast<T*>(smraw);
   __shared__ int s_chunk;
   __shared__ int s_bb[6];
+  chain_wait();
   const int nchunks = ctrl->nchunks;
   while (true) {
     if (threadIdx.x == 0) {
@@ -935,6 +936,7 @@ __global__ void __launch_bounds__(PB_THREADS) k_push_deferred(GridP g, const T* 
                                                                Particles<T> p, Chunk* chunks, Ctrl* ctrl,
                                                                PushDefer pd, PushConst pc, int nblk,
                                                                AntennaStep ant, const double* ant_xs) {
+  chain_wait();
   if ((int)blockIdx.x >= nblk) {
     antenna_column<T>(g, gJ + g.cs, ant_xs, ant, ((int)blockIdx.x - nblk) * PB_THREADS + threadIdx.x);
     return;
@@ -1242,6 +1244,7 @@ __device__ __forceinline__ void inject_block(const GridP& g, const Particles<T>&
 
 template <class T>
 __global__ void k_inject(GridP g, Particles<T> p, Chunk* chunks, Ctrl* ctrl, InjectP ip, int cap, int chunk_cap) {
+  chain_wait();
   inject_block<T>(g, p, chunks, ctrl, ip, cap, chunk_cap, blockIdx.x, blockIdx.y, gridDim.x,
                   gridDim.x * gridDim.y);
 }
@@ -1413,22 +1416,22 @@ void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* c
   const T* gB = nodal ? f.nB[0] : f.fB[0];
   if (order == 3 && !nodal) {
     cudaFuncSetAttribute(k_push<T, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_push<T, 3, false><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
+    launch_chained(k_push<T, 3, false>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
   } else if (order == 3) {
     cudaFuncSetAttribute(k_push<T, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_push<T, 3, true><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
+    launch_chained(k_push<T, 3, true>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
   } else if (!nodal) {
     cudaFuncSetAttribute(k_push<T, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_push<T, 1, false><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
+    launch_chained(k_push<T, 1, false>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
   } else {
     cudaFuncSetAttribute(k_push<T, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_push<T, 1, true><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
+    launch_chained(k_push<T, 1, true>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
   }
   // the global-memory pass over what the window kernel left (usually nothing: its blocks exit at once), and the antenna
   const int gb = grid_blocks < 304 ? grid_blocks : 304;
   const int ga = gb + (ant_xs ? (g.nx + PB_THREADS) / PB_THREADS : 0);
   auto second = [&](auto kernel) {
-    kernel<<<ga, PB_THREADS, 0, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, pd, pc, gb, ant, ant_xs);
+    launch_chained(kernel, ga, PB_THREADS, 0, s, g, gE, gB, f.J[0], p, chunks, ctrl, pd, pc, gb, ant, ant_xs);
   };
   if (order == 3 && !nodal) second(k_push_deferred<T, 3, false>);
   else if (order == 3) second(k_push_deferred<T, 3, true>);
@@ -1492,7 +1495,7 @@ void launch_inject(const GridP& g, Particles<T> p, Chunk* chunks, Ctrl* ctrl, co
   if (nrows <= 0) return;
   const int ncx = g.gx_hi - g.gx_lo;
   dim3 grd((ncx + ip.xblock - 1) / ip.xblock, (unsigned)((nrows + ip.rblock - 1) / ip.rblock));
-  k_inject<T><<<grd, 256, 0, s>>>(g, p, chunks, ctrl, ip, cap, chunk_cap);
+  launch_chained(k_inject<T>, grd, 256, 0, s, g, p, chunks, ctrl, ip, cap, chunk_cap);
 }
 
 #define INST(T)                                                                                                 \
