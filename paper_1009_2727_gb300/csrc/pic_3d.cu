@@ -1004,29 +1004,41 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
         shape_w<T, ORD>(Xs - fl, wg[a][h]);
         bl[a][h] = (int)fl - SH + WGM;
       }
-    T EB[6];
+    // Yee locations; every component at the nodes for the 'momentum conserving' gather (MC). The tensor-product sum is
+    // taken axis by axis: z within each (x, y) row, then y, then x. The x planes are a rolled loop (the x weights rotate
+    // past index 0) and the rest unrolled: fully unrolled, this and the deposit came to some 80 KB of instructions and a
+    // third of the stalls were instruction fetches (2.4 M electrons on 256 x 128 x 128 cells: 1310 us, rolled 887 us).
+    T EB[6] = {};
+    {
+      const T* F[6];
 #pragma unroll
-    for (int c = 0; c < 6; c++) {
-      // Yee locations; every component at the nodes for the 'momentum conserving' gather (MC). The
-      // tensor-product sum taken axis by axis: z within each (x, y) row, then y, then x
-      const int hx = MC ? 0 : c < 3 ? (c == 0) : (c != 3), hy = MC ? 0 : c < 3 ? (c == 1) : (c != 4),
-                hz = MC ? 0 : c < 3 ? (c == 2) : (c != 5);
-      const T* F = sF + c * WGN + (bl[0][hx] * WGY + bl[1][hy]) * WGZ + bl[2][hz];
-      T acc = T(0);
-#pragma unroll
-      for (int l0 = 0; l0 < NS; l0++) {
-        T accy = T(0);
-#pragma unroll
-        for (int l1 = 0; l1 < NS; l1++) {
-          const T* row = F + (l0 * WGY + l1) * WGZ;
-          T accz = T(0);
-#pragma unroll
-          for (int l2 = 0; l2 < NS; l2++) accz += row[l2] * wg[2][hz][l2];
-          accy += wg[1][hy][l1] * accz;
-        }
-        acc += wg[0][hx][l0] * accy;
+      for (int c = 0; c < 6; c++) {
+        const int hx = MC ? 0 : c < 3 ? (c == 0) : (c != 3), hy = MC ? 0 : c < 3 ? (c == 1) : (c != 4),
+                  hz = MC ? 0 : c < 3 ? (c == 2) : (c != 5);
+        F[c] = sF + c * WGN + (bl[0][hx] * WGY + bl[1][hy]) * WGZ + bl[2][hz];
       }
-      EB[c] = acc;
+#pragma unroll 1
+      for (int l0 = 0; l0 < NS; l0++) {
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+          const int hx = MC ? 0 : c < 3 ? (c == 0) : (c != 3), hy = MC ? 0 : c < 3 ? (c == 1) : (c != 4),
+                    hz = MC ? 0 : c < 3 ? (c == 2) : (c != 5);
+          T accy = T(0);
+#pragma unroll
+          for (int l1 = 0; l1 < NS; l1++) {
+            T accz = T(0);
+#pragma unroll
+            for (int l2 = 0; l2 < NS; l2++) accz += F[c][l1 * WGZ + l2] * wg[2][hz][l2];
+            accy += wg[1][hy][l1] * accz;
+          }
+          EB[c] += wg[0][hx][0] * accy;
+          F[c] += WGY * WGZ;
+        }
+#pragma unroll
+        for (int h = 0; h < (MC ? 1 : 2); h++)
+#pragma unroll
+          for (int m = 0; m < NS - 1; m++) wg[0][h][m] = wg[0][h][m + 1];
+      }
     }
     T u[3] = {p.ux[j], p.uy[j], p.uz[j]};
     boris3<T>(u, EB, EB + 3, kq);
@@ -1041,6 +1053,7 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
     // Esirkepov into the shared window
     T S0[3][W], DS[3][W];
     int base[3];
+    bool crossed[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       const T f0 = floor(X[a]), f1 = floor(X1[a]);
@@ -1050,6 +1063,7 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
       shape_w<T, ORD>(X1[a] - f1, wb);
       // each stencil starts at base or one cell above (moves below one cell): select with constant indices
       const bool up0 = f0 > f1, up1 = f1 > f0;
+      crossed[a] = up0 || up1;
 #pragma unroll
       for (int m = 0; m < W; m++) {
         const T s0 = up0 ? (m > 0 ? wa[m - 1] : T(0)) : (m < NS ? wa[m] : T(0));
@@ -1059,24 +1073,13 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
       }
       base[a] += WM;
     }
-    // the prefix along q of W_q = DS_q tr(u, v) factorises: J_q(m_q, m_u, m_v) = cq tr(m_u, m_v) C_q(m_q),
-    // C_q the running sum of DS_q; all loops unrolled so that the stencils stay in registers
-    // C_q at the W - 1 edges between the stencil's nodes (its value past the last node is the total change
-    // of the shape, zero)
-    T Cm[3][W - 1];
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-      T run = T(0);
-#pragma unroll
-      for (int m = 0; m < W - 1; m++) {
-        run += DS[a][m];
-        Cm[a][m] = run;
-      }
-    }
+    // the prefix along q of W_q = DS_q tr(u, v) factorises: J_q(m_q, m_u, m_v) = cq tr(m_u, m_v) C_q(m_q), C_q the
+    // running sum of DS_q at the W - 1 edges between the stencil's nodes (its value past the last node is the total
+    // change of the shape, zero; so is the last edge's of a particle that stays in its cell along q, whose last node is
+    // empty). The planes along u are a rolled loop, the u weights rotating past index 0 (see the gather); every term's
+    // offset from its plane is a compile-time constant.
     const T wj = p.w[j];
-    // the window offset of the stencil's first node; every term's offset from it is a compile-time
-    // constant once the loops are unrolled
-    const int off0 = (base[0] * WY + base[1]) * WZ + base[2];
+    T* J0 = sJ + (base[0] * WY + base[1]) * WZ + base[2];   // the stencil's first node
 #pragma unroll
     for (int q = 0; q < 3; q++) {
       const int u1 = (q + 1) % 3, v1 = (q + 2) % 3;
@@ -1084,8 +1087,12 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
 #pragma unroll
       for (int m = 0; m < W; m++) moved |= DS[q][m] != T(0);
       if (!moved) continue;
+      T Cm[W - 1];
+      T run = T(0);
+#pragma unroll
+      for (int m = 0; m < W - 1; m++) { run += DS[q][m]; Cm[m] = run; }
+      if (!crossed[q]) Cm[W - 2] = T(0);
       const T cq = cqw[q] * wj;
-      T* Jq = sJ + q * WN + off0;
       // tr(u, v) = S0_u S0_v + DS_u S0_v / 2 + S0_u DS_v / 2 + DS_u DS_v / 3
       //          = S0_u (S0_v + DS_v / 2) + DS_u (S0_v / 2 + DS_v / 3), times cq
       T Av[W], Bv[W];
@@ -1094,19 +1101,26 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
         Av[mv] = cq * (S0[v1][mv] + T(0.5) * DS[v1][mv]);
         Bv[mv] = cq * (T(0.5) * S0[v1][mv] + DS[v1][mv] * T(1.0 / 3.0));
       }
-#pragma unroll
-      for (int mu = 0; mu < W; mu++)
+      T* plane = J0 + q * WN;
+#pragma unroll 1
+      for (int mu = 0; mu < W; mu++, plane += wstride(u1)) {
+        const T su0 = S0[u1][0], du0 = DS[u1][0];
 #pragma unroll
         for (int mv = 0; mv < W; mv++) {
-          const T ct = S0[u1][mu] * Av[mv] + DS[u1][mu] * Bv[mv];
+          const T ct = su0 * Av[mv] + du0 * Bv[mv];
           if (ct == T(0)) continue;
 #pragma unroll
           for (int mq = 0; mq < W - 1; mq++) {
-            const T v = ct * Cm[q][mq];
+            const T v = ct * Cm[mq];
             if (v == T(0)) continue;
-            atomicAdd(Jq + mq * wstride(q) + mu * wstride(u1) + mv * wstride(v1), v);
+            atomicAdd(plane + mq * wstride(q) + mv * wstride(v1), v);
           }
         }
+#pragma unroll
+        for (int m = 0; m < W - 1; m++) { S0[u1][m] = S0[u1][m + 1]; DS[u1][m] = DS[u1][m + 1]; }
+        S0[u1][W - 1] = su0;
+        DS[u1][W - 1] = du0;
+      }
     }
     const double pn[3] = {pos[0] + (double)Dm[0], pos[1] + (double)Dm[1], pos[2] + (double)Dm[2]};
     p.x[j] = pn[0]; p.y[j] = pn[1]; p.z[j] = pn[2];
