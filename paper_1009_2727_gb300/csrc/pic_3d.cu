@@ -814,8 +814,8 @@ constexpr int WGM = 2;
 constexpr int WGX = TX + 2 * WGM + 1, WGY = TY + 2 * WGM + 1, WGZ = TZ + 2 * WGM + 1;
 constexpr int WGN = WGX * WGY * WGZ;
 // shared memory of the 3D push: the six gathered fields on the field window, the current on its window
-template <class T>
-constexpr int push3_smem() { return (int)((6 * WGN + 3 * WN) * sizeof(T)); }
+template <class T, bool FEW>
+constexpr int push3_smem() { return (int)((6 * WGN + (FEW ? 0 : 3 * WN)) * sizeof(T)); }
 
 // The sort of every step: particles by tile and, inside a tile, by cell (z fastest), so that the lanes of a push warp
 // gather and deposit on neighbouring words: in tile order alone the shared-memory pipe spent half its wavefronts on
@@ -937,14 +937,34 @@ __global__ void k3_tile_scatter(Parts3<T> src, Parts3<T> dst, Tiles3 t, int n_ol
   dst.w[q] = src.w[j]; dst.id[q] = src.id[j]; dst.fl[q] = 1;
 }
 
-template <class T, int ORD, bool MC>
+// entry h of v with h a lane's own (a dynamic index would put v into local memory)
+template <class T, int N>
+__device__ __forceinline__ T pick(const T (&v)[N], int h) {
+  T x = v[0];
+#pragma unroll
+  for (int m = 1; m < N; m++) x = h == m ? v[m] : x;
+  return x;
+}
+
+// FEW: for a run with fewer particles than the chip has threads (the launch's rule). A tile's particles are split over
+// kSplit blocks, four lanes share a particle, each gathers one x plane and deposits every fourth plane, straight into J.
+// One block per tile and one lane per particle left most of the chip idle, and in a tile with several particles per cell
+// the lanes met on every shared add (a compare-and-swap loop); J in global memory takes adds without an answer.
+constexpr int kQuad = 4, kSplit = 8;
+
+template <class T, int ORD, bool MC, bool FEW>
 __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<T> p, Tiles3 t, Ctrl3* ctrl, T kq,
                                                      Cq3<T> cq) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sF = reinterpret_cast<T*>(smraw);        // 6 x WGN gather fields
   T* sJ = sF + 6 * WGN;                       // 3 x WN current
   const int tile = blockIdx.x;
-  const int p0 = t.start[tile], p1 = t.start[tile + 1];
+  int p0 = t.start[tile], p1 = t.start[tile + 1];
+  if constexpr (FEW) {
+    const int np = p1 - p0;
+    p1 = p0 + np * ((int)blockIdx.y + 1) / kSplit;
+    p0 += np * (int)blockIdx.y / kSplit;
+  }
   if (p1 <= p0) return;
   const int tz = tile % t.nt[2], r = tile / t.nt[2];
   const int ty = r % t.nt[1], tx = r / t.nt[1];
@@ -982,7 +1002,8 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
     for (int u = 0; u < SU; u++)
       if (l0 + u < NL && lane < WGZ) sF[(l0 + u) * WGZ + lane] = v[u];
   }
-  for (int e = threadIdx.x; e < 3 * WN; e += blockDim.x) sJ[e] = T(0);
+  if constexpr (!FEW)
+    for (int e = threadIdx.x; e < 3 * WN; e += blockDim.x) sJ[e] = T(0);
   __syncthreads();
   constexpr int NS = ORD == 3 ? 4 : 2;
   constexpr int SH = ORD == 3 ? 1 : 0;
@@ -1007,9 +1028,10 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
   for (int a = 0; a < 3; a++) cqw[a] = cq.v[a];
   // a thread takes consecutive particles: with as many per cell throughout, the lanes of a warp then hold particles of
   // different, neighbouring cells at any time (particles of one cell would meet on every shared add)
-  const int per = (p1 - p0 + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int j0 = p0 + (int)threadIdx.x * per, j1 = min(p1, j0 + per);
-  for (int j = j0; j < j1; j++) {
+  const int h = FEW ? threadIdx.x % kQuad : 0;   // the lane's part of its particle
+  const int per = FEW ? 1 : (p1 - p0 + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int j0 = FEW ? p0 + (int)threadIdx.x / kQuad : p0 + (int)threadIdx.x * per, j1 = FEW ? p1 : min(p1, j0 + per);
+  for (int j = j0; j < j1; j += FEW ? (int)blockDim.x / kQuad : 1) {
     const double pos[3] = {p.x[j], p.y[j], p.z[j]};
     T X[3];
     bool inside = true;
@@ -1051,8 +1073,14 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
                   hz = MC ? 0 : c < 3 ? (c == 2) : (c != 5);
         F[c] = sF + c * WGN + (bl[0][hx] * WGY + bl[1][hy]) * WGZ + bl[2][hz];
       }
+      if constexpr (FEW) {
+#pragma unroll
+        for (int c = 0; c < 6; c++) F[c] += h * (WGY * WGZ);
+#pragma unroll
+        for (int k = 0; k < (MC ? 1 : 2); k++) wg[0][k][0] = pick(wg[0][k], h);
+      }
 #pragma unroll 1
-      for (int l0 = 0; l0 < NS; l0++) {
+      for (int l0 = FEW ? h : 0; l0 < NS; l0 += FEW ? kQuad : 1) {
 #pragma unroll
         for (int c = 0; c < 6; c++) {
           const int hx = MC ? 0 : c < 3 ? (c == 0) : (c != 3), hy = MC ? 0 : c < 3 ? (c == 1) : (c != 4),
@@ -1072,6 +1100,14 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
         for (int h = 0; h < (MC ? 1 : 2); h++)
 #pragma unroll
           for (int m = 0; m < NS - 1; m++) wg[0][h][m] = wg[0][h][m + 1];
+      }
+    }
+    if constexpr (FEW) {   // the planes' sum, the same in the four lanes (they hold the same particle and are all here)
+      const unsigned mask = 0xfu << (threadIdx.x & 28);
+#pragma unroll
+      for (int c = 0; c < 6; c++) {
+        EB[c] += __shfl_xor_sync(mask, EB[c], 1);
+        EB[c] += __shfl_xor_sync(mask, EB[c], 2);
       }
     }
     T u[3] = {p.ux[j], p.uy[j], p.uz[j]};
@@ -1105,7 +1141,6 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
         S0[a][m] = s0;
         DS[a][m] = s1 - s0;
       }
-      base[a] += WM;
     }
     // the prefix along q of W_q = DS_q tr(u, v) factorises: J_q(m_q, m_u, m_v) = cq tr(m_u, m_v) C_q(m_q), C_q the
     // running sum of DS_q at the W - 1 edges between the stencil's nodes (its value past the last node is the total
@@ -1113,7 +1148,9 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
     // empty). The planes along u are a rolled loop, the u weights rotating past index 0 (see the gather); every term's
     // offset from its plane is a compile-time constant.
     const T wj = p.w[j];
-    T* J0 = sJ + (base[0] * WY + base[1]) * WZ + base[2];   // the stencil's first node
+    // the stencil's first node in the window, and on the grid
+    T* J0 = sJ + ((base[0] + WM) * WY + base[1] + WM) * WZ + base[2] + WM;
+    const int gn[3] = {c0[0] + base[0], c0[1] + base[1], c0[2] + base[2]};
 #pragma unroll
     for (int q = 0; q < 3; q++) {
       const int u1 = (q + 1) % 3, v1 = (q + 2) % 3;
@@ -1134,6 +1171,27 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
       for (int mv = 0; mv < W; mv++) {
         Av[mv] = cq * (S0[v1][mv] + T(0.5) * DS[v1][mv]);
         Bv[mv] = cq * (T(0.5) * S0[v1][mv] + DS[v1][mv] * T(1.0 / 3.0));
+      }
+      if constexpr (FEW) {
+        const long st[3] = {line_stride, g.ldz, 1};
+        T* Jq = f.J[q] + (long)gn[0] * line_stride + (long)gn[1] * g.ldz + gn[2];
+#pragma unroll 1
+        for (int mu = h; mu < W; mu += kQuad) {
+          if ((unsigned)(gn[u1] + mu) > (unsigned)g.n[u1]) continue;   // the window's margin off the grid holds nothing
+          const T su = pick(S0[u1], mu), du = pick(DS[u1], mu);
+#pragma unroll
+          for (int mv = 0; mv < W; mv++) {
+            const T ct = su * Av[mv] + du * Bv[mv];
+            if (ct == T(0) || (unsigned)(gn[v1] + mv) > (unsigned)g.n[v1]) continue;
+#pragma unroll
+            for (int mq = 0; mq < W - 1; mq++) {
+              const T v = ct * Cm[mq];
+              if (v == T(0) || (unsigned)(gn[q] + mq) > (unsigned)g.n[q]) continue;
+              atomicAdd(Jq + mq * st[q] + mu * st[u1] + mv * st[v1], v);
+            }
+          }
+        }
+        continue;
       }
       T* plane = J0 + q * WN;
 #pragma unroll 1
@@ -1156,6 +1214,10 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
         DS[u1][W - 1] = du0;
       }
     }
+    if constexpr (FEW) {
+      __syncwarp(0xfu << (threadIdx.x & 28));   // the four have read the particle before one writes it back
+      if (h) continue;
+    }
     const double pn[3] = {pos[0] + (double)Dm[0], pos[1] + (double)Dm[1], pos[2] + (double)Dm[2]};
     p.x[j] = pn[0]; p.y[j] = pn[1]; p.z[j] = pn[2];
     p.ux[j] = u[0]; p.uy[j] = u[1]; p.uz[j] = u[2];
@@ -1175,6 +1237,7 @@ __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<
     }
     if (out) p.fl[j] = 0;
   }
+  if constexpr (FEW) return;
   __syncthreads();
   // the window's current added to J line by line, as it was staged
   for (int line = warp; line < 3 * WX * WY; line += nwarps) {
@@ -1976,6 +2039,7 @@ struct Sim3 : Sim3Api {
   int64_t compactions = 0;
   Tiles3 tl{};
   int ntiles = 0, nsum = 0;
+  long few_max = 0;       // up to this many particles the push splits tiles over blocks and particles over lanes
   long key_cap = 0;
   // plasma
   bool loaded = false;
@@ -2156,11 +2220,18 @@ struct Sim3 : Sim3Api {
     tl.ccnt = dal<int>((size_t)ntiles * TC + nsum);
     if (!tl.cnt || !tl.start || !tl.ccnt) return fail(PIC_ENOMEM, "allocation failed");
     tl.bsum = tl.ccnt + (size_t)ntiles * TC;
-    const int smem = push3_smem<T>();
-    cudaFuncSetAttribute(k3_push_tiles<T, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k3_push_tiles<T, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k3_push_tiles<T, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k3_push_tiles<T, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const auto set_smem = [](auto* few, auto* many) {
+      cudaFuncSetAttribute(few, cudaFuncAttributeMaxDynamicSharedMemorySize, push3_smem<T, true>());
+      cudaFuncSetAttribute(many, cudaFuncAttributeMaxDynamicSharedMemorySize, push3_smem<T, false>());
+    };
+    set_smem(k3_push_tiles<T, 3, false, true>, k3_push_tiles<T, 3, false, false>);
+    set_smem(k3_push_tiles<T, 1, false, true>, k3_push_tiles<T, 1, false, false>);
+    set_smem(k3_push_tiles<T, 3, true, true>, k3_push_tiles<T, 3, true, false>);
+    set_smem(k3_push_tiles<T, 1, true, true>, k3_push_tiles<T, 1, true, false>);
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    few_max = 256L * nsm;
     cudaEventCreate(&ev0);
     cudaEventCreate(&ev1);
     return cudaGetLastError() == cudaSuccess ? PIC_OK : fail(PIC_ECUDA, "CUDA error in 3D init");
@@ -2480,6 +2551,15 @@ struct Sim3 : Sim3Api {
     tev.clear();
   }
 
+  template <int ORD, bool MC>
+  void launch_push(const Fld3<T>& f, T kq) {
+    if (count_ub <= few_max)
+      k3_push_tiles<T, ORD, MC, true><<<dim3(ntiles, kSplit), 256, push3_smem<T, true>(), s>>>(g, f, P2[cur], tl, ctrl, kq,
+                                                                                              cq_e);
+    else
+      k3_push_tiles<T, ORD, MC, false><<<ntiles, 256, push3_smem<T, false>(), s>>>(g, f, P2[cur], tl, ctrl, kq, cq_e);
+  }
+
   int one_step() {
     const long nn = nodes();
     const long n3 = 3 * g.cs;
@@ -2509,16 +2589,11 @@ struct Sim3 : Sim3Api {
     const T kq = T(-kQe * g.dt / (2.0 * kMe));
     if (loaded && count_ub > 0) {
       sort_tiles();
-      const int smem = push3_smem<T>();
       tbeg(0);
-      if (cfg.shape_order == 3 && !nodal)
-        k3_push_tiles<T, 3, false><<<ntiles, 256, smem, s>>>(g, f, P2[cur], tl, ctrl, kq, cq_e);
-      else if (cfg.shape_order == 3)
-        k3_push_tiles<T, 3, true><<<ntiles, 256, smem, s>>>(g, f, P2[cur], tl, ctrl, kq, cq_e);
-      else if (!nodal)
-        k3_push_tiles<T, 1, false><<<ntiles, 256, smem, s>>>(g, f, P2[cur], tl, ctrl, kq, cq_e);
-      else
-        k3_push_tiles<T, 1, true><<<ntiles, 256, smem, s>>>(g, f, P2[cur], tl, ctrl, kq, cq_e);
+      if (cfg.shape_order == 3 && !nodal) launch_push<3, false>(f, kq);
+      else if (cfg.shape_order == 3) launch_push<3, true>(f, kq);
+      else if (!nodal) launch_push<1, false>(f, kq);
+      else launch_push<1, true>(f, kq);
       nl++;
       tend(0);
     }
