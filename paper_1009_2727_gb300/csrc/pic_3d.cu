@@ -102,7 +102,8 @@ struct Cq3 {
 struct Ctrl3 {
   int count;
   int status;
-  int pad[2];
+  int inj_done;   // blocks of k3_inject that have read the count
+  int pad;
   double red[8];
 };
 
@@ -115,12 +116,12 @@ struct Taps3 {
 // ---------------------------------------------------------------------------
 // fields
 // Faraday with the enlarged operator, Friedman's E_eff and the split PML for B (PR-1, PR-2), over a tile
-// of FX x FY x FZ nodes. E_eff = c1 E^n - c2 E^{n-1} + c3 E-bar^{n-2} is formed while the tile and a
+// of FX x FY x FZ nodes (FX: see the launch). E_eff = c1 E^n - c2 E^{n-1} + c3 E-bar^{n-2} is formed while the tile and a
 // one-node halo are staged in shared memory (zero off the grid); each thread then updates the three B
 // components of FX nodes along x.
 //   Delta*_a F at a node (result half a cell above along a) = (alpha D(0,0) + beta (four axial neighbours)
 //   + gamma (four diagonal neighbours)) / d_a, D the difference along a on the transverse offsets.
-constexpr int FX = 4, FY = 8, FZ = 32;
+constexpr int FY = 8, FZ = 32;
 // z nodes per thread of the other grid sweeps (a block width apart)
 constexpr int KPT = 4;
 
@@ -142,11 +143,12 @@ __device__ __forceinline__ T dstar_s(const T* S, int a, int c0, T ca, T cb, T cg
   return (ca * D[1][1] + cb * s1 + cg * s2) * inv_d;
 }
 
-template <class T>
+template <class T, int FX>
 __global__ void __launch_bounds__(256) k3_faraday_tile(G3 g, Pml3<T> pm, const T* __restrict__ E,
                                                        const T* __restrict__ Ep, const T* __restrict__ Eb,
                                                        T* __restrict__ B, T* __restrict__ Bs, T* __restrict__ fB, T c1,
                                                        T c2, T c3, T ca, T cb, T cg, T dtT) {
+  if constexpr (FX < 4) chain_wait();   // (a few hundred cycles per block: not on a grid that fills the chip)
   constexpr int SX = FX + 2, SY = FY + 2, SZ = FZ + 2, SN = SX * SY * SZ;
   __shared__ T se[3][SN];   // index (x * SY + y) * SZ + z, tile origin at (1, 1, 1)
   const int i0 = blockIdx.z * FX, j0 = blockIdx.y * FY, k0 = blockIdx.x * FZ;
@@ -203,14 +205,26 @@ __global__ void __launch_bounds__(256) k3_faraday_tile(G3 g, Pml3<T> pm, const T
 }
 
 // Friedman history (PR-1): E-bar <- (1 - theta/2) E + (theta/2) E-bar, E^{n-1} <- E, gather copy <- E
+// (n a multiple of 16 bytes, the arrays aligned to them)
 template <class T>
-__global__ void k3_friedman(long n, const T* E, T* Ep, T* Eb, T* fE, T a, T b) {
-  const long p = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const T e = E[p];
-  Eb[p] = a * e + b * Eb[p];
-  Ep[p] = e;
-  fE[p] = e;
+__global__ void __launch_bounds__(256) k3_friedman(long n, const T* E, T* Ep, T* Eb, T* fE, T a, T b) {
+  chain_wait();
+  typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type V;
+  constexpr int VL = 16 / (int)sizeof(T);
+  const long nv = n / VL, step = (long)gridDim.x * blockDim.x;
+  for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < nv; p += step) {
+    const V e = reinterpret_cast<const V*>(E)[p];
+    V v = reinterpret_cast<V*>(Eb)[p];
+    v.x = a * e.x + b * v.x;
+    v.y = a * e.y + b * v.y;
+    if constexpr (VL == 4) {
+      v.z = a * e.z + b * v.z;
+      v.w = a * e.w + b * v.w;
+    }
+    reinterpret_cast<V*>(Eb)[p] = v;
+    reinterpret_cast<V*>(Ep)[p] = e;
+    reinterpret_cast<V*>(fE)[p] = e;
+  }
 }
 
 template <class T>
@@ -257,6 +271,7 @@ __device__ __forceinline__ void ampere_node(const G3& g, const Pml3<T>& pm, T* _
 template <class T>
 __global__ void __launch_bounds__(128) k3_ampere(G3 g, Pml3<T> pm, T* __restrict__ E, T* __restrict__ Es,
                                                  const T* __restrict__ B, const T* __restrict__ J, T dtc2, T dte) {
+  chain_wait();
   const int k0 = blockIdx.x * blockDim.x * KPT + threadIdx.x, j = blockIdx.y, i = blockIdx.z;
 #pragma unroll
   for (int kk = 0; kk < KPT; kk++) {
@@ -369,22 +384,28 @@ __device__ __forceinline__ void ld16(const double* p, double* v) {
 // z axis of the composed filter (stride 1): each block stages a row segment of 128 * ZR nodes and an
 // 8-node halo in shared memory; each thread reads its ZR + 16 staged values with 16-byte loads and sums
 // the taps of ZR consecutive outputs in the same order as k3_filter_axis.
+// nb blocks per row; components c0, c0 + 1, ... follow one another along blockIdx.x (src0: one block of nodes for each;
+// dst03, dst35: the blocks of components 0..2 and 3..5).
 // A row's last block also takes a remainder of up to ZTAIL nodes past its segment (a row of 2^m + 1 nodes
 // would otherwise need a block for its last node); longer remainders get a block of their own.
 constexpr int ZR = 8, ZHA = 8, ZTAIL = 32;
 template <class T, int PT>
-__global__ void __launch_bounds__(128) k3_filter_zs(G3 g, const T* __restrict__ src, T* __restrict__ dst, int comp,
-                                                    Taps3<T> t) {
+__global__ void __launch_bounds__(128) k3_filter_zs(G3 g, const T* __restrict__ src0, T* __restrict__ dst03,
+                                                    T* __restrict__ dst35, int c0, int nb, Taps3<T> t) {
+  chain_wait();
   static_assert(PT <= ZHA, "filter halo above the staged halo");
   constexpr int SEG = 128 * ZR, NV = ZR + 2 * ZHA, VL = 16 / (int)sizeof(T);
   constexpr int ROW = SEG + 2 * ZHA + ZTAIL, NVEC = ROW / VL, UV = (NVEC + 127) / 128;
   static_assert(ROW % VL == 0 && ZHA % VL == 0, "16-byte vectors tile the staged row");
   typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type V;
   __shared__ __align__(16) T row[ROW];
-  const int kb = blockIdx.x * SEG, j = blockIdx.y, i = blockIdx.z;
+  const int part = (int)blockIdx.x / nb, bx = (int)blockIdx.x - part * nb, comp = c0 + part;
+  const T* src = src0 + part * g.cs;
+  T* dst = (comp < 3 ? dst03 : dst35) + comp % 3 * g.cs;
+  const int kb = bx * SEG, j = blockIdx.y, i = blockIdx.z;
   const int n = g.n[2];
   // nodes past this segment that this block also filters (the row's last block only)
-  const int tail = blockIdx.x + 1 == gridDim.x ? min(max(n + 1 - (kb + SEG), 0), ZTAIL) : 0;
+  const int tail = bx + 1 == nb ? min(max(n + 1 - (kb + SEG), 0), ZTAIL) : 0;
   const long base = nid(g, i, j, 0);   // 16-byte aligned: ldz is padded to 128 bytes
   // the staged row in 16-byte vectors, every thread's loads issued before any is stored (an element
   // q of the row is node kb - ZHA + q; off the row: zero)
@@ -421,6 +442,7 @@ __global__ void __launch_bounds__(128) k3_filter_zs(G3 g, const T* __restrict__ 
   vr(comp, 2, g, lo2, hi2);
   const bool other = i >= lo0 && i <= hi0 && j >= lo1 && j <= hi1;
   const int l0 = ZR * threadIdx.x;
+  if (kb + l0 > n) return;   // past the row's end (and then there is no tail): in FP64 their sums cost as much as any
   T v[NV];
 #pragma unroll
   for (int q = 0; q < NV / VL; q++) ld16(row + l0 + q * VL, v + q * VL);
@@ -468,13 +490,16 @@ inline unsigned zs_blocks(int n) {
 // as zero), filters it along x into a scratch box that keeps the y halo, then along y, and writes the
 // XYT x XYT x ZB outputs: one read and one write of the component instead of two of each. Each thread
 // slides a register window along its line, summing the taps in the same order as k3_filter_axis, and the
-// outputs of either pass at invalid nodes of the component are zero, as in the separate sweeps.
+// outputs of either pass at invalid nodes of the component are zero, as in the separate sweeps. Components as in
+// k3_filter_zs (dst0: one block of nodes for each).
 constexpr int XYT = 16, ZB = 16;
 constexpr long kWait3 = 1L << 24;
 
 template <class T, int PT>
-__global__ void __launch_bounds__(256) k3_filter_xy(G3 g, const __grid_constant__ CUtensorMap map, int slot,
-                                                    T* __restrict__ dst, int comp, Taps3<T> t, Ctrl3* ctrl) {
+__global__ void __launch_bounds__(256) k3_filter_xy(G3 g, const __grid_constant__ CUtensorMap map03,
+                                                    const __grid_constant__ CUtensorMap map35, T* __restrict__ dst0,
+                                                    int c0, int nb, Taps3<T> t, Ctrl3* ctrl) {
+  if ((int)gridDim.x > nb) chain_wait();   // components share the launch: a small grid
   constexpr int W = 2 * PT + 1, XW = XYT + 2 * PT;
   extern __shared__ __align__(128) unsigned char raw3[];
   T* S = reinterpret_cast<T*>(raw3 + ((128u - ((uint32_t)__cvta_generic_to_shared(raw3) & 127u)) & 127u));
@@ -483,7 +508,9 @@ __global__ void __launch_bounds__(256) k3_filter_xy(G3 g, const __grid_constant_
   constexpr int XP = XW * ZB + 16;
   T* X1 = S + XW * XW * ZB;
   __shared__ __align__(8) uint64_t bar;
-  const int k0 = blockIdx.x * ZB, j0 = blockIdx.y * XYT, i0 = blockIdx.z * XYT;
+  const int part = (int)blockIdx.x / nb, comp = c0 + part;
+  T* dst = dst0 + part * g.cs;
+  const int k0 = ((int)blockIdx.x - part * nb) * ZB, j0 = blockIdx.y * XYT, i0 = blockIdx.z * XYT;
   const int tid = threadIdx.x;
   const uint32_t sbar = (uint32_t)__cvta_generic_to_shared(&bar);
   if (tid == 0) {
@@ -499,7 +526,7 @@ __global__ void __launch_bounds__(256) k3_filter_xy(G3 g, const __grid_constant_
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
         "[%6];" ::"r"((uint32_t)__cvta_generic_to_shared(S)),
-        "l"((unsigned long long)&map), "r"(k0), "r"(j0 - PT), "r"(i0 - PT), "r"(slot), "r"(sbar)
+        "l"((unsigned long long)(comp < 3 ? &map03 : &map35)), "r"(k0), "r"(j0 - PT), "r"(i0 - PT), "r"(comp % 3), "r"(sbar)
         : "memory");
   }
   // one warp polls the mbarrier; the others wait at the barrier below, taking no issue slots
@@ -622,10 +649,13 @@ bool encode_xy_map(CUtensorMap* m, const T* base, const G3& g, int halo) {
 }
 
 template <class T, int PT>
-void launch_filter_xy(const G3& g, const CUtensorMap& map, int slot, T* dst, int comp, const Taps3<T>& t,
-                      Ctrl3* ctrl, cudaStream_t s) {
-  const dim3 grid(nblk(g.n[2] + 1, ZB), nblk(g.n[1] + 1, XYT), nblk(g.n[0] + 1, XYT));
-  k3_filter_xy<T, PT><<<grid, 256, filter_xy_smem<T, PT>(), s>>>(g, map, slot, dst, comp, t, ctrl);
+void launch_filter_xyz(const G3& g, const CUtensorMap& map03, const CUtensorMap& map35, T* F03, T* F35, T* tmp, int c0,
+                       int nc, const Taps3<T>& t, Ctrl3* ctrl, cudaStream_t s) {
+  const int nb = (int)nblk(g.n[2] + 1, ZB), nz = (int)zs_blocks(g.n[2]);
+  const dim3 grid(nb * nc, nblk(g.n[1] + 1, XYT), nblk(g.n[0] + 1, XYT));
+  if (nc > 1) launch_chained(k3_filter_xy<T, PT>, grid, dim3(256), filter_xy_smem<T, PT>(), s, g, map03, map35, tmp, c0, nb, t, ctrl);
+  else k3_filter_xy<T, PT><<<grid, 256, filter_xy_smem<T, PT>(), s>>>(g, map03, map35, tmp, c0, nb, t, ctrl);
+  launch_chained(k3_filter_zs<T, PT>, dim3(nz * nc, g.n[1] + 1, g.n[0] + 1), dim3(128), 0, s, g, tmp, F03, F35, c0, nz, t);
 }
 
 template <class T>
@@ -640,7 +670,9 @@ void set_filter_xy_smem() {
 template <class T, int PT>
 void launch_filter_fast(const G3& g, const T* src, T* dst, int comp, int axis, const Taps3<T>& t, cudaStream_t s) {
   if (axis == 2) {
-    k3_filter_zs<T, PT><<<dim3(zs_blocks(g.n[2]), g.n[1] + 1, g.n[0] + 1), 128, 0, s>>>(g, src, dst, comp, t);
+    T* d0 = dst - comp % 3 * g.cs;
+    const int nz = (int)zs_blocks(g.n[2]);
+    k3_filter_zs<T, PT><<<dim3(nz, g.n[1] + 1, g.n[0] + 1), 128, 0, s>>>(g, src, d0, d0, comp, nz, t);
   } else {
     // segments of about 32 nodes along the axis: enough lines in flight to cover the load latency
     const int n1 = (axis == 0 ? g.n[0] : g.n[1]) + 1;
@@ -679,6 +711,7 @@ void launch_filter_axis(const G3& g, dim3 grid, const T* src, T* dst, int comp, 
 template <class T>
 __global__ void __launch_bounds__(128) k3_nodal(G3 g, const T* __restrict__ fE, const T* __restrict__ fB,
                                                 T* __restrict__ dst) {
+  chain_wait();
   const int k0 = blockIdx.x * blockDim.x * KPT + threadIdx.x, j = blockIdx.y, i = blockIdx.z;
   const long sx = (long)(g.n[1] + 1) * g.ldz, sy = g.ldz;
 #pragma unroll
@@ -848,6 +881,7 @@ __device__ __forceinline__ int cell_of(const G3& g, const Tiles3& t, const doubl
 // device count, so that the scatter reads no stale key
 template <class T>
 __global__ void k3_tile_key(G3 g, Parts3<T> p, const Ctrl3* ctrl, Tiles3 t, int n) {
+  chain_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   int key = -1;
@@ -861,6 +895,7 @@ __global__ void k3_tile_key(G3 g, Parts3<T> p, const Ctrl3* ctrl, Tiles3 t, int 
 
 // one warp per tile: its cells' counts become offsets inside the tile; the tile's total
 __global__ void __launch_bounds__(256) k3_tile_cells(Tiles3 t, int ntiles) {
+  chain_wait();
   const int tile = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (tile >= ntiles) return;   // warp-uniform
   int4* c = reinterpret_cast<int4*>(t.ccnt + (long)tile * TC) + 2 * lane;
@@ -888,6 +923,7 @@ __global__ void __launch_bounds__(256) k3_tile_cells(Tiles3 t, int ntiles) {
 // exclusive scan of the tile counts, SCB tiles per block; a block sums the totals of the blocks before it itself. The
 // total becomes the particle count.
 __global__ void __launch_bounds__(256) k3_scan_tiles(Tiles3 t, int n, Ctrl3* ctrl) {
+  chain_wait();
   constexpr int PER = SCB / 256;
   __shared__ int ws[8], s_base;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -927,6 +963,7 @@ __global__ void __launch_bounds__(256) k3_scan_tiles(Tiles3 t, int n, Ctrl3* ctr
 
 template <class T>
 __global__ void k3_tile_scatter(Parts3<T> src, Parts3<T> dst, Tiles3 t, int n_old) {
+  chain_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_old) return;
   const int key = t.key[j];
@@ -949,12 +986,14 @@ __device__ __forceinline__ T pick(const T (&v)[N], int h) {
 // FEW: for a run with fewer particles than the chip has threads (the launch's rule). A tile's particles are split over
 // kSplit blocks, four lanes share a particle, each gathers one x plane and deposits every fourth plane, straight into J.
 // One block per tile and one lane per particle left most of the chip idle, and in a tile with several particles per cell
-// the lanes met on every shared add (a compare-and-swap loop); J in global memory takes adds without an answer.
+// the lanes met on every shared add (a compare-and-swap loop); J in global memory takes adds without an answer. 3000 electrons
+// in FP64: 119 us, split 55 us.
 constexpr int kQuad = 4, kSplit = 8;
 
 template <class T, int ORD, bool MC, bool FEW>
 __global__ void __launch_bounds__(256, 3) k3_push_tiles(G3 g, Fld3<T> f, Parts3<T> p, Tiles3 t, Ctrl3* ctrl, T kq,
                                                      Cq3<T> cq) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sF = reinterpret_cast<T*>(smraw);        // 6 x WGN gather fields
   T* sJ = sF + 6 * WGN;                       // 3 x WN current
@@ -1276,29 +1315,39 @@ struct Rows8 {
 };
 
 template <class T>
-__global__ void k3_inject(G3 g, Parts3<T> p, const Ctrl3* ctrl, Lat3 L, Rows8 rows, double t) {
+__global__ void k3_inject(G3 g, Parts3<T> p, Ctrl3* ctrl, Lat3 L, Rows8 rows, double t) {
+  chain_wait();
   const long per = (long)L.nxl * L.nyl;
   const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= per * rows.n) return;
-  const int r = (int)(e / per);
-  const long ab = e - (long)r * per;
-  const int a = (int)(ab / L.nyl), b = (int)(ab - (long)a * L.nyl);
-  const long long m = rows.m[r];
-  const double zlat = (m + 0.5) * L.h;
-  const double n = L.gamma * lab_density3(L, L.gamma * zlat);
-  const long q = (long)ctrl->count + e;
-  p.x[q] = (g.lo[0] + (a + 0.5) / L.ppc[0]) * g.d[0];
-  p.y[q] = (g.lo[1] + (b + 0.5) / L.ppc[1]) * g.d[1];
-  p.z[q] = zlat - L.beta * kC * t;
-  p.ux[q] = T(0);
-  p.uy[q] = T(0);
-  p.uz[q] = T(-L.gamma * L.beta * kC);
-  p.w[q] = T(n * g.d[0] * g.d[1] * g.d[2] / (double)(L.ppc[0] * L.ppc[1] * L.ppc[2]));
-  p.id[q] = (uint32_t)((unsigned long long)m * (unsigned long long)per + (unsigned long long)(a * (long)L.nyl + b));
-  p.fl[q] = 1;
+  const int count = ctrl->count;
+  if (e < per * rows.n) {
+    const int r = (int)(e / per);
+    const long ab = e - (long)r * per;
+    const int a = (int)(ab / L.nyl), b = (int)(ab - (long)a * L.nyl);
+    const long long m = rows.m[r];
+    const double zlat = (m + 0.5) * L.h;
+    const double n = L.gamma * lab_density3(L, L.gamma * zlat);
+    const long q = (long)count + e;
+    p.x[q] = (g.lo[0] + (a + 0.5) / L.ppc[0]) * g.d[0];
+    p.y[q] = (g.lo[1] + (b + 0.5) / L.ppc[1]) * g.d[1];
+    p.z[q] = zlat - L.beta * kC * t;
+    p.ux[q] = T(0);
+    p.uy[q] = T(0);
+    p.uz[q] = T(-L.gamma * L.beta * kC);
+    p.w[q] = T(n * g.d[0] * g.d[1] * g.d[2] / (double)(L.ppc[0] * L.ppc[1] * L.ppc[2]));
+    p.id[q] = (uint32_t)((unsigned long long)m * (unsigned long long)per + (unsigned long long)(a * (long)L.nyl + b));
+    p.fl[q] = 1;
+  }
+  // the last block to have read the count adds the rows' particles to it
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&ctrl->inj_done, 1) == (int)gridDim.x - 1) {
+      ctrl->inj_done = 0;
+      ctrl->count = count + (int)(per * rows.n);
+    }
+  }
 }
-
-__global__ void k3_add_count(Ctrl3* c, int d) { c->count += d; }
 
 // sum over n >= 0 of S(u + n): the prefix of the shape samples (Esirkepov's 1D flux)
 __device__ __forceinline__ double cum_shape(int order, double u) {
@@ -1317,37 +1366,12 @@ __device__ __forceinline__ double cum_shape(int order, double u) {
   return acc;
 }
 
-// Z(k) = sum over the live ion rows of w_m (C(Z1 - k) - C(Z0 - k)): the z-prefix of the rows' shape change.
-// One warp per z node, its lanes over the rows near the node (strided), then a warp sum: the FP64 shape
-// sums are latency-bound, so they are spread over many warps instead of run one node per thread.
-__global__ void k3_ion_z(G3 g, Lat3 L, int order, long long mlo, long long mhi, double t0, double t1, double* Zs) {
-  const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (k > g.n[2]) return;   // warp-uniform
-  const double dz = g.d[2], idz = g.id[2];
-  const double vsh = L.beta * kC;
-  long long m0 = (long long)floor(((k - 4) * dz + vsh * t0) / L.h - 0.5);
-  long long m1 = (long long)ceil(((k + 4) * dz + vsh * t0) / L.h - 0.5);
-  if (m0 < mlo) m0 = mlo;
-  if (m1 > mhi - 1) m1 = mhi - 1;
-  double acc = 0.0;
-  for (long long m = m0 + lane; m <= m1; m += 32) {
-    const double zl = (m + 0.5) * L.h;
-    const double n = L.gamma * lab_density3(L, L.gamma * zl);
-    if (n <= 0.0) continue;
-    const double w = n * g.d[0] * g.d[1] * g.d[2] / (double)(L.ppc[0] * L.ppc[1] * L.ppc[2]);
-    const double Z0 = (zl - vsh * t0) * idz, Z1 = (zl - vsh * t1) * idz;
-    acc += w * (cum_shape(order, Z1 - k) - cum_shape(order, Z0 - k));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if (lane == 0) Zs[k] = acc;
-}
-
 // J_z += coef Tx(i) Ty(j) Z(k), coef = -q_ion/(dx dy dt), on the nodes where T_x T_y is non-zero
 // (i0 + blockIdx.z, j0 + blockIdx.y); KPT z nodes per thread, a block width apart
 template <class T>
 __global__ void __launch_bounds__(128) k3_ion_jz(G3 g, const double* Tx, const double* Ty, const double* Zs,
                                                  double coef, int i0, int j0, T* Jz) {
+  chain_wait();
   const int i = i0 + blockIdx.z, j = j0 + blockIdx.y;
   const double f = coef * Tx[i] * Ty[j];
   if (f == 0.0) return;
@@ -1431,10 +1455,38 @@ struct Ant3 {
   int order;
 };
 
+// Z(k) = sum over the live ion rows of w_m (C(Z1 - k) - C(Z0 - k)): the z-prefix of the rows' shape change.
+// One warp per z node, its lanes over the rows near the node (strided), then a warp sum: the FP64 shape
+// sums are latency-bound, so they are spread over many warps instead of run one node per thread.
+__device__ __forceinline__ void ion_z(const G3& g, const Lat3& L, int order, long long mlo, long long mhi, double t0,
+                                      double t1, double* Zs, int k) {
+  const int lane = threadIdx.x & 31;
+  if (k > g.n[2]) return;   // warp-uniform
+  const double dz = g.d[2], idz = g.id[2];
+  const double vsh = L.beta * kC;
+  long long m0 = (long long)floor(((k - 4) * dz + vsh * t0) / L.h - 0.5);
+  long long m1 = (long long)ceil(((k + 4) * dz + vsh * t0) / L.h - 0.5);
+  if (m0 < mlo) m0 = mlo;
+  if (m1 > mhi - 1) m1 = mhi - 1;
+  double acc = 0.0;
+  for (long long m = m0 + lane; m <= m1; m += 32) {
+    const double zl = (m + 0.5) * L.h;
+    const double n = L.gamma * lab_density3(L, L.gamma * zl);
+    if (n <= 0.0) continue;
+    const double w = n * g.d[0] * g.d[1] * g.d[2] / (double)(L.ppc[0] * L.ppc[1] * L.ppc[2]);
+    const double Z0 = (zl - vsh * t0) * idz, Z1 = (zl - vsh * t1) * idz;
+    acc += w * (cum_shape(order, Z1 - k) - cum_shape(order, Z0 - k));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if (lane == 0) Zs[k] = acc;
+}
+
+// four lanes per pair, each the terms of one z node of its stencil
 template <class T>
-__global__ void k3_antenna(G3 g, T* Jy, Ant3 a) {
+__device__ __forceinline__ void antenna_pairs(const G3& g, T* Jy, const Ant3& a, int tid) {
   const int nyp = g.hi[1] - g.lo[1] + 1;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int e = tid / 4, lz = tid % 4;
   if (e >= (g.hi[0] - g.lo[0] + 1) * nyp) return;
   const int i = g.lo[0] + e / nyp, j = g.lo[1] + e % nyp;
   const double x = i * g.d[0], y = j * g.d[1];
@@ -1463,7 +1515,7 @@ __global__ void k3_antenna(G3 g, T* Jy, Ant3 a) {
     const int bx = (int)fx - SH, bz = (int)fz - SH;
     // J_y(j+1/2) - J_y(j-1/2) = -Q/(dx dz dt) W_y, W_y = DS_y S0_z S0_x
     const double cy = -a.Q / (g.d[0] * g.d[2] * g.dt);
-    for (int lz = 0; lz < NS; lz++)
+    if (lz < NS)
       for (int lx = 0; lx < NS; lx++) {
         const double tr = wz[lz] * wx[lx];
         if (tr == 0.0) continue;
@@ -1477,6 +1529,17 @@ __global__ void k3_antenna(G3 g, T* Jy, Ant3 a) {
         }
       }
   }
+}
+
+// the ions' Z(k) and the antenna's current in one launch of one-warp blocks (the first npair / 8 for the antenna, then one
+// per z node): both are chains of FP64 work that a few warps per SM would queue for
+template <class T>
+__global__ void __launch_bounds__(32) k3_ion_antenna(G3 g, Lat3 L, int order, long long mlo, long long mhi, double t0,
+                                                     double t1, double* Zs, T* Jy, Ant3 a, int nant) {
+  chain_wait();
+  const int b = (int)blockIdx.x;
+  if (b < nant) antenna_pairs<T>(g, Jy, a, b * 32 + threadIdx.x);
+  else ion_z(g, L, order, mlo, mhi, t0, t1, Zs, b - nant);
 }
 
 // charge of the antenna pairs (the moving partner +Q, its fixed twin -Q) added to rho
@@ -2024,7 +2087,7 @@ struct Sim3 : Sim3Api {
   // the fused x-y filter: tensor maps of the blocks it reads (gather copies and current), when it applies
   bool xy_ok = false;
   CUtensorMap xy_map[3];
-  const T* xy_base[3] = {nullptr, nullptr, nullptr};
+  int ntmp = 1;           // components of tmp
   Cq3<T> cq_e;
   bool nodal = false;     // 'momentum conserving' gather (pic_config.gather_scheme = 1)
   T* nF = nullptr;        // its node values: Ex, Ey, Ez, Bx, By, Bz
@@ -2038,7 +2101,7 @@ struct Sim3 : Sim3Api {
   long blk_cap = 0;
   int64_t compactions = 0;
   Tiles3 tl{};
-  int ntiles = 0, nsum = 0;
+  int ntiles = 0, nsum = 0, nsm = 0;
   long few_max = 0;       // up to this many particles the push splits tiles over blocks and particles over lanes
   long key_cap = 0;
   // plasma
@@ -2143,13 +2206,21 @@ struct Sim3 : Sim3Api {
     g.ldz = ((c->nz + 1 + align - 1) / align) * align;
     g.cs = (long)(c->nx + 1) * (c->ny + 1) * g.ldz;
     const size_t cs = (size_t)g.cs;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    // components share their filter launches up to some blocks per SM for one of them (step without plasma, 45 blocks:
+    // 110 us, shared 49 us in FP32, 282 and 186 us in FP64; 825 blocks: 284 and 236 us, 1511 and 1423 us); on larger grids
+    // a component at a time keeps tmp in L2 and small
+    const long xy_blocks = (long)nblk(c->nz + 1, ZB) * nblk(c->ny + 1, XYT) * nblk(c->nx + 1, XYT);
+    ntmp = xy_blocks <= 6L * nsm ? 6 : 1;
     E = dal<T>(3 * cs); B = dal<T>(3 * cs); J = dal<T>(3 * cs); Ep = dal<T>(3 * cs); Eb = dal<T>(3 * cs);
     nodal = c->gather_scheme == 1;
     if (nodal) {
       nF = dal<T>(6 * cs);
       if (!nF) return fail(PIC_ENOMEM, "allocation failed");
     }
-    fE = dal<T>(3 * cs); fB = dal<T>(3 * cs); tmp = dal<T>(cs); tmp2 = dal<T>(cs);
+    fE = dal<T>(3 * cs); fB = dal<T>(3 * cs); tmp = dal<T>(ntmp * cs); tmp2 = dal<T>(cs);
     Es = dal<T>(6 * cs); Bs = dal<T>(6 * cs);
     ctrl = dal<Ctrl3>(1);
     bacc = dal<double>(8);
@@ -2205,9 +2276,9 @@ struct Sim3 : Sim3Api {
     taps.s = wide ? 1 : c->filter_stride;
     // stride-1 filters of up to five taps a side take the fused x-y pass (one TMA-staged box per CTA)
     if (taps.s == 1 && taps.P >= 1 && taps.P <= 5) {
-      xy_base[0] = fE; xy_base[1] = fB; xy_base[2] = J;
+      const T* base[3] = {fE, fB, J};
       xy_ok = true;
-      for (int q = 0; q < 3; q++) xy_ok = xy_ok && encode_xy_map<T>(&xy_map[q], xy_base[q], g, taps.P);
+      for (int q = 0; q < 3; q++) xy_ok = xy_ok && encode_xy_map<T>(&xy_map[q], base[q], g, taps.P);
       if (xy_ok) set_filter_xy_smem<T>();
     }
     tl.nt[0] = (g.n[0] + TX - 1) / TX;
@@ -2228,9 +2299,6 @@ struct Sim3 : Sim3Api {
     set_smem(k3_push_tiles<T, 1, false, true>, k3_push_tiles<T, 1, false, false>);
     set_smem(k3_push_tiles<T, 3, true, true>, k3_push_tiles<T, 3, true, false>);
     set_smem(k3_push_tiles<T, 1, true, true>, k3_push_tiles<T, 1, true, false>);
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     few_max = 256L * nsm;
     cudaEventCreate(&ev0);
     cudaEventCreate(&ev1);
@@ -2293,10 +2361,11 @@ struct Sim3 : Sim3Api {
   // particles into tile and cell order (dropping the dead ones) in the other buffer set
   void sort_tiles() {
     cudaMemsetAsync(tl.ccnt, 0, sizeof(int) * ((size_t)ntiles * TC + nsum), s);
-    k3_tile_key<T><<<nblk(count_ub, 256), 256, 0, s>>>(g, P2[cur], ctrl, tl, (int)count_ub);
-    k3_tile_cells<<<nblk(ntiles, 8), 256, 0, s>>>(tl, ntiles);
-    k3_scan_tiles<<<nsum, 256, 0, s>>>(tl, ntiles, ctrl);
-    k3_tile_scatter<T><<<nblk(count_ub, 256), 256, 0, s>>>(P2[cur], P2[1 - cur], tl, (int)count_ub);
+    launch_chained(k3_tile_key<T>, dim3(nblk(count_ub, 256)), dim3(256), 0, s, g, P2[cur], ctrl, tl, (int)count_ub);
+    launch_chained(k3_tile_cells, dim3(nblk(ntiles, 8)), dim3(256), 0, s, tl, ntiles);
+    launch_chained(k3_scan_tiles, dim3(nsum), dim3(256), 0, s, tl, ntiles, ctrl);
+    launch_chained(k3_tile_scatter<T>, dim3(nblk(count_ub, 256)), dim3(256), 0, s, P2[cur], P2[1 - cur], tl,
+                   (int)count_ub);
     nl += 4;
     cur = 1 - cur;
     compactions++;
@@ -2354,9 +2423,9 @@ struct Sim3 : Sim3Api {
       R.n = (int)std::min<size_t>(8, rows.size() - r0);
       for (int q = 0; q < R.n; q++) R.m[q] = rows[r0 + q];
       const long n = per * R.n;
-      k3_inject<T><<<nblk(n, 256), 256, 0, s>>>(g, P2[cur], ctrl, lat, R, t);
-      k3_add_count<<<1, 1, 0, s>>>(ctrl, (int)n);
-      nl += 2;
+      // one-warp blocks: the density's FP64 chain per particle, on as many SMs as there are warps
+      launch_chained(k3_inject<T>, dim3(nblk(n, 32)), dim3(32), 0, s, g, P2[cur], ctrl, lat, R, t);
+      nl++;
       count_ub += n;
     }
     return PIC_OK;
@@ -2499,23 +2568,26 @@ struct Sim3 : Sim3Api {
 
   dim3 grid3() const { return dim3(nblk(g.n[2] + 1, 128 * KPT), g.n[1] + 1, g.n[0] + 1); }
 
-  void filter3(T* F, int comp) {
-    // F inside one of the mapped blocks: x and y in one TMA-staged pass F -> tmp, then z: tmp -> F
-    for (int q = 0; xy_ok && q < 3; q++) {
-      const long d = F - xy_base[q];
-      if (d < 0 || d >= 3 * g.cs || d % g.cs != 0) continue;
-      const int slot = (int)(d / g.cs);
-      switch (taps.P) {
-        case 1: launch_filter_xy<T, 1>(g, xy_map[q], slot, tmp, comp, taps, ctrl, s); break;
-        case 2: launch_filter_xy<T, 2>(g, xy_map[q], slot, tmp, comp, taps, ctrl, s); break;
-        case 3: launch_filter_xy<T, 3>(g, xy_map[q], slot, tmp, comp, taps, ctrl, s); break;
-        case 4: launch_filter_xy<T, 4>(g, xy_map[q], slot, tmp, comp, taps, ctrl, s); break;
-        default: launch_filter_xy<T, 5>(g, xy_map[q], slot, tmp, comp, taps, ctrl, s); break;
+  // components c0 .. c0 + nc - 1 (0..2 in the block F03, 3..5 in F35)
+  void filter3(T* F03, T* F35, int c0, int nc) {
+    if (xy_ok) {   // x and y in one TMA-staged pass F -> tmp, then z: tmp -> F
+      const CUtensorMap &m03 = xy_map[F03 == J ? 2 : 0], &m35 = xy_map[1];
+      for (int c = c0, n; c < c0 + nc; c += n) {
+        n = ntmp > 1 ? nc : 1;
+        switch (taps.P) {
+          case 1: launch_filter_xyz<T, 1>(g, m03, m35, F03, F35, tmp, c, n, taps, ctrl, s); break;
+          case 2: launch_filter_xyz<T, 2>(g, m03, m35, F03, F35, tmp, c, n, taps, ctrl, s); break;
+          case 3: launch_filter_xyz<T, 3>(g, m03, m35, F03, F35, tmp, c, n, taps, ctrl, s); break;
+          case 4: launch_filter_xyz<T, 4>(g, m03, m35, F03, F35, tmp, c, n, taps, ctrl, s); break;
+          default: launch_filter_xyz<T, 5>(g, m03, m35, F03, F35, tmp, c, n, taps, ctrl, s); break;
+        }
+        nl += 2;
       }
-      launch_filter_axis<T>(g, grid3(), tmp, F, comp, 2, taps, s);
-      nl += 2;
       return;
     }
+    for (int c = c0; c < c0 + nc; c++) filter3_axes((c < 3 ? F03 : F35) + c % 3 * g.cs, c);
+  }
+  void filter3_axes(T* F, int comp) {
     // x: F -> tmp, y: tmp -> tmp2, z: tmp2 -> F
     launch_filter_axis<T>(g, grid3(), F, tmp, comp, 0, taps, s);
     launch_filter_axis<T>(g, grid3(), tmp, tmp2, comp, 1, taps, s);
@@ -2554,10 +2626,11 @@ struct Sim3 : Sim3Api {
   template <int ORD, bool MC>
   void launch_push(const Fld3<T>& f, T kq) {
     if (count_ub <= few_max)
-      k3_push_tiles<T, ORD, MC, true><<<dim3(ntiles, kSplit), 256, push3_smem<T, true>(), s>>>(g, f, P2[cur], tl, ctrl, kq,
-                                                                                              cq_e);
+      launch_chained(k3_push_tiles<T, ORD, MC, true>, dim3(ntiles, kSplit), dim3(256), push3_smem<T, true>(), s, g, f,
+                     P2[cur], tl, ctrl, kq, cq_e);
     else
-      k3_push_tiles<T, ORD, MC, false><<<ntiles, 256, push3_smem<T, false>(), s>>>(g, f, P2[cur], tl, ctrl, kq, cq_e);
+      launch_chained(k3_push_tiles<T, ORD, MC, false>, dim3(ntiles), dim3(256), push3_smem<T, false>(), s, g, f, P2[cur], tl,
+                     ctrl, kq, cq_e);
   }
 
   int one_step() {
@@ -2568,13 +2641,21 @@ struct Sim3 : Sim3Api {
     btd_part(1, 0);
     // 1. Faraday + Friedman + PML-B (B^{n-1/2} -> B^{n+1/2}), gather copies
     tbeg(1);
-    k3_faraday_tile<T><<<dim3(nblk(g.n[2] + 1, FZ), nblk(g.n[1] + 1, FY), nblk(g.n[0] + 1, FX)), dim3(FZ, FY), 0, s>>>(
-        g, pm, E, Ep, Eb, B, Bs, fB, T(1.0 + th / 4.0), T(0.5), T(0.5 - th / 4.0), T(cfg.ck_alpha), T(cfg.ck_beta),
-        T(cfg.ck_gamma), T(g.dt));
-    k3_friedman<T><<<nblk(n3, 256), 256, 0, s>>>(n3, E, Ep, Eb, fE, T(1.0 - th / 2.0), T(th / 2.0));
+    // x nodes per tile: 4 (a halo plane read per two); 2 where tiles of 4 are fewer than SMs, FP64 then taking as long as
+    // a tile has nodes (65 x 25 x 25 nodes: 58 us, 34 us with 2)
+    const auto faraday = [&](auto kernel, int fx) {
+      const dim3 grid(nblk(g.n[2] + 1, FZ), nblk(g.n[1] + 1, FY), nblk(g.n[0] + 1, fx)), block(FZ, FY);
+      const T c1 = T(1.0 + th / 4.0), c2 = T(0.5), c3 = T(0.5 - th / 4.0);
+      const T ca = T(cfg.ck_alpha), cb = T(cfg.ck_beta), cg = T(cfg.ck_gamma);
+      if (fx < 4) launch_chained(kernel, grid, block, 0, s, g, pm, E, Ep, Eb, B, Bs, fB, c1, c2, c3, ca, cb, cg, T(g.dt));
+      else kernel<<<grid, block, 0, s>>>(g, pm, E, Ep, Eb, B, Bs, fB, c1, c2, c3, ca, cb, cg, T(g.dt));
+    };
+    if ((long)nblk(g.n[2] + 1, FZ) * nblk(g.n[1] + 1, FY) * nblk(g.n[0] + 1, 4) < nsm) faraday(k3_faraday_tile<T, 2>, 2);
+    else faraday(k3_faraday_tile<T, 4>, 4);
+    launch_chained(k3_friedman<T>, dim3((unsigned)std::min<long>(nblk(n3 * sizeof(T) / 16, 256), 16L * nsm)), dim3(256), 0, s, n3, E, Ep, Eb, fE, T(1.0 - th / 2.0), T(th / 2.0));
     nl += 2;
     if (cfg.filter_gather && P > 0)
-      for (int c = 0; c < 3; c++) { filter3(fE + c * g.cs, c); filter3(fB + c * g.cs, 3 + c); }
+      filter3(fE, fB, 0, 6);
     tend(1);
     // 2. particles
     cudaMemsetAsync(J, 0, sizeof(T) * 3 * g.cs, s);
@@ -2582,7 +2663,7 @@ struct Sim3 : Sim3Api {
     for (int c = 0; c < 3; c++) { f.fE[c] = fE + c * g.cs; f.fB[c] = fB + c * g.cs; f.J[c] = J + c * g.cs; }
     if (nodal) {
       // 'momentum conserving' gather: the copies interpolated to the nodes
-      k3_nodal<T><<<grid3(), 128, 0, s>>>(g, fE, fB, nF);
+      launch_chained(k3_nodal<T>, grid3(), dim3(128), 0, s, g, fE, fB, nF);
       nl++;
       for (int c = 0; c < 3; c++) { f.fE[c] = nF + c * g.cs; f.fB[c] = nF + (3 + c) * g.cs; }
     }
@@ -2598,12 +2679,6 @@ struct Sim3 : Sim3Api {
       tend(0);
     }
     const double tn = time_of(step), tn1 = time_of(step + 1);
-    if (loaded && ions && row_next > mlo) {
-      k3_ion_z<<<nblk(g.n[2] + 1, 4), 128, 0, s>>>(g, lat, cfg.shape_order, mlo, row_next, tn, tn1, Zs);
-      k3_ion_jz<T><<<dim3(nblk(g.n[2] + 1, 128 * KPT), ion_j1 - ion_j0 + 1, ion_i1 - ion_i0 + 1), 128, 0, s>>>(
-          g, Tx, Ty, Zs, -kQe / (g.d[0] * g.d[1] * g.dt), ion_i0, ion_j0, J + 2 * g.cs);
-      nl += 2;
-    }
     if (has_beam) {
       if (cfg.shape_order == 3)
         k3_beam_push<T, 3><<<nblk(bm.n, 128), 128, 0, s>>>(g, f, bm, tn, tn1, bacc, kq, nodal ? 1 : 0);
@@ -2611,21 +2686,32 @@ struct Sim3 : Sim3Api {
         k3_beam_push<T, 1><<<nblk(bm.n, 128), 128, 0, s>>>(g, f, bm, tn, tn1, bacc, kq, nodal ? 1 : 0);
       nl++;
     }
-    // 3. antenna: the moving partners' displacement G(x, y) D_n -> G D_{n+1}
+    // 3. ions; antenna: the moving partners' displacement G(x, y) D_n -> G D_{n+1}
+    const bool ion_rows = loaded && ions && row_next > mlo;
+    int nant = 0;
+    Ant3 a{};
     if (antenna_inside()) {
       const double th_ = tn + 0.5 * g.dt;
       const double dD = -2.0 * kEps0 * kC * emit_t(th_) * g.d[0] * g.d[1] / Qpair * g.dt;
-      const Ant3 a = ant_params(Dn, Dn + dD);
-      const int npair = (g.hi[0] - g.lo[0] + 1) * (g.hi[1] - g.lo[1] + 1);
-      k3_antenna<T><<<nblk(npair, 128), 128, 0, s>>>(g, J + g.cs, a);
-      nl++;
+      a = ant_params(Dn, Dn + dD);
+      nant = (int)nblk(4L * (g.hi[0] - g.lo[0] + 1) * (g.hi[1] - g.lo[1] + 1), 32);
       Dn += dD;
+    }
+    if (nant + ion_rows > 0) {
+      launch_chained(k3_ion_antenna<T>, dim3(nant + (ion_rows ? g.n[2] + 1 : 0)), dim3(32), 0, s, g, lat, cfg.shape_order,
+                     mlo, row_next, tn, tn1, Zs, J + g.cs, a, nant);
+      nl++;
+    }
+    if (ion_rows) {
+      launch_chained(k3_ion_jz<T>, dim3(nblk(g.n[2] + 1, 128 * KPT), ion_j1 - ion_j0 + 1, ion_i1 - ion_i0 + 1), dim3(128),
+                     0, s, g, Tx, Ty, Zs, -kQe / (g.d[0] * g.d[1] * g.dt), ion_i0, ion_j0, J + 2 * g.cs);
+      nl++;
     }
     // 4. current filter, Ampere + PML-E
     tbeg(1);
     if (cfg.filter_J && P > 0)
-      for (int c = 0; c < 3; c++) filter3(J + c * g.cs, c);
-    k3_ampere<T><<<grid3(), 128, 0, s>>>(g, pm, E, Es, B, J, T(g.dt * kC * kC), T(g.dt / kEps0));
+      filter3(J, nullptr, 0, 3);
+    launch_chained(k3_ampere<T>, grid3(), dim3(128), 0, s, g, pm, E, Es, B, J, T(g.dt * kC * kC), T(g.dt / kEps0));
     nl++;
     tend(1);
     btd_part(0, 1);
