@@ -516,41 +516,58 @@ uint64_t splitmix64(uint64_t& s) {
 }
 
 // ---------------------------------------------------------------------------
-// Tensor-core inference (tcgen05): one CTA takes 128 rows through every layer. Each layer's weights
-// come as a prepacked BF16 image (K-major, no swizzle, padded to multiples of 16) by one bulk TMA copy
-// into shared memory; the activations of the 128 rows sit in shared memory in the same canonical layout;
-// one thread issues the K/16 tcgen05.mma (M = 128, N = padded width, BF16 x BF16 -> FP32) into a TMEM
-// accumulator; the four warps read their 32 TMEM lanes (one row per thread), add the bias, apply GELU
-// and write the next layer's operand (or the FP32 outputs) in place.
+// Tensor-core inference (tcgen05): one CTA takes 128 rows through every layer. The weights come as a prepacked BF16 image
+// (K-major, padded to multiples of 16, in chunks of TC_KC columns) by bulk TMA copies through a ring of shared-memory
+// slots that runs across the layers; the activations of the 128 rows sit in shared memory; both in swizzled layouts. One
+// warp issues the K/16 tcgen05.mma (M = 128, N = padded width, BF16 x BF16 -> FP32) into a TMEM accumulator, one thread
+// copies; sixteen warps read the accumulator's lanes (one row per thread), add the bias, apply GELU and write the next
+// layer's operand (or the FP32 outputs) in place.
+// The epilogue bounds it: two special-function instructions per GELU (4100 cycles per 128 x 256 layer; with the other 15
+// instructions 5800 alone, 7000 with two CTAs), then the products and their waits (5000 per 256 x 256 layer). With a ring
+// of 3 slots two CTAs share an SM (shared memory, 64 registers a thread, 256 TMEM columns each), one's products and copies
+// under the other's epilogue. Where there are no more tiles than SMs a ring of 8 holds a whole layer and the next one's
+// copies run under the epilogue. 6-256-256-256-4: 100 000 rows 151.6 us, now 79.1; up to 19 456 rows 33.4, now 25 to 26
+// (before: one CTA per SM, a layer's weights in one copy, a clock read in every wait, scalar arithmetic).
 constexpr int TC_M = 128;
 constexpr int TC_THREADS = 512;                            // 16 warps: 4 TMEM lane groups x 4 column groups
 constexpr int TC_MAXW = 256;                              // padded width limit of this kernel
+constexpr int TC_KC = 32;                                 // weight columns per chunk
 constexpr int TC_A_BYTES = TC_M * TC_MAXW * 2;            // activations
-constexpr int TC_B_BYTES = TC_MAXW * TC_MAXW * 2;         // one layer's weights
-constexpr int TC_SMEM = TC_A_BYTES + TC_B_BYTES + 64;
+constexpr int TC_C_BYTES = TC_MAXW * TC_KC * 2;           // one chunk
+constexpr int tc_smem(int ring) { return TC_A_BYTES + ring * TC_C_BYTES + (2 * ring + 1) * 8 + 8; }
 constexpr int TC_MAXL = 16;
 
 __host__ __device__ inline int pad16(int v) { return (v + 15) & ~15; }
 
-// byte offset of element (r, k) of an operand with Kp columns: 8 x 8 core matrices of 128 contiguous
-// bytes (a row of 8 elements every 16 bytes), K-groups 128 bytes apart, 8-row groups Kp * 16 bytes apart
-__host__ __device__ inline uint32_t canon_off(int r, int k, int Kp) {
-  return (uint32_t)((r >> 3) * (Kp * 16) + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
+// byte offset of element (r, k) of the activations: K-major with 128-byte swizzle, blocks of 64 columns (128 rows x 128
+// bytes), the eight 16-byte pieces of a row exchanged by the row's place in its group of eight
+__host__ __device__ inline uint32_t act_off(int r, int k) {
+  return (uint32_t)((k >> 6) * (TC_M * 128) + r * 128 + ((((k >> 3) & 7) ^ (r & 7)) << 4) + (k & 7) * 2);
 }
+// byte offset of element (r, k) of a chunk of weights: K-major with 64-byte swizzle, rows of TC_KC = 32 columns
+__host__ __device__ inline uint32_t chunk_off(int r, int k) {
+  return (uint32_t)(r * 64 + ((((k >> 3) & 3) ^ ((r >> 1) & 3)) << 4) + (k & 7) * 2);
+}
+__host__ __device__ inline int tc_chunks(int Kp) { return (Kp + TC_KC - 1) / TC_KC; }
+// columns per copy: as many chunks of a layer Np wide as fill a slot
+inline int tc_copy_cols(int Np) { return TC_KC * (TC_MAXW / Np); }
 
 __global__ void k_next_epoch(int* eidx) { *eidx += 1; }
 
-__global__ void k_pack_weights(const __nv_bfloat16* W, int N, int K, int Np, int Kp, __nv_bfloat16* img) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= Np * Kp) return;
-  const int r = e / Kp, k = e - r * Kp;
-  img[canon_off(r, k, Kp) >> 1] = (r < N && k < K) ? W[(long)r * K + k] : __float2bfloat16(0.0f);
+// the image of one layer: its weights chunk by chunk (zero beyond its columns), then its biases in FP32
+__global__ void k_pack_weights(const __nv_bfloat16* W, const float* bias, int N, int K, int Np, int chunks,
+                               __nv_bfloat16* img) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x, Kc = chunks * TC_KC;
+  if (e < Np) reinterpret_cast<float*>(img + Np * Kc)[e] = e < N ? bias[e] : 0.0f;
+  if (e >= Np * Kc) return;
+  const int r = e / Kc, k = e - r * Kc, c = k / TC_KC;
+  img[c * TC_KC * Np + (chunk_off(r, k - c * TC_KC) >> 1)] = (r < N && k < K) ? W[(long)r * K + k] : __float2bfloat16(0.0f);
 }
 
 struct TcLayer {
   const __nv_bfloat16* img;
-  const float* bias;
   int N, K, Np, Kp;
+  int cols, copies;   // columns per copy of weights, copies
 };
 struct TcNet {
   TcLayer l[TC_MAXL];
@@ -559,11 +576,17 @@ struct TcNet {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// shared-memory matrix descriptor: start, LBO (K direction), SBO (8-row groups), fixed version bits 46-47,
-// no swizzle
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+// D (+)= A B on the tensor cores, M = 128, K = 16, operands in shared memory. An operand's matrix descriptor: low word the
+// address in 16 bytes (in the units of which it advances along K) and a fixed leading distance, high word the distance of
+// the 8-row groups in 16 bytes, fixed version bits 14-15 and the swizzle mode (2: 128 bytes, 4: 64 bytes) from bit 29.
+constexpr uint32_t kDescAct = (1024u >> 4) | (1u << 14) | (2u << 29), kDescChunk = (512u >> 4) | (1u << 14) | (4u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr >> 4) & 0x3FFFu) | (1u << 16); }
+__device__ __forceinline__ void mma_k16(uint32_t tmem, uint32_t a, uint32_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %4, 0;\n mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %6};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(tmem),
+      "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(kDescAct), "r"(kDescChunk)
+      : "memory");
 }
 
 __device__ __forceinline__ uint64_t global_ns() {
@@ -572,58 +595,147 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
-// wait for the phase of an mbarrier, giving up after about half a second (then the error flag is set)
-__device__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err) {
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// wait for the phase of an mbarrier, giving up after about half a second (then the error flag is set); the clock, whose
+// reading costs more than most of these waits, is looked at every 64 polls
+__device__ __noinline__ bool mbar_wait_long(uint32_t bar, uint32_t parity, int* err) {
   const uint64_t t0 = global_ns();
   while (true) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
+    for (int poll = 0; poll < 64; poll++)
+      if (mbar_try(bar, parity)) return true;
     if (global_ns() - t0 > 500000000ull) {
       atomicExch(err, 1);
       return false;
     }
   }
 }
-
-// erf by Abramowitz & Stegun, Handbook of Mathematical Functions, 7.1.26 (Hastings' rational
-// approximation; |error| <= 1.5e-7 for x >= 0, far below the BF16 rounding that every activation takes):
-// erf(x) = 1 - t (a1 + a2 t + a3 t^2 + a4 t^3 + a5 t^4) exp(-x^2), t = 1 / (1 + p x), odd in x.
-// About half the instructions of the library erf in the serving epilogue, which bounds the kernel.
-__device__ __forceinline__ float erf_as(float x) {
-  const float ax = fabsf(x);
-  const float t = __fdividef(1.0f, fmaf(0.3275911f, ax, 1.0f));
-  const float poly =
-      t * fmaf(fmaf(fmaf(fmaf(1.061405429f, t, -1.453152027f), t, 1.421413741f), t, -0.284496736f), t,
-               0.254829592f);
-  return copysignf(fmaf(-poly, __expf(-ax * ax), 1.0f), x);
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err) {
+  if (mbar_try(bar, parity) || mbar_try(bar, parity)) return true;
+  return mbar_wait_long(bar, parity, err);
 }
 
-// exact (erf-form) GELU of the serving path
-__device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.0f + erf_as(z * 0.70710678118654752f)); }
+// one lane of a converged warp, always the same
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
 
-__global__ void __launch_bounds__(TC_THREADS, 1) k_mlp_fwd_tc(TcNet net, const float* __restrict__ x, long n,
-                                                             float* __restrict__ y, int* err) {
+// two FP32 values in one register pair: packed instructions round each as the scalar one does
+typedef unsigned long long F2;
+__device__ __forceinline__ F2 f2(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ F2 f2(float v) { return f2(v, v); }
+__device__ __forceinline__ float lo(F2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a;
+}
+__device__ __forceinline__ float hi(F2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return b;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float ex2_approx(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// GELU, z (1 + erf(z / sqrt 2)) / 2, of two values, with erf by Abramowitz & Stegun, Handbook of Mathematical Functions,
+// 7.1.26 (Hastings' rational approximation; |error| <= 1.5e-7 for x >= 0, far below the BF16 rounding that every
+// activation takes): erf(x) = 1 - t (a1 + a2 t + a3 t^2 + a4 t^3 + a5 t^4) exp(-x^2), t = 1 / (1 + p x), odd in x.
+__device__ __forceinline__ F2 gelu2(F2 z) {
+  const F2 x = mul2(z, f2(0.70710678118654752f));
+  const F2 ax = x & 0x7fffffff7fffffffull;
+  const F2 d = fma2(f2(0.3275911f), ax, f2(1.0f));
+  const F2 t = f2(rcp_approx(lo(d)), rcp_approx(hi(d)));
+  F2 q = fma2(f2(-1.061405429f), t, f2(1.453152027f));   // minus the polynomial
+  q = fma2(q, t, f2(-1.421413741f));
+  q = fma2(q, t, f2(0.284496736f));
+  q = fma2(q, t, f2(-0.254829592f));
+  q = mul2(t, q);
+  // exp(-x^2) = 2^(-x^2 log2 e)
+  const F2 w = mul2(mul2(x, x), f2(-1.44269504088896341f));
+  const F2 e = f2(ex2_approx(lo(w)), ex2_approx(hi(w)));
+  const F2 v = fma2(q, e, f2(1.0f));
+  const F2 erf = (v & 0x7fffffff7fffffffull) | (x & 0x8000000080000000ull);
+  return mul2(mul2(f2(0.5f), z), add2(f2(1.0f), erf));
+}
+
+template <int RING, int CTAS>
+__global__ void __launch_bounds__(TC_THREADS, CTAS) k_mlp_fwd_tc(const __grid_constant__ TcNet net,
+                                                                 const float* __restrict__ x, long n,
+                                                                 float* __restrict__ y, int* err) {
   extern __shared__ __align__(1024) unsigned char sm[];
   unsigned char* A = sm;
   unsigned char* Bw = sm + TC_A_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + TC_A_BYTES + TC_B_BYTES);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + TC_A_BYTES + RING * TC_C_BYTES);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2 * RING + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // TMEM lanes 32 (warp % 4) .. +31 are this warp's rows; chunks of 16 columns go round-robin to warp / 4
   const int lgrp = warp & 3, cgrp = warp >> 2;
   const int rloc = lgrp * 32 + lane;
   const long row0 = (long)blockIdx.x * TC_M;
-  const uint32_t barW = smem_u32(&bars[0]), barM = smem_u32(&bars[1]);
+  // a slot's copy has landed; a slot's products have completed; the layer's products have completed
+  const uint32_t bar_full = smem_u32(bars), bar_free = smem_u32(bars + RING), bar_acc = smem_u32(bars + 2 * RING);
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barW) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barM) : "memory");
+    for (int q = 0; q < 2 * RING + 1; q++)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[q])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // the weights' copies, numbered through all layers: warp 0 multiplies (c_mma so far), thread LOADER copies (c_in so
+  // far) and waits for the slots, so that the products never wait for a slot to be given back
+  constexpr int LOADER = 32;
+  int c_in = 0, c_mma = 0, load_l = 0, load_k = 0;
+  auto load_chunk = [&]() {
+    if (load_l >= net.L) return;
+    const int Np = net.l[load_l].Np, Kp = net.l[load_l].Kp, slot = c_in % RING;
+    const int cols = min(net.l[load_l].cols, tc_chunks(Kp) * TC_KC - load_k);
+    const uint32_t bytes = (uint32_t)(Np * cols * 2), bar = bar_full + 8 * slot;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(Bw) + slot * TC_C_BYTES),
+                 "l"(net.l[load_l].img + (long)load_k * Np), "r"(bytes), "r"(bar)
+                 : "memory");
+    c_in++;
+    load_k += cols;
+    if (load_k >= Kp) { load_l++; load_k = 0; }
+  };
+  __syncthreads();
+  if (tid == LOADER)
+    for (int q = 0; q < RING; q++) load_chunk();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(tslot))
                  : "memory");
@@ -641,58 +753,67 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_mlp_fwd_tc(TcNet net, const f
         const int k = k8 * 8 + q;
         v[q] = __float2bfloat16((r < n && k < net.k0) ? x[r * net.k0 + k] : 0.0f);
       }
-      *reinterpret_cast<uint4*>(A + canon_off(rr, k8 * 8, Kp)) = *reinterpret_cast<const uint4*>(v);
+      *reinterpret_cast<uint4*>(A + act_off(rr, k8 * 8)) = *reinterpret_cast<const uint4*>(v);
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tslot;
-  uint32_t phW = 0, phM = 0;
-  bool ok = true;
-  // the weights of layer l arrive by one bulk copy, issued for the next layer as soon as the current
-  // layer's products have completed (it overlaps the epilogue)
-  auto load_weights = [&](int l) {
-    const uint32_t bytes = (uint32_t)(net.l[l].Np * net.l[l].Kp * 2);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(barW), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(Bw)),
-                 "l"(net.l[l].img), "r"(bytes), "r"(barW)
-                 : "memory");
-  };
-  if (tid == 0) load_weights(0);
+  const uint32_t tmem = *tslot, a_lo = desc_lo(smem_u32(A)), b_lo = desc_lo(smem_u32(Bw));
   for (int l = 0; l < net.L; l++) {
-    const TcLayer Ly = net.l[l];
-    ok = __syncthreads_and(mbar_wait(barW, phW, err) ? 1 : 0) != 0;
-    phW ^= 1u;
-    if (!ok) break;
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(Ly.Np >> 3) << 17) |
+    const TcLayer& Ly = net.l[l];
+    const int Np = Ly.Np;
+    bool ok = true;
+    if (warp == 0) {   // the whole warp walks the chunks (uniform descriptors), one lane issues
+      const int Kp = Ly.Kp;
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(Np >> 3) << 17) |
                              ((uint32_t)(TC_M >> 4) << 24);
-      const uint32_t sbo = (uint32_t)(Ly.Kp * 16);
-      for (int ks = 0; ks < Ly.Kp / 16; ks++) {
-        const uint64_t ad = smem_desc(smem_u32(A) + ks * 256, 128, sbo);
-        const uint64_t bd = smem_desc(smem_u32(Bw) + ks * 256, 128, sbo);
-        const uint32_t acc = ks > 0 ? 1u : 0u;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-            : "memory");
+      const int cols = Ly.cols;
+      for (int k = 0; k < Kp; k += cols, c_mma++) {
+        const int slot = c_mma % RING;
+        ok = mbar_wait(bar_full + 8 * slot, (c_mma / RING) & 1, err);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        uint32_t b = b_lo + slot * (TC_C_BYTES >> 4);
+        if (elect_one()) {
+          const int end = min(Kp, k + cols);
+          for (int c = k; c < end; c += TC_KC, b += Np * (TC_KC * 2 >> 4)) {
+            const uint32_t a = a_lo + (act_off(0, c) >> 4);
+            mma_k16(tmem, a, b, idesc, c > 0);
+            if (c + 16 < Kp) mma_k16(tmem, a + 2, b + 2, idesc, 1);
+          }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                           bar_free + 8 * slot)
+                       : "memory");
+        }
+        __syncwarp();
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(barM)
-                   : "memory");
+      if (ok && elect_one())
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_acc)
+                     : "memory");
+    } else if (tid == LOADER) {
+      const int end = c_mma + Ly.copies;
+      for (; c_mma < end && ok; c_mma++) {
+        if (load_l >= net.L) continue;
+        ok = mbar_wait(bar_free + 8 * (c_mma % RING), (c_mma / RING) & 1, err);
+        if (ok) load_chunk();
+      }
     }
-    ok = __syncthreads_and(mbar_wait(barM, phM, err) ? 1 : 0) != 0;
-    phM ^= 1u;
-    if (!ok) break;
-    if (tid == 0 && l + 1 < net.L) load_weights(l + 1);
+    // one warp waits for the products, the others at the barrier (polls would take the epilogue's issue slots)
+    __syncwarp();
+    if (warp == 0) {
+      if (ok) ok = mbar_wait(bar_acc, l & 1, err);
+    }
+    if (__syncthreads_and(ok ? 1 : 0) == 0) break;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const bool last = l == net.L - 1;
     const long r = row0 + rloc;
-    for (int c0 = 16 * cgrp; c0 < Ly.Np; c0 += 64) {
+    const float* bias = reinterpret_cast<const float*>(Ly.img + Np * tc_chunks(Ly.Kp) * TC_KC);
+    for (int c0 = 16 * cgrp; c0 < Np; c0 += 64) {
+      float b[16];
+#pragma unroll
+      for (int q = 0; q < 4; q++) *reinterpret_cast<float4*>(b + 4 * q) = __ldg(reinterpret_cast<const float4*>(bias + c0) + q);
       uint32_t v[16];
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -701,19 +822,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_mlp_fwd_tc(TcNet net, const f
           : "r"(tmem + ((uint32_t)(lgrp * 32) << 16) + (uint32_t)c0)
           : "memory");
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      float f[16];
-#pragma unroll
-      for (int q = 0; q < 16; q++) f[q] = __uint_as_float(v[q]) + (c0 + q < Ly.N ? Ly.bias[c0 + q] : 0.0f);
       if (!last) {
-        __align__(16) __nv_bfloat16 h[16];
+        // (the columns of the padding have zero weights and biases, and GELU(0) = 0)
+        __align__(16) __nv_bfloat162 h[8];
 #pragma unroll
-        for (int q = 0; q < 16; q++) h[q] = __float2bfloat16(c0 + q < Ly.N ? gelu_f(f[q]) : 0.0f);
-        *reinterpret_cast<uint4*>(A + canon_off(rloc, c0, Ly.Np)) = *reinterpret_cast<const uint4*>(h);
-        *reinterpret_cast<uint4*>(A + canon_off(rloc, c0 + 8, Ly.Np)) = *reinterpret_cast<const uint4*>(h + 8);
+        for (int q = 0; q < 8; q++) {
+          const F2 g = gelu2(add2(f2(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1])), f2(b[2 * q], b[2 * q + 1])));
+          h[q] = __floats2bfloat162_rn(lo(g), hi(g));
+        }
+        *reinterpret_cast<uint4*>(A + act_off(rloc, c0)) = *reinterpret_cast<const uint4*>(h);
+        *reinterpret_cast<uint4*>(A + act_off(rloc, c0 + 8)) = *reinterpret_cast<const uint4*>(h + 4);
       } else if (r < n) {
 #pragma unroll
         for (int q = 0; q < 16; q++)
-          if (c0 + q < Ly.N) y[r * Ly.N + c0 + q] = f[q];
+          if (c0 + q < Ly.N) y[r * Ly.N + c0 + q] = __uint_as_float(v[q]) + b[q];
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -721,6 +843,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_mlp_fwd_tc(TcNet net, const f
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   }
+  // after a wait that gave up: copies still in flight land before the block's memory is given back
+  if (tid == LOADER)
+    for (int c = max(0, c_in - RING); c < c_in; c++) mbar_wait(bar_full + 8 * (c % RING), (c / RING) & 1, err);
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
 }
@@ -762,6 +887,7 @@ struct pic_mlp {
   bool tc_ok = false;                   // every padded width <= 256
   bool tc_dirty = true;
   bool use_tc = true;
+  int nsm = 0;                          // SMs of the device
   std::vector<__nv_bfloat16*> img;
   int* err = nullptr;                   // device flag: a tensor-core wait gave up
   cudaStream_t s = nullptr;
@@ -969,9 +1095,14 @@ int pic_mlp_create(int n_layers, const int* widths, uint64_t seed, pic_alloc_fn 
   m->tc_ok = n_layers <= TC_MAXL;
   for (int l = 0; l <= n_layers; l++) m->tc_ok = m->tc_ok && pad16(widths[l]) <= TC_MAXW;
   if (m->tc_ok) {
-    for (int l = 1; l <= n_layers; l++) m->img.push_back(mlp_al<__nv_bfloat16>(m, (size_t)pad16(widths[l]) * pad16(widths[l - 1])));
+    for (int l = 1; l <= n_layers; l++) 
+      m->img.push_back(mlp_al<__nv_bfloat16>(m, (size_t)pad16(widths[l]) * (tc_chunks(pad16(widths[l - 1])) * TC_KC + 2)));
     for (auto* q : m->img) m->tc_ok = m->tc_ok && q;
-    cudaFuncSetAttribute(k_mlp_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    cudaFuncSetAttribute(k_mlp_fwd_tc<3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(3));
+    cudaFuncSetAttribute(k_mlp_fwd_tc<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(8));
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&m->nsm, cudaDevAttrMultiProcessorCount, dev);
   }
   if (!m->p || !m->pb || !m->g || !m->m || !m->v || !m->loss || !m->err) {
     mlp_release(m);
@@ -1037,7 +1168,9 @@ int pic_mlp_infer(pic_mlp* m, const float* x, int64_t n, float* y) {
     if (m->tc_dirty) {
       for (int l = 1; l <= m->L; l++) {
         const int N = m->w[l], K = m->w[l - 1], Np = pad16(N), Kp = pad16(K);
-        k_pack_weights<<<(Np * Kp + 255) / 256, 256, 0, m->s>>>(m->pb + m->off_w[l - 1], N, K, Np, Kp, m->img[l - 1]);
+        const int nc = tc_chunks(Kp);
+        k_pack_weights<<<(Np * nc * TC_KC + 255) / 256, 256, 0, m->s>>>(m->pb + m->off_w[l - 1], m->p + m->off_b[l - 1], N, K,
+                                                                        Np, nc, m->img[l - 1]);
       }
       m->tc_dirty = false;
     }
@@ -1047,14 +1180,18 @@ int pic_mlp_infer(pic_mlp* m, const float* x, int64_t n, float* y) {
     for (int l = 1; l <= m->L; l++) {
       TcLayer& t = net.l[l - 1];
       t.img = m->img[l - 1];
-      t.bias = m->p + m->off_b[l - 1];
       t.N = m->w[l];
       t.K = m->w[l - 1];
       t.Np = pad16(t.N);
       t.Kp = pad16(t.K);
+      t.cols = tc_copy_cols(t.Np);
+      t.copies = (t.Kp + t.cols - 1) / t.cols;
     }
     const long blocks = (n + TC_M - 1) / TC_M;
-    k_mlp_fwd_tc<<<(unsigned)blocks, TC_THREADS, TC_SMEM, m->s>>>(net, x, (long)n, y, m->err);
+    if (blocks > m->nsm)
+      k_mlp_fwd_tc<3, 2><<<(unsigned)blocks, TC_THREADS, tc_smem(3), m->s>>>(net, x, (long)n, y, m->err);
+    else
+      k_mlp_fwd_tc<8, 1><<<(unsigned)blocks, TC_THREADS, tc_smem(8), m->s>>>(net, x, (long)n, y, m->err);
     return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
   }
   const int chunk = 65536;
