@@ -251,6 +251,26 @@ struct Sim : SimBase {
     pt.cx_i = dx_t + 4 * nx1; pt.cx_h = dx_t + 5 * nx1;
     pt.sz_i = dz_t; pt.sz_h = dz_t + nz1; pt.xz_i = dz_t + 2 * nz1; pt.xz_h = dz_t + 3 * nz1;
     pt.cz_i = dz_t + 4 * nz1; pt.cz_h = dz_t + 5 * nz1;
+    // the FP32 pairs (pml_step): B's, then E's
+    const auto pairs = [](const std::vector<double>& v, int n1, std::vector<float4>& out) {
+      const auto hi = [](double a) { return (float)a; };
+      const auto lo = [](double a) { return (float)(a - (double)(float)a); };
+      out.resize(2 * n1);
+      for (int i = 0; i < n1; i++) {
+        const double xb = v[3 * n1 + i], cb = v[5 * n1 + i], xe = v[2 * n1 + i], ce = (kC * kC) * v[4 * n1 + i];
+        out[i] = make_float4(hi(xb), lo(xb), hi(cb), lo(cb));
+        out[n1 + i] = make_float4(hi(xe), lo(xe), hi(ce), lo(ce));
+      }
+    };
+    std::vector<float4> px, pz;
+    pairs(hx, nx1, px);
+    pairs(hz, nz1, pz);
+    float4* dpx = al<float4>(px.size());
+    float4* dpz = al<float4>(pz.size());
+    if (!dpx || !dpz) return c->fail(PIC_ENOMEM, "allocation failed");
+    cudaMemcpyAsync(dpx, px.data(), px.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
+    cudaMemcpyAsync(dpz, pz.data(), pz.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
+    pt.bx = dpx; pt.ex = dpx + nx1; pt.bz = dpz; pt.ez = dpz + nz1;
     // interior index ranges, where the field kernels skip the PML branches
     auto interior = [](const std::vector<double>& v, int n, int& lo, int& hi) {
       lo = 0; hi = n;

@@ -77,6 +77,9 @@ __host__ __device__ inline void valid_range(int comp, int nx, int nz, int& i0, i
 struct PmlTabs {
   const double *sx_i, *sx_h, *xx_i, *xx_h, *cx_i, *cx_h;
   const double *sz_i, *sz_h, *xz_i, *xz_h, *cz_i, *cz_h;
+  // the coefficients of B (half-integer tables) and E (integer tables, c^2 in cx and cz) as pairs of FP32 values: xi high,
+  // xi low, coefficient high, low
+  const float4 *bx, *bz, *ex, *ez;
   int iin0, iin1, kin0, kin1;   // nodes whose sigma is zero at both staggerings (the interior)
 };
 

@@ -40,6 +40,35 @@ __device__ __forceinline__ void load_tile_b(const GridP& g, const FieldPtrs<T>& 
   }
 }
 
+// xi a + cf b of the split-field PML (f cf: E's c^2), rounded once. The coefficients are FP64; FP32 fields take them as
+// pairs of FP32 values and the products and the sum with their rounding errors, about 2^-47 of the larger term before the
+// final rounding; where the terms cancel to a thousandth, FP64 as for FP64 fields. (4 million values over all ranges of the
+// coefficients and with cancelling terms: the same results as FP64 arithmetic, bit for bit.) FP64 itself (conversions included) bounded the field kernels: a warp's FP64 instruction occupies the SM for 16
+// cycles, and the SMs with PML tiles were busy with them 70 to 90 % of the time.
+template <class T>
+__device__ __forceinline__ T pml_step(const double* x, const double* c, const float4* t, int q, double f, T a, T b,
+                                      bool minus) {
+  if (minus) b = -b;
+  if constexpr (sizeof(T) == 4) {
+    const float4 w = t[q];
+    const float p = __fmul_rn(w.x, a), pe = __fmaf_rn(w.x, a, -p);
+    const float r = __fmul_rn(w.z, b), re = __fmaf_rn(w.z, b, -r);
+    const float s = __fadd_rn(p, r), v = __fadd_rn(s, -p);
+    if (!(fabsf(s) < 0x1p-10f * fabsf(p))) {
+      float e = __fadd_rn(__fadd_rn(p, -__fadd_rn(s, -v)), __fadd_rn(r, -v));
+      e = __fadd_rn(e, __fadd_rn(pe, re));
+      e = __fmaf_rn(w.y, a, e);
+      e = __fmaf_rn(w.w, b, e);
+      return fabsf(s) < INFINITY ? __fadd_rn(s, e) : s;   // (an infinite field has no rounding error)
+    }
+  }
+  return T(x[q] * (double)a + f * c[q] * (double)b);
+}
+// sigma > 0 (by the bits: an FP64 comparison takes the FP64 pipe)
+__device__ __forceinline__ bool damped(const double* sigma, int q) {
+  return __double_as_longlong(sigma[q]) > 0;
+}
+
 // B update of one tile from E_eff staged in shared memory: Ee[c] holds the tile and a one-node halo, row
 // stride SZ, node (i0 - 1 + li, k0 - 1 + lk) at li * SZ + lk (zero outside the grid); b: the tile's
 // B^{n-1/2} (load_tile_b). PML = false: a tile clear of the PML (no table reads, no FP64 in the
@@ -84,7 +113,7 @@ __device__ __forceinline__ void faraday_update_t(const GridP& g, const FieldPtrs
       const T d = dsz(EY);
       const T bo = bx0[r];
       T bn;
-      if (!interior && pt.sz_h[k] > 0.0) bn = T(pt.xz_h[k] * (double)bo + pt.cz_h[k] * (double)d);
+      if (!interior && damped(pt.sz_h, k)) bn = pml_step(pt.xz_h, pt.cz_h, pt.bz, k, 1.0, bo, d, false);
       else bn = bo + dt * d;
       f.B[0][p] = bn;
       f.Bavg[0][p] = T(0.5) * (bo + bn);
@@ -94,7 +123,7 @@ __device__ __forceinline__ void faraday_update_t(const GridP& g, const FieldPtrs
       const T d = dsx(EY);
       const T bo = bz0[r];
       T bn;
-      if (!interior && pt.sx_h[i] > 0.0) bn = T(pt.xx_h[i] * (double)bo - pt.cx_h[i] * (double)d);
+      if (!interior && damped(pt.sx_h, i)) bn = pml_step(pt.xx_h, pt.cx_h, pt.bx, i, 1.0, bo, d, true);
       else bn = bo - dt * d;
       f.B[2][p] = bn;
       f.Bavg[2][p] = T(0.5) * (bo + bn);
@@ -105,12 +134,12 @@ __device__ __forceinline__ void faraday_update_t(const GridP& g, const FieldPtrs
       const T b = dsx(EZ);
       const T bo = by0[r];
       T bn;
-      if (!interior && (pt.sx_h[i] > 0.0 || pt.sz_h[k] > 0.0)) {
-        double yz = pt.xz_h[k] * (double)f.Byz[p] - pt.cz_h[k] * (double)a;
-        double yx = pt.xx_h[i] * (double)f.Byx[p] + pt.cx_h[i] * (double)b;
-        f.Byz[p] = T(yz);
-        f.Byx[p] = T(yx);
-        bn = T(yx) + T(yz);
+      if (!interior && (damped(pt.sx_h, i) || damped(pt.sz_h, k))) {
+        const T yz = pml_step(pt.xz_h, pt.cz_h, pt.bz, k, 1.0, f.Byz[p], a, true);
+        const T yx = pml_step(pt.xx_h, pt.cx_h, pt.bx, i, 1.0, f.Byx[p], b, false);
+        f.Byz[p] = yz;
+        f.Byx[p] = yx;
+        bn = yx + yz;
       } else {
         bn = bo - dt * (a - b);
       }
@@ -657,6 +686,16 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
     mbar_init(&bar[1]);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // the rigid ion column's factors on the staged box, FP64 work done once per row and column of the tile (every thread
+  // its own kept the FP64 pipe busy for a third of the kernel)
+  __shared__ T ion_ix[DIRECT ? 1 : 256], ion_cz[DIRECT ? 1 : 256];   // (a staged box is at most 256 wide)
+  if (!DIRECT && ion_x != nullptr) {
+    for (int q = threadIdx.y * FT_Z + threadIdx.x; q < tm.BX + tm.BZ; q += FT_Z * FT_TY) {
+      const int gi = gi0 + q, lk = q - tm.BX, gk = gk0 + lk;
+      if (lk < 0) ion_ix[q] = gi >= 0 && gi <= g.nx ? T(ion_coef * ion_x[gi]) : T(0);
+      else ion_cz[lk] = gk >= 0 && gk <= g.nz ? T(ion_c[gk]) : T(0);
+    }
+  }
   __syncthreads();
   if (!DIRECT && leader) stage<T>(tile0, pmapJ, 0, gk0, gi0, &bar[0], tm);
   const T dt = grid_dt<T>(g);
@@ -697,18 +736,16 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
       return;
     }
     if (!DIRECT && c == 2 && ion_x != nullptr) {
-      // rigid ion-column current added to Jz before the filter (each thread
-      // converts its columns' factors once)
+      // rigid ion-column current added to Jz before the filter
       T cz[(256 + FT_Z - 1) / FT_Z];
 #pragma unroll
       for (int u = 0; u < (256 + FT_Z - 1) / FT_Z; u++) {
-        const int lk = threadIdx.x + u * FT_Z, gk = gk0 + lk;
-        cz[u] = (lk < tm.BZ && gk >= 0 && gk <= g.nz) ? T(ion_c[gk]) : T(0);
+        const int lk = threadIdx.x + u * FT_Z;
+        cz[u] = lk < tm.BZ ? ion_cz[lk] : T(0);
       }
       for (int li = threadIdx.y; li < tm.BX; li += FT_TY) {
-        const int gi = gi0 + li;
-        if (gi < 0 || gi > g.nx) continue;
-        const T ix = T(ion_coef * ion_x[gi]);
+        if (gi0 + li < 0 || gi0 + li > g.nx) continue;
+        const T ix = ion_ix[li];
 #pragma unroll
         for (int u = 0; u < (256 + FT_Z - 1) / FT_Z; u++) {
           const int lk = threadIdx.x + u * FT_Z;
@@ -739,21 +776,21 @@ __device__ __forceinline__ void ampere_tile(const GridP& g, const FieldPtrs<T>& 
       T en;
       if (c == 0) {
         T d = (ba[r] - bb[r]) * idz;
-        if (!interior && pt.sz_i[k] > 0.0) en = T(pt.xz_i[k] * (double)eo - c2d * pt.cz_i[k] * (double)d);
+        if (!interior && damped(pt.sz_i, k)) en = pml_step(pt.xz_i, pt.cz_i, pt.ez, k, c2d, eo, d, true);
         else en = eo - dt * (c2 * d + jv * ie0);
       } else if (c == 2) {
         T d = (ba[r] - bb[r]) * idx;
-        if (!interior && pt.sx_i[i] > 0.0) en = T(pt.xx_i[i] * (double)eo + c2d * pt.cx_i[i] * (double)d);
+        if (!interior && damped(pt.sx_i, i)) en = pml_step(pt.xx_i, pt.cx_i, pt.ex, i, c2d, eo, d, false);
         else en = eo + dt * (c2 * d - jv * ie0);
       } else {
         T dbx = (ba[r] - bb[r]) * idz;
         T dbz = (bc[r] - bd[r]) * idx;
-        if (!interior && (pt.sx_i[i] > 0.0 || pt.sz_i[k] > 0.0)) {
-          double yz = pt.xz_i[k] * (double)f.Eyz[p] + c2d * pt.cz_i[k] * (double)dbx;
-          double yx = pt.xx_i[i] * (double)f.Eyx[p] - c2d * pt.cx_i[i] * (double)dbz;
-          f.Eyz[p] = T(yz);
-          f.Eyx[p] = T(yx);
-          en = T(yx) + T(yz);
+        if (!interior && (damped(pt.sx_i, i) || damped(pt.sz_i, k))) {
+          const T yz = pml_step(pt.xz_i, pt.cz_i, pt.ez, k, c2d, f.Eyz[p], dbx, false);
+          const T yx = pml_step(pt.xx_i, pt.cx_i, pt.ex, i, c2d, f.Eyx[p], dbz, true);
+          f.Eyz[p] = yz;
+          f.Eyx[p] = yx;
+          en = yx + yz;
         } else {
           en = eo + dt * (c2 * (dbx - dbz) - jv * ie0);
         }
@@ -904,6 +941,14 @@ __global__ void __launch_bounds__(WXC* WXG) k_wide_x(GridP g, const __grid_const
 #pragma unroll
   for (int q = 0; q < CV; q++) cz[q] = (ion && k + q <= g.nz) ? T(job.ion_c[k + q]) : T(0);
   const int n = NX + 2 * H + 8;
+  __shared__ T ixs[NIN];   // the rows' factors of the ion current, FP64 work done once per row
+  if (ion) {               // block-uniform
+    for (int e = gy * WXC + lane; e < n; e += WXC * WXG) {
+      const int i = i0 - H + e;
+      ixs[e] = i >= 0 && i <= g.nx ? T(job.coef * job.ion_x[i]) : T(0);
+    }
+    __syncthreads();
+  }
   // six rows' loads of a thread in flight
   constexpr int U = 6;
   for (int l0 = gy; l0 < n; l0 += WXG * U) {
@@ -921,7 +966,7 @@ __global__ void __launch_bounds__(WXC* WXG) k_wide_x(GridP g, const __grid_const
 #pragma unroll
       for (int q = 0; q < CV; q++) v[u][q] = k + q <= g.nz ? xp[q] : T(0);
       if (ion) {
-        const T ix = T(job.coef * job.ion_x[i]);
+        const T ix = ixs[li];
 #pragma unroll
         for (int q = 0; q < CV; q++) v[u][q] += ix * cz[q];
       }
