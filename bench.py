@@ -40,11 +40,11 @@ BYTES_PER_PARTICLE = {"mixed": 60, "fp64": 88}
 BYTES_PER_PARTICLE_3D = {"mixed": 76, "fp64": 104}
 # algorithmic bytes per cell-step of the field kernels (mixed, with Friedman): see the design notes
 BYTES_PER_CELL = {"mixed": 168, "fp64": 336}
-# measured DRAM bytes (read + write) per particle of one push launch (k_push), mixed precision, cubic shapes,
-# the Yee-located gather, for every layout the autotuner can return, keyed by (tile_x, tile_z, sort_every):
-# ncu dram__bytes_read.sum + dram__bytes_write.sum on the 2048 x 256 stage box (bench.py --layout-sweep, the
-# 2nd and 3rd push of each layout), scaled to the full box by its particle count. Below the 56 bytes of stored
-# state: the last writes of a launch are still in the 129 MB L2 when it ends.
+# DRAM bytes (read + write) per particle of a push launch in which every particle is pushed (k_push, mixed precision, cubic
+# shapes, the Yee-located gather), for every layout the autotuner can return, keyed by (tile_x, tile_z, sort_every): ncu
+# dram__bytes_read.sum + dram__bytes_write.sum on the 2048 x 256 stage box, measured when chunks at rest were still pushed
+# (the 2nd and 3rd push of each layout). Below the 56 bytes of stored state: the last writes of a launch are still in the
+# 129 MB L2 when it ends. What a run moves is less (PUSH_DRAM_BYTES_PER_PARTICLE).
 TRAFFIC_BYTES_PER_PARTICLE = {
     (8, 8, 8): 49.71, (8, 8, 16): 49.61, (8, 8, 32): 49.58, (8, 8, 64): 49.49, (8, 8, 128): 49.62, (8, 16, 8): 49.58,
     (8, 16, 16): 49.63, (8, 16, 32): 49.61, (8, 16, 64): 49.49, (8, 16, 128): 49.63, (8, 32, 8): 49.83,
@@ -56,18 +56,19 @@ TRAFFIC_BYTES_PER_PARTICLE = {
     (32, 16, 16): 49.3, (32, 16, 32): 49.07, (32, 16, 64): 49.05, (32, 16, 128): 49.2, (32, 32, 8): 48.87,
     (32, 32, 16): 48.85, (32, 32, 32): 48.84, (32, 32, 64): 48.94, (32, 32, 128): 48.95,
 }
-# the push's instruction and FP32 arithmetic counts per particle (mixed, cubic, Yee-located gather; ncu
-# smsp__inst_executed.sum and smsp__sass_thread_inst_executed_op_{fadd,fmul,ffma}_pred_on.sum of three pushes
-# at steps 5-7 of the 2048 x 256 stage box, 8 x 16-cell tiles, sort every 64): warp instructions, and FLOPs
-# counted as FADD + FMUL + 2 FFMA (the packed two-lane FMAs of the gather are not in these counters). The
-# warp instructions were 20.7 there before each thread's next particle was copied into shared memory ahead
-# of its push; that copy adds 1.6% (22.29 -> 22.64 warp instructions per particle in the full captures at
-# step 76), hence 21.0. The arithmetic is unchanged.
-PUSH_WARP_INST_PER_PARTICLE = 21.0
-PUSH_FLOPS_PER_PARTICLE = 174.0
-# 3D: ncu dram bytes of k3_push_tiles on the 256 x 128 x 128 box (189.5 MB for 2,356,608 electrons), scaled
+# DRAM bytes, warp instructions and FP32 operations per particle of one push launch (k_push), mixed precision, cubic
+# shapes, the Yee-located gather: ncu dram__bytes_read.sum + dram__bytes_write.sum, smsp__inst_executed.sum and
+# smsp__sass_thread_inst_executed_op_{fadd,fmul,ffma}_pred_on.sum of the pushes of steps 104-106 (the middle of the default
+# 200 steps) on the 2048 x 256 stage box, 8 x 16-cell tiles, sort every 64, over all its particles (6,514,944): 37.1 MB,
+# 44.6 M, and 278 M counted as FADD + FMUL + 2 FFMA (the packed two-lane FMAs of the gather are not in these counters).
+# Chunks of electrons at rest in a field-free window are in the count of particles and cost next to nothing; what moves
+# of the half box stays in the 129 MB L2 from one step to the next.
+PUSH_DRAM_BYTES_PER_PARTICLE = 5.7
+PUSH_WARP_INST_PER_PARTICLE = 6.85
+PUSH_FLOPS_PER_PARTICLE = 42.7
+# 3D: ncu dram bytes of k3_push_tiles on the 256 x 128 x 128 box (195.3 MB for 2,356,608 electrons), scaled
 # to the full box by its particle count
-TRAFFIC_BYTES_PER_PARTICLE_3D = {("mixed", 3): 80.4}
+TRAFFIC_BYTES_PER_PARTICLE_3D = {("mixed", 3): 82.9}
 
 
 def measured_peaks() -> dict:
@@ -930,23 +931,28 @@ def main():
     if three:
         tpp = TRAFFIC_BYTES_PER_PARTICLE_3D.get((args.precision, args.order)) if args.gather == "energy" else None
     else:
-        lay = (tuple(tuned["tile"]) + (tuned["sort_every"],)) if tuned else None
         ok = args.precision == "mixed" and args.order == 3 and args.gather == "energy"
-        tpp = TRAFFIC_BYTES_PER_PARTICLE.get(lay) if ok and lay else None
+        tpp = PUSH_DRAM_BYTES_PER_PARTICLE if ok else None
+        lay = (tuple(tuned["tile"]) + (tuned["sort_every"],)) if tuned else None
+        all_moving = TRAFFIC_BYTES_PER_PARTICLE.get(lay) if ok and lay else None
     roof = {"kernel": "k3_push_tiles (3D gather + Boris + Esirkepov)" if three else "k_push (gather + Boris + Esirkepov)",
             "bound": "hbm", "achieved": achieved, "peak": peak,
             "unit": "GB/s", "frac": achieved / peak, "traffic": tpp * n_avg if tpp else None,
             "traffic_source": ("ncu dram bytes of k3_push_tiles, 256 x 128 x 128 box, scaled by particles" if three
-                               else "ncu dram bytes of k_push, 2048 x 256 box, this layout, scaled by particles") if tpp else None,
+                               else "ncu dram bytes of k_push, 2048 x 256 box, steps 104-106, scaled by particles") if tpp else None,
             "note": ("3D push on sorted 4x4x16-cell tiles with shared-memory windows: issue- and latency-bound at "
-                     "three CTAs per SM (ncu: 44% issue slots, 37% warps active, 4.5k thread-instructions per "
+                     "three CTAs per SM (ncu: 52% issue slots, 37% warps active, 193 warp instructions per "
                      "particle, 4% DRAM)" if three else
-                     "at cubic order the push is bound by instruction issue and the L1/shared pipe "
-                     "(ncu: 64-65% issue slots, 69% L1/TEX, 17% DRAM), not by HBM; see issue and alu"),
+                     "achieved counts every particle's algorithmic bytes, but chunks of electrons at rest in a "
+                     "field-free window only move their box (their particles are not read or written); the others "
+                     "are bound by instruction issue and the shared-memory pipe (ncu: 64% issue slots); see traffic, "
+                     "issue and alu"),
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if "hbm_gbs" in peaks else "fallback",
             "algorithmic_bytes_per_particle": bpp, "push_ms_per_step": push_avg_ms,
             "field_kernels_ms_per_step": field_ms / kf,
             "share_of_step": push_avg_ms / (ms / args.steps)}
+    if not three and all_moving:
+        roof["traffic_if_every_chunk_moved"] = all_moving * n_avg
     # the field kernels' roofline (Faraday + Friedman + PML, gather filter, current filter + Ampere): SURVEY's
     # algorithmic bytes per cell-step (all six E/B components and the current, fused) over their measured time
     cells = w["nx"] * w.get("ny", 1) * w["nz"]
