@@ -322,6 +322,7 @@ __global__ void k_beam_push(GridP g, FieldPtrs<T> f, Beam<T> b, int order, doubl
 // gather; the batched step carries no node-interpolated runs)
 template <class T>
 __global__ void k_beam_push_batch(const StepArgs<T>* a) {
+  chain_wait();
   const StepArgs<T>& A = a[blockIdx.y];
   if (!A.beam_on) return;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -614,6 +615,7 @@ __global__ void k_shift_particles(GridP g, Particles<T> p, const Ctrl* ctrl, int
 // batched antenna (each run's blocks also clear its ion-column sums for the next kernel)
 template <class T>
 __global__ void k_antenna_batch(const StepArgs<T>* a, const int* off, int nruns) {
+  chain_wait();
   __shared__ int s_r;
   if (threadIdx.x == 0) s_r = batch_run(off, nruns, blockIdx.x);
   __syncthreads();
@@ -627,6 +629,7 @@ __global__ void k_antenna_batch(const StepArgs<T>* a, const int* off, int nruns)
 // batched rigid-ion column current: rows [ion_mlo, ion_mhi) of each run, one thread per row
 template <class T>
 __global__ void k_ion_current_batch(const StepArgs<T>* a, const int* off, int nruns) {
+  chain_wait();
   __shared__ int s_r;
   if (threadIdx.x == 0) s_r = batch_run(off, nruns, blockIdx.x);
   __syncthreads();
@@ -656,8 +659,8 @@ __global__ void k_ion_current_batch(const StepArgs<T>* a, const int* off, int nr
 
 template <class T>
 void launch_antenna_ion_batch(const StepArgs<T>* a, const BatchGrid& bg, bool any_ion, cudaStream_t s) {
-  k_antenna_batch<T><<<bg.ant_blocks, 128, 0, s>>>(a, bg.ant_off, bg.nruns);
-  if (any_ion) k_ion_current_batch<T><<<bg.ion_blocks, 256, 0, s>>>(a, bg.ion_off, bg.nruns);
+  launch_chained(k_antenna_batch<T>, dim3(bg.ant_blocks), dim3(128), 0, s, a, bg.ant_off, bg.nruns);
+  if (any_ion) launch_chained(k_ion_current_batch<T>, dim3(bg.ion_blocks), dim3(256), 0, s, a, bg.ion_off, bg.nruns);
 }
 
 // ---------------------------------------------------------------------------
@@ -849,7 +852,8 @@ void launch_beam_init(Beam<T> b, const double* lx, const double* lz, const doubl
 
 template <class T>
 void launch_beam_push_batch(const StepArgs<T>* a, int nruns, int beam_max, cudaStream_t s) {
-  if (beam_max > 0) k_beam_push_batch<T><<<dim3((beam_max + BEAM_TB - 1) / BEAM_TB, nruns), BEAM_TB, 0, s>>>(a);
+  if (beam_max > 0)
+    launch_chained(k_beam_push_batch<T>, dim3((beam_max + BEAM_TB - 1) / BEAM_TB, nruns), dim3(BEAM_TB), 0, s, a);
 }
 
 template <class T>

@@ -1069,17 +1069,6 @@ __device__ __forceinline__ void tensormap_acquire(const CUtensorMap* m) {
   asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(m) : "memory");
 }
 
-// A run's arguments copied to shared memory by the block (a barrier follows): read in place, every pointer is a dependent
-// global load again after each store. 8 runs of 512 x 160 cells: Faraday 57.9 us, Ampere 46.1 us; copied 47.2 us and 42.6 us
-// (Faraday with its taps by value; Ampere has no registers for them, and in shared memory they cost 1.8 us).
-template <class X>
-__device__ __forceinline__ void to_shared(X* dst, const X* src) {
-  static_assert(sizeof(X) % 4 == 0 && alignof(X) >= 4, "copied in 4-byte words");
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x, n = blockDim.x * blockDim.y;
-  for (int q = tid; q < (int)(sizeof(X) / 4); q += n)
-    reinterpret_cast<unsigned*>(dst)[q] = reinterpret_cast<const unsigned*>(src)[q];
-}
-
 // the taps of an unrolled filter by value (constant indices throughout: they stay in registers)
 template <class T, int PT>
 __device__ __forceinline__ decltype(auto) taps_of(const FilterTaps<T>& t) {

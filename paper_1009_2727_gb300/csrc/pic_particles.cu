@@ -1265,13 +1265,15 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push_batch(con
   __shared__ PushConst s_pc;
   __shared__ GridP s_g;
   __shared__ Particles<T> s_p;
+  chain_wait();
+  // (one thread would wait for three dependent loads per run, and below for a run's arguments word by word; with the same in
+  // the deferred pass and dependent launches, a step of eight stage runs took 8 us less of 220)
+  for (int r = threadIdx.x; r < nruns; r += PB_THREADS) s_pref[r + 1] = a[r].push_on ? a[r].ctrl->nchunks : 0;
+  __syncthreads();
   if (threadIdx.x == 0) {
     int acc = 0;
-    for (int r = 0; r < nruns; r++) {
-      s_pref[r] = acc;
-      if (a[r].push_on) acc += a[r].ctrl->nchunks;
-    }
-    s_pref[nruns] = acc;
+    s_pref[0] = 0;
+    for (int r = 1; r <= nruns; r++) s_pref[r] = acc += s_pref[r];
   }
   __syncthreads();
   const int total = s_pref[nruns];
@@ -1296,7 +1298,9 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push_batch(con
     if (w >= total) break;
     const int r = s_r;
     if (r != cur) {
-      if (threadIdx.x == 0) { s_pc = a[r].pc; s_g = a[r].g; s_p = a[r].p; }
+      to_shared(&s_pc, &a[r].pc);
+      to_shared(&s_g, &a[r].g);
+      to_shared(&s_p, &a[r].p);
       __syncthreads();
       cur = r;
     }
@@ -1309,10 +1313,16 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push_batch(con
 // the global-memory pass of every run (usually nothing to do)
 template <class T, int ORDER>
 __global__ void __launch_bounds__(PB_THREADS) k_push_deferred_batch(const StepArgs<T>* a, int nruns) {
+  chain_wait();
+  __shared__ int2 s_n[MAX_BATCH_RUNS];   // all runs' counts at once: one run after another cost a round trip each
+  for (int r = threadIdx.x; r < nruns; r += PB_THREADS)
+    s_n[r] = a[r].push_on ? make_int2(min(a[r].ctrl->n_ovf, a[r].pd.ovf_cap), min(a[r].ctrl->n_defer, a[r].pd.defer_cap))
+                          : make_int2(0, 0);
+  __syncthreads();
   for (int r = 0; r < nruns; r++) {
+    const int novf = s_n[r].x, ndef = s_n[r].y;
+    if (novf == 0 && ndef == 0) continue;
     const StepArgs<T>& A = a[r];
-    if (!A.push_on) continue;
-    const int novf = min(A.ctrl->n_ovf, A.pd.ovf_cap), ndef = min(A.ctrl->n_defer, A.pd.defer_cap);
     for (int j = blockIdx.x; j < novf * OVF_SLICES; j += gridDim.x) {
       const int c = A.pd.ovf[j / OVF_SLICES];
       const Chunk ch = A.chunks[c];
@@ -1344,6 +1354,7 @@ __global__ void __launch_bounds__(PB_THREADS) k_push_deferred_batch(const StepAr
 // run's rows idle
 template <class T>
 __global__ void k_inject_batch(const StepArgs<T>* a, const int* off, int nruns) {
+  chain_wait();
   __shared__ int s_r;
   if (threadIdx.x == 0) s_r = batch_run(off, nruns, blockIdx.x);
   __syncthreads();
@@ -1364,18 +1375,20 @@ void launch_push_batch(const StepArgs<T>* a, const BatchGrid& bg, int order, int
   const int gb = grid_blocks < 304 ? grid_blocks : 304;
   if (order == 3) {
     cudaFuncSetAttribute(k_push_batch<T, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_push_batch<T, 3><<<grid_blocks, PB_THREADS, sm, s>>>(a, bg.nruns, bg.push_counter, smem_nodes, tile_z);
-    k_push_deferred_batch<T, 3><<<gb, PB_THREADS, 0, s>>>(a, bg.nruns);
+    launch_chained(k_push_batch<T, 3>, dim3(grid_blocks), dim3(PB_THREADS), sm, s, a, bg.nruns, bg.push_counter, smem_nodes,
+                   tile_z);
+    launch_chained(k_push_deferred_batch<T, 3>, dim3(gb), dim3(PB_THREADS), 0, s, a, bg.nruns);
   } else {
     cudaFuncSetAttribute(k_push_batch<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_push_batch<T, 1><<<grid_blocks, PB_THREADS, sm, s>>>(a, bg.nruns, bg.push_counter, smem_nodes, tile_z);
-    k_push_deferred_batch<T, 1><<<gb, PB_THREADS, 0, s>>>(a, bg.nruns);
+    launch_chained(k_push_batch<T, 1>, dim3(grid_blocks), dim3(PB_THREADS), sm, s, a, bg.nruns, bg.push_counter, smem_nodes,
+                   tile_z);
+    launch_chained(k_push_deferred_batch<T, 1>, dim3(gb), dim3(PB_THREADS), 0, s, a, bg.nruns);
   }
 }
 
 template <class T>
 void launch_inject_batch(const StepArgs<T>* a, const BatchGrid& bg, cudaStream_t s) {
-  k_inject_batch<T><<<bg.inj_blocks, 256, 0, s>>>(a, bg.inj_off, bg.nruns);
+  launch_chained(k_inject_batch<T>, dim3(bg.inj_blocks), dim3(256), 0, s, a, bg.inj_off, bg.nruns);
 }
 
 PushConst push_const(const GridP& g, double q, double m, double gamma_b, int fr1_sz, float fr1_fz, int pairs,
