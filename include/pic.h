@@ -365,7 +365,7 @@ int pic_autotune_window(const pic_config* cfg, const pic_plasma* plasma, const p
  *    and particle layout; at most 512 runs; a test beam rides along): all runs
  *    share one non-blocking stream and an ensemble step is one launch per kernel
  *    class over all runs (Faraday, gather filter, push, its global pass, test
- *    beams, antenna, ion current, Ampere, inflow, counts; the runs' sorts every
+ *    beams, antenna, ion current, Ampere, inflow; the runs' sorts every
  *    sort_every steps), the per-run
  *    arguments of the step in one block of device memory filled from the same
  *    host decisions as pic_step. From the third step on, each step replays a

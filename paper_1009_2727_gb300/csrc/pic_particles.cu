@@ -3,8 +3,11 @@
 //    takes one chunk (a contiguous run of particles whose cells lie in a known
 //    bounding box), stages the six gather fields of the box in shared memory,
 //    deposits J into a shared-memory copy of the box with shared atomics and
-//    adds the box to the global current once. A chunk whose box exceeds the
-//    shared-memory capacity runs the same arithmetic on global memory.
+//    adds the box to the global current once. A mixed-precision chunk whose
+//    electrons are all at rest with their ions in a field-free window only
+//    moves its box. k_push_deferred runs the same arithmetic on global memory
+//    for a chunk whose box exceeds the shared-memory capacity, and carries the
+//    antenna in further blocks;
 //  - tile sort (counting sort into tiles; within a tile, particles are grouped
 //    by their rank inside their cell so that the lanes of a warp usually hold
 //    particles of different cells and their shared atomics do not collide);

@@ -43,3 +43,22 @@ def test_3d_push_forms(orc, many, order, gather):
     for k in ("x", "y", "z", "w"):
         assert rel(pg[k][ig], po[k][io]) <= TOL64, k
     assert rel(np.stack([pg[k][ig] for k in ("ux", "uy", "uz")]), np.stack([po[k][io] for k in ("ux", "uy", "uz")])) <= TOL64
+
+
+def test_3d_grid_that_fills_the_chip(orc):
+    """a grid past the lines below which a filter pass takes all components in one launch and Faraday tiles of two x nodes:
+    antenna in vacuum with PML, compensated filter and damping against the oracle, 1e-10"""
+    from paper_1009_2727_gb300.pic import Simulation
+    w = W.shrink3(W.parity_3d(), 49, 50, 1000, theta=0.2, filter_passes=2, filter_compensate=1)
+    del w["plasma"]
+    w["laser"]["t_peak"] = 4e-15
+    g = Simulation(w, precision="fp64")
+    o = orc.Sim3(w)
+    g.step(8)
+    o.step(8)
+    g.sync()
+    assert np.abs(o.field(1)).max() > 0
+    for grp in ((0, 1, 2), (3, 4, 5)):
+        a = np.stack([g.field(c) for c in grp])
+        b = np.stack([o.field(c) for c in grp])
+        assert rel(a, b) <= TOL64, grp
