@@ -357,7 +357,7 @@ constexpr int push_threads1() { return sizeof(T) == 8 ? 64 : 128; }
 constexpr int JW1 = 192;
 
 template <class T, int ORD, bool MC>
-__global__ void __launch_bounds__(push_threads1<T>()) k1_push(G1 g, const T* __restrict__ fE, const T* __restrict__ fB, T* J,
+__global__ void __launch_bounds__(push_threads1<T>()) k1_push(G1 g, const T* fE, const T* fB, T* J,
                                                Parts1<T> p, int count, Ctrl1* ctrl, T kq, T qe, double zlo,
                                                double zhi1, Lat1 L, Rows1 rows, Ions1 ions, Ant1 ant, int nbp) {
   constexpr int NG = ORD + 1, ND = NG + 1, OFF = ORD == 3 ? 1 : 0, PB1 = push_threads1<T>();

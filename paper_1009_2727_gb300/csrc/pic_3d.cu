@@ -143,12 +143,14 @@ __device__ __forceinline__ T dstar_s(const T* S, int a, int c0, T ca, T cb, T cg
   return (ca * D[1][1] + cb * s1 + cg * s2) * inv_d;
 }
 
+// A kernel that waits for its predecessor on the device takes plain pointers: restrict on its parameters would promise
+// that nothing writes the data from the kernel's start on, which the predecessor still does. Where the promise is worth
+// having (loads ahead of the loop's earlier stores) the work is a function called after the wait.
 template <class T, int FX>
-__global__ void __launch_bounds__(256) k3_faraday_tile(G3 g, Pml3<T> pm, const T* __restrict__ E,
-                                                       const T* __restrict__ Ep, const T* __restrict__ Eb,
-                                                       T* __restrict__ B, T* __restrict__ Bs, T* __restrict__ fB, T c1,
-                                                       T c2, T c3, T ca, T cb, T cg, T dtT) {
-  if constexpr (FX < 4) chain_wait();   // (a few hundred cycles per block: not on a grid that fills the chip)
+__device__ __forceinline__ void faraday_tile3(const G3& g, const Pml3<T>& pm, const T* __restrict__ E,
+                                              const T* __restrict__ Ep, const T* __restrict__ Eb, T* __restrict__ B,
+                                              T* __restrict__ Bs, T* __restrict__ fB, T c1, T c2, T c3, T ca, T cb, T cg,
+                                              T dtT) {
   constexpr int SX = FX + 2, SY = FY + 2, SZ = FZ + 2, SN = SX * SY * SZ;
   __shared__ T se[3][SN];   // index (x * SY + y) * SZ + z, tile origin at (1, 1, 1)
   const int i0 = blockIdx.z * FX, j0 = blockIdx.y * FY, k0 = blockIdx.x * FZ;
@@ -202,6 +204,13 @@ __global__ void __launch_bounds__(256) k3_faraday_tile(G3 g, Pml3<T> pm, const T
       fB[q * g.cs + p] = T(0.5) * (old + nw);
     }
   }
+}
+
+template <class T, int FX>
+__global__ void __launch_bounds__(256) k3_faraday_tile(G3 g, Pml3<T> pm, const T* E, const T* Ep, const T* Eb, T* B, T* Bs,
+                                                       T* fB, T c1, T c2, T c3, T ca, T cb, T cg, T dtT) {
+  if constexpr (FX < 4) chain_wait();   // (a few hundred cycles per block: not on a grid that fills the chip)
+  faraday_tile3<T, FX>(g, pm, E, Ep, Eb, B, Bs, fB, c1, c2, c3, ca, cb, cg, dtT);
 }
 
 // Friedman history (PR-1): E-bar <- (1 - theta/2) E + (theta/2) E-bar, E^{n-1} <- E, gather copy <- E
@@ -269,9 +278,8 @@ __device__ __forceinline__ void ampere_node(const G3& g, const Pml3<T>& pm, T* _
 }
 
 template <class T>
-__global__ void __launch_bounds__(128) k3_ampere(G3 g, Pml3<T> pm, T* __restrict__ E, T* __restrict__ Es,
-                                                 const T* __restrict__ B, const T* __restrict__ J, T dtc2, T dte) {
-  chain_wait();
+__device__ __forceinline__ void ampere_nodes(const G3& g, const Pml3<T>& pm, T* __restrict__ E, T* __restrict__ Es,
+                                             const T* __restrict__ B, const T* __restrict__ J, T dtc2, T dte) {
   const int k0 = blockIdx.x * blockDim.x * KPT + threadIdx.x, j = blockIdx.y, i = blockIdx.z;
 #pragma unroll
   for (int kk = 0; kk < KPT; kk++) {
@@ -279,6 +287,12 @@ __global__ void __launch_bounds__(128) k3_ampere(G3 g, Pml3<T> pm, T* __restrict
     if (k > g.n[2]) break;
     ampere_node<T>(g, pm, E, Es, B, J, dtc2, dte, i, j, k);
   }
+}
+
+template <class T>
+__global__ void __launch_bounds__(128) k3_ampere(G3 g, Pml3<T> pm, T* E, T* Es, const T* B, const T* J, T dtc2, T dte) {
+  chain_wait();
+  ampere_nodes<T>(g, pm, E, Es, B, J, dtc2, dte);
 }
 
 // one axis of the composed filter: out = sum_m c_m F(node + (m - P) s e_axis), zero off the valid range.
@@ -390,8 +404,8 @@ __device__ __forceinline__ void ld16(const double* p, double* v) {
 // would otherwise need a block for its last node); longer remainders get a block of their own.
 constexpr int ZR = 8, ZHA = 8, ZTAIL = 32;
 template <class T, int PT>
-__global__ void __launch_bounds__(128) k3_filter_zs(G3 g, const T* __restrict__ src0, T* __restrict__ dst03,
-                                                    T* __restrict__ dst35, int c0, int nb, Taps3<T> t) {
+__global__ void __launch_bounds__(128) k3_filter_zs(G3 g, const T* src0, T* dst03, T* dst35, int c0, int nb,
+                                                    Taps3<T> t) {
   chain_wait();
   static_assert(PT <= ZHA, "filter halo above the staged halo");
   constexpr int SEG = 128 * ZR, NV = ZR + 2 * ZHA, VL = 16 / (int)sizeof(T);
@@ -497,7 +511,7 @@ constexpr long kWait3 = 1L << 24;
 
 template <class T, int PT>
 __global__ void __launch_bounds__(256) k3_filter_xy(G3 g, const __grid_constant__ CUtensorMap map03,
-                                                    const __grid_constant__ CUtensorMap map35, T* __restrict__ dst0,
+                                                    const __grid_constant__ CUtensorMap map35, T* dst0,
                                                     int c0, int nb, Taps3<T> t, Ctrl3* ctrl) {
   if ((int)gridDim.x > nb) chain_wait();   // components share the launch: a small grid
   constexpr int W = 2 * PT + 1, XW = XYT + 2 * PT;
@@ -709,9 +723,8 @@ void launch_filter_axis(const G3& g, dim3 grid, const T* src, T* dst, int comp, 
 // staggered values along each half-integer axis of the component (two along one axis, four along two);
 // values off the grid count as zero. dst holds Ex, Ey, Ez, Bx, By, Bz, cs elements each.
 template <class T>
-__global__ void __launch_bounds__(128) k3_nodal(G3 g, const T* __restrict__ fE, const T* __restrict__ fB,
-                                                T* __restrict__ dst) {
-  chain_wait();
+__device__ __forceinline__ void nodal_values(const G3& g, const T* __restrict__ fE, const T* __restrict__ fB,
+                                             T* __restrict__ dst) {
   const int k0 = blockIdx.x * blockDim.x * KPT + threadIdx.x, j = blockIdx.y, i = blockIdx.z;
   const long sx = (long)(g.n[1] + 1) * g.ldz, sy = g.ldz;
 #pragma unroll
@@ -745,6 +758,12 @@ __global__ void __launch_bounds__(128) k3_nodal(G3 g, const T* __restrict__ fE, 
       dst[c * g.cs + p] = cnt == 4 ? T(0.25) * acc : cnt == 2 ? T(0.5) * acc : acc;
     }
   }
+}
+
+template <class T>
+__global__ void __launch_bounds__(128) k3_nodal(G3 g, const T* fE, const T* fB, T* dst) {
+  chain_wait();
+  nodal_values<T>(g, fE, fB, dst);
 }
 
 // ---------------------------------------------------------------------------
