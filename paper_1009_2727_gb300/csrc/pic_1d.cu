@@ -23,6 +23,7 @@
 
 #include "pic_3d.h"
 #include "pic_common.cuh"
+#include "pic_dst.h"
 
 namespace picgb {
 namespace {
@@ -1063,6 +1064,7 @@ class Sim1 : public Sim3Api {
   int get_field(int comp, double* dst, int on_device) override {
     if (comp < 0 || comp > PIC_RHO) return fail(PIC_EINVAL, "bad component");
     const int n1 = g.nz + 1;
+    if (on_device && !ddst.order(s)) return fail(PIC_ECUDA, "CUDA error in get_field");
     if (comp == PIC_RHO) {
       cudaMemsetAsync(rho, 0, sizeof(double) * g.n1p, s);
       if (loaded && count_ub > 0) {
@@ -1210,6 +1212,7 @@ class Sim1 : public Sim3Api {
   pic_laser las{};
   long long row_next = 0, mlo = 0, shifts = 0, step = 0;
   int64_t nl = 0, compactions = 0;
+  DeviceDst ddst;        // get_field to device memory
   bool timing_on = false;
   int timing_which = 0;
   double t_ms = 0;

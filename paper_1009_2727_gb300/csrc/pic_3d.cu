@@ -28,6 +28,7 @@
 
 #include "pic_3d.h"
 #include "pic_common.cuh"
+#include "pic_dst.h"
 
 namespace picgb {
 namespace {
@@ -2100,6 +2101,7 @@ struct Sim3 : Sim3Api {
   T *Es = nullptr, *Bs = nullptr;     // 6 split parts each
   T *fE = nullptr, *fB = nullptr, *tmp = nullptr, *tmp2 = nullptr;
   double* rho = nullptr;              // scratch for PIC_RHO
+  DeviceDst ddst;         // get_field to device memory
   double* out_d = nullptr;            // copy-out scratch
   Pml3<T> pm;
   Taps3<T> taps;
@@ -2800,6 +2802,7 @@ struct Sim3 : Sim3Api {
   int get_field(int comp, double* dst, int on_device) override {
     if (comp < 0 || comp > PIC_RHO) return fail(PIC_EINVAL, "bad component");
     const long nn = nodes();
+    if (on_device && !ddst.order(s)) return fail(PIC_ECUDA, "CUDA error in get_field");
     // a device destination is written in place, a host one through out_d
     double* o = dst;
     if (!on_device) {

@@ -14,6 +14,7 @@
 #include "pic_3d.h"
 #include "pic_batch.h"
 #include "pic_common.cuh"
+#include "pic_dst.h"
 
 namespace picgb {
 int push_occupancy(int order, bool dbl, int smem_nodes);
@@ -159,12 +160,11 @@ struct Sim : SimBase {
   int timing_which = 0;
   std::vector<cudaEvent_t> ev;
   int64_t timed_launches = 0;
-  cudaEvent_t dst_ready = nullptr;   // get_field: the default stream's work before a device destination is written
+  DeviceDst ddst;       // get_field to device memory
 
   explicit Sim(pic_ctx* ctx) : c(ctx) {}
   ~Sim() override {
     for (auto e : ev) cudaEventDestroy(e);
-    if (dst_ready) cudaEventDestroy(dst_ready);
     if (hmirror) cudaFreeHost(hmirror);
     if (hstats) cudaFreeHost(hstats);
   }
@@ -892,14 +892,7 @@ struct Sim : SimBase {
 
   int get_field(int comp, double* dst, int on_device) {
     set_ptrs_for_step();
-    if (on_device && c->stream) {
-      // dst is written on the context's stream: after the work already queued on the default stream, where the caller's
-      // earlier use of that memory may still run
-      if (!dst_ready && cudaEventCreateWithFlags(&dst_ready, cudaEventDisableTiming) != cudaSuccess)
-        return c->fail(PIC_ECUDA, "event creation failed");
-      cudaEventRecord(dst_ready, nullptr);
-      cudaStreamWaitEvent(c->stream, dst_ready, 0);
-    }
+    if (on_device && !ddst.order(c->stream)) return c->fail(PIC_ECUDA, "CUDA error in get_field");
     const size_t n = stage_n;
     if (comp >= PIC_EX && comp <= PIC_JZ) {
       const T* src = comp < 3 ? f.E[comp] : comp < 6 ? f.B[comp - 3] : f.Jn[comp - 6];
