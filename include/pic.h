@@ -241,7 +241,9 @@ int pic_free(pic_ctx* ctx);
 /* Accessors (synchronise the stream). */
 /* Copy one grid component (PIC_EX..PIC_JZ, or PIC_RHO = charge density of
  * electrons and ions at the current positions) into dst: (nx+1)*(nz+1) values
- * of type double (always converted to double). on_device selects dst memory. */
+ * of type double (always converted to double). on_device selects dst memory: any
+ * that cudaMemcpy reaches as a device pointer, written after the work already
+ * queued on the default stream; the call returns when dst is complete. */
 int pic_get_field(pic_ctx* ctx, int comp, double* dst, int on_device);
 /* Overwrite one of the six E/B components from a host array of doubles (tests). */
 int pic_set_field(pic_ctx* ctx, int comp, const double* src);

@@ -1077,9 +1077,12 @@ class Sim1 : public Sim3Api {
       }
       cudaMemcpyAsync(dst, rho, sizeof(double) * n1, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
     } else {
-      k1_out<T><<<nb1(n1, 256), 256, 0, s>>>(n1, comp_ptr(comp), on_device ? dst : outd);
+      // written in place where a kernel may, else through the scratch
+      double* out = on_device && DeviceDst::in_place(dst) ? dst : outd;
+      k1_out<T><<<nb1(n1, 256), 256, 0, s>>>(n1, comp_ptr(comp), out);
       nl++;
-      if (!on_device) cudaMemcpyAsync(dst, outd, sizeof(double) * n1, cudaMemcpyDeviceToHost, s);
+      if (out != dst)
+        cudaMemcpyAsync(dst, outd, sizeof(double) * n1, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
     }
     return cudaStreamSynchronize(s) == cudaSuccess ? PIC_OK : fail(PIC_ECUDA, "CUDA error in get_field");
   }

@@ -2803,9 +2803,9 @@ struct Sim3 : Sim3Api {
     if (comp < 0 || comp > PIC_RHO) return fail(PIC_EINVAL, "bad component");
     const long nn = nodes();
     if (on_device && !ddst.order(s)) return fail(PIC_ECUDA, "CUDA error in get_field");
-    // a device destination is written in place, a host one through out_d
+    // written in place where a kernel may, else through out_d
     double* o = dst;
-    if (!on_device) {
+    if (!on_device || !DeviceDst::in_place(dst)) {
       if (!out_d) { out_d = dal<double>(nn); if (!out_d) return fail(PIC_ENOMEM, "allocation failed"); }
       o = out_d;
     }
@@ -2830,7 +2830,8 @@ struct Sim3 : Sim3Api {
       k3_out_field<T><<<nblk(nn, 256), 256, 0, s>>>(g, comp_ptr(comp), o);
     }
     nl++;
-    if (!on_device) cudaMemcpyAsync(dst, out_d, sizeof(double) * nn, cudaMemcpyDeviceToHost, s);
+    if (o != dst)
+      cudaMemcpyAsync(dst, out_d, sizeof(double) * nn, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
     return cudaStreamSynchronize(s) == cudaSuccess ? PIC_OK : fail(PIC_ECUDA, "CUDA error in get_field");
   }
 

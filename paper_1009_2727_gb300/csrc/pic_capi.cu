@@ -894,25 +894,26 @@ struct Sim : SimBase {
     set_ptrs_for_step();
     if (on_device && !ddst.order(c->stream)) return c->fail(PIC_ECUDA, "CUDA error in get_field");
     const size_t n = stage_n;
+    // written in place where a kernel may, else through the scratch
+    double* out = on_device && DeviceDst::in_place(dst) ? dst : stage;
     if (comp >= PIC_EX && comp <= PIC_JZ) {
       const T* src = comp < 3 ? f.E[comp] : comp < 6 ? f.B[comp - 3] : f.Jn[comp - 6];
-      launch_convert<T>(src, on_device ? dst : stage, g, c->stream);
+      launch_convert<T>(src, out, g, c->stream);
     } else if (comp == PIC_RHO) {
-      double* rho = on_device ? dst : stage;
-      cudaMemsetAsync(rho, 0, n * 8, c->stream);
-      if (loaded) launch_rho<T>(g, P, ctrl, cap, c->cfg.shape_order, -kQe, rho, c->stream);
+      cudaMemsetAsync(out, 0, n * 8, c->stream);
+      if (loaded) launch_rho<T>(g, P, ctrl, cap, c->cfg.shape_order, -kQe, out, c->stream);
       if (ions && loaded) {
         const double t = time_of(step);
         long long mlo = std::max(row_first, (long long)std::ceil((zlo_prev + c->hg.beta * kC * t) / ip.h - 0.5));
         if (step == 0) mlo = row_first;
         launch_ion_rows(g, mlo, row_next, t, ip, c->cfg.shape_order, ion_R0, c->stream);
-        launch_ion_rho(g, ion_x, ion_R0, kQe / (g.dx * g.dz), rho, c->stream);
+        launch_ion_rho(g, ion_x, ion_R0, kQe / (g.dx * g.dz), out, c->stream);
       }
     } else {
       return c->fail(PIC_EINVAL, "unknown component");
     }
-    // a device destination was written in place (on this stream); the call returns when it is there
-    if (!on_device) cudaMemcpyAsync(dst, stage, n * 8, cudaMemcpyDeviceToHost, c->stream);
+    if (out != dst)
+      cudaMemcpyAsync(dst, stage, n * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream);
     cudaStreamSynchronize(c->stream);
     return cudaGetLastError() == cudaSuccess ? PIC_OK : c->fail(PIC_ECUDA, "CUDA error in get_field");
   }
