@@ -823,12 +823,19 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) k_mlp_fwd_tc(const __grid_co
           : "memory");
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       if (!last) {
-        // (the columns of the padding have zero weights and biases, and GELU(0) = 0)
         __align__(16) __nv_bfloat162 h[8];
 #pragma unroll
         for (int q = 0; q < 8; q++) {
           const F2 g = gelu2(add2(f2(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1])), f2(b[2 * q], b[2 * q + 1])));
           h[q] = __floats2bfloat162_rn(lo(g), hi(g));
+        }
+        // the padding's columns are zero whatever the row holds (their products are not where an activation is infinite)
+        if (c0 + 16 > Ly.N) {
+#pragma unroll
+          for (int q = 0; q < 8; q++) {
+            if (c0 + 2 * q >= Ly.N) h[q].x = __float2bfloat16(0.0f);
+            if (c0 + 2 * q + 1 >= Ly.N) h[q].y = __float2bfloat16(0.0f);
+          }
         }
         *reinterpret_cast<uint4*>(A + act_off(rloc, c0)) = *reinterpret_cast<const uint4*>(h);
         *reinterpret_cast<uint4*>(A + act_off(rloc, c0 + 8)) = *reinterpret_cast<const uint4*>(h + 4);
