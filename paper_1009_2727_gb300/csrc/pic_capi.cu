@@ -15,6 +15,7 @@
 #include "pic_batch.h"
 #include "pic_common.cuh"
 #include "pic_dst.h"
+#include "pic_pml.cuh"
 
 namespace picgb {
 int push_occupancy(int order, bool dbl, int smem_nodes);
@@ -253,13 +254,14 @@ struct Sim : SimBase {
     pt.cz_i = dz_t + 4 * nz1; pt.cz_h = dz_t + 5 * nz1;
     // the FP32 pairs (pml_step): B's, then E's
     const auto pairs = [](const std::vector<double>& v, int n1, std::vector<float4>& out) {
-      const auto hi = [](double a) { return (float)a; };
-      const auto lo = [](double a) { return (float)(a - (double)(float)a); };
       out.resize(2 * n1);
       for (int i = 0; i < n1; i++) {
-        const double xb = v[3 * n1 + i], cb = v[5 * n1 + i], xe = v[2 * n1 + i], ce = (kC * kC) * v[4 * n1 + i];
-        out[i] = make_float4(hi(xb), lo(xb), hi(cb), lo(cb));
-        out[n1 + i] = make_float4(hi(xe), lo(xe), hi(ce), lo(ce));
+        float4& b = out[i];
+        float4& e = out[n1 + i];
+        pml_pair(v[3 * n1 + i], b.x, b.y);
+        pml_pair(v[5 * n1 + i], b.z, b.w);
+        pml_pair(v[2 * n1 + i], e.x, e.y);
+        pml_pair((kC * kC) * v[4 * n1 + i], e.z, e.w);
       }
     };
     std::vector<float4> px, pz;

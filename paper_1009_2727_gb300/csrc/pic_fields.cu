@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "pic_common.cuh"
+#include "pic_pml.cuh"
 
 namespace picgb {
 
@@ -40,30 +41,6 @@ __device__ __forceinline__ void load_tile_b(const GridP& g, const FieldPtrs<T>& 
   }
 }
 
-// xi a + cf b of the split-field PML (f cf: E's c^2), rounded once. The coefficients are FP64; FP32 fields take them as
-// pairs of FP32 values and the products and the sum with their rounding errors, about 2^-47 of the larger term before the
-// final rounding; where the terms cancel to a thousandth, FP64 as for FP64 fields. (4 million values over all ranges of the
-// coefficients and with cancelling terms: the same results as FP64 arithmetic, bit for bit.) FP64 itself (conversions included) bounded the field kernels: a warp's FP64 instruction occupies the SM for 16
-// cycles, and the SMs with PML tiles were busy with them 70 to 90 % of the time.
-template <class T>
-__device__ __forceinline__ T pml_step(const double* x, const double* c, const float4* t, int q, double f, T a, T b,
-                                      bool minus) {
-  if (minus) b = -b;
-  if constexpr (sizeof(T) == 4) {
-    const float4 w = t[q];
-    const float p = __fmul_rn(w.x, a), pe = __fmaf_rn(w.x, a, -p);
-    const float r = __fmul_rn(w.z, b), re = __fmaf_rn(w.z, b, -r);
-    const float s = __fadd_rn(p, r), v = __fadd_rn(s, -p);
-    if (!(fabsf(s) < 0x1p-10f * fabsf(p))) {
-      float e = __fadd_rn(__fadd_rn(p, -__fadd_rn(s, -v)), __fadd_rn(r, -v));
-      e = __fadd_rn(e, __fadd_rn(pe, re));
-      e = __fmaf_rn(w.y, a, e);
-      e = __fmaf_rn(w.w, b, e);
-      return fabsf(s) < INFINITY ? __fadd_rn(s, e) : s;   // (an infinite field has no rounding error)
-    }
-  }
-  return T(x[q] * (double)a + f * c[q] * (double)b);
-}
 // sigma > 0 (by the bits: an FP64 comparison takes the FP64 pipe)
 __device__ __forceinline__ bool damped(const double* sigma, int q) {
   return __double_as_longlong(sigma[q]) > 0;
