@@ -181,6 +181,19 @@ __host__ __device__ inline void frame_z(uint32_t c, float oz, int sz, float fz, 
   tz = t;
 }
 
+// the grid rows z0 .. z1 of the stored positions with keys lo .. hi (z_key) for the frame shift (sz, fz)
+__host__ __device__ inline void key_rows(uint32_t lo, uint32_t hi, int sz, float fz, int& z0, int& z1) {
+  float t;
+  frame_z((lo >> 16) & 0xffffu, (float)(lo & 0xffffu) * (1.0f / 65536.0f), sz, fz, z0, t);
+  frame_z((hi >> 16) & 0xffffu, (float)(hi & 0xffffu) * (1.0f / 65536.0f), sz, fz, z1, t);
+}
+// all of them in the rows iz0 .. iz1 of their chunk's box, the rows whose fields its window holds
+__host__ __device__ inline bool key_rows_in(uint32_t lo, uint32_t hi, int sz, float fz, int iz0, int iz1) {
+  int z0, z1;
+  key_rows(lo, hi, sz, fz, z0, z1);
+  return iz0 <= z0 && z0 <= z1 && z1 <= iz1;
+}
+
 // Lattice site (row m, column a) of a plasma particle: the stored cell and
 // offsets (z in the drifting frame) that the particle gets at injection, and
 // that its lab-fixed ion keeps for ever (row m at z = (m + 1/2) dz / ppcz).

@@ -734,10 +734,11 @@ __device__ __forceinline__ bool chunk_at_rest(const Particles<T>& p, const Chunk
     if (lo > hi) return false;
   }
   lo += zref; hi += zref;
+  // an electron outside the box (the FP64 rows of the inflow's box and the frame's can differ at a cell's edge; a pushed
+  // particle would take the global path) may have a field that the window does not show
+  if (!key_rows_in(lo, hi, pc.fr0_sz, pc.fr0_fz, ch.iz0, ch.iz1) || x0 < ch.ix0 || x1 > ch.ix1) return false;
   int z0, z1;
-  float t;
-  frame_z((lo >> 16) & 0xffffu, (float)(lo & 0xffffu) * (1.0f / 65536.0f), pc.fr1_sz, pc.fr1_fz, z0, t);
-  frame_z((hi >> 16) & 0xffffu, (float)(hi & 0xffffu) * (1.0f / 65536.0f), pc.fr1_sz, pc.fr1_fz, z1, t);
+  key_rows(lo, hi, pc.fr1_sz, pc.fr1_fz, z0, z1);
   // everything clear of the domain's edges by a cell, before and after: nothing leaves, every ion row stays live
   if (ch.iz0 <= pc.cz_lo || z0 <= pc.cz_lo || z0 > z1 || z1 + 1 >= pc.cz_hi || x0 < pc.cx_lo || x1 >= pc.cx_hi)
     return false;
