@@ -43,8 +43,8 @@ BYTES_PER_CELL = {"mixed": 168, "fp64": 336}
 # DRAM bytes (read + write) per particle of a push launch in which every particle is pushed (k_push, mixed precision, cubic
 # shapes, the Yee-located gather), for every layout the autotuner can return, keyed by (tile_x, tile_z, sort_every): ncu
 # dram__bytes_read.sum + dram__bytes_write.sum on the 2048 x 256 stage box, measured when chunks at rest were still pushed
-# (the 2nd and 3rd push of each layout). Below the 56 bytes of stored state: the last writes of a launch are still in the
-# 129 MB L2 when it ends. What a run moves is less (PUSH_DRAM_BYTES_PER_PARTICLE).
+# (the 2nd and 3rd push of each layout; --layout-sweep pushes every chunk). Below the 56 bytes of stored state: the last
+# writes of a launch are still in the 129 MB L2 when it ends.
 TRAFFIC_BYTES_PER_PARTICLE = {
     (8, 8, 8): 49.71, (8, 8, 16): 49.61, (8, 8, 32): 49.58, (8, 8, 64): 49.49, (8, 8, 128): 49.62, (8, 16, 8): 49.58,
     (8, 16, 16): 49.63, (8, 16, 32): 49.61, (8, 16, 64): 49.49, (8, 16, 128): 49.63, (8, 32, 8): 49.83,
@@ -56,16 +56,13 @@ TRAFFIC_BYTES_PER_PARTICLE = {
     (32, 16, 16): 49.3, (32, 16, 32): 49.07, (32, 16, 64): 49.05, (32, 16, 128): 49.2, (32, 32, 8): 48.87,
     (32, 32, 16): 48.85, (32, 32, 32): 48.84, (32, 32, 64): 48.94, (32, 32, 128): 48.95,
 }
-# DRAM bytes, warp instructions and FP32 operations per particle of one push launch (k_push), mixed precision, cubic
-# shapes, the Yee-located gather: ncu dram__bytes_read.sum + dram__bytes_write.sum, smsp__inst_executed.sum and
-# smsp__sass_thread_inst_executed_op_{fadd,fmul,ffma}_pred_on.sum of the pushes of steps 104-106 (the middle of the default
-# 200 steps) on the 2048 x 256 stage box, 8 x 16-cell tiles, sort every 64, over all its particles (6,514,944): 37.1 MB,
-# 44.6 M, and 278 M counted as FADD + FMUL + 2 FFMA (the packed two-lane FMAs of the gather are not in these counters).
-# Chunks of electrons at rest in a field-free window are in the count of particles and cost next to nothing; what moves
-# of the half box stays in the 129 MB L2 from one step to the next.
-PUSH_DRAM_BYTES_PER_PARTICLE = 5.7
-PUSH_WARP_INST_PER_PARTICLE = 6.85
-PUSH_FLOPS_PER_PARTICLE = 42.7
+# Warp instructions and FP32 operations that a pushed particle takes at least (mixed precision, cubic shapes, the Yee-located
+# gather): ncu smsp__inst_executed.sum and smsp__sass_thread_inst_executed_op_{fadd,fmul,ffma}_pred_on.sum of pushes of plasma
+# at rest with every chunk pushed, where most terms of the deposit are zero and skipped (2048 x 256 stage box, 8 x 16-cell
+# tiles, sort every 64; counted as FADD + FMUL + 2 FFMA, without the packed two-lane FMAs of the gather). With no term zero
+# (--push-all, steps 104-106) it is 39.7 and 351. The staging of windows for chunks at rest comes on top.
+PUSH_WARP_INST_PER_PARTICLE = 21.0
+PUSH_FLOPS_PER_PARTICLE = 174.0
 # 3D: ncu dram bytes of k3_push_tiles on the 256 x 128 x 128 box (195.3 MB for 2,356,608 electrons), scaled
 # to the full box by its particle count
 TRAFFIC_BYTES_PER_PARTICLE_3D = {("mixed", 3): 82.9}
@@ -512,6 +509,7 @@ def run_1d(args):
     sampler.start()
     torch.cuda.synchronize()
     l0 = sim.launches()
+    counts0 = None if three else sim.push_counts()
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
     ev0.record(stream)
@@ -520,6 +518,7 @@ def run_1d(args):
     torch.cuda.synchronize()
     clocks = sampler.stop()
     launches = sim.launches() - l0
+    counts1 = None if three else sim.push_counts()
     ms = ev0.elapsed_time(ev1)
     push_ms, push_n = sim.timing(False)
     n1 = sim.stats()["n_electrons"]
@@ -658,8 +657,8 @@ def run_stage3d(args):  # noqa: C901
 def run_layout_sweep(args):
     """every particle layout the autotuner can return (tiles {8, 16, 32}^2, sort cadences 8, 16, 32, 64, 128;
     --sweep-cadences restricts the cadences) on the given box, a few steps each: run under ncu with the DRAM
-    byte counters to tabulate the push kernel's traffic per particle for each layout (prints one line per
-    layout with its electron count)"""
+    byte counters to tabulate the push kernel's traffic per particle for each layout, every particle pushed (prints
+    one line per layout with its electron count)"""
     import torch
     from paper_1009_2727_gb300 import workloads as W
     from paper_1009_2727_gb300.pic import Simulation
@@ -671,6 +670,7 @@ def run_layout_sweep(args):
         for tz in (8, 16, 32):
             for se in (int(v) for v in args.sweep_cadences.split(",")):
                 sim = Simulation(w, precision=args.precision, tile=(tx, tz), sort_every=se)
+                push_all(sim)
                 sim.step(args.steps)
                 sim.sync()
                 print(json.dumps({"tile": [tx, tz], "sort_every": se, "steps": args.steps,
@@ -777,6 +777,26 @@ def wide_band(w, strides, three):
     return w
 
 
+def push_all(sim):
+    """1e-25 V/m and T on every node: no chunk's window is field-free, so that every particle is pushed, and nothing moves
+    by it (counters of the push; not the benchmark)"""
+    import numpy as np
+    for c in range(6):
+        sim.set_field(c, np.full(sim.shape, 1e-25))
+
+
+def push_roofline(pushed, at_rest, push_ms, bytes_per_particle, traffic_per_particle, peak):
+    """the push's rates over one step: algorithmic bytes of the particles pushed; its DRAM traffic where every particle is
+    pushed and the particles' stored state is well above the 129 MB L2 (the state the traffic figures were measured in)"""
+    achieved = pushed * bytes_per_particle / (push_ms * 1e-3) / 1e9 if push_ms > 0 else None
+    measured = traffic_per_particle and at_rest <= 0.01 * pushed and 56.0 * pushed >= 2 * 129e6
+    return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+            "frac": achieved / peak if achieved is not None else None,
+            "traffic": traffic_per_particle * pushed if measured else None,
+            "algorithmic_bytes_per_particle": bytes_per_particle,
+            "particles_pushed_per_step": pushed, "particles_at_rest_per_step": at_rest}
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -815,6 +835,9 @@ def main():
                     help="instability level (high-k E_z power at fixed times) against c dt/dz for both gather schemes")
     ap.add_argument("--solver-accuracy", action="store_true",
                     help="Sec. 5.1.2: beam gain of the scaled stage at gamma 2-13 with CK, Yee-Friedman and Yee + S(1:2:4)")
+    ap.add_argument("--push-all", action="store_true",
+                    help="a field too weak to move anything on every node, so that no chunk counts as at rest (for "
+                         "counters of the push with every particle pushed)")
     ap.add_argument("--layout-sweep", action="store_true",
                     help="step every layout the autotuner can return, a few steps each (for a DRAM traffic table)")
     ap.add_argument("--stage3d", type=int, default=0,
@@ -889,6 +912,8 @@ def main():
     else:
         sim = Simulation(w, precision=args.precision, sort_every=args.sort_every)
     stream = torch.cuda.current_stream()
+    if args.push_all:
+        push_all(sim)
     for _ in range(max(args.warmup, 3)):
         sim.step(1)
     sim.sync()
@@ -900,6 +925,7 @@ def main():
     barrier(ws)
     torch.cuda.synchronize()
     l0 = sim.launches()
+    counts0 = None if three else sim.push_counts()
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
     ev0.record(stream)
@@ -909,6 +935,7 @@ def main():
     barrier(ws)
     clocks = sampler.stop()
     launches = sim.launches() - l0
+    counts1 = None if three else sim.push_counts()
     ms = ev0.elapsed_time(ev1)
     push_ms, push_n = sim.timing(False)
     # field kernels (Faraday, filters, Ampere) over a shorter run after the timed region
@@ -927,32 +954,29 @@ def main():
     peak = peaks.get("hbm_gbs", 6800.0)
     bpp = (BYTES_PER_PARTICLE_3D if three else BYTES_PER_PARTICLE)[args.precision]
     push_avg_ms = push_ms / max(push_n, 1)
-    achieved = n_avg * bpp / (push_avg_ms * 1e-3) / 1e9
+    standard = args.precision == "mixed" and args.order == 3 and args.gather == "energy"
     if three:
+        pushed, at_rest = n_avg, 0.0
         tpp = TRAFFIC_BYTES_PER_PARTICLE_3D.get((args.precision, args.order)) if args.gather == "energy" else None
     else:
-        ok = args.precision == "mixed" and args.order == 3 and args.gather == "energy"
-        tpp = PUSH_DRAM_BYTES_PER_PARTICLE if ok else None
+        pushed, at_rest = ((b - a) / args.steps for a, b in zip(counts0, counts1))
         lay = (tuple(tuned["tile"]) + (tuned["sort_every"],)) if tuned else None
-        all_moving = TRAFFIC_BYTES_PER_PARTICLE.get(lay) if ok and lay else None
+        tpp = TRAFFIC_BYTES_PER_PARTICLE.get(lay) if standard and lay else None
     roof = {"kernel": "k3_push_tiles (3D gather + Boris + Esirkepov)" if three else "k_push (gather + Boris + Esirkepov)",
-            "bound": "hbm", "achieved": achieved, "peak": peak,
-            "unit": "GB/s", "frac": achieved / peak, "traffic": tpp * n_avg if tpp else None,
-            "traffic_source": ("ncu dram bytes of k3_push_tiles, 256 x 128 x 128 box, scaled by particles" if three
-                               else "ncu dram bytes of k_push, 2048 x 256 box, steps 104-106, scaled by particles") if tpp else None,
+            **push_roofline(pushed, at_rest, push_avg_ms, bpp, tpp, peak),
+            "traffic_source": ("ncu dram bytes of k3_push_tiles, 256 x 128 x 128 box, scaled by particles" if three else
+                               "ncu dram bytes of k_push with every particle pushed, 2048 x 256 box, by layout, scaled by "
+                               "particles (null where chunks are at rest or the particles fit in L2)") if tpp else None,
             "note": ("3D push on sorted 4x4x16-cell tiles with shared-memory windows: issue- and latency-bound at "
                      "three CTAs per SM (ncu: 52% issue slots, 37% warps active, 193 warp instructions per "
                      "particle, 4% DRAM)" if three else
-                     "achieved counts every particle's algorithmic bytes, but chunks of electrons at rest in a "
-                     "field-free window only move their box (their particles are not read or written); the others "
-                     "are bound by instruction issue and the shared-memory pipe (ncu: 64% issue slots); see traffic, "
-                     "issue and alu"),
+                     "the particles pushed (pic_push_counts); those of chunks at rest in a field-free window are neither "
+                     "read nor written, but the windows that show their fields are read and staged, in the same time. Chunks "
+                     "in motion are bound by instruction issue and the shared-memory pipe (at least: issue and alu)"),
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if "hbm_gbs" in peaks else "fallback",
-            "algorithmic_bytes_per_particle": bpp, "push_ms_per_step": push_avg_ms,
+            "push_ms_per_step": push_avg_ms,
             "field_kernels_ms_per_step": field_ms / kf,
             "share_of_step": push_avg_ms / (ms / args.steps)}
-    if not three and all_moving:
-        roof["traffic_if_every_chunk_moved"] = all_moving * n_avg
     # the field kernels' roofline (Faraday + Friedman + PML, gather filter, current filter + Ampere): SURVEY's
     # algorithmic bytes per cell-step (all six E/B components and the current, fused) over their measured time
     cells = w["nx"] * w.get("ny", 1) * w["nz"]
@@ -964,27 +988,29 @@ def main():
                              "peak": peak, "unit": "GB/s", "frac": field_ach / peak if field_ach else None,
                              "algorithmic_bytes_per_cell": bpc, "ms_per_step": field_avg_ms,
                              "cell_steps_per_s": cells / (field_avg_ms * 1e-3) if field_avg_ms > 0 else None}
-    if not three and args.precision == "mixed" and args.order == 3 and args.gather == "energy":
-        # the push's instruction-issue and FP32 rooflines: instruction and FLOP counts per particle from ncu,
-        # time from the CUDA events above; issue peak = 4 warp-instructions per SM per cycle at the median SM
+    if not three and standard:
+        # the push's instruction-issue and FP32 rooflines, from below: the fewest instructions and FLOPs a pushed particle
+        # takes, the particles pushed as counted, time from the CUDA events above; issue peak = 4 warp-instructions per SM per cycle at the median SM
         # clock sampled during the timed steps; FP32 peak measured by the library's FMA microbenchmark
         nsm = torch.cuda.get_device_properties(0).multi_processor_count
         mhz = clocks.get("sm_mhz") or 2070.0
         issue_peak = 4.0 * nsm * mhz * 1e6
-        issue_ach = PUSH_WARP_INST_PER_PARTICLE * n_avg / (push_avg_ms * 1e-3)
+        issue_ach = PUSH_WARP_INST_PER_PARTICLE * pushed / (push_avg_ms * 1e-3)
         import ctypes
         from paper_1009_2727_gb300 import capi
         sc, pk = ctypes.c_double(0.0), ctypes.c_double(0.0)
         fp32_peak = None
         if capi.load().pic_measure_fp32_peak(ctypes.byref(sc), ctypes.byref(pk)) == 0:
             fp32_peak = max(sc.value, pk.value)
-        alu_ach = PUSH_FLOPS_PER_PARTICLE * n_avg / (push_avg_ms * 1e-3) / 1e12
+        alu_ach = PUSH_FLOPS_PER_PARTICLE * pushed / (push_avg_ms * 1e-3) / 1e12
         roof["issue"] = {"achieved": issue_ach, "peak": issue_peak, "unit": "warp-instructions/s",
-                         "frac": issue_ach / issue_peak, "warp_instructions_per_particle": PUSH_WARP_INST_PER_PARTICLE,
+                         "frac": issue_ach / issue_peak, "warp_instructions_per_pushed_particle": PUSH_WARP_INST_PER_PARTICLE,
+                         "note": "at least: a moving particle takes up to 39.7, staging windows at rest comes on top",
                          "peak_source": f"4 per SM per cycle x {nsm} SMs x {mhz:g} MHz (sampled)"}
         roof["alu"] = {"achieved": alu_ach, "peak": fp32_peak, "unit": "TFLOP/s",
                        "frac": alu_ach / fp32_peak if fp32_peak else None,
-                       "flops_per_particle": PUSH_FLOPS_PER_PARTICLE,
+                       "flops_per_pushed_particle": PUSH_FLOPS_PER_PARTICLE,
+                       "note": "at least: a moving particle takes up to 351",
                        "peak_source": "pic_measure_fp32_peak (FMA microbenchmark, measured in this run)"}
     sim.close()
     del sim

@@ -306,6 +306,14 @@ int pic_get_rho_noalloc(pic_ctx* ctx, double* dst_device);
 /* Number of kernel launches enqueued so far by this context (bench accounting). */
 int64_t pic_kernel_launches(pic_ctx* ctx);
 
+/* Particle slots that the 2D push has taken since the context was made, summed
+ * over its steps: those of the chunks it pushed, and those of the chunks of
+ * electrons at rest in a field-free window (mixed precision), of which only the
+ * box moves with the frame: neither read nor written (bench accounting: what a
+ * push works on is the first). 2D contexts only (PIC_EINVAL otherwise);
+ * synchronises the stream. */
+int pic_push_counts(pic_ctx* ctx, int64_t* pushed, int64_t* at_rest);
+
 /* Measured FP32 arithmetic peak of the current device, in TFLOP/s: the best of
  * five launches of a kernel whose threads run eight independent FMA chains
  * over every SM (two FLOPs per FMA lane), once with scalar FMAs and once with

@@ -28,7 +28,7 @@ STATUS_NAMES = {0: "PIC_OK", -1: "PIC_EINVAL", -2: "PIC_ENOMEM", -3: "PIC_ECFL",
 EXPORTS = ("pic_init", "pic_load_plasma", "pic_inject_laser", "pic_step", "pic_sync", "pic_boosted_to_lab_diag",
            "pic_free", "pic_get_field", "pic_set_field", "pic_get_particles", "pic_get_stats",
            "pic_get_particles_y", "pic_last_error",
-           "pic_kernel_launches", "pic_kernel_timing", "pic_get_rho_noalloc", "pic_autotune",
+           "pic_kernel_launches", "pic_kernel_timing", "pic_get_rho_noalloc", "pic_push_counts", "pic_autotune",
            "pic_autotune_window",
            "pic_ensemble_create", "pic_ensemble_step", "pic_ensemble_sync", "pic_ensemble_size",
            "pic_ensemble_member", "pic_ensemble_free", "pic_ensemble_autotune",
@@ -171,6 +171,7 @@ def load(build_if_missing: bool = True):
         L.pic_kernel_launches.restype = ctypes.c_int64
         L.pic_kernel_timing.argtypes = [vp, ctypes.c_int, ctypes.c_int, _D, ctypes.POINTER(ctypes.c_int64)]
         L.pic_get_rho_noalloc.argtypes = [vp, _D]
+        L.pic_push_counts.argtypes = [vp, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
         L.pic_ensemble_create.argtypes = [ctypes.c_int, ctypes.POINTER(PicConfig), ctypes.POINTER(PicPlasma),
                                           ctypes.POINTER(PicLaser), ALLOC_FN, FREE_FN, vp, vp, ctypes.POINTER(vp)]
         L.pic_ensemble_step.argtypes = [vp, ctypes.c_int]

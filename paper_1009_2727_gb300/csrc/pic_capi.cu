@@ -1086,6 +1086,15 @@ struct Sim : SimBase {
     return PIC_OK;
   }
 
+  int push_counts(int64_t* pushed, int64_t* at_rest) {
+    Ctrl hc;
+    cudaMemcpyAsync(&hc, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream);
+    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return c->fail(PIC_ECUDA, "CUDA error in pic_push_counts");
+    *pushed = (int64_t)hc.n_pushed;
+    *at_rest = (int64_t)hc.n_rest;
+    return PIC_OK;
+  }
+
   int kernel_timing(int enable, int which, double* ms, int64_t* nl) {
     if (enable) {
       for (auto e : ev) cudaEventDestroy(e);
@@ -1491,6 +1500,13 @@ int pic_get_rho_noalloc(pic_ctx* c, double* dst_device) {
   if (c->s3) return c->fail(PIC_EINVAL, "pic_get_rho_noalloc: 2D contexts only");
   if (c->cfg.nz > PIC_NOALLOC_MAX_NZ) return c->fail(PIC_EINVAL, "pic_get_rho_noalloc: nz exceeds PIC_NOALLOC_MAX_NZ");
   return DISPATCH(c, get_rho_noalloc(dst_device));
+}
+
+int pic_push_counts(pic_ctx* c, int64_t* pushed, int64_t* at_rest) {
+  if (!c || !pushed || !at_rest) return PIC_EINVAL;
+  if (c->status != PIC_OK) return c->status;
+  if (c->s3) return PIC_EINVAL;
+  return DISPATCH(c, push_counts(pushed, at_rest));
 }
 
 int pic_beam_self_field(pic_ctx* c) {

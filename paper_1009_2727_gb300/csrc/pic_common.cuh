@@ -236,6 +236,8 @@ struct Ctrl {
   int n_defer;        // particles of this step's push left for the global-memory pass
   int n_ovf;          // chunks of this step's push left for the global-memory pass (window too large)
   int inj_done;       // blocks of the running injection that have finished
+  unsigned long long n_pushed;   // since the start: particle slots of the chunks pushed
+  unsigned long long n_rest;     // since the start: particle slots of the chunks at rest, whose boxes moved
   double red[8];      // reduction scratch
 };
 

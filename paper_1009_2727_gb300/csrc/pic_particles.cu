@@ -815,6 +815,7 @@ __device__ __forceinline__ void push_chunk(const GridP& g, const T* gE, const T*
       if constexpr (CellPos<T>::value) {
         if (!__syncthreads_or((field & 0x7fffffffu) != 0)) {
           if (chunk_at_rest<T>(p, ch, pc, chunks + c, s_bb)) {
+            if (threadIdx.x == 0) atomicAdd(&ctrl->n_rest, (unsigned long long)(ch.p1 - ch.p0));
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
             return;
@@ -898,6 +899,7 @@ __device__ __forceinline__ void push_chunk(const GridP& g, const T* gE, const T*
     }
     __syncthreads();
     if (threadIdx.x == 0) {
+      atomicAdd(&ctrl->n_pushed, (unsigned long long)(ch.p1 - ch.p0));
       Chunk o = ch;
       o.rest = 0;
       o.ix0 = s_bb[0]; o.ix1 = s_bb[1]; o.iz0 = s_bb[2]; o.iz1 = s_bb[3];

@@ -298,6 +298,12 @@ class Simulation:
     def launches(self) -> int:
         return int(self.L.pic_kernel_launches(self.h))
 
+    def push_counts(self) -> tuple:
+        """particle slots (pushed, at rest) of every push so far (2D; see pic_push_counts)"""
+        n = (ctypes.c_int64(0), ctypes.c_int64(0))
+        self._check(self.L.pic_push_counts(self.h, ctypes.byref(n[0]), ctypes.byref(n[1])), "pic_push_counts")
+        return int(n[0].value), int(n[1].value)
+
     def timing(self, enable: bool, which: int = 0):
         ms = ctypes.c_double(0.0)
         nl = ctypes.c_int64(0)
