@@ -337,6 +337,8 @@ int pic_kernel_timing(pic_ctx* ctx, int enable, int which, double* ms_total, int
  * trial that brings the GPU to its clocks) of contexts built from cfg, plasma and
  * laser (laser may be NULL) through
  * pic_init/pic_load_plasma/pic_inject_laser with the given allocator and stream.
+ * The trials push every chunk of particles, those at rest in a field-free window
+ * too, which a run's push leaves out: the layout is chosen for plasma in motion.
  * The result is cached per (nx, nz, ppc_x, ppc_z, shape order, precision,
  * gamma_boost, warm-up and timed steps) for the life of the process; a cached answer comes back without
  * timing and with cached = 1. out->struct_size must be set by the caller.
@@ -346,7 +348,7 @@ typedef struct pic_tune_result {
   uint32_t struct_size;
   uint32_t version;
   int32_t tile_x, tile_z, sort_every;   /* the chosen layout */
-  double ms_per_step;                   /* its time per step in the trials */
+  double ms_per_step;                   /* its time per step in the trials, with every chunk pushed */
   int32_t n_trials;
   int32_t trial_tile_x[PIC_TUNE_MAX_TRIALS];
   int32_t trial_tile_z[PIC_TUNE_MAX_TRIALS];

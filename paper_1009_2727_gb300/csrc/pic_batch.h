@@ -23,4 +23,8 @@ struct Batch {
 // beam, lab samples or moving window, created on the stream s.
 Batch* make_batch(pic_ctx* const* runs, int n, cudaStream_t s, std::string* why);
 
+// 2D contexts: push every chunk, those at rest in a field-free window too (for timing the push on a run's first steps, when
+// the pulse has not reached most of the plasma)
+void push_every_chunk(pic_ctx* ctx);
+
 }  // namespace picgb

@@ -152,6 +152,7 @@ struct Sim : SimBase {
   long long step = 0;
   long long shifts = 0;
   int64_t sorts = 0;
+  bool push_all = false;   // also push the chunks at rest (the autotuner's trials)
   double* stats_buf = nullptr;
   double* stage = nullptr;    // (nx+1)*(nz+1) doubles
   size_t stage_n = 0;
@@ -677,7 +678,7 @@ struct Sim : SimBase {
       frame_of(frame_shift(step + 1), fr1_sz, fr1_fz);
       launch_push<T>(g, f, P, chunks, ctrl, cf.shape_order, push_grid, smem_nodes, sb.tz, -kQe, kMe, c->hg.gamma,
                      c->hg.beta,
-                     fr1_sz, fr1_fz, (pairs && ions) ? 1 : 0, (int)mlo, nodal ? 1 : 0, pdef, ast,
+                     fr1_sz, fr1_fz, (pairs && ions) ? 1 : 0, (int)mlo, !push_all, nodal ? 1 : 0, pdef, ast,
                      ant_on ? ant_xs : nullptr, c->stream);
       tstop(0);
       c->launches += 2;
@@ -775,7 +776,7 @@ struct Sim : SimBase {
     int fr1_sz;
     float fr1_fz;
     frame_of(frame_shift(step + 1), fr1_sz, fr1_fz);
-    a.pc = push_const(g, -kQe, kMe, c->hg.gamma, fr1_sz, fr1_fz, (pairs && ions) ? 1 : 0, (int)mlo);
+    a.pc = push_const(g, -kQe, kMe, c->hg.gamma, fr1_sz, fr1_fz, (pairs && ions) ? 1 : 0, (int)mlo, !push_all);
     a.p = P;
     a.chunks = chunks;
     a.ctrl = ctrl;
@@ -1299,6 +1300,12 @@ struct BatchImpl : Batch {
 };
 
 }  // namespace
+
+void picgb::push_every_chunk(pic_ctx* c) {
+  if (c->s3) return;
+  if (c->cfg.precision == PIC_FP64) S<double>(c)->push_all = true;
+  else S<float>(c)->push_all = true;
+}
 
 Batch* picgb::make_batch(pic_ctx* const* runs, int n, cudaStream_t s, std::string* why) {
   if (n < 1 || !runs[0]->sim) {

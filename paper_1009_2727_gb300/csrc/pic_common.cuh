@@ -260,6 +260,7 @@ struct PushConst {
   // site (pairs; power-of-two particles per cell); ion rows below mlo have left
   // the particle domain; the stored id is (row << kb) | column
   int pairs, mlo;
+  int rest;   // a chunk of electrons at rest in a field-free window only moves its box (pairs, exact z keys)
   int kb, lpx, lpz, gx_lo, z0_cells;
 };
 
@@ -384,7 +385,8 @@ struct PushDefer {
 template <class T>
 void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* chunks, Ctrl* ctrl, int order,
                  int grid_blocks, int smem_nodes, int tile_z, double q, double m, double gamma_b, double beta_b,
-                 int fr1_sz, float fr1_fz, int pairs, int mlo, int nodal, const PushDefer& pd, const AntennaStep& ant,
+                 int fr1_sz, float fr1_fz, int pairs, int mlo, int rest, int nodal, const PushDefer& pd,
+                 const AntennaStep& ant,
                  const double* ant_xs, cudaStream_t s);
 
 struct SortBufs {
@@ -561,7 +563,7 @@ struct BatchGrid {
 // the push's constants for one step (q, m: charge and mass; fr1: frame shift at t^{n+1}; pairs, mlo: the
 // electron-ion pairs and the first live ion row)
 PushConst push_const(const GridP& g, double q, double m, double gamma_b, int fr1_sz, float fr1_fz, int pairs,
-                     int mlo);
+                     int mlo, int rest);
 // tile grid of the field kernels (tiles along z, along x) and their Faraday coefficients
 void field_tiles(const GridP& g, int& tiles_k, int& tiles_i);
 template <class T>

@@ -189,8 +189,10 @@ int pic_ensemble_autotune(int n, const pic_config* cfgs, const pic_plasma* plasm
     }
     pic_ens* e = nullptr;
     double ms = -1.0;
-    if (pic_ensemble_create(n, c.data(), plasmas, lasers, alloc, free_fn, alloc_user, cuda_stream, &e) == PIC_OK &&
-        pic_ensemble_step(e, 4) == PIC_OK && pic_ensemble_sync(e) == PIC_OK) {
+    const int made = pic_ensemble_create(n, c.data(), plasmas, lasers, alloc, free_fn, alloc_user, cuda_stream, &e);
+    if (made == PIC_OK)   // every chunk pushed, as in pic_autotune
+      for (pic_ctx* m : e->ctx) picgb::push_every_chunk(m);
+    if (made == PIC_OK && pic_ensemble_step(e, 4) == PIC_OK && pic_ensemble_sync(e) == PIC_OK) {
       cudaEventRecord(e0, st);
       const int rr = pic_ensemble_step(e, steps);
       cudaEventRecord(e1, st);

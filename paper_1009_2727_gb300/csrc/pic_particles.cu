@@ -697,7 +697,7 @@ __device__ __noinline__ void push_global_guarded(const T* gE, const T* gB, T* gJ
 template <class T>
 __device__ __forceinline__ bool chunk_at_rest(const Particles<T>& p, const Chunk& ch, const PushConst& pc, Chunk* out,
                                               int* s_bb) {
-  if (!pc.pairs || pc.lpz > 14) return false;
+  if (!pc.rest) return false;
   // keys relative to a stored cell below every cell of the chunk, so that they do not wrap
   const uint32_t zref = (uint32_t)((pc.fr0_sz + ch.iz0 - 1) & 0xffff) << 16;
   uint32_t lo = ch.zlo - zref, hi = ch.zhi - zref;
@@ -1398,7 +1398,7 @@ void launch_inject_batch(const StepArgs<T>* a, const BatchGrid& bg, cudaStream_t
 }
 
 PushConst push_const(const GridP& g, double q, double m, double gamma_b, int fr1_sz, float fr1_fz, int pairs,
-                     int mlo) {
+                     int mlo, int rest) {
   PushConst pc;
   pc.dx = g.dx; pc.dz = g.dz; pc.dt = g.dt; pc.z0 = g.z0;
   pc.idx = g.idx; pc.idz = g.idz;
@@ -1419,16 +1419,17 @@ PushConst push_const(const GridP& g, double q, double m, double gamma_b, int fr1
   pc.lpx = 0; pc.lpz = 0;
   while ((1 << pc.lpx) < g.il_ppcx) pc.lpx++;
   while ((1 << pc.lpz) < g.il_ppcz) pc.lpz++;
+  pc.rest = rest && pairs && pc.lpz <= 14;   // a site's offset in 16 bits
   return pc;
 }
 
 template <class T>
 void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* chunks, Ctrl* ctrl, int order,
                  int grid_blocks, int smem_nodes, int tile_z, double q, double m, double gamma_b, double beta_b,
-                 int fr1_sz, float fr1_fz, int pairs, int mlo, int nodal, const PushDefer& pd,
+                 int fr1_sz, float fr1_fz, int pairs, int mlo, int rest, int nodal, const PushDefer& pd,
                  const AntennaStep& ant, const double* ant_xs, cudaStream_t s) {
   (void)beta_b;
-  const PushConst pc = push_const(g, q, m, gamma_b, fr1_sz, fr1_fz, pairs, mlo);
+  const PushConst pc = push_const(g, q, m, gamma_b, fr1_sz, fr1_fz, pairs, mlo, rest);
   const size_t sm = (size_t)9 * smem_nodes * sizeof(T) + push_stage_bytes<T>();
   // 'momentum conserving' gather: the node-interpolated copies; else the Yee-located gather copies
   const T* gE = nodal ? f.nE[0] : f.fE[0];
@@ -1519,7 +1520,7 @@ void launch_inject(const GridP& g, Particles<T> p, Chunk* chunks, Ctrl* ctrl, co
 
 #define INST(T)                                                                                                 \
   template void launch_push<T>(const GridP&, const FieldPtrs<T>&, Particles<T>, Chunk*, Ctrl*, int, int, int,   \
-                               int, double, double, double, double, int, float, int, int, int, const PushDefer&, \
+                               int, double, double, double, double, int, float, int, int, int, int, const PushDefer&, \
                                const AntennaStep&, const double*, cudaStream_t);                                                                   \
   template void launch_sort<T>(const GridP&, Particles<T>, Particles<T>, SortBufs, Chunk*, Ctrl*, int, int, int,\
                                cudaStream_t);                                                                   \

@@ -1,7 +1,8 @@
 // Autotuner of the particle layout: the tile shape of the particle sort and the
 // sort cadence, timed on a window of steps of the run itself (by default its first
-// steps) and cached per run shape and window. Every trial is an ordinary context built through the public ABI, so a
-// tuned configuration is exactly what the caller then runs.
+// steps) and cached per run shape and window. Every trial is an ordinary context built through the public ABI, with
+// every chunk pushed: on the first steps nearly all plasma is at rest, where chunks only move their boxes, and a layout chosen
+// there is one for a push that has next to nothing to do (the run's costs grow with the pulse's way through the plasma).
 #include <cuda_runtime.h>
 
 #include <map>
@@ -9,6 +10,7 @@
 #include <tuple>
 
 #include "../../include/pic.h"
+#include "pic_batch.h"
 
 namespace {
 
@@ -36,6 +38,7 @@ double trial(const pic_config* cfg0, const pic_plasma* pl, const pic_laser* lase
   cfg.sort_every = sort_every;
   pic_ctx* ctx = nullptr;
   if (pic_init(&cfg, alloc, free_fn, user, stream, &ctx) != PIC_OK) return -1.0;
+  picgb::push_every_chunk(ctx);
   double ms = -1.0;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (pic_load_plasma(ctx, pl) == PIC_OK && (!laser || pic_inject_laser(ctx, laser) == PIC_OK) &&
