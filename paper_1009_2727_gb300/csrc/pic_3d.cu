@@ -2241,7 +2241,22 @@ struct Sim3 : Sim3Api {
       nF = dal<T>(6 * cs);
       if (!nF) return fail(PIC_ENOMEM, "allocation failed");
     }
-    fE = dal<T>(3 * cs); fB = dal<T>(3 * cs); tmp = dal<T>(ntmp * cs); tmp2 = dal<T>(cs);
+    tl.nt[0] = (g.n[0] + TX - 1) / TX;
+    tl.nt[1] = (g.n[1] + TY - 1) / TY;
+    tl.nt[2] = (g.n[2] + TZ - 1) / TZ;
+    ntiles = tl.nt[0] * tl.nt[1] * tl.nt[2];
+    nsum = (ntiles + SCB - 1) / SCB;
+    fE = dal<T>(3 * cs); fB = dal<T>(3 * cs);
+    tmp = dal<T>(ntmp * cs);
+    if (!tmp && ntmp > 1) {   // then a component at a time
+      cudaGetLastError();
+      ntmp = 1;
+      tmp = dal<T>(cs);
+    }
+    // the filter's second scratch also holds the sort's counts per cell: a filter is never under way in a sort
+    const size_t ncc = (size_t)ntiles * TC + nsum;
+    tmp2 = dal<T>(std::max(cs, (ncc * sizeof(int) + sizeof(T) - 1) / sizeof(T)));
+    tl.ccnt = reinterpret_cast<int*>(tmp2);
     Es = dal<T>(6 * cs); Bs = dal<T>(6 * cs);
     ctrl = dal<Ctrl3>(1);
     bacc = dal<double>(8);
@@ -2302,15 +2317,9 @@ struct Sim3 : Sim3Api {
       for (int q = 0; q < 3; q++) xy_ok = xy_ok && encode_xy_map<T>(&xy_map[q], base[q], g, taps.P);
       if (xy_ok) set_filter_xy_smem<T>();
     }
-    tl.nt[0] = (g.n[0] + TX - 1) / TX;
-    tl.nt[1] = (g.n[1] + TY - 1) / TY;
-    tl.nt[2] = (g.n[2] + TZ - 1) / TZ;
-    ntiles = tl.nt[0] * tl.nt[1] * tl.nt[2];
     tl.cnt = dal<int>(ntiles + 1);
     tl.start = dal<int>(ntiles + 1);
-    nsum = (ntiles + SCB - 1) / SCB;
-    tl.ccnt = dal<int>((size_t)ntiles * TC + nsum);
-    if (!tl.cnt || !tl.start || !tl.ccnt) return fail(PIC_ENOMEM, "allocation failed");
+    if (!tl.cnt || !tl.start) return fail(PIC_ENOMEM, "allocation failed");
     tl.bsum = tl.ccnt + (size_t)ntiles * TC;
     const auto set_smem = [](auto* few, auto* many) {
       cudaFuncSetAttribute(few, cudaFuncAttributeMaxDynamicSharedMemorySize, push3_smem<T, true>());

@@ -75,10 +75,28 @@ struct pic_ctx {
     void* p = nullptr;
     if (alloc) p = alloc(bytes, (void*)stream, user);
     else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
-    if (!p) return nullptr;
+    if (!p) {
+      cudaGetLastError();   // a refused allocation is the caller's to report
+      if (!spare) return nullptr;
+      drop_spare();
+      return dalloc(bytes);
+    }
     allocs.push_back({p, bytes});
     cudaMemsetAsync(p, 0, bytes, stream);
     return p;
+  }
+  // scratch that a step is faster with and can do without: given back when another allocation fails
+  void* spare = nullptr;
+  void drop_spare() {
+    cudaStreamSynchronize(stream);
+    for (size_t i = 0; i < allocs.size(); i++)
+      if (allocs[i].p == spare) {
+        if (freef) freef(allocs[i].p, allocs[i].n, (void*)stream, user);
+        else cudaFree(allocs[i].p);
+        allocs.erase(allocs.begin() + i);
+        break;
+      }
+    spare = nullptr;
   }
   void release_all() {
     for (auto& a : allocs) {
@@ -152,6 +170,7 @@ struct Sim : SimBase {
   long long step = 0;
   long long shifts = 0;
   int64_t sorts = 0;
+  bool wide = false, wide_tried = false;   // a filter for the wide kernels; their scratch has been asked for
   bool push_all = false;   // also push the chunks at rest (the autotuner's trials)
   double* stats_buf = nullptr;
   double* stage = nullptr;    // (nx+1)*(nz+1) doubles
@@ -205,11 +224,7 @@ struct Sim : SimBase {
     if (filt_gather) ok = ok && block(f.fE) && block(f.fB);
     nodal = cf.gather_scheme == 1;
     if (nodal) ok = ok && block(f.nE) && block(f.nB);
-    if ((filt_gather || filt_J) && filter_is_wide<T>(fs)) {
-      f.wide = al<T>(6 * N);
-      ok = ok && f.wide;
-      if (filt_J) ok = ok && block(f.Jf);
-    }
+    wide = (filt_gather || filt_J) && filter_is_wide<T>(fs, cf.nx);
     if (!ok) return c->fail(PIC_ENOMEM, "field allocation failed");
     if (cf.pml_cells > 0) {
       f.Byx = grid(); f.Byz = grid(); f.Eyx = grid(); f.Eyz = grid();
@@ -630,7 +645,22 @@ struct Sim : SimBase {
     }
   }
 
+  // The wide filters' scratch (nine node arrays, six without a filtered current), taken at the first step, after everything
+  // that a run cannot do without; where it is not to be had, the tile kernels filter. Runs of a batched ensemble, whose
+  // steps do not use it, never take it.
+  void wide_scratch() {
+    const size_t N = (size_t)g.cs;
+    if (!wide_tried) {
+      wide_tried = true;
+      c->spare = al<T>((filt_J ? 9 : 6) * N);
+    }
+    T* b = (T*)c->spare;
+    f.wide = b;
+    for (int q = 0; q < 3; q++) f.Jf[q] = b && filt_J ? b + (6 + q) * N : nullptr;
+  }
+
   int one_step() {
+    if (wide) wide_scratch();
     const pic_config& cf = c->cfg;
     const HostGeom& h = c->hg;
     const double tn = time_of(step), tn1 = time_of(step + 1);

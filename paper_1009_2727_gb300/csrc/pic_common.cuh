@@ -344,10 +344,10 @@ template <class T>
 bool launch_faraday_fused(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, double a2, double b2,
                           double theta, bool friedman, const FilterSpec& fs, bool filt_gather, const TileMaps& tm,
                           Ctrl* ctrl, cudaStream_t s);
-// a filter the tile kernels have no unrolled form for, with a halo of at least eight cells: it takes the two-pass
-// kernels, with f.wide (and f.Jf for the current) allocated
+// a filter the tile kernels have no unrolled form for, with a halo of at least eight cells, on a grid within the launch's
+// limits: it takes the two-pass kernels where f.wide (and f.Jf for the current) is had
 template <class T>
-bool filter_is_wide(const FilterSpec& fs);
+bool filter_is_wide(const FilterSpec& fs, int nx);
 template <class T>
 void launch_ampere(const GridP& g, const FieldPtrs<T>& f, const PmlTabs& pt, const FilterSpec& fs, bool filter_on,
                    const double* ion_x, const double* ion_c, double ion_coef, const TileMaps& tm, Ctrl* ctrl,

@@ -1430,9 +1430,9 @@ static void run_wide(const GridP& g, const WideTaps<T>& w, const WideJob<T>& job
 }
 
 template <class T>
-bool filter_is_wide(const FilterSpec& fs) {
+bool filter_is_wide(const FilterSpec& fs, int nx) {
   const FilterTaps<T> ft = make_taps<T>(fs);
-  return ft.H >= WMINH && filter_pt(ft) == 0;
+  return ft.H >= WMINH && filter_pt(ft) == 0 && (nx + WZB) / WZB <= 65535;   // k_wide_z's rows of blocks
 }
 
 template <class T>
@@ -1582,7 +1582,7 @@ size_t tile_smem_bytes(const TileMaps& tm, int H) { return tile_smem<T>(tm, H); 
 
 #define INSTF(T)                                                                                                 \
   template FarK<T> faraday_coefs<T>(double, double, double);                                                     \
-  template bool filter_is_wide<T>(const FilterSpec&);                                                            \
+  template bool filter_is_wide<T>(const FilterSpec&, int);                                                            \
   template FilterTaps<T> filter_taps<T>(const FilterSpec&);                                                      \
   template int filter_taps_class<T>(const FilterTaps<T>&);                                                       \
   template size_t tile_smem_bytes<T>(const TileMaps&, int);                                                      \
