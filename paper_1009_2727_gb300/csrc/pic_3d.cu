@@ -668,9 +668,11 @@ void launch_filter_xyz(const G3& g, const CUtensorMap& map03, const CUtensorMap&
                        int nc, const Taps3<T>& t, Ctrl3* ctrl, cudaStream_t s) {
   const int nb = (int)nblk(g.n[2] + 1, ZB), nz = (int)zs_blocks(g.n[2]);
   const dim3 grid(nb * nc, nblk(g.n[1] + 1, XYT), nblk(g.n[0] + 1, XYT));
-  if (nc > 1) launch_chained(k3_filter_xy<T, PT>, grid, dim3(256), filter_xy_smem<T, PT>(), s, g, map03, map35, tmp, c0, nb, t, ctrl);
-  else k3_filter_xy<T, PT><<<grid, 256, filter_xy_smem<T, PT>(), s>>>(g, map03, map35, tmp, c0, nb, t, ctrl);
-  launch_chained(k3_filter_zs<T, PT>, dim3(nz * nc, g.n[1] + 1, g.n[0] + 1), dim3(128), 0, s, g, tmp, F03, F35, c0, nz, t);
+  constexpr size_t sm = filter_xy_smem<T, PT>();
+  if (nc > 1) launch_chained(k3_filter_xy<T, PT>, grid, dim3(256), sm, s, g, map03, map35, tmp, c0, nb, t, ctrl);
+  else k3_filter_xy<T, PT><<<grid, 256, sm, s>>>(g, map03, map35, tmp, c0, nb, t, ctrl);
+  const dim3 zgrid(nz * nc, g.n[1] + 1, g.n[0] + 1);
+  launch_chained(k3_filter_zs<T, PT>, zgrid, dim3(128), 0, s, g, tmp, F03, F35, c0, nz, t);
 }
 
 template <class T>
@@ -2682,7 +2684,8 @@ struct Sim3 : Sim3Api {
     };
     if ((long)nblk(g.n[2] + 1, FZ) * nblk(g.n[1] + 1, FY) * nblk(g.n[0] + 1, 4) < nsm) faraday(k3_faraday_tile<T, 2>, 2);
     else faraday(k3_faraday_tile<T, 4>, 4);
-    launch_chained(k3_friedman<T>, dim3((unsigned)std::min<long>(nblk(n3 * sizeof(T) / 16, 256), 16L * nsm)), dim3(256), 0, s, n3, E, Ep, Eb, fE, T(1.0 - th / 2.0), T(th / 2.0));
+    const unsigned fblocks = (unsigned)std::min<long>(nblk(n3 * sizeof(T) / 16, 256), 16L * nsm);
+    launch_chained(k3_friedman<T>, dim3(fblocks), dim3(256), 0, s, n3, E, Ep, Eb, fE, T(1.0 - th / 2.0), T(th / 2.0));
     nl += 2;
     if (cfg.filter_gather && P > 0)
       filter3(fE, fB, 0, 6);

@@ -861,7 +861,6 @@ struct Sim : SimBase {
         a.inj_xblocks = inj_xblocks();
         a.cap = cap;
         a.chunk_cap = chunk_cap;
-        a.add_count = (int)add;
         a.add_chunks = a.inj_xblocks * rblocks;
         count_ub += add;
       }

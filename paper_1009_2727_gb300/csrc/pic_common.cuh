@@ -521,7 +521,7 @@ struct StepArgs {
   // plasma rows entering through the +z plane
   int inj_on, inj_xblocks;
   InjectP ip;
-  int cap, chunk_cap, add_count, add_chunks;
+  int cap, chunk_cap, add_chunks;
   // test beam (pushed after the plasma, before the antenna)
   int beam_on, beam_order;
   Beam<T> beam;

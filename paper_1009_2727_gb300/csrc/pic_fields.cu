@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(FT_Z* FT_TY, sizeof(T) == 4 ? 4 : 2) k_ampere(
 }
 
 // ---------------------------------------------------------------------------
-// Wide filters (halo above six cells, or strided): along x into a scratch block, then along z, one launch each for all
+// Wide filters (filter_is_wide: a halo of eight cells or more and no unrolled form): along x into a scratch block, then along z, one launch each for all
 // components. The tile kernels above stage a 16 x 64 tile with its halo on both axes; with the 35-cell halo of S(1:2:4)
 // that is 86 x 136 nodes read and 220 products per output, a third of which refill the halo. Here the halo is paid along
 // one axis at a time, each thread sums 16 outputs from a register window (128 products per eight inputs and 15 or 23
@@ -1122,8 +1122,8 @@ __global__ void __launch_bounds__(FT_Z* FT_TY) k_filter_fields_batch(const StepA
 }
 
 template <class T, bool FILT, int PT>
-__global__ void __launch_bounds__(FT_Z* FT_TY, sizeof(T) == 4 ? 4 : 2) k_ampere_batch(const StepArgs<T>* a, const int* off, int nruns,
-                                                                                  int* push_counter) {
+__global__ void __launch_bounds__(FT_Z* FT_TY, sizeof(T) == 4 ? 4 : 2)
+    k_ampere_batch(const StepArgs<T>* a, const int* off, int nruns, int* push_counter) {
   __shared__ int s_r;
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     if (blockIdx.x == 0) *push_counter = 0;
@@ -1241,8 +1241,8 @@ static void run_faraday_staged(dim3 grd, dim3 blk, cudaStream_t s, const GridP& 
   const size_t sm = (size_t)9 * ring_stride<T>() * sizeof(T) + 128;
   const int e = tm.Ebase[0] == (const void*)f.E[0] ? 0 : 1, b = tm.Ebbase[0] == (const void*)f.Eb[0] ? 0 : 1;
   cudaFuncSetAttribute(k_faraday_fused<T, true, CK, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  launch_chained(k_faraday_fused<T, true, CK, 0>, grd, blk, sm, s, g, f, pt, q, FilterTaps<T>{}, tm.Er[e], tm.Er[1 - e], tm.Eb[b],
-                                                        ctrl);
+  launch_chained(k_faraday_fused<T, true, CK, 0>, grd, blk, sm, s, g, f, pt, q, FilterTaps<T>{}, tm.Er[e], tm.Er[1 - e],
+                 tm.Eb[b], ctrl);
 }
 
 template <class T>

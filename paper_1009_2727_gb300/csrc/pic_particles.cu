@@ -910,9 +910,9 @@ __device__ __forceinline__ void push_chunk(const GridP& g, const T* gE, const T*
 }
 
 template <class T, int ORDER, bool MC>
-__global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push(GridP g, const T* gE, const T* gB, T* gJ, Particles<T> p,
-                                                     Chunk* chunks, Ctrl* ctrl, int cap_nodes, int tile_z,
-                                                     PushDefer pd, PushConst pc) {
+__global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
+    k_push(GridP g, const T* gE, const T* gB, T* gJ, Particles<T> p, Chunk* chunks, Ctrl* ctrl, int cap_nodes, int tile_z,
+           PushDefer pd, PushConst pc) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
   __shared__ int s_chunk;
@@ -933,9 +933,8 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push(GridP g, 
 
 // The global-memory pass after k_push: whole chunks whose window did not fit in shared memory (OVF_SLICES
 // blocks each), then single particles that were outside their chunk's box (one thread each); the blocks past nblk add
-// the antenna. Both add their
-// current with global atomics and widen their chunk's box atomically (k_push has written the box of the
-// particles it pushed; an overflow chunk's box starts empty).
+// the antenna. Both add their current with global atomics and widen their chunk's box atomically (k_push has written the
+// box of the particles it pushed; an overflow chunk's box starts empty).
 constexpr int OVF_SLICES = 8;
 template <class T, int ORDER, bool MC>
 __global__ void __launch_bounds__(PB_THREADS) k_push_deferred(GridP g, const T* gE, const T* gB, T* gJ,
@@ -1216,24 +1215,24 @@ __device__ __forceinline__ void inject_block(const GridP& g, const Particles<T>&
     if (ci >= chunk_cap || start + cnt > cap) {
       atomicOr(&ctrl->status, ST_OVERFLOW);
     } else {
-    Chunk c;
-    c.p0 = (int)start; c.p1 = (int)(start + cnt);
-    c.ix0 = g.gx_lo + cx0; c.ix1 = g.gx_lo + cx0 + ncx - 1;
-    const double za = ((ip.m_beg + r0 + 0.5) * ip.h - ip.beta * kC * ip.t - g.z0) * g.idz;
-    const double zb = ((ip.m_beg + r0 + nr - 1 + 0.5) * ip.h - ip.beta * kC * ip.t - g.z0) * g.idz;
-    c.iz0 = (int)floor(za); c.iz1 = (int)floor(zb);
-    c.rest = 0; c.zlo = c.zhi = 0;
-    if constexpr (CellPos<T>::value) {
-      // every electron starts at rest at its site
-      uint32_t cell;
-      float sox, soz;
-      lattice_site((int)(ip.m_beg + r0), 0, ip.ppc_x, ip.ppc_z, g.gx_lo, g.z0_cells, cell, sox, soz);
-      c.zlo = z_key(cell_z(cell), soz);
-      lattice_site((int)(ip.m_beg + r0 + nr - 1), 0, ip.ppc_x, ip.ppc_z, g.gx_lo, g.z0_cells, cell, sox, soz);
-      c.zhi = z_key(cell_z(cell), soz);
-      c.rest = 1;
-    }
-    chunks[ci] = c;
+      Chunk c;
+      c.p0 = (int)start; c.p1 = (int)(start + cnt);
+      c.ix0 = g.gx_lo + cx0; c.ix1 = g.gx_lo + cx0 + ncx - 1;
+      const double za = ((ip.m_beg + r0 + 0.5) * ip.h - ip.beta * kC * ip.t - g.z0) * g.idz;
+      const double zb = ((ip.m_beg + r0 + nr - 1 + 0.5) * ip.h - ip.beta * kC * ip.t - g.z0) * g.idz;
+      c.iz0 = (int)floor(za); c.iz1 = (int)floor(zb);
+      c.rest = 0; c.zlo = c.zhi = 0;
+      if constexpr (CellPos<T>::value) {
+        // every electron starts at rest at its site
+        uint32_t cell;
+        float sox, soz;
+        lattice_site((int)(ip.m_beg + r0), 0, ip.ppc_x, ip.ppc_z, g.gx_lo, g.z0_cells, cell, sox, soz);
+        c.zlo = z_key(cell_z(cell), soz);
+        lattice_site((int)(ip.m_beg + r0 + nr - 1), 0, ip.ppc_x, ip.ppc_z, g.gx_lo, g.z0_cells, cell, sox, soz);
+        c.zhi = z_key(cell_z(cell), soz);
+        c.rest = 1;
+      }
+      chunks[ci] = c;
     }
   }
   // the last of the injection's nblocks blocks to finish adds the counts (every block has read them by then)
@@ -1262,8 +1261,8 @@ constexpr int MAX_BATCH_RUNS = 512;
 // the window kernel over all runs' chunks: blocks take (run, chunk) pairs from one queue; the run's push
 // constants, geometry and particle arrays are copied to shared memory when a block changes run
 template <class T, int ORDER>
-__global__ void __launch_bounds__(PB_THREADS, push_blocks<T>()) k_push_batch(const StepArgs<T>* a, int nruns, int* counter,
-                                                           int cap_nodes, int tile_z) {
+__global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
+    k_push_batch(const StepArgs<T>* a, int nruns, int* counter, int cap_nodes, int tile_z) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
   __shared__ int s_pref[MAX_BATCH_RUNS + 1];
@@ -1436,16 +1435,20 @@ void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* c
   const T* gB = nodal ? f.nB[0] : f.fB[0];
   if (order == 3 && !nodal) {
     cudaFuncSetAttribute(k_push<T, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push<T, 3, false>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
+    launch_chained(k_push<T, 3, false>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes,
+                   tile_z, pd, pc);
   } else if (order == 3) {
     cudaFuncSetAttribute(k_push<T, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push<T, 3, true>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
+    launch_chained(k_push<T, 3, true>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes,
+                   tile_z, pd, pc);
   } else if (!nodal) {
     cudaFuncSetAttribute(k_push<T, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push<T, 1, false>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
+    launch_chained(k_push<T, 1, false>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes,
+                   tile_z, pd, pc);
   } else {
     cudaFuncSetAttribute(k_push<T, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push<T, 1, true>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd, pc);
+    launch_chained(k_push<T, 1, true>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes,
+                   tile_z, pd, pc);
   }
   // the global-memory pass over what the window kernel left (usually nothing: its blocks exit at once), and the antenna
   const int gb = grid_blocks < 304 ? grid_blocks : 304;
@@ -1521,7 +1524,7 @@ void launch_inject(const GridP& g, Particles<T> p, Chunk* chunks, Ctrl* ctrl, co
 #define INST(T)                                                                                                 \
   template void launch_push<T>(const GridP&, const FieldPtrs<T>&, Particles<T>, Chunk*, Ctrl*, int, int, int,   \
                                int, double, double, double, double, int, float, int, int, int, int, const PushDefer&, \
-                               const AntennaStep&, const double*, cudaStream_t);                                                                   \
+                               const AntennaStep&, const double*, cudaStream_t);                                \
   template void launch_sort<T>(const GridP&, Particles<T>, Particles<T>, SortBufs, Chunk*, Ctrl*, int, int, int,\
                                cudaStream_t);                                                                   \
   template void launch_inject<T>(const GridP&, Particles<T>, Chunk*, Ctrl*, const InjectP&, int, int, cudaStream_t); \

@@ -1,8 +1,10 @@
 // Autotuner of the particle layout: the tile shape of the particle sort and the
 // sort cadence, timed on a window of steps of the run itself (by default its first
-// steps) and cached per run shape and window. Every trial is an ordinary context built through the public ABI, with
-// every chunk pushed: on the first steps nearly all plasma is at rest, where chunks only move their boxes, and a layout chosen
-// there is one for a push that has next to nothing to do (the run's costs grow with the pulse's way through the plasma).
+// steps) and cached per run shape and window. Every trial is an ordinary context
+// built through the public ABI, with every chunk pushed: on the first steps nearly
+// all plasma is at rest, where chunks only move their boxes, and a layout chosen
+// there is one for a push that has next to nothing to do (the run's costs grow
+// with the pulse's way through the plasma).
 #include <cuda_runtime.h>
 
 #include <map>
