@@ -1376,17 +1376,15 @@ __global__ void k_inject_batch(const StepArgs<T>* a, const int* off, int nruns) 
 template <class T>
 void launch_push_batch(const StepArgs<T>* a, const BatchGrid& bg, int order, int grid_blocks, int smem_nodes,
                        int tile_z, cudaStream_t s) {
-  const size_t sm = (size_t)9 * smem_nodes * sizeof(T) + push_stage_bytes<T>();
+  const size_t sm = (size_t)9 * smem_nodes * sizeof(T) + push_stage_bytes<T>();   // (on idle SMs: see launch_push)
   const int gb = grid_blocks < 304 ? grid_blocks : 304;
   if (order == 3) {
     cudaFuncSetAttribute(k_push_batch<T, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push_batch<T, 3>, dim3(grid_blocks), dim3(PB_THREADS), sm, s, a, bg.nruns, bg.push_counter, smem_nodes,
-                   tile_z);
+    k_push_batch<T, 3><<<grid_blocks, PB_THREADS, sm, s>>>(a, bg.nruns, bg.push_counter, smem_nodes, tile_z);
     launch_chained(k_push_deferred_batch<T, 3>, dim3(gb), dim3(PB_THREADS), 0, s, a, bg.nruns);
   } else {
     cudaFuncSetAttribute(k_push_batch<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push_batch<T, 1>, dim3(grid_blocks), dim3(PB_THREADS), sm, s, a, bg.nruns, bg.push_counter, smem_nodes,
-                   tile_z);
+    k_push_batch<T, 1><<<grid_blocks, PB_THREADS, sm, s>>>(a, bg.nruns, bg.push_counter, smem_nodes, tile_z);
     launch_chained(k_push_deferred_batch<T, 1>, dim3(gb), dim3(PB_THREADS), 0, s, a, bg.nruns);
   }
 }
@@ -1430,25 +1428,30 @@ void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* c
   (void)beta_b;
   const PushConst pc = push_const(g, q, m, gamma_b, fr1_sz, fr1_fz, pairs, mlo, rest);
   const size_t sm = (size_t)9 * smem_nodes * sizeof(T) + push_stage_bytes<T>();
+  // k_push does not start while its predecessor ends: an SM's split between shared memory and L1 is set when a kernel
+  // finds it idle, and blocks that join the filter's (220 KB an SM) leave the push with its spills, and the second launch
+  // with its gathers from global memory, 28 KB of L1. Over 6000 steps of the 4096 x 256 stage (13.2 M electrons): 7.76 s
+  // so started, 5.94 s on an idle SM; a heated stage, where over a thousand chunks a step exceed the window, 4.5 ms a step
+  // and 2.7; the first steps 0.26 ms either way, small runs (256 x 64, FP64) the same.
   // 'momentum conserving' gather: the node-interpolated copies; else the Yee-located gather copies
   const T* gE = nodal ? f.nE[0] : f.fE[0];
   const T* gB = nodal ? f.nB[0] : f.fB[0];
   if (order == 3 && !nodal) {
     cudaFuncSetAttribute(k_push<T, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push<T, 3, false>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes,
-                   tile_z, pd, pc);
+    k_push<T, 3, false><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd,
+                                                          pc);
   } else if (order == 3) {
     cudaFuncSetAttribute(k_push<T, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push<T, 3, true>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes,
-                   tile_z, pd, pc);
+    k_push<T, 3, true><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd,
+                                                          pc);
   } else if (!nodal) {
     cudaFuncSetAttribute(k_push<T, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push<T, 1, false>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes,
-                   tile_z, pd, pc);
+    k_push<T, 1, false><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd,
+                                                          pc);
   } else {
     cudaFuncSetAttribute(k_push<T, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_chained(k_push<T, 1, true>, grid_blocks, PB_THREADS, sm, s, g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes,
-                   tile_z, pd, pc);
+    k_push<T, 1, true><<<grid_blocks, PB_THREADS, sm, s>>>(g, gE, gB, f.J[0], p, chunks, ctrl, smem_nodes, tile_z, pd,
+                                                          pc);
   }
   // the global-memory pass over what the window kernel left (usually nothing: its blocks exit at once), and the antenna
   const int gb = grid_blocks < 304 ? grid_blocks : 304;
