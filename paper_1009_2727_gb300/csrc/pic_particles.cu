@@ -1430,9 +1430,9 @@ void launch_push(const GridP& g, const FieldPtrs<T>& f, Particles<T> p, Chunk* c
   const size_t sm = (size_t)9 * smem_nodes * sizeof(T) + push_stage_bytes<T>();
   // k_push does not start while its predecessor ends: an SM's split between shared memory and L1 is set when a kernel
   // finds it idle, and blocks that join the filter's (220 KB an SM) leave the push with its spills, and the second launch
-  // with its gathers from global memory, 28 KB of L1. Over 6000 steps of the 4096 x 256 stage (13.2 M electrons): 7.76 s
-  // so started, 5.94 s on an idle SM; a heated stage, where over a thousand chunks a step exceed the window, 4.5 ms a step
-  // and 2.7; the first steps 0.26 ms either way, small runs (256 x 64, FP64) the same.
+  // with its gathers from global memory, 28 KB of L1. The first 4750 steps of the 4096 x 256 stage (13.2 M electrons):
+  // 3.28 s so started, 3.07 s on idle SMs; at step 4800, when it has heated up and hundreds of chunks a step exceed the
+  // window, 2.5 ms a step and 1.8; the first steps 0.26 ms either way, small runs (256 x 64, FP64) the same.
   // 'momentum conserving' gather: the node-interpolated copies; else the Yee-located gather copies
   const T* gE = nodal ? f.nE[0] : f.fE[0];
   const T* gB = nodal ? f.nB[0] : f.fB[0];

@@ -54,7 +54,7 @@ def test_waiting_kernel_takes_plain_pointers(k):
 
 def test_the_push_starts_on_idle_sms():
     """its shared memory and L1 are split when a kernel finds an SM idle: started beside the filter's blocks, the push and
-    its global-memory pass have a sixth of their L1 (a heated stage takes 4.5 ms a step instead of 2.7)"""
+    its global-memory pass have a sixth of their L1 (a heated stage takes 2.5 ms a step instead of 1.8)"""
     src = re.sub(r"//[^\n]*", "", open(os.path.join(SRC, "pic_particles.cu")).read())
     assert not re.search(r"launch_chained\(\s*k_push(_batch)?\s*<", src)
     assert re.search(r"k_push<T, 3, false>\s*<<<", src) and re.search(r"k_push_batch<T, 3>\s*<<<", src)
