@@ -207,11 +207,20 @@ __device__ __forceinline__ void faraday_tile3(const G3& g, const Pml3<T>& pm, co
   }
 }
 
-template <class T, int FX>
-__global__ void __launch_bounds__(256) k3_faraday_tile(G3 g, Pml3<T> pm, const T* E, const T* Ep, const T* Eb, T* B, T* Bs,
-                                                       T* fB, T c1, T c2, T c3, T ca, T cb, T cg, T dtT) {
-  if constexpr (FX < 4) chain_wait();   // (a few hundred cycles per block: not on a grid that fills the chip)
-  faraday_tile3<T, FX>(g, pm, E, Ep, Eb, B, Bs, fB, c1, c2, c3, ca, cb, cg, dtT);
+// on a grid that fills the chip, where the wait would cost a few hundred cycles per block: an ordinary launch, whose
+// read-only loads take 409 us at 1024 x 128 x 128 (437 without the qualifiers)
+template <class T>
+__global__ void __launch_bounds__(256) k3_faraday_tile(G3 g, Pml3<T> pm, const T* __restrict__ E,
+                                                       const T* __restrict__ Ep, const T* __restrict__ Eb,
+                                                       T* __restrict__ B, T* __restrict__ Bs, T* __restrict__ fB, T c1,
+                                                       T c2, T c3, T ca, T cb, T cg, T dtT) {
+  faraday_tile3<T, 4>(g, pm, E, Ep, Eb, B, Bs, fB, c1, c2, c3, ca, cb, cg, dtT);
+}
+template <class T>
+__global__ void __launch_bounds__(256) k3_faraday_few(G3 g, Pml3<T> pm, const T* E, const T* Ep, const T* Eb, T* B, T* Bs,
+                                                      T* fB, T c1, T c2, T c3, T ca, T cb, T cg, T dtT) {
+  chain_wait();
+  faraday_tile3<T, 2>(g, pm, E, Ep, Eb, B, Bs, fB, c1, c2, c3, ca, cb, cg, dtT);
 }
 
 // Friedman history (PR-1): E-bar <- (1 - theta/2) E + (theta/2) E-bar, E^{n-1} <- E, gather copy <- E
@@ -2682,8 +2691,8 @@ struct Sim3 : Sim3Api {
       if (fx < 4) launch_chained(kernel, grid, block, 0, s, g, pm, E, Ep, Eb, B, Bs, fB, c1, c2, c3, ca, cb, cg, T(g.dt));
       else kernel<<<grid, block, 0, s>>>(g, pm, E, Ep, Eb, B, Bs, fB, c1, c2, c3, ca, cb, cg, T(g.dt));
     };
-    if ((long)nblk(g.n[2] + 1, FZ) * nblk(g.n[1] + 1, FY) * nblk(g.n[0] + 1, 4) < nsm) faraday(k3_faraday_tile<T, 2>, 2);
-    else faraday(k3_faraday_tile<T, 4>, 4);
+    if ((long)nblk(g.n[2] + 1, FZ) * nblk(g.n[1] + 1, FY) * nblk(g.n[0] + 1, 4) < nsm) faraday(k3_faraday_few<T>, 2);
+    else faraday(k3_faraday_tile<T>, 4);
     const unsigned fblocks = (unsigned)std::min<long>(nblk(n3 * sizeof(T) / 16, 256), 16L * nsm);
     launch_chained(k3_friedman<T>, dim3(fblocks), dim3(256), 0, s, n3, E, Ep, Eb, fE, T(1.0 - th / 2.0), T(th / 2.0));
     nl += 2;

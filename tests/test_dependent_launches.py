@@ -42,7 +42,7 @@ WAITING = [k for k in kernels() if WAIT.search(k[3])]
 
 def test_the_waiting_kernels_are_found():
     names = {k[1] for k in WAITING}
-    assert {"k1_push", "k3_ampere", "k3_faraday_tile", "k3_filter_zs", "k_push", "k_sb_fwd"} <= names and len(names) > 25
+    assert {"k1_push", "k3_ampere", "k3_faraday_few", "k3_filter_zs", "k_push", "k_sb_fwd"} <= names and len(names) > 25
 
 
 @pytest.mark.parametrize("k", WAITING, ids=lambda k: f"{k[0]}-{k[1]}")
