@@ -221,9 +221,11 @@ class Simulation:
         t = self.torch.empty(self.shape, dtype=self.torch.float64, device=self.device)
         # the library writes after the default stream's work: on another current stream the tensor may be memory that work
         # queued there still uses
-        cur, dflt = self.torch.cuda.current_stream(self.device), self.torch.cuda.default_stream(self.device)
-        if cur != dflt and cur != self.stream:
-            dflt.wait_stream(cur)
+        # (the handle alone, 0 for the default stream: stream objects cost 2 us each)
+        if self.torch._C._cuda_getCurrentRawStream(self.device.index):
+            cur = self.torch.cuda.current_stream(self.device)
+            if cur != self.stream:
+                self.torch.cuda.default_stream(self.device).wait_stream(cur)
         ptr = ctypes.cast(ctypes.c_void_p(t.data_ptr()), _D)
         self._check(self.L.pic_get_field(self.h, comp, ptr, 1), "pic_get_field")
         return t
