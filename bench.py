@@ -509,7 +509,6 @@ def run_1d(args):
     sampler.start()
     torch.cuda.synchronize()
     l0 = sim.launches()
-    counts0 = None if three else sim.push_counts()
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
     ev0.record(stream)
@@ -518,7 +517,6 @@ def run_1d(args):
     torch.cuda.synchronize()
     clocks = sampler.stop()
     launches = sim.launches() - l0
-    counts1 = None if three else sim.push_counts()
     ms = ev0.elapsed_time(ev1)
     push_ms, push_n = sim.timing(False)
     n1 = sim.stats()["n_electrons"]

@@ -28,3 +28,22 @@ def test_traffic_only_where_it_was_measured():
 def test_instruction_constants_are_of_pushed_particles():
     # a particle's gather, push and deposit are hundreds of operations; an average over resting ones was 42.7
     assert bench.PUSH_WARP_INST_PER_PARTICLE > 15 and bench.PUSH_FLOPS_PER_PARTICLE > 150
+
+
+def test_every_name_is_defined():
+    """the bench's modes mostly run on a GPU only: no function may read a global that the module has not"""
+    import builtins
+    import dis
+    import types
+
+    def functions(code):
+        yield code
+        for c in code.co_consts:
+            if isinstance(c, types.CodeType):
+                yield from functions(c)
+
+    code = compile(open(bench.__file__).read(), "bench.py", "exec")
+    missing = {(f.co_name, i.argval) for f in functions(code) for i in dis.get_instructions(f)
+               if i.opname in ("LOAD_GLOBAL", "LOAD_NAME") and f is not code
+               and not hasattr(bench, i.argval) and not hasattr(builtins, i.argval)}
+    assert not {m for m in missing if not m[1].startswith("__")}, missing
