@@ -332,7 +332,7 @@ int pic_kernel_timing(pic_ctx* ctx, int enable, int which, double* ms_total, int
 /* ---- Autotuner of the particle layout (no counterpart in the paper) ----
  * Picks the particle tile (tile_x, tile_z) from {8, 16, 32}^2 at a cadence of 32,
  * then the sort cadence from {8, 16, 32, 64, 128} for that tile, by timing `steps`
- * steps (after 4 warm-up steps; a cadence trial runs at least two sort periods;
+ * steps (after 4 warm-up steps; the cadence trials run at least 256;
  * each tile is timed twice and the faster time is recorded, after one untimed
  * trial that brings the GPU to its clocks) of contexts built from cfg, plasma and
  * laser (laser may be NULL) through
@@ -348,7 +348,7 @@ typedef struct pic_tune_result {
   uint32_t struct_size;
   uint32_t version;
   int32_t tile_x, tile_z, sort_every;   /* the chosen layout */
-  double ms_per_step;                   /* its time per step in the trials, with every chunk pushed */
+  double ms_per_step;                   /* its time per step in the trials */
   int32_t n_trials;
   int32_t trial_tile_x[PIC_TUNE_MAX_TRIALS];
   int32_t trial_tile_z[PIC_TUNE_MAX_TRIALS];
@@ -360,10 +360,11 @@ typedef struct pic_tune_result {
 int pic_autotune(const pic_config* cfg, const pic_plasma* plasma, const pic_laser* laser, int steps,
                  pic_alloc_fn alloc, pic_free_fn free_fn, void* alloc_user, void* cuda_stream,
                  pic_tune_result* out);
-/* The same with the window of the run that the trials time: `warm` untimed steps (instead of 4), then
- * `steps` timed steps; a layout that is best while the plasma is still cold need not be best once the
- * laser has reached it, so a caller that times a later window tunes on that window. The cache key
- * includes warm and steps. Errors as pic_autotune (warm < 0: PIC_EINVAL). */
+/* The same on a window of the run itself: `warm` untimed steps (instead of 4), then `steps` timed steps,
+ * with chunks at rest left out of the push as the run leaves them out; a layout that is best while the
+ * plasma is still cold need not be best once the laser has reached it, so a caller that times a later
+ * window tunes on that window. The cache key includes the window, the laser, the plasma and the
+ * configuration but for tiles and cadence. Errors as pic_autotune (warm < 0: PIC_EINVAL). */
 int pic_autotune_window(const pic_config* cfg, const pic_plasma* plasma, const pic_laser* laser, int warm,
                         int steps, pic_alloc_fn alloc, pic_free_fn free_fn, void* alloc_user, void* cuda_stream,
                         pic_tune_result* out);

@@ -125,8 +125,9 @@ def torch_allocator(device_index: int):
 
 
 def autotune(w: dict, steps: int = 16, precision: str | None = None, stream=None, warm: int = 4) -> dict:
-    """Tile shape and sort cadence for this workload, timed on `steps` steps after `warm` untimed ones
-    (pic_autotune_window; the result is cached per run shape and window inside the library)."""
+    """Tile shape and sort cadence for this workload, timed on `steps` steps after `warm` untimed ones: with warm = 4 with
+    every chunk pushed (pic_autotune), else on the run's own steps of that window (pic_autotune_window). The result is
+    cached inside the library."""
     import torch
     L = capi.load()
     prec = precision or w.get("precision", "fp64")
@@ -138,9 +139,9 @@ def autotune(w: dict, steps: int = 16, precision: str | None = None, stream=None
     acb, fcb = torch_allocator(torch.cuda.current_device())
     out = capi.PicTuneResult()
     out.struct_size = ctypes.sizeof(capi.PicTuneResult)
-    r = L.pic_autotune_window(ctypes.byref(c), ctypes.byref(pl), ctypes.byref(la) if la is not None else None,
-                              int(warm), int(steps), acb, fcb, None, ctypes.c_void_p(st.cuda_stream),
-                              ctypes.byref(out))
+    args = (ctypes.byref(c), ctypes.byref(pl), ctypes.byref(la) if la is not None else None)
+    rest = (int(steps), acb, fcb, None, ctypes.c_void_p(st.cuda_stream), ctypes.byref(out))
+    r = L.pic_autotune(*args, *rest) if int(warm) == 4 else L.pic_autotune_window(*args, int(warm), *rest)
     if r != 0:
         raise PicError(f"pic_autotune failed: {capi.STATUS_NAMES.get(r, r)}")
     n = out.n_trials

@@ -1,6 +1,7 @@
 """The autotuner's trials push every chunk: on a stage that no pulse has reached yet, where a run's push only moves boxes,
 their time per step is that of a push that works (on this box of 3.3 million electrons the push is most of it), while the
-tuned run itself still leaves its resting chunks out."""
+tuned run itself still leaves its resting chunks out. On a window that the caller names, the trials are the run's own steps,
+and a layout found without a pulse is not handed to a run with one."""
 import numpy as np
 import pytest
 
@@ -45,3 +46,16 @@ def test_ensemble():
     tuned = ens.tuned[0]["ms_per_step"]
     ens.close()
     assert rest > pushed and tuned > 1.4 * own, (tuned, own)
+
+
+def test_window_of_the_run():
+    from paper_1009_2727_gb300.pic import Simulation, autotune
+    w = dark(1024)
+    t = autotune(w, warm=8, steps=16)
+    sim = Simulation(w, tile=t["tile"], sort_every=t["sort_every"])
+    own = min(ms_per_step(sim) for _ in range(3))
+    sim.close()
+    assert not t["cached"] and t["ms_per_step"] < 1.4 * own, (t["ms_per_step"], own)
+    assert autotune(w, warm=8, steps=16)["cached"]
+    lit = dict(w, laser=W.shrink(W.stage_2d(), 256, 1024)["laser"])
+    assert not autotune(lit, warm=8, steps=16)["cached"]
