@@ -753,7 +753,8 @@ __device__ __forceinline__ bool chunk_at_rest(const Particles<T>& p, const Chunk
 
 // One chunk of the window kernel: stage the six gather fields of the chunk's box (+ halo) in shared memory,
 // push its particles (gather, Boris, move, Esirkepov into a shared current window), add the window to J once,
-// and store the box of the particles' new cells. Called by every thread of the block; s_bb is shared.
+// and store the box of the particles' new cells. Called by every thread of the block; s_bb is shared: the box and key
+// minima and maxima, then (thread 0) the particle slots of the chunks pushed and at rest.
 template <class T, int ORDER, bool MC>
 __device__ __forceinline__ void push_chunk(const GridP& g, const T* gE, const T* gB, T* gJ, const Particles<T>& p,
                                            Chunk* chunks, Ctrl* ctrl, int cap_nodes, int tile_z,
@@ -815,7 +816,7 @@ __device__ __forceinline__ void push_chunk(const GridP& g, const T* gE, const T*
       if constexpr (CellPos<T>::value) {
         if (!__syncthreads_or((field & 0x7fffffffu) != 0)) {
           if (chunk_at_rest<T>(p, ch, pc, chunks + c, s_bb)) {
-            if (threadIdx.x == 0) atomicAdd(&ctrl->n_rest, (unsigned long long)(ch.p1 - ch.p0));
+            if (threadIdx.x == 0) s_bb[7] += ch.p1 - ch.p0;
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
             return;
@@ -899,7 +900,7 @@ __device__ __forceinline__ void push_chunk(const GridP& g, const T* gE, const T*
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      atomicAdd(&ctrl->n_pushed, (unsigned long long)(ch.p1 - ch.p0));
+      s_bb[6] += ch.p1 - ch.p0;
       Chunk o = ch;
       o.rest = 0;
       o.ix0 = s_bb[0]; o.ix1 = s_bb[1]; o.iz0 = s_bb[2]; o.iz1 = s_bb[3];
@@ -909,6 +910,13 @@ __device__ __forceinline__ void push_chunk(const GridP& g, const T* gE, const T*
   }
 }
 
+// a block's counts added to its run's, once: the queue's counter, which every chunk adds to, lies in the same cache line
+__device__ __forceinline__ void add_push_counts(Ctrl* ctrl, int* s_bb) {
+  if (s_bb[6]) atomicAdd(&ctrl->n_pushed, (unsigned long long)s_bb[6]);
+  if (s_bb[7]) atomicAdd(&ctrl->n_rest, (unsigned long long)s_bb[7]);
+  s_bb[6] = s_bb[7] = 0;
+}
+
 template <class T, int ORDER, bool MC>
 __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
     k_push(GridP g, const T* gE, const T* gB, T* gJ, Particles<T> p, Chunk* chunks, Ctrl* ctrl, int cap_nodes, int tile_z,
@@ -916,8 +924,9 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
   __shared__ int s_chunk;
-  __shared__ int s_bb[6];
+  __shared__ int s_bb[8];
   chain_wait();
+  if (threadIdx.x == 0) s_bb[6] = s_bb[7] = 0;
   const int nchunks = ctrl->nchunks;
   while (true) {
     if (threadIdx.x == 0) {
@@ -929,6 +938,7 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
     if (c >= nchunks) break;
     push_chunk<T, ORDER, MC>(g, gE, gB, gJ, p, chunks, ctrl, cap_nodes, tile_z, pd, pc, c, sm, s_bb);
   }
+  if (threadIdx.x == 0) add_push_counts(ctrl, s_bb);
 }
 
 // The global-memory pass after k_push: whole chunks whose window did not fit in shared memory (OVF_SLICES
@@ -1266,7 +1276,7 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
   __shared__ int s_pref[MAX_BATCH_RUNS + 1];
-  __shared__ int s_w, s_r, s_bb[6];
+  __shared__ int s_w, s_r, s_bb[8];
   __shared__ PushConst s_pc;
   __shared__ GridP s_g;
   __shared__ Particles<T> s_p;
@@ -1283,6 +1293,7 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
   __syncthreads();
   const int total = s_pref[nruns];
   int cur = -1;
+  if (threadIdx.x == 0) s_bb[6] = s_bb[7] = 0;
   while (true) {
     if (threadIdx.x == 0) {
       const int w = atomicAdd(counter, 1);
@@ -1303,6 +1314,7 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
     if (w >= total) break;
     const int r = s_r;
     if (r != cur) {
+      if (threadIdx.x == 0 && cur >= 0) add_push_counts(a[cur].ctrl, s_bb);
       to_shared(&s_pc, &a[r].pc);
       to_shared(&s_g, &a[r].g);
       to_shared(&s_p, &a[r].p);
@@ -1313,6 +1325,7 @@ __global__ void __launch_bounds__(PB_THREADS, push_blocks<T>())
     push_chunk<T, ORDER, false>(s_g, A.f.fE[0], A.f.fB[0], A.f.J[0], s_p, A.chunks, A.ctrl, cap_nodes, tile_z, A.pd,
                                 s_pc, w - s_pref[r], sm, s_bb);
   }
+  if (threadIdx.x == 0 && cur >= 0) add_push_counts(a[cur].ctrl, s_bb);
 }
 
 // the global-memory pass of every run (usually nothing to do)
