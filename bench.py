@@ -42,25 +42,24 @@ BYTES_PER_PARTICLE_3D = {"mixed": 76, "fp64": 104}
 BYTES_PER_CELL = {"mixed": 168, "fp64": 336}
 # DRAM bytes (read + write) per particle of a push launch in which every particle is pushed (k_push, mixed precision, cubic
 # shapes, the Yee-located gather), for every layout the autotuner can return, keyed by (tile_x, tile_z, sort_every): ncu
-# dram__bytes_read.sum + dram__bytes_write.sum on the 2048 x 256 stage box, measured when chunks at rest were still pushed
-# (the 2nd and 3rd push of each layout; --layout-sweep pushes every chunk). Below the 56 bytes of stored state: the last
-# writes of a launch are still in the 129 MB L2 when it ends.
+# dram__bytes_read.sum + dram__bytes_write.sum on the 2048 x 256 stage box, the 2nd and 3rd push of each layout of
+# --layout-sweep. Below the 56 bytes of stored state: the last writes of a launch are still in the 129 MB L2 when it ends.
 TRAFFIC_BYTES_PER_PARTICLE = {
-    (8, 8, 8): 49.71, (8, 8, 16): 49.61, (8, 8, 32): 49.58, (8, 8, 64): 49.49, (8, 8, 128): 49.62, (8, 16, 8): 49.58,
-    (8, 16, 16): 49.63, (8, 16, 32): 49.61, (8, 16, 64): 49.49, (8, 16, 128): 49.63, (8, 32, 8): 49.83,
-    (8, 32, 16): 49.81, (8, 32, 32): 49.78, (8, 32, 64): 49.71, (8, 32, 128): 49.74, (16, 8, 8): 49.64,
-    (16, 8, 16): 49.6, (16, 8, 32): 49.74, (16, 8, 64): 49.58, (16, 8, 128): 49.72, (16, 16, 8): 49.79,
-    (16, 16, 16): 49.73, (16, 16, 32): 49.78, (16, 16, 64): 49.69, (16, 16, 128): 49.68, (16, 32, 8): 49.07,
-    (16, 32, 16): 49.13, (16, 32, 32): 49.08, (16, 32, 64): 48.96, (16, 32, 128): 49.09, (32, 8, 8): 49.53,
-    (32, 8, 16): 49.53, (32, 8, 32): 49.54, (32, 8, 64): 49.52, (32, 8, 128): 49.47, (32, 16, 8): 49.05,
-    (32, 16, 16): 49.3, (32, 16, 32): 49.07, (32, 16, 64): 49.05, (32, 16, 128): 49.2, (32, 32, 8): 48.87,
-    (32, 32, 16): 48.85, (32, 32, 32): 48.84, (32, 32, 64): 48.94, (32, 32, 128): 48.95,
+    (8, 8, 8): 51.07, (8, 8, 16): 51.2, (8, 8, 32): 51.12, (8, 8, 64): 51.14, (8, 8, 128): 51.08, (8, 16, 8): 51.02,
+    (8, 16, 16): 50.75, (8, 16, 32): 50.96, (8, 16, 64): 50.78, (8, 16, 128): 50.72, (8, 32, 8): 50.52,
+    (8, 32, 16): 50.69, (8, 32, 32): 50.66, (8, 32, 64): 50.76, (8, 32, 128): 50.74, (16, 8, 8): 50.91,
+    (16, 8, 16): 50.7, (16, 8, 32): 50.85, (16, 8, 64): 50.9, (16, 8, 128): 50.94, (16, 16, 8): 51.13,
+    (16, 16, 16): 51.06, (16, 16, 32): 51.26, (16, 16, 64): 51.14, (16, 16, 128): 51.21, (16, 32, 8): 50.24,
+    (16, 32, 16): 50.29, (16, 32, 32): 50.12, (16, 32, 64): 50.4, (16, 32, 128): 50.43, (32, 8, 8): 50.34,
+    (32, 8, 16): 50.46, (32, 8, 32): 50.71, (32, 8, 64): 50.4, (32, 8, 128): 50.32, (32, 16, 8): 49.83,
+    (32, 16, 16): 49.77, (32, 16, 32): 49.77, (32, 16, 64): 49.75, (32, 16, 128): 49.93, (32, 32, 8): 49.94,
+    (32, 32, 16): 50.11, (32, 32, 32): 50, (32, 32, 64): 50.09, (32, 32, 128): 50.03,
 }
 # Warp instructions and FP32 operations that a pushed particle takes at least (mixed precision, cubic shapes, the Yee-located
 # gather): ncu smsp__inst_executed.sum and smsp__sass_thread_inst_executed_op_{fadd,fmul,ffma}_pred_on.sum of pushes of plasma
 # at rest with every chunk pushed, where most terms of the deposit are zero and skipped (2048 x 256 stage box, 8 x 16-cell
 # tiles, sort every 64; counted as FADD + FMUL + 2 FFMA, without the packed two-lane FMAs of the gather). With no term zero
-# (--push-all, steps 104-106) it is 39.7 and 351. The staging of windows for chunks at rest comes on top.
+# (--push-all, steps 104-106) it is 39.9 and 353. The staging of windows for chunks at rest comes on top.
 PUSH_WARP_INST_PER_PARTICLE = 21.0
 PUSH_FLOPS_PER_PARTICLE = 174.0
 # 3D: ncu dram bytes of k3_push_tiles on the 256 x 128 x 128 box (195.3 MB for 2,356,608 electrons), scaled
@@ -1003,12 +1002,12 @@ def main():
         alu_ach = PUSH_FLOPS_PER_PARTICLE * pushed / (push_avg_ms * 1e-3) / 1e12
         roof["issue"] = {"achieved": issue_ach, "peak": issue_peak, "unit": "warp-instructions/s",
                          "frac": issue_ach / issue_peak, "warp_instructions_per_pushed_particle": PUSH_WARP_INST_PER_PARTICLE,
-                         "note": "at least: a moving particle takes up to 39.7, staging windows at rest comes on top",
+                         "note": "at least: a moving particle takes up to 39.9, staging windows at rest comes on top",
                          "peak_source": f"4 per SM per cycle x {nsm} SMs x {mhz:g} MHz (sampled)"}
         roof["alu"] = {"achieved": alu_ach, "peak": fp32_peak, "unit": "TFLOP/s",
                        "frac": alu_ach / fp32_peak if fp32_peak else None,
                        "flops_per_pushed_particle": PUSH_FLOPS_PER_PARTICLE,
-                       "note": "at least: a moving particle takes up to 351",
+                       "note": "at least: a moving particle takes up to 353",
                        "peak_source": "pic_measure_fp32_peak (FMA microbenchmark, measured in this run)"}
     sim.close()
     del sim
