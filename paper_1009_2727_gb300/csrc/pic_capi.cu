@@ -650,7 +650,9 @@ struct Sim : SimBase {
   // steps do not use it, never take it.
   void wide_scratch() {
     const size_t N = (size_t)g.cs;
-    if (!wide_tried) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    // (a stream under capture cannot allocate: that step takes the tile kernels)
+    if (!wide_tried && cudaStreamIsCapturing(c->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
       wide_tried = true;
       c->spare = al<T>((filt_J ? 9 : 6) * N);
     }
